@@ -58,7 +58,6 @@ void fill_geometry(FilmDesc& d, int Lx, int Ly, int Lz, int y_mode, int x_mode, 
   d.n = (uint32_t)Lz / 2;
   d.W = (d.n + 31) / 32;
   d.Wp = d.W;  // rows contiguous: no padding words
-  d.nq = (d.Wp + 3) / 4;
   const uint32_t r = d.n - 32 * (d.W - 1);  // valid sites of the last word, 1..32
   uint32_t mask = 0;
   for (uint32_t l = 0; l < r; l++) mask |= 1u << bitpos(l);
@@ -72,7 +71,6 @@ void fill_geometry(FilmDesc& d, int Lx, int Ly, int Lz, int y_mode, int x_mode, 
     d.rk0[k] = d.key0 + k * kWeyl0;
     d.rk1[k] = d.key1 + k * kWeyl1;
   }
-  d.upd_items = d.Lx * (d.Ly - 1) * d.W;
   d.meas_bpl = std::max<uint32_t>(1, (d.Ly * d.W + kMeasureItemsPerBlock - 1) / kMeasureItemsPerBlock);
   d.meas_lpu = 1;
   if (2 * d.Ly * d.W <= kMeasureItemsPerBlock)
@@ -80,57 +78,65 @@ void fill_geometry(FilmDesc& d, int Lx, int Ly, int Lz, int y_mode, int x_mode, 
   d.active = 1;
   d.sweep_end = 0xFFFFFFFFu;
   fastdiv_magic(d.W, &d.divw_m, &d.divw_l);
-  fastdiv_magic(d.Ly > 2 ? d.Ly - 2 : 1, &d.divy_m, &d.divy_l);  // rows ky = 2 .. Ly-1 of a layer
-  // thin films: the one-word grid kernels update 4 (at most 8 sites per
-  // array) or 2 (at most 16) rows per packed word; the first and the last
-  // group of a layer must differ.  Two rows pay only on films of at least
-  // kPack2Rows rows: packing halves a film's threads and doubles each one's
-  // chain of Philox calls, which a small film's few waves cannot hide
-  // (measured on GB300: the beta-integration set's films of 1200-3000 rows
-  // lose 6%, the line-tension set's of 13824 rows gain)
-  d.pack = 1;
-  if (d.W == 1 && d.n <= 8 && d.Ly % 4 == 0 && d.Ly >= 8) d.pack = 4;
-  else if (d.W == 1 && d.n <= 16 && d.Ly % 2 == 0 && d.Ly >= 4 && d.Lx * d.Ly >= kPack2Rows) d.pack = 2;
+  // thin films: a word of the grid kernels holds 4 (at most 8 sites per array)
+  // or 2 (at most 16) rows; the first and the last group of a layer must
+  // differ.  Two rows pay only on films of at least kPack2Rows rows: packing
+  // halves a film's threads and doubles each one's chain of Philox calls,
+  // which a small film's few waves cannot hide (measured on GB300: the
+  // beta-integration set's films of 1200-3000 rows lose 6%, the line-tension
+  // set's of 13824 rows gain).  On the slab path films pack whenever they can
+  // (slab_rows decides).
+  d.sl_pack = 1;
+  if (d.W == 1 && d.n <= 8 && d.Ly % 4 == 0 && d.Ly >= 8) d.sl_pack = 4;
+  else if (d.W == 1 && d.n <= 16 && d.Ly % 2 == 0 && d.Ly >= 4) d.sl_pack = 2;
+  d.pack = (d.sl_pack == 2 && d.Lx * d.Ly < kPack2Rows) ? 1 : d.sl_pack;
   const uint32_t groups = d.Ly / d.pack;
-  d.pk_items = d.Lx * (groups - 1);
-  fastdiv_magic(groups > 2 ? groups - 2 : 1, &d.pk_divm, &d.pk_divl);
+  for (uint32_t i = 0; i < 3; i++) {
+    const uint32_t len = column_len(i);
+    d.cols[i] = (groups - 2 + len - 1) / len;
+    fastdiv_magic(std::max<uint32_t>(d.cols[i], 1), &d.divc_m[i], &d.divc_l[i]);
+  }
 }
 
 void build_tables(FilmDesc& d, double J, double H, double H1, double T) {
-  const int Lx = (int)d.Lx;
-  d.has_never = 0;
   for (int cls = 0; cls < 4; cls++) {
-    bool present = false;  // does some layer kx have this class?
-    for (int kx = 1; kx <= Lx && !present; kx = (kx == 1 && Lx > 2) ? Lx - 1 : kx + 1)
-      present = row_class((uint32_t)kx, (uint32_t)Lx) == (uint32_t)cls;
     const bool first = cls & 1, lastl = (cls & 2) != 0;
-    uint32_t always = 0;
     // classes that cannot occur for this Lx keep a harmless table
-    const int n_nb = 6 - (d.x_pbc ? 0 : ((first ? 1 : 0) + (lastl ? 1 : 0)));
+    const int D = 6 - (d.x_pbc ? 0 : ((first ? 1 : 0) + (lastl ? 1 : 0)));
     double h = H;
     if (first) h += H1;
     if (lastl) h += -H1;
-    for (int idx = 0; idx < 16; idx++) {
-      const int sbit = idx & 1, nal = idx >> 1;
-      d.thr[cls][idx] = 0;
-      if (nal > n_nb) continue;
-      const int s = sbit ? 1 : -1;
-      const int sigma = s * (2 * nal - n_nb);  // sum of the neighbour spins
-      const double dE = 2.0 * (double)s * (J * (double)sigma + h);
-      if (dE <= 0.0) {
-        always |= 1u << idx;
-        continue;
+    ClassDraw& c = d.cls[cls];
+    std::memset(&c, 0, sizeof c);
+    for (int k = 0; k <= D; k++) {
+      // Eq. 1's move of either spin at k up neighbours: always, or for a
+      // word below a threshold
+      const int sigma = 2 * k - D;
+      bool always[2];
+      uint32_t thr[2];
+      for (int sb = 0; sb < 2; sb++) {
+        const double s = sb ? 1.0 : -1.0;
+        const double dE = 2.0 * s * (J * (double)sigma + h);
+        const double t = dE <= 0.0 ? 0.0 : std::floor(std::ldexp(std::exp(-dE / T), 32));
+        always[sb] = dE <= 0.0 || t >= 4294967296.0;
+        thr[sb] = always[sb] ? 0u : (uint32_t)t;
       }
-      const double t = std::floor(std::ldexp(std::exp(-dE / T), 32));
-      if (t >= 4294967296.0) {
-        always |= 1u << idx;
-        continue;
+      if (always[0] && always[1]) {
+        c.alw |= 1u << k;
+      } else if (!always[1]) {
+        c.t[k] = thr[1];
+        c.up |= 1u << k;
+        if (!always[0]) c.frz |= 1u << k;  // dE is not a number: neither spin moves
+      } else {
+        c.t[k] = thr[0];
       }
-      d.thr[cls][idx] = (uint32_t)t;
-      if (t == 0.0 && present) d.has_never = 1;
     }
-    d.always[cls] = always;
-    (void)Lx;
+    bool sym = D == 6 && (c.alw & 8u) && !c.frz;
+    for (int k = 0; k < 3 && sym; k++) {
+      const bool a = (c.alw >> k) & 1u, b = (c.alw >> (6 - k)) & 1u;
+      sym = a == b && (a || (c.t[k] == c.t[6 - k] && !((c.up >> k) & 1u) && ((c.up >> (6 - k)) & 1u)));
+    }
+    c.sym = sym ? 1u : 0u;
   }
 }
 
@@ -156,7 +162,7 @@ void FilmSet::layout(bool assign_part) {
     d.upd_block_begin = ub;
     d.meas_block_begin = mb;
     if (assign_part) d.part_off = po;
-    ub += (grid_items(d, items) + words_per_block(items) - 1) / words_per_block(items);
+    ub += update_blocks(d, items);
     mb += meas_units(d);
     po += part_len(d);
   }
@@ -189,7 +195,7 @@ int FilmSet::upload() {
   uint32_t* om = ou + hh.upd_blocks;
   for (size_t f = 0; f < nf; f++) {
     const FilmDesc& d = h[f];
-    const uint32_t nb = (grid_items(d, items) + words_per_block(items) - 1) / words_per_block(items);
+    const uint32_t nb = update_blocks(d, items);
     for (uint32_t b = 0; b < nb; b++) ou[d.upd_block_begin + b] = (uint32_t)f;
     for (uint32_t b = 0; b < meas_units(d); b++) om[d.meas_block_begin + b] = (uint32_t)f;
   }
@@ -209,11 +215,8 @@ uint32_t FilmSet::fin_grid() const { return std::min<uint32_t>(hh.n_films, (uint
 int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n, bool all_meas, bool fixed_grid) {
   const uint32_t ug = fixed_grid ? upd_grid_max() : upd_grid();
   const uint32_t fg = fixed_grid ? (uint32_t)(2 * n_sm) : fin_grid();
-  bool exact = false, pack = false;
-  for (const auto& d : h) {
-    exact = exact || (d.active && d.has_never);
-    pack = pack || d.pack > 1;
-  }
+  bool pack = false;
+  for (const auto& d : h) pack = pack || d.pack > 1;
   bool prev_meas = false;
   for (uint32_t k = k0; k < k0 + n; k++) {
     bool meas = all_meas;
@@ -226,8 +229,8 @@ int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n, bool all_meas, bool fixed_g
         }
     // records: half-sweep 1 accumulates the sums; the next half-sweep 0
     // writes them, or, after the last sweep of the call, a small kernel
-    ISG_CK(launch_update(L, ug, pool, 0, k, exact, items, pack, part, rec, false, prev_meas ? k : 0, stream));
-    ISG_CK(launch_update(L, ug, pool, 1, k, exact, items, pack, part, rec, meas, 0, stream));
+    ISG_CK(launch_update(L, ug, pool, 0, k, items, pack, part, rec, false, prev_meas ? k : 0, k == k0, stream));
+    ISG_CK(launch_update(L, ug, pool, 1, k, items, pack, part, rec, meas, 0, false, stream));
     if (meas && k + 1 == k0 + n) ISG_CK(launch_record(L, fg, part, rec, k + 1, stream));
     prev_meas = meas;
   }
@@ -268,6 +271,15 @@ using namespace isg;
 
 // ---------------------------------------------------------------- one film
 
+namespace {
+
+struct SlabLaunch {
+  uint32_t C = 0, smem = 0, threads = 0;
+  bool tasks = false;
+};
+
+}  // namespace
+
 struct ising {
   FilmSet fs;
   double J = 1.0, H = 0.0, H1 = 0.0, T = 1.0;
@@ -279,11 +291,10 @@ struct ising {
   int8_t* d_stage = nullptr;
   bool dirty = true;
   int shape = ISING_SHAPE_AUTO;
-  uint32_t* d_cl_list = nullptr;  // the cluster path's film list: one cluster, this film
-  // cluster size of this film (film_cluster_size), cached for the table
-  // variant it was found for (cl_exact: 0 fast, 1 exact, -1 none yet)
-  uint32_t cl_size = 0;
-  int cl_exact = -1;
+  // launch parameters of the cluster and the resident path, looked up once (the
+  // geometry of a handle never changes): cl_size -1 and resident.C 0, not yet
+  int cl_size = -1;
+  SlabLaunch cluster, resident;
   // asynchronous record copies (ising_read_series_async): records
   // [inflight_lo, inflight_hi) of the ring counters are still being copied
   // on copy_stream until ev_copied
@@ -302,32 +313,41 @@ int ensure_stage(ising* h) {
   return ISING_OK;
 }
 
-// CTAs per cluster of a single film on the cluster path: the most (up to
-// kClusterMaxSize) its layers and shared memory allow and the GPU can hold
-// as one cluster, 0 if none.
-uint32_t film_cluster_size(const FilmDesc& d) {
-  const bool exact = d.has_never != 0;
-  for (uint32_t C = kClusterMaxSize; C >= 1; C--) {
-    const uint32_t m = cluster_smem_bytes(d, C);
-    if (m && cluster_capacity(C, 1, m, cluster_threads(d, C, exact, 1), exact) > 0) return C;
-  }
-  return 0;
+// Launch parameters of a film on clusters of C CTAs (C = 1: the resident path);
+// false if it does not qualify or the GPU cannot hold such a cluster.
+bool film_slab(const FilmDesc& d, uint32_t C, SlabLaunch* o) {
+  if (C > 1 ? !cluster_smem_bytes(d, C) : !resident_smem_bytes(d)) return false;
+  o->C = C;
+  o->tasks = slab_tasks_fit(d, C);
+  o->threads = cluster_threads(d, C, 1, o->tasks);
+  const uint32_t smem = C == 1 && !o->tasks ? resident_smem_bytes(d) : slab_dyn_bytes(d, C, o->tasks);
+  return cluster_capacity(C, 1, smem, o->threads, o->tasks, &o->smem) > 0;
 }
 
-// film_cluster_size of the handle's film, looked up once per table variant
-// (the geometry of a handle never changes; its table variant can).
+// The most CTAs per cluster (up to kClusterMaxSize) that the film's layers and
+// shared memory allow and the GPU can hold as one cluster, 0 if none.
+uint32_t film_cluster_size(const FilmDesc& d, SlabLaunch* o) {
+  for (uint32_t C = kClusterMaxSize; C >= 2; C--)
+    if (film_slab(d, C, o)) return C;
+  // one CTA: beyond the resident path's films too
+  o->C = 1;
+  o->tasks = slab_tasks_fit(d, 1);
+  o->threads = cluster_threads(d, 1, 1, o->tasks);
+  return cluster_smem_bytes(d, 1) &&
+                 cluster_capacity(1, 1, slab_dyn_bytes(d, 1, o->tasks), o->threads, o->tasks, &o->smem) > 0 ? 1u : 0u;
+}
+
+// film_cluster_size of the handle's film, looked up once.
 uint32_t handle_cluster_size(ising* h) {
-  const int exact = h->d().has_never != 0 ? 1 : 0;
-  if (h->cl_exact != exact) {
-    h->cl_size = film_cluster_size(h->d());
-    h->cl_exact = exact;
-  }
-  return h->cl_size;
+  if (h->cl_size < 0) h->cl_size = (int)film_cluster_size(h->d(), &h->cluster);
+  return (uint32_t)h->cl_size;
 }
 
 // The launch shape of an ising_sweep call: the pinned one, else the
 // autotuner's choice for this film shape and record interval, else the
-// resident kernel up to kResidentAutoSites spins and one word per thread above.
+// resident kernel up to kResidentAutoSites spins, a cluster up to
+// kClusterAutoSites, and one word per thread above; a film that no cluster
+// takes (one layer) is resident up to kResidentOnlySites.
 int resolve_shape(ising* h, uint32_t measure_every) {
   const FilmDesc& d = h->d();
   if (h->shape != ISING_SHAPE_AUTO) return h->shape;
@@ -336,7 +356,9 @@ int resolve_shape(ising* h, uint32_t measure_every) {
       (s != ISING_SHAPE_CLUSTER || handle_cluster_size(h)))
     return s;
   const uint64_t sites = (uint64_t)d.Lx * d.Ly * d.Lz;
-  return (sites <= kResidentAutoSites && resident_smem_bytes(d)) ? ISING_SHAPE_RESIDENT : ISING_SHAPE_GRID_1;
+  if (sites <= kResidentAutoSites && resident_smem_bytes(d)) return ISING_SHAPE_RESIDENT;
+  if (sites <= kClusterAutoSites && handle_cluster_size(h) > 1) return ISING_SHAPE_CLUSTER;
+  return (sites <= kResidentOnlySites && resident_smem_bytes(d)) ? ISING_SHAPE_RESIDENT : ISING_SHAPE_GRID_1;
 }
 
 int sync_desc(ising* h) {
@@ -627,7 +649,7 @@ int ising_autotune(ising* h, uint32_t measure_every, int* shape) {
   std::vector<int64_t> drain;
   for (int cand = ISING_SHAPE_RESIDENT; !rc && cand <= ISING_SHAPE_CLUSTER; cand++) {
     if (cand == ISING_SHAPE_RESIDENT && !resident_smem_bytes(d)) continue;
-    if (cand == ISING_SHAPE_CLUSTER && !film_cluster_size(d)) continue;
+    if (cand == ISING_SHAPE_CLUSTER && !handle_cluster_size(s)) continue;
     s->shape = cand;
     float ms = 3.0e38f;
     for (int rep = 0; !rc && rep < 3; rep++) {  // the first run warms up
@@ -681,19 +703,12 @@ int ising_sweep(ising* h, uint64_t n, uint32_t measure_every) {
   if (shape == ISING_SHAPE_CLUSTER) {
     // every sweep of the call in one launch: one cluster holds the film in
     // distributed shared memory
-    if (!h->d_cl_list) {
-      const uint32_t list[3] = {0u, 1u, 0u};  // cluster 0 sweeps film 0
-      if (dev_alloc(&h->d_cl_list, sizeof list) != cudaSuccess)
-        return fail(ISING_ENOMEM, "cannot allocate the cluster film list");
-      ISG_CK(cudaMemcpy(h->d_cl_list, list, sizeof list, cudaMemcpyHostToDevice));
-    }
     const uint32_t C = handle_cluster_size(h);
-    const bool exact = d.has_never != 0;
     if (C == 0) return fail(ISING_EINVAL, "film too large for the cluster kernel");
     for (uint64_t done = 0; done < n;) {
       const uint32_t k = (uint32_t)std::min<uint64_t>(n - done, 4096);
-      ISG_CK(launch_cluster(h->fs.L.films, h->d_cl_list, 1, C, 1, cluster_smem_bytes(d, C),
-                            cluster_threads(d, C, exact, 1), exact, h->fs.pool, h->fs.rec, k, h->fs.stream));
+      ISG_CK(launch_cluster(h->fs.L.films, nullptr, 1, C, h->cluster.smem, h->cluster.threads, h->cluster.tasks,
+                            h->fs.pool, h->fs.rec, k, h->fs.stream));
       done += k;
     }
     d.sweep = (uint32_t)(s0 + n);
@@ -702,10 +717,13 @@ int ising_sweep(ising* h, uint64_t n, uint32_t measure_every) {
     return ISING_OK;
   }
   if (shape == ISING_SHAPE_RESIDENT) {
-    const uint32_t smem = resident_smem_bytes(d);
     // small film: every sweep of the call in one launch, planes in shared memory
-    ISG_CK(launch_resident(h->fs.L.films, 1, smem, resident_threads(d), d.has_never != 0, h->fs.pool, h->fs.rec,
-                           (uint32_t)n, h->fs.stream));
+    if (!h->resident.C && !film_slab(d, 1, &h->resident)) {
+      h->resident.C = 0;
+      return fail(ISING_EINVAL, "film too large for the resident kernel");
+    }
+    ISG_CK(launch_cluster(h->fs.L.films, nullptr, 1, 1, h->resident.smem, h->resident.threads, h->resident.tasks,
+                          h->fs.pool, h->fs.rec, (uint32_t)n, h->fs.stream));
     d.sweep = (uint32_t)(s0 + n);
     d.rec_next += (uint32_t)nrec;
     h->rec_written += nrec;
@@ -828,7 +846,6 @@ int ising_destroy(ising* h) {
   h->fs.release();
   if (h->d_direct) cudaFree(h->d_direct);
   if (h->d_stage) cudaFree(h->d_stage);
-  if (h->d_cl_list) cudaFree(h->d_cl_list);
   delete h;
   return ISING_OK;
 }

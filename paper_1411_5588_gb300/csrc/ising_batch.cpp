@@ -35,8 +35,8 @@ struct Lane {
   cudaEvent_t ev_done = nullptr;               // the lane's last sweep call has finished
   // cluster-resident path (CTAs per film; 0: the grid kernels), with the
   // launch's shared memory and threads per CTA and its table variant
-  uint32_t cl_size = 0, cl_per_sm = 1, cl_smem = 0, cl_threads = 0;
-  bool cl_exact = false;
+  uint32_t cl_size = 0, cl_smem = 0, cl_threads = 0;
+  bool cl_tasks = false;           // the task form (slab_tasks_fit)
   uint32_t cl_clusters = 0;        // clusters of the lane's launch
   uint32_t* d_cl_list = nullptr;   // their film lists (launch_cluster's list)
 
@@ -131,18 +131,19 @@ int lane_apply_items(Lane* b, uint32_t items) {
 
 // Launch parameters of the cluster path with C CTAs per film, per_sm CTAs per
 // SM, for every film of the lane; EINVAL if some film does not qualify.
-int lane_cluster_params(const Lane* b, uint32_t C, uint32_t per_sm, uint32_t* smem, uint32_t* threads, bool* exact) {
+int lane_cluster_params(const Lane* b, uint32_t C, uint32_t per_sm, uint32_t* smem, uint32_t* threads, bool* tasks) {
   *smem = 0;
   *threads = 0;
-  *exact = false;
-  for (const FilmDesc& d : b->fs.h) *exact = *exact || d.has_never != 0;
+  *tasks = true;  // a film too large for it takes the whole launch to columns
   for (const FilmDesc& d : b->fs.h) {
-    const uint32_t m = cluster_smem_bytes(d, C);
-    if (m == 0) return fail(ISING_EINVAL, "film %ux%ux%u does not fit clusters of %u CTAs", d.Lx, d.Ly, d.Lz, C);
-    *smem = std::max(*smem, m);
-    *threads = std::max(*threads, cluster_threads(d, C, *exact, per_sm));
+    if (!cluster_smem_bytes(d, C)) return fail(ISING_EINVAL, "film %ux%ux%u does not fit clusters of %u CTAs", d.Lx, d.Ly, d.Lz, C);
+    *tasks = *tasks && slab_tasks_fit(d, C);
   }
-  const int cap = cluster_capacity(C, per_sm, *smem, *threads, *exact);
+  for (const FilmDesc& d : b->fs.h) {
+    *smem = std::max(*smem, slab_dyn_bytes(d, C, *tasks));
+    *threads = std::max(*threads, cluster_threads(d, C, per_sm, *tasks));
+  }
+  const int cap = cluster_capacity(C, per_sm, *smem, *threads, *tasks, smem);
   if (cap < 0) return fail(ISING_ECUDA, "cluster occupancy query failed");
   if (cap == 0) return fail(ISING_EINVAL, "this GPU cannot hold a cluster of %u CTAs of this size", C);
   return ISING_OK;
@@ -160,10 +161,10 @@ double cluster_film_work(const FilmDesc& d) {
 int lane_apply_cluster(Lane* b, uint32_t C, uint32_t n_clusters) {
   const uint32_t per_sm = 1;
   uint32_t smem = 0, threads = 0;
-  bool exact = false;
+  bool tasks = false;
   const size_t nf = b->fs.h.size();
   if (C) {
-    int rc = lane_cluster_params(b, C, per_sm, &smem, &threads, &exact);
+    int rc = lane_cluster_params(b, C, per_sm, &smem, &threads, &tasks);
     if (rc) return rc;
     n_clusters = (uint32_t)std::min<size_t>(std::max<uint32_t>(n_clusters, 1), nf);
   }
@@ -204,10 +205,9 @@ int lane_apply_cluster(Lane* b, uint32_t C, uint32_t n_clusters) {
   }
   b->cl_size = C;
   b->cl_clusters = C ? n_clusters : 0;
-  b->cl_per_sm = per_sm;
   b->cl_smem = smem;
   b->cl_threads = threads;
-  b->cl_exact = exact;
+  b->cl_tasks = tasks;
   b->drop_graphs();
   return ISING_OK;
 }
@@ -218,8 +218,8 @@ int lane_cluster_sweeps(Lane* b, uint64_t n) {
   FilmSet& fs = b->fs;
   while (n) {
     const uint32_t k = (uint32_t)std::min<uint64_t>(n, 4096);
-    ISG_CK(launch_cluster(fs.L.films, b->d_cl_list, b->cl_clusters, b->cl_size, b->cl_per_sm, b->cl_smem,
-                          b->cl_threads, b->cl_exact, fs.pool, fs.rec, k, fs.stream));
+    ISG_CK(launch_cluster(fs.L.films, b->d_cl_list, b->cl_clusters, b->cl_size, b->cl_smem,
+                          b->cl_threads, b->cl_tasks, fs.pool, fs.rec, k, fs.stream));
     for (auto& d : fs.h) d.sweep += k;
     b->sweeps += k;
     n -= k;
@@ -610,9 +610,9 @@ int ising_batch_set_cluster_size(ising_batch* b, uint32_t cluster_size) {
   if (cluster_size > kClusterMaxSize) return fail(ISING_EINVAL, "clusters hold at most %u CTAs", kClusterMaxSize);
   if (cluster_size) {  // every film must qualify before anything changes
     uint32_t smem, threads;
-    bool exact;
+    bool tasks;
     for (Lane* l : b->lanes) {
-      int rc = lane_cluster_params(l, cluster_size, 1, &smem, &threads, &exact);
+      int rc = lane_cluster_params(l, cluster_size, 1, &smem, &threads, &tasks);
       if (rc) return rc;
     }
   }
@@ -670,8 +670,8 @@ int ising_batch_autotune(ising_batch* b, int* shape) {
       bool ok = true;
       for (const Lane* l : b->lanes) {
         uint32_t smem = 0, threads = 0;
-        bool exact = false;
-        ok = ok && lane_cluster_params(l, C, per_sm, &smem, &threads, &exact) == ISING_OK;
+              bool tasks = false;
+              ok = ok && lane_cluster_params(l, C, per_sm, &smem, &threads, &tasks) == ISING_OK;
       }
       clear_error();
       if (ok) cands.push_back({ISING_SHAPE_CLUSTER, C});
@@ -681,7 +681,9 @@ int ising_batch_autotune(ising_batch* b, int* shape) {
     const int cand = cands[ci].first;
     rc = cand == ISING_SHAPE_CLUSTER ? batch_apply_cluster(s, cands[ci].second) : batch_apply_items(s, shape_items(cand));
     float ms = 3.0e38f;
-    for (int rep = 0; !rc && rep < 3; rep++) {  // the first run captures the graphs
+    // the first run captures the graphs; the first candidate gets three more,
+    // or it would be timed on a GPU that is still raising its clocks
+    for (int rep = ci ? 0 : -3; !rc && rep < 3; rep++) {
       if (cudaEventRecord(e0, s->stream()) != cudaSuccess) rc = fail(ISING_ECUDA, "event record failed");
       if (!rc) rc = batch_sweep(s, n, 1);
       if (!rc && cudaEventRecord(e1, s->stream()) != cudaSuccess) rc = fail(ISING_ECUDA, "event record failed");

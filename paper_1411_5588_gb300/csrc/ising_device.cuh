@@ -30,15 +30,27 @@ enum : uint32_t { kYGapbc = 0, kYPbc = 1, kYApbc = 2 };
 
 // One film of a launch.  Lives in device memory; counters `sweep` and
 // `rec_next` are advanced by kernels so that captured graphs can be replayed.
+// Acceptance data of one row class, by k = the site's up neighbours (0 .. D):
+// dE of the two spins at one k are each other's negatives, so at most one of
+// the two moves costs energy.  It happens for a word u < t[k], or always
+// where bit k of alw is set (T = infinity); the other always happens.
+struct ClassDraw {
+  uint32_t t[7];
+  uint32_t alw;   // bit k: both moves always happen
+  uint32_t up;    // bit k: the costly move starts from an up spin
+  uint32_t frz;   // bit k: neither spin moves (couplings whose dE is not a number)
+  uint32_t sym;   // D = 6, t[k] = t[6 - k], k = 3 free, up = (k > 3): the three-mask form holds
+  uint32_t pad;
+};
+
 struct FilmDesc {
   uint32_t Lx, Ly, Lz, n, W;   // n = Lz/2 sites per array, W words per array
-  uint32_t Wp, nq;             // row stride in words (= W), nq = ceil(Wp / 4)
+  uint32_t Wp;                 // row stride in words (= W)
   uint32_t y_mode, x_pbc;
   uint32_t key0, key1;         // Philox key
   uint32_t last_mask;          // valid bits of word W-1
   uint32_t last_calls;         // Philox calls needed by word W-1 (1..8)
   uint32_t upd_block_begin;    // first block of this film in the update grid
-  uint32_t upd_items;          // Lx*(Ly-1)*W (one item = one word of a row)
   uint32_t meas_block_begin;   // first block in the measurement grid
   uint32_t meas_bpl;           // measurement blocks per layer
   uint32_t measure_every;      // 0 = never
@@ -51,15 +63,14 @@ struct FilmDesc {
   uint64_t rec_off;            // int64 offset of the record ring
   uint64_t part_off;           // int64 offset of this film's partial sums
   uint32_t divw_m, divw_l;     // n / W = (umulhi(n, m) + n) >> l  (n < 2^31)
-  uint32_t divy_m, divy_l;     // the same for Ly - 2 (for 1 when Ly = 2)
-  uint32_t thr[4][16];         // Metropolis thresholds [class][s + 2*n_aligned]
-  uint32_t always[4];          // bit (s + 2*n_aligned): accept without a draw
-  uint32_t has_never;          // some reachable entry has dE > 0 and thr = 0
+  ClassDraw cls[4];            // acceptance by row class (row_class)
   uint32_t meas_lpu;           // layers per measurement block (> 1 only when meas_bpl = 1)
   uint32_t rk0[10], rk1[10];   // Philox round keys: key + r * Weyl constant
-  uint32_t pack;               // rows per packed word in the one- and two-word grid kernels (1, 2, 4)
-  uint32_t pk_items;           // their items when pack > 1: Lx * (Ly / pack - 1) groups of pack rows
-  uint32_t pk_divm, pk_divl;   // division by Ly / pack - 2 (by 1 when that is 0)
+  uint32_t pack;               // rows per packed word in the grid kernels (1, 2, 4)
+  uint32_t cols[3];            // columns of a layer without its pairs, by launch shape (column_len)
+  uint32_t divc_m[3], divc_l[3];  // division by them (by 1 when there are none)
+  uint32_t sl_pack;            // the most rows a packed word holds on the slab path (1, 2, 4)
+  uint32_t pad[2];
 };
 
 // Division by a runtime constant d < 2^31 for numerators n < 2^31 (round-up
@@ -111,74 +122,12 @@ __device__ __forceinline__ void philox10(uint32_t c0, uint32_t c1, uint32_t c2, 
   out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// Philox calls that share the row, sweep and parity words of the counter:
-// the first round and half of the second depend only on those, so they are
-// computed once per row and reused for the calls of a word.  rk0/rk1 are the
-// round keys (key + r * Weyl constant, r = 0..9).
-struct PhiloxRow {
-  uint32_t r1_hi1, r1_c3, r2_c0, r2_c1;
-  uint32_t r1_x2;
-  const uint32_t* rk0;
-  const uint32_t* rk1;
-  __device__ __forceinline__ PhiloxRow(uint32_t row, uint32_t sweep, uint32_t parity, const uint32_t* k0,
-                                       const uint32_t* k1)
-      : rk0(k0), rk1(k1) {
-    // round 1 with counter (row, c1, sweep, parity): words 1..3 of the result
-    // do not depend on c1.
-    const uint64_t p0 = (uint64_t)kPhiloxM0 * row, p1 = (uint64_t)kPhiloxM1 * sweep;
-    r1_hi1 = (uint32_t)(p1 >> 32);  // x0 = hi1 ^ c1 ^ k0
-    const uint32_t x1 = (uint32_t)p1;
-    r1_x2 = (uint32_t)(p0 >> 32) ^ parity ^ rk1[0];
-    r1_c3 = (uint32_t)p0;
-    // round 2: the products of x2 are c1-independent
-    const uint64_t q1 = (uint64_t)kPhiloxM1 * r1_x2;
-    r2_c0 = (uint32_t)(q1 >> 32) ^ x1 ^ rk0[1];
-    r2_c1 = (uint32_t)q1;
-  }
-  // Full Philox4x32-10 output for counter word 1 = c1.
-  __device__ __forceinline__ void draw(uint32_t c1, uint32_t out[4]) const {
-    const uint32_t x0 = r1_hi1 ^ c1 ^ rk0[0];  // end of round 1 (x1 = lo1, x2 = r1_x2, x3 = r1_c3)
-    const uint64_t pp = (uint64_t)kPhiloxM0 * x0;
-    uint32_t c0 = r2_c0, c1w = r2_c1, c2 = (uint32_t)(pp >> 32) ^ r1_c3 ^ rk1[1], c3 = (uint32_t)pp;
-#pragma unroll
-    for (int r = 2; r < 10; r++) {
-      const uint64_t p0 = (uint64_t)kPhiloxM0 * c0, p1 = (uint64_t)kPhiloxM1 * c2;
-      c0 = (uint32_t)(p1 >> 32) ^ c1w ^ rk0[r];
-      c1w = (uint32_t)p1;
-      c2 = (uint32_t)(p0 >> 32) ^ c3 ^ rk1[r];
-      c3 = (uint32_t)p0;
-    }
-    out[0] = c0; out[1] = c1w; out[2] = c2; out[3] = c3;
-  }
-  // Two Philox calls (counter words 1 = c1a and c1b) computed side by side.
-  __device__ __forceinline__ void draw2(uint32_t c1a, uint32_t c1b, uint32_t oa[4], uint32_t ob[4]) const {
-    const uint32_t xa = r1_hi1 ^ c1a ^ rk0[0], xb = r1_hi1 ^ c1b ^ rk0[0];
-    const uint64_t pa = (uint64_t)kPhiloxM0 * xa, pb = (uint64_t)kPhiloxM0 * xb;
-    uint32_t a0 = r2_c0, a1 = r2_c1, a2 = (uint32_t)(pa >> 32) ^ r1_c3 ^ rk1[1], a3 = (uint32_t)pa;
-    uint32_t b0 = r2_c0, b1 = r2_c1, b2 = (uint32_t)(pb >> 32) ^ r1_c3 ^ rk1[1], b3 = (uint32_t)pb;
-#pragma unroll
-    for (int r = 2; r < 10; r++) {
-      const uint64_t pa0 = (uint64_t)kPhiloxM0 * a0, pa1 = (uint64_t)kPhiloxM1 * a2;
-      const uint64_t pb0 = (uint64_t)kPhiloxM0 * b0, pb1 = (uint64_t)kPhiloxM1 * b2;
-      a0 = (uint32_t)(pa1 >> 32) ^ a1 ^ rk0[r];
-      a1 = (uint32_t)pa1;
-      a2 = (uint32_t)(pa0 >> 32) ^ a3 ^ rk1[r];
-      a3 = (uint32_t)pa0;
-      b0 = (uint32_t)(pb1 >> 32) ^ b1 ^ rk0[r];
-      b1 = (uint32_t)pb1;
-      b2 = (uint32_t)(pb0 >> 32) ^ b3 ^ rk1[r];
-      b3 = (uint32_t)pb0;
-    }
-    oa[0] = a0; oa[1] = a1; oa[2] = a2; oa[3] = a3;
-    ob[0] = b0; ob[1] = b1; ob[2] = b2; ob[3] = b3;
-  }
-};
-
-// The same calls with one more product hoisted: round 2's word 0 does not
-// depend on c1 either, so neither does round 3's product of it.  Each call
-// then starts at round 2 with one product there and one in round 3 (16 wide
-// multiplies per call instead of 17).  It keeps two more words live across
-// the calls, which the single-film kernel has room for.
+// Philox calls that share the row, sweep and parity words of the counter.
+// Round 1's words 1..3, round 2's words 0 and 1 and round 3's product of the
+// former depend on those alone, so they are computed once per row and word;
+// each call then starts at round 2 with one product there and one in round 3
+// (16 wide products per call instead of 20).  rk0/rk1 are the round keys (key +
+// r * Weyl constant, r = 0..9).
 struct PhiloxRow3 {
   uint32_t r1_hi1, r1_c3;  // round 1: hi(M1 * sweep) (x0 before the c1 and key xor), x3
   uint32_t r2_c1;          // round 2: y1

@@ -132,7 +132,7 @@ struct DeviceGuard {
 // shape (ISING_SHAPE_*) measured for a film shape, boundary, table variant
 // and record interval.
 struct TuneKey {
-  uint32_t Lx, Ly, Lz, y_mode, x_pbc, exact, m_class;
+  uint32_t Lx, Ly, Lz, y_mode, x_pbc, m_class;
   bool operator<(const TuneKey& o) const;
 };
 TuneKey tune_key(const FilmDesc& d, uint32_t measure_every);

@@ -19,9 +19,8 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <type_traits>
 
-#include "ising_device.cuh"
+#include "ising_draw.cuh"
 
 #include "ising_launch.h"
 
@@ -61,78 +60,6 @@ __device__ __forceinline__ bool oob(uint64_t idx, uint64_t lim, uint32_t site) {
 #define ISG_ST(p, idx, lim, site, v) ((void)(lim), (p)[(idx)] = (v))
 #endif
 
-__device__ __forceinline__ uint32_t maj3(uint32_t a, uint32_t b, uint32_t c) {
-  return (a & b) | (c & (a ^ b));
-}
-
-// acc | bit when u <= t: one compare setting a predicate and one predicated OR.
-__device__ __forceinline__ void or_if_le(uint32_t& acc, uint32_t u, uint32_t t, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\tsetp.le.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-      : "+r"(acc) : "r"(u), "r"(t), "r"(bit));
-}
-
-// The same with the bit as an immediate operand.
-template <uint32_t BIT>
-__device__ __forceinline__ void or_if_le_c(uint32_t& acc, uint32_t u, uint32_t t) {
-  asm("{\n\t.reg .pred p;\n\tsetp.le.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-      : "+r"(acc) : "r"(u), "r"(t), "n"(BIT));
-}
-template <uint32_t BIT>
-__device__ __forceinline__ void or_if_lt_c(uint32_t& acc, uint32_t u, uint32_t t) {
-  asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-      : "+r"(acc) : "r"(u), "r"(t), "n"(BIT));
-}
-
-// acc | bit when u < t.
-__device__ __forceinline__ void or_if_lt(uint32_t& acc, uint32_t u, uint32_t t, uint32_t bit) {
-  asm("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p or.b32 %0, %0, %3;\n\t}"
-      : "+r"(acc) : "r"(u), "r"(t), "r"(bit));
-}
-
-// Decisions of the sites at bits Q + 8I (Philox call Q, word u[I]) and
-// Q + 4 + 8I (call Q + 4, word v[I]) of a word.
-template <bool FAST, uint32_t Q, uint32_t I>
-__device__ __forceinline__ void site_pair(uint32_t& lt, const char* tb, uint32_t Y, uint32_t Y2, uint32_t u,
-                                          uint32_t v, bool two) {
-  uint32_t t, t2;
-  const uint32_t base = (uint32_t)__cvta_generic_to_shared(tb);
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(base + __byte_perm(Y, 0, 0x4440 + I)));
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t2) : "r"(base + __byte_perm(Y2, 0, 0x4440 + I)));
-  if (FAST) {
-    // table word thr - 1, or 0xFFFFFFFF for "always" (dE <= 0)
-    or_if_le_c<1u << (Q + 8 * I)>(lt, u, t);
-    if (two) or_if_le_c<1u << (Q + 4 + 8 * I)>(lt, v, t2);
-  } else {
-    or_if_lt_c<1u << (Q + 8 * I)>(lt, u, t);
-    if (two) or_if_lt_c<1u << (Q + 4 + 8 * I)>(lt, v, t2);
-  }
-}
-
-// Decision of the site at bit Q + 8I (Philox call Q, word u).
-template <bool FAST, uint32_t Q, uint32_t I>
-__device__ __forceinline__ void site_one(uint32_t& lt, const char* tb, uint32_t Y, uint32_t u) {
-  uint32_t t;
-  const uint32_t base = (uint32_t)__cvta_generic_to_shared(tb);
-  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(base + __byte_perm(Y, 0, 0x4440 + I)));
-  if (FAST) or_if_le_c<1u << (Q + 8 * I)>(lt, u, t);
-  else or_if_lt_c<1u << (Q + 8 * I)>(lt, u, t);
-}
-
-// Per-launch constants of one film, kept in registers.
-struct FilmCtx {
-  uint32_t* plane0;
-  uint32_t* plane1;
-  uint32_t Lx, Ly, n, W, Wp, y_mode, x_pbc, last_mask, last_calls;
-  uint32_t plane_words;  // words of one plane (Lx * Ly * Wp), for checked builds
-  uint32_t seam_same;    // the y-wrap bonds join sites of one colour (Lx+Ly even under Eq. 11, Ly odd otherwise)
-  uint32_t pack;         // rows per packed word (1, 2 or 4) in the grid kernels' items
-  // decision path of the film's words (kFull, kPartial, kSingle or kMixed)
-  __device__ __forceinline__ uint32_t path() const;
-  const uint32_t* rk0;  // Philox round keys (constant bank or shared memory)
-  const uint32_t* rk1;
-  uint32_t colour, sweep;
-};
-
 __host__ __device__ inline uint32_t seam_joins_one_colour(uint32_t Lx, uint32_t Ly, uint32_t y_mode) {
   return y_mode == kYGapbc ? ((Lx + Ly) % 2 == 0) : (Ly % 2 == 1);
 }
@@ -148,45 +75,6 @@ __device__ __forceinline__ bool measured_now(const FilmDesc& F, uint32_t done, i
   return force || records_after(F, F.sweep, done);
 }
 
-// The words one thread needs to update word w of row (kx, ky), loaded ahead
-// of the arithmetic so that the loads of the next word overlap the current
-// word's Philox draws.
-struct Fetched {
-  uint32_t S, xm, xp, ym, yp, z0, za, zf;
-  uint32_t kx, ky, w;
-};
-
-__device__ __forceinline__ void fetch_word(const FilmCtx& c, uint32_t kx, uint32_t ky, uint32_t w, Fetched& f) {
-  const uint32_t Lx = c.Lx, Ly = c.Ly, W = c.W, Wp = c.Wp;
-  const uint32_t row = (kx - 1) * Ly + (ky - 1);
-  const uint32_t X = (kx + ky + 1 + c.colour) & 1u;
-  const uint32_t* __restrict__ P = X ? c.plane1 : c.plane0;
-  const uint32_t* __restrict__ Q = X ? c.plane0 : c.plane1;
-  const uint32_t rbase = row * Wp;  // planes hold < 2^31 words
-  const uint32_t base = rbase + w;
-  const uint32_t LyWp = Ly * Wp;
-  const uint32_t gkx = (c.y_mode == kYGapbc) ? (Lx - kx) : (kx - 1);  // 0-based layer of the wrap row
-  f.kx = kx; f.ky = ky; f.w = w;
-  const uint32_t lim = c.plane_words;
-  f.S = ISG_LD(P, base, lim, 1);
-  f.xm = (kx > 1) ? ISG_LD(P, base - LyWp, lim, 2)
-                  : (c.x_pbc ? ISG_LD(P, base + (Lx - 1) * LyWp, lim, 3) : 0u);
-  f.xp = (kx < Lx) ? ISG_LD(P, base + LyWp, lim, 4)
-                   : (c.x_pbc ? ISG_LD(P, base - (Lx - 1) * LyWp, lim, 5) : 0u);
-  f.ym = (ky > 1) ? ISG_LD(P, base - Wp, lim, 6) : ISG_LD(P, (gkx * Ly + (Ly - 1)) * Wp + w, lim, 7);
-  f.yp = (ky < Ly) ? ISG_LD(P, base + Wp, lim, 8) : ISG_LD(P, gkx * LyWp + w, lim, 9);
-  f.z0 = ISG_LD(Q, base, lim, 10);
-  if (X == 0)  // previous word, or the row's last
-    f.za = (w > 0) ? ISG_LD(Q, base - 1, lim, 11) : ISG_LD(Q, rbase + W - 1, lim, 12);
-  else  // next word, or the row's first
-    f.za = (w + 1 < W) ? ISG_LD(Q, base + 1, lim, 13) : ISG_LD(Q, rbase, lim, 14);
-  f.zf = ISG_LD(Q, rbase, lim, 15);
-}
-
-// Metropolis decisions for the up to 32 sites of the fetched word; returns
-// the mask of sites that flip.  QUARTER: only Philox calls qsel and qsel + 4
-// (the sites at bits qsel and qsel + 4 of each byte), for a word shared by
-// four lanes.
 __device__ __forceinline__ int64_t block_sum(int64_t v, int64_t* s_red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xFFFFFFFFu, v, o);
@@ -238,71 +126,11 @@ __device__ __noinline__ void write_record(FilmDesc* Fg, const FilmDesc& F, uint3
   }
 }
 
-// Record sums of half-sweep 1.  After its update every neighbour word a
-// thread loaded is final -- it holds the other colour -- except the -y word
-// of a ky = 1 row when the seam joins one colour: that is its wrap partner,
-// which the same thread updates right after it.  So each thread can add up,
-// for its word, the magnetisation of the row's two words w and
-// sum sigma_b S_i S_j over the bonds from the word's sites to their
-// neighbours (an empty x slot is no bond), and every bond of the film is
-// counted once; the seam cases are settled in the partner step.
-//
-// The bonds come from the bit-sliced aligned-neighbour count (c0, c1, c2) of
-// the decision: a flip toggles every aligned mask of its site, so over the
-// D bond slots of the word
-//   sum_d popc(a'_d) = n_old + D popc(fl) - 2 n_fl,
-// n_old and n_fl being the aligned counts summed over the valid and over the
-// flipped sites.  decide_word parks c0, c1, c2 and the row's other word z0 in
-// slots 0-3 of the thread's kStashSlots consecutive shared-memory words
-// (thread-major; the odd stride keeps a warp's accesses on distinct banks)
-// across the Philox draws, so the sums cost no registers there; slot 4 holds
-// a partner word's seam adjustment across its draws.
-constexpr uint32_t kStashSlots = 5;
-
+// One word's record sums; layer: 0-based kx, none when 0xFFFFFFFF.
 struct LayerSums {
-  uint32_t layer = 0xFFFFFFFFu;  // 0-based kx, none when 0xFFFFFFFF
+  uint32_t layer = 0xFFFFFFFFu;
   int m = 0, b = 0;
 };
-
-__device__ __forceinline__ void stash_counts(uint32_t* stash, uint32_t c0, uint32_t c1, uint32_t c2, uint32_t z0) {
-  stash[0] = c0;
-  stash[1] = c1;
-  stash[2] = c2;
-  stash[3] = z0;
-}
-
-// Sums of the word of layer kx (1-based) whose flips were fl and whose new
-// value is v, from the counts decide_word parked.
-__device__ __forceinline__ LayerSums word_sums(const FilmCtx& c, uint32_t kx, uint32_t w, uint32_t fl, uint32_t v,
-                                               const uint32_t* stash) {
-  const uint32_t valid = (w + 1 == c.W) ? c.last_mask : 0xFFFFFFFFu;
-  const int nv = __popc(valid);
-  const uint32_t c0 = stash[0], c1 = stash[1], c2 = stash[2];
-  const uint32_t z0 = stash[3];
-  const int D = 4 + ((kx > 1 || c.x_pbc) ? 1 : 0) + ((kx < c.Lx || c.x_pbc) ? 1 : 0);
-  const int n_old = __popc(c0 & valid) + 2 * __popc(c1 & valid) + 4 * __popc(c2 & valid);
-  const int n_fl = __popc(c0 & fl) + 2 * __popc(c1 & fl) + 4 * __popc(c2 & fl);
-  LayerSums r;
-  r.layer = kx - 1;
-  r.b = 2 * (n_old + D * __popc(fl) - 2 * n_fl) - D * nv;
-  r.m = 2 * (__popc(v & valid) + __popc(z0 & valid)) - 2 * nv;
-  return r;
-}
-
-// Seam correction of a ky = 1 word (new value v, other word z0f) and its
-// partner word g (just fetched) when the seam joins one colour: the word's
-// -y count used the partner's old word, so it comes out again (the partner
-// counts that bond from its +y side with both final words), and the seam
-// bonds between the two rows' other arrays, which no one else holds, go in.
-__device__ __forceinline__ int seam_adjust(const FilmCtx& c, uint32_t w, uint32_t v, uint32_t z0f,
-                                           const Fetched& g) {
-  const uint32_t valid = (w + 1 == c.W) ? c.last_mask : 0xFFFFFFFFu;
-  const int nv = __popc(valid);
-  const bool neg = c.y_mode != kYPbc;
-  const int stale = 2 * __popc(~(v ^ g.S ^ (neg ? 0xFFFFFFFFu : 0u)) & valid) - nv;
-  const int other = nv - 2 * __popc((z0f ^ g.z0) & valid);
-  return (neg ? -other : other) - stale;
-}
 
 // Adds the sums of every lane that has some into the film's per-layer int64
 // accumulators [2 kx (magnetisation), 2 kx + 1 (bonds)].  All 32 lanes call
@@ -334,768 +162,551 @@ __device__ __forceinline__ void add_lane_sums(unsigned long long* acc, const Lay
   atomicAdd(acc + 2 * (size_t)r.layer + 1, (unsigned long long)(long long)r.b);
 }
 
-// The same into a block's shared counters (resident films: int32 suffices
-// below 2^16 sites): layer sums s_m[kx], and the totals s_tot = {B, M}.  All
-// 32 lanes call it.
-__device__ __forceinline__ void add_layer_sums_shared(int* s_m, int* s_tot, const LayerSums& r) {
-  const bool on = r.layer != 0xFFFFFFFFu;
-  const uint32_t act = __ballot_sync(0xFFFFFFFFu, on);
-  if (act == 0) return;
-  const int lead = __ffs(act) - 1;
-  const uint32_t l0 = __shfl_sync(0xFFFFFFFFu, r.layer, lead);
-  const bool in0 = on && r.layer == l0;
-  const int m0 = __reduce_add_sync(0xFFFFFFFFu, in0 ? r.m : 0);
-  const int b = __reduce_add_sync(0xFFFFFFFFu, on ? r.b : 0);
-  const int m = __reduce_add_sync(0xFFFFFFFFu, on ? r.m : 0);
-  if ((int)(threadIdx.x & 31u) == lead) {
-    atomicAdd(&s_m[l0], m0);
-    atomicAdd(&s_tot[0], b);
-    atomicAdd(&s_tot[1], m);
-  } else if (on && !in0) {
-    atomicAdd(&s_m[r.layer], r.m);
-  }
-}
 
-// The other array's word w shifted by one site onto this word's sites, so
-// that each site meets its second z-neighbour: site j of array 0 meets site
-// j - 1 of array 1, site j of array 1 meets site j + 1 of array 0, and the
-// row's ends meet through the periodic z wrap.
-template <bool FULL>
-__device__ __forceinline__ uint32_t z_shifted(const FilmCtx& c, const Fetched& f, uint32_t X, bool partial) {
-  if (X == 0) {
-    const uint32_t pw = (f.w > 0) ? f.za : (((f.za >> bitpos((c.n - 1) & 31u)) & 1u) << 31);
-    return shift_prev(f.z0, pw);
-  }
-  uint32_t Zs = shift_next(f.z0, f.za);
-  if (!FULL && partial) Zs |= (f.zf & 1u) << bitpos((c.n - 1) & 31u);
-  return Zs;
-}
+// ------------------------------------------------------------ grid path
 
-// Decision paths of a word, chosen per film (so that a warp issues one):
-//   kFull     32 valid sites, eight Philox calls;
-//   kPartial  the row's only word (W = 1), partial: the film's last_mask and
-//             last_calls (5..7 calls: calls Q and Q + 4 drawn together);
-//   kSingle   the same with at most four calls, each drawn alone;
-//   kMixed    rows of full words and a partial last word (W >= 2): each
-//             word's own mask and call count.
-enum : uint32_t { kFull = 0, kPartial = 1, kSingle = 2, kMixed = 3 };
-
-__device__ __forceinline__ uint32_t FilmCtx::path() const {
-  if (last_mask == 0xFFFFFFFFu) return kFull;
-  if (W >= 2) return kMixed;
-  return last_calls <= 4 ? kSingle : kPartial;
-}
-
-template <uint32_t PATH, bool FAST, bool QUARTER, bool MEAS = false, bool H3 = false>
-__device__ __forceinline__ uint32_t decide_word(const FilmCtx& c, const Fetched& f,
-                                                const uint32_t* __restrict__ s_thr,
-                                                const uint32_t* __restrict__ s_alw, uint32_t qsel,
-                                                uint32_t* stash = nullptr) {
-  const uint32_t Lx = c.Lx, Ly = c.Ly;
-  const uint32_t kx = f.kx, ky = f.ky, w = f.w;
-  const uint32_t row = (kx - 1) * Ly + (ky - 1);
-  const uint32_t X = (kx + ky + 1 + c.colour) & 1u;
-  const uint32_t S = f.S;
-  // aligned-with-S masks of the six neighbour slots (free x surface: empty
-  // slot, mask 0; Eq. 11 wrap: the partner's spin enters with reversed sign)
-  const uint32_t xm_on = (kx > 1 || c.x_pbc) ? 0xFFFFFFFFu : 0u;
-  const uint32_t xp_on = (kx < Lx || c.x_pbc) ? 0xFFFFFFFFu : 0u;
-  const uint32_t negm = (c.y_mode != kYPbc) ? 0xFFFFFFFFu : 0u;
-  const uint32_t a0 = ~(S ^ f.xm) & xm_on;
-  const uint32_t a1 = ~(S ^ f.xp) & xp_on;
-  const uint32_t a2 = ~(S ^ f.ym ^ (ky > 1 ? 0u : negm));
-  const uint32_t a3 = ~(S ^ f.yp ^ (ky < Ly ? 0u : negm));
-  constexpr bool FULL = PATH == kFull, SINGLE = PATH == kSingle;
-  const bool partial = PATH == kMixed ? (w + 1 == c.W) : !FULL;  // the word holds fewer than 32 sites
-  const uint32_t Zs = z_shifted<FULL>(c, f, X, partial);
-  const uint32_t a4 = ~(S ^ f.z0);
-  const uint32_t a5 = ~(S ^ Zs);
-
-  // bit-sliced count of aligned neighbours: n = c0 + 2 c1 + 4 c2
-  const uint32_t s1 = a0 ^ a1 ^ a2, k1 = maj3(a0, a1, a2);
-  const uint32_t s2 = a3 ^ a4 ^ a5, k2 = maj3(a3, a4, a5);
-  const uint32_t c0 = s1 ^ s2, k3 = s1 & s2;
-  const uint32_t c1 = k1 ^ k2 ^ k3, c2 = maj3(k1, k2, k3);
-  if (MEAS) stash_counts(stash, c0, c1, c2, f.z0);  // for word_sums after the draws
-
-  const uint32_t cls = row_class(kx, Lx);
-  uint32_t alw = 0;
-  if (!FAST) {
-  // "always accept" (dE <= 0) as a 4-input function of (S, c0, c1, c2)
-  const uint4* m4 = reinterpret_cast<const uint4*>(s_alw + cls * 16);
-  const uint4 ma = m4[0], mb = m4[1], mc = m4[2], md = m4[3];
-  const uint32_t v0 = (S & ma.y) | (~S & ma.x);
-  const uint32_t v1 = (S & ma.w) | (~S & ma.z);
-  const uint32_t v2 = (S & mb.y) | (~S & mb.x);
-  const uint32_t v3 = (S & mb.w) | (~S & mb.z);
-  const uint32_t v4 = (S & mc.y) | (~S & mc.x);
-  const uint32_t v5 = (S & mc.w) | (~S & mc.z);
-  const uint32_t v6 = (S & md.y) | (~S & md.x);
-  const uint32_t v7 = (S & md.w) | (~S & md.z);
-  const uint32_t w0 = (c0 & v1) | (~c0 & v0);
-  const uint32_t w1 = (c0 & v3) | (~c0 & v2);
-  const uint32_t w2 = (c0 & v5) | (~c0 & v4);
-  const uint32_t w3 = (c0 & v7) | (~c0 & v6);
-  const uint32_t x0 = (c1 & w1) | (~c1 & w0);
-  const uint32_t x1 = (c1 & w3) | (~c1 & w2);
-  alw = (c2 & x1) | (~c2 & x0);
-  }
-
-  // transpose the planes (S, c0, c1, c2) into nibbles: nibble r of U[a] holds
-  // the 4-bit table index S + 2*n of bit position 4r + a
-  const uint32_t T0 = (S & 0x55555555u) | ((c0 & 0x55555555u) << 1);
-  const uint32_t T1 = ((S >> 1) & 0x55555555u) | (c0 & 0xAAAAAAAAu);
-  const uint32_t T2 = (c1 & 0x55555555u) | ((c2 & 0x55555555u) << 1);
-  const uint32_t T3 = ((c1 >> 1) & 0x55555555u) | (c2 & 0xAAAAAAAAu);
-  uint32_t U[4];
-  U[0] = (T0 & 0x33333333u) | ((T2 & 0x33333333u) << 2);
-  U[1] = (T1 & 0x33333333u) | ((T3 & 0x33333333u) << 2);
-  U[2] = ((T0 >> 2) & 0x33333333u) | (T2 & 0xCCCCCCCCu);
-  U[3] = ((T1 >> 2) & 0x33333333u) | (T3 & 0xCCCCCCCCu);
-
-  const uint32_t ncalls = FULL ? 8u : PATH == kMixed ? (partial ? c.last_calls : 8u) : c.last_calls;
-  const uint32_t clsb = (cls * 64u) * 0x01010101u;  // byte offset of this class's table
-  const char* tb = reinterpret_cast<const char*>(s_thr);
-  using Row = typename std::conditional<H3, PhiloxRow3, PhiloxRow>::type;
-  const Row pr(row, c.sweep, X, c.rk0, c.rk1);
-  uint32_t lt = 0;
-  // calls Q and Q + 4 are drawn together (two independent Philox chains),
-  // except on the kSingle path
-  auto calls = [&](auto qc, uint32_t Uq) {
-    constexpr uint32_t Q = decltype(qc)::value;
-    if (FULL || Q < ncalls) {
-      uint32_t u[4], v[4];
-      if (SINGLE) {
-        // a partial word of at most four calls: call Q alone
-        pr.draw(8u * w + Q, u);
-        const uint32_t Y = ((Uq << 2) & 0x3C3C3C3Cu) | clsb;
-        site_one<FAST, Q, 0>(lt, tb, Y, u[0]);
-        site_one<FAST, Q, 1>(lt, tb, Y, u[1]);
-        site_one<FAST, Q, 2>(lt, tb, Y, u[2]);
-        site_one<FAST, Q, 3>(lt, tb, Y, u[3]);
-      } else {
-        pr.draw2(8u * w + Q, 8u * w + Q + 4, u, v);
-        const bool two = FULL || Q + 4 < ncalls;
-        const uint32_t Y = ((Uq << 2) & 0x3C3C3C3Cu) | clsb;
-        const uint32_t Y2 = ((Uq >> 2) & 0x3C3C3C3Cu) | clsb;
-        site_pair<FAST, Q, 0>(lt, tb, Y, Y2, u[0], v[0], two);
-        site_pair<FAST, Q, 1>(lt, tb, Y, Y2, u[1], v[1], two);
-        site_pair<FAST, Q, 2>(lt, tb, Y, Y2, u[2], v[2], two);
-        site_pair<FAST, Q, 3>(lt, tb, Y, Y2, u[3], v[3], two);
-      }
-    }
-  };
-  using Q0 = std::integral_constant<uint32_t, 0>;
-  using Q1 = std::integral_constant<uint32_t, 1>;
-  using Q2 = std::integral_constant<uint32_t, 2>;
-  using Q3 = std::integral_constant<uint32_t, 3>;
-  if (QUARTER) {
-    // one code path for the four lanes (a switch on qsel would run all four
-    // bodies one after another): runtime call index, bit in a register
-    const uint32_t Uq = qsel == 0 ? U[0] : qsel == 1 ? U[1] : qsel == 2 ? U[2] : U[3];
-    if (FULL || qsel < ncalls) {
-      uint32_t u[4], v[4];
-      pr.draw2(8u * w + qsel, 8u * w + qsel + 4, u, v);
-      const bool two = FULL || qsel + 4 < ncalls;
-      const uint32_t Y = ((Uq << 2) & 0x3C3C3C3Cu) | clsb;
-      const uint32_t Y2 = ((Uq >> 2) & 0x3C3C3C3Cu) | clsb;
-      const uint32_t base = (uint32_t)__cvta_generic_to_shared(tb);
-#pragma unroll
-      for (uint32_t i = 0; i < 4; i++) {
-        uint32_t t, t2;
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(base + __byte_perm(Y, 0, 0x4440 + i)));
-        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(t2) : "r"(base + __byte_perm(Y2, 0, 0x4440 + i)));
-        if (FAST) {
-          or_if_le(lt, u[i], t, 1u << (qsel + 8 * i));
-          if (two) or_if_le(lt, v[i], t2, 1u << (qsel + 4 + 8 * i));
-        } else {
-          or_if_lt(lt, u[i], t, 1u << (qsel + 8 * i));
-          if (two) or_if_lt(lt, v[i], t2, 1u << (qsel + 4 + 8 * i));
-        }
-      }
-    }
-  } else {
-    calls(Q0{}, U[0]);
-    calls(Q1{}, U[1]);
-    calls(Q2{}, U[2]);
-    calls(Q3{}, U[3]);
-  }
-  const uint32_t valid = FULL ? 0xFFFFFFFFu : PATH == kMixed ? (partial ? c.last_mask : 0xFFFFFFFFu) : c.last_mask;
-  return (lt | alw) & valid;
-}
-
-// decide_word on the film's path (uniform across the film, so across a
-// warp).  PATHS4 = false keeps two bodies only (for the kernel whose register
-// budget has no room for more): full words on kFull, a partial last word on
-// kPartial, chosen per word.
-template <bool FAST, bool QUARTER, bool MEAS, bool PATHS4, bool H3 = false>
-__device__ __forceinline__ uint32_t decide_any(const FilmCtx& c, const Fetched& f, const uint32_t* s_thr,
-                                               const uint32_t* s_alw, uint32_t qsel, uint32_t* stash) {
-  if (!PATHS4) {
-    if (f.w + 1 < c.W || c.last_mask == 0xFFFFFFFFu)
-      return decide_word<kFull, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-    return decide_word<kPartial, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-  }
-  const uint32_t path = c.path();
-  if (path == kFull) return decide_word<kFull, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-  if (path == kMixed) return decide_word<kMixed, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-  if (!QUARTER && path == kSingle)
-    return decide_word<kSingle, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-  return decide_word<kPartial, FAST, QUARTER, MEAS, H3>(c, f, s_thr, s_alw, qsel, stash);
-}
-
-__device__ __forceinline__ void store_word(const FilmCtx& c, const Fetched& f, uint32_t v) {
-  const uint32_t row = (f.kx - 1) * c.Ly + (f.ky - 1);
-  const uint32_t X = (f.kx + f.ky + 1 + c.colour) & 1u;
-  uint32_t* __restrict__ P = X ? c.plane1 : c.plane0;
-  ISG_ST(P, row * c.Wp + f.w, c.plane_words, 16, v);
-}
-
-// Word of update item `item`.  The first Lx * W items are the words of the
-// ky = 1 rows, whose threads then also update the wrap partner's word: kept
-// together, they fill whole warps instead of putting one lane that does twice
-// the work into a third of the warps of a small film.  The other items are
-// the rows ky = 2 .. Ly-1, layer by layer.  (dym, dyl) divide by Ly - 2 (by 1
-// when Ly = 2, which has no such rows).
-__device__ __forceinline__ void item_word(const FilmCtx& c, uint32_t item, uint32_t dwm, uint32_t dwl,
-                                          uint32_t dym, uint32_t dyl, uint32_t& kx, uint32_t& ky, uint32_t& w) {
-  const uint32_t rp = fastdiv(item, dwm, dwl);  // the region boundary Lx * W is a whole number of rows
-  w = item - rp * c.W;
-  const bool pair = rp < c.Lx;
-  const uint32_t rq = pair ? 0u : rp - c.Lx;
-  const uint32_t q = fastdiv(rq, dym, dyl);
-  kx = (pair ? rp : q) + 1;
-  ky = pair ? 1u : rq - q * (c.Ly - 2) + 2;
-}
-
-// MEAS: also return the record sums of the word (r1) and of its partner word
-// (r2, ky = 1 only), using the thread's stash slots.
-template <bool FAST, bool MEAS = false, bool PATHS4 = true, bool H3 = false>
-__device__ __forceinline__ void update_fetched(const FilmCtx& c, const Fetched& f, const uint32_t* s_thr,
-                                               const uint32_t* s_alw, uint32_t* stash = nullptr,
-                                               LayerSums* r1 = nullptr, LayerSums* r2 = nullptr) {
-  const uint32_t fl = decide_any<FAST, false, MEAS, PATHS4, H3>(c, f, s_thr, s_alw, 0, stash);
-  const uint32_t v = f.S ^ fl;
-  store_word(c, f, v);
-  if (MEAS) *r1 = word_sums(c, f.kx, f.w, fl, v, stash);
-  // ky = 1 rows then update their wrap partner row (kx', Ly); its wrap
-  // neighbour is the word just written, so it is fetched only now
-  if (f.ky == 1) {
-    const uint32_t kx2 = (c.y_mode == kYGapbc) ? (c.Lx + 1 - f.kx) : f.kx;
-    Fetched g;
-    fetch_word(c, kx2, c.Ly, f.w, g);
-    if (MEAS) stash[4] = c.seam_same ? (uint32_t)seam_adjust(c, f.w, v, stash[3], g) : 0u;
-    const uint32_t fl2 = decide_any<FAST, false, MEAS, PATHS4, H3>(c, g, s_thr, s_alw, 0, stash);
-    const uint32_t v2 = g.S ^ fl2;
-    store_word(c, g, v2);
-    if (MEAS) {
-      *r2 = word_sums(c, kx2, g.w, fl2, v2, stash);
-      r2->b += (int)stash[4];
-    }
-  }
-}
-
-// The same for a word shared by the four lanes 4j..4j+3 of a warp (lane qsel
-// draws Philox calls qsel and qsel + 4); gmask holds the lanes whose group has
-// a word.  The lanes merge their flip masks and the group's lane 0 stores
-// (and, MEAS, takes the record sums).
-template <bool FAST, bool MEAS>
-__device__ __forceinline__ void update_fetched_quarter(const FilmCtx& c, const Fetched& f, bool on, uint32_t qsel,
-                                                       uint32_t gmask, const uint32_t* s_thr,
-                                                       const uint32_t* s_alw, uint32_t* stash, LayerSums& r1,
-                                                       LayerSums& r2) {
-  uint32_t fl = 0;
-  if (on) fl = decide_any<FAST, true, MEAS, true>(c, f, s_thr, s_alw, qsel, stash);
-  if (!on) return;
-  fl |= __shfl_xor_sync(gmask, fl, 1);
-  fl |= __shfl_xor_sync(gmask, fl, 2);
-  const uint32_t v = f.S ^ fl;
-  if (qsel == 0) store_word(c, f, v);
-  if (MEAS && qsel == 0) r1 = word_sums(c, f.kx, f.w, fl, v, stash);
-  // ky = 1 words then update their wrap partner word (see update_fetched)
-  const uint32_t pmask = __ballot_sync(gmask, f.ky == 1);
-  if (f.ky != 1) return;
-  __syncwarp(pmask);  // the partner's wrap neighbour is the word stored above
-  const uint32_t kx2 = (c.y_mode == kYGapbc) ? (c.Lx + 1 - f.kx) : f.kx;
-  Fetched g;
-  fetch_word(c, kx2, c.Ly, f.w, g);
-  if (MEAS) stash[4] = c.seam_same ? (uint32_t)seam_adjust(c, f.w, v, stash[3], g) : 0u;
-  uint32_t fl2 = decide_any<FAST, true, MEAS, true>(c, g, s_thr, s_alw, qsel, stash);
-  fl2 |= __shfl_xor_sync(pmask, fl2, 1);
-  fl2 |= __shfl_xor_sync(pmask, fl2, 2);
-  const uint32_t v2 = g.S ^ fl2;
-  if (qsel == 0) store_word(c, g, v2);
-  if (MEAS && qsel == 0) {
-    r2 = word_sums(c, kx2, g.w, fl2, v2, stash);
-    r2.b += (int)stash[4];
-  }
-}
-
-// ---- thin films: several rows per register
-//
-// A film whose rows hold one partial word per parity array (W = 1) with at
-// most 8 sites (R = 4) or 16 sites (R = 2) per array spends the per-word work
-// -- neighbour count, table indices, stores -- on a quarter or a half of a
-// word's 32 sites.  The grid kernels then update R rows (kx, ky0 .. ky0+R-1)
-// of one layer at once: row j's bits, which sit in the low B = 8/R bits of
-// each byte, move up by j*B bits into one register, and the decision runs
-// once on the packed word.  Packed bit j*B + q + 8*I is row j's site
-// 4q + I, served by that row's Philox call q: the bit-to-call rule of a full
-// word holds with "call" Q = j*B + q and the row's own counter.  The
-// checkerboard is unchanged: consecutive rows update opposite arrays, and
-// none reads an array another updates in the same half-sweep.  The memory
-// layout is the same as for every other film; only the grid update kernels
-// (one or two items per thread) pack.
-
-// Packed operands of R rows (wrap signs folded into ym, yp).
-struct Packed {
-  uint32_t S, xm, xp, ym, yp, z0, Zs;
-  uint32_t kx, ky0;
+// Per-launch constants of one film.
+struct FilmCtx {
+  uint32_t* plane0;
+  uint32_t* plane1;
+  uint32_t Lx, Ly, W, y_mode, x_pbc, last_mask, last_calls;
+  uint32_t pos;          // bit of a row's last site in its last word
+  uint32_t plane_words;  // words of one plane (Lx * Ly * W), for checked builds
+  uint32_t neg;          // all ones where the y wrap reverses the sign
+  uint32_t seam_same;    // the y-wrap bonds join sites of one colour (Lx+Ly even under Eq. 11, Ly odd otherwise)
+  const ClassDraw* cls;
+  const uint32_t* rk0;   // Philox round keys (constant bank or shared memory)
+  const uint32_t* rk1;
+  uint32_t colour, sweep;
 };
 
-// Row mask of the low B bits of each byte.
-template <uint32_t R>
+__device__ __forceinline__ void film_ctx(FilmCtx& c, const FilmDesc& d, uint32_t* pool, uint32_t colour,
+                                         uint32_t sweep) {
+  c.Lx = d.Lx; c.Ly = d.Ly; c.W = d.W;
+  c.y_mode = d.y_mode; c.x_pbc = d.x_pbc;
+  c.last_mask = d.last_mask; c.last_calls = d.last_calls;
+  c.pos = bitpos((d.n - 1) & 31u);
+  c.plane_words = d.Lx * d.Ly * d.W;
+  c.neg = d.y_mode != kYPbc ? 0xFFFFFFFFu : 0u;
+  c.seam_same = seam_joins_one_colour(d.Lx, d.Ly, d.y_mode);
+  c.cls = d.cls; c.rk0 = d.rk0; c.rk1 = d.rk1;
+  c.colour = colour; c.sweep = sweep;
+  c.plane0 = pool + d.spin_off;
+  c.plane1 = c.plane0 + (size_t)d.Lx * d.Ly * d.W;
+}
+
+// The masks of a word drawn ahead: the three-mask form fills m[4..6].
+struct Drawn {
+  uint32_t m[7];
+};
+
+// Masks of one word of R rows from row `row` (parity array X) of class cl;
+// any7: the warp takes the general form (ROLL: as a
+// loop over the calls, in fewer registers).  calls: the word's (R > 1: a row's)
+// Philox calls; full: every word of the film has eight.
+template <int R, bool ROLL = false>
+__device__ __forceinline__ void draw_any(Drawn& o, bool any7, const ClassDraw& cl, uint32_t row, uint32_t X,
+                                         uint32_t w, uint32_t calls, bool full, bool paired, uint32_t sweep,
+                                         const uint32_t* rk0, const uint32_t* rk1) {
+  if (!any7) {
+    Masks<3> a;
+    const uint32_t t[3] = {cl.t[4], cl.t[5], cl.t[6]};
+    if (R == 1 && full) draw_masks<1, true, 3>(a, t, row, X, 8u * w, 8u, true, sweep, rk0, rk1);
+    else draw_masks<R, false, 3>(a, t, row, X, 8u * w, calls, paired, sweep, rk0, rk1);
+    // all ones where t_k would be 2^32 (T = infinity)
+    if (cl.alw & 0x70u) {
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+        if ((cl.alw >> (4 + k)) & 1u) a.m[k] = 0xFFFFFFFFu;
+    }
+    // every mask is set, so that none is live from one drawing to the next
+    o = Drawn{{0, 0, 0, 0, a.m[0], a.m[1], a.m[2]}};
+  } else {
+    Masks<7> a;
+    draw_masks<R, false, 7, ROLL>(a, cl.t, row, X, 8u * w, calls, paired, sweep, rk0, rk1);
+#pragma unroll
+    for (int k = 0; k < 7; k++) o.m[k] = (cl.alw >> k) & 1u ? 0xFFFFFFFFu : a.m[k];
+  }
+}
+
+__device__ __forceinline__ uint32_t decide(const Hood& h, const Count& k, bool any7, const Drawn& a,
+                                           const ClassDraw& cl) {
+  if (!any7) return flips3(h.S, k, a.m[4], a.m[5], a.m[6]);
+  return flips7(h.S, k, a.m, cl.up, cl.frz);
+}
+
+// Slot masks of a word of R packed rows: the rows' first-site bits, and the
+// bits of row 0.
+template <int R>
+__device__ __forceinline__ constexpr uint32_t first_bits() {
+  return R == 1 ? 0x01u : R == 2 ? 0x11u : 0x55u;
+}
+template <int R>
 __device__ __forceinline__ constexpr uint32_t slot_mask() {
   return 0x01010101u * ((1u << (8 / R)) - 1u);
 }
 
-template <uint32_t R>
-__device__ __forceinline__ void fetch_packed(const FilmCtx& c, uint32_t kx, uint32_t ky0, Packed& p) {
-  constexpr uint32_t B = 8 / R;
-  p.kx = kx;
-  p.ky0 = ky0;
-  p.S = p.xm = p.xp = p.ym = p.yp = p.z0 = p.Zs = 0;
-  const uint32_t valid = c.last_mask;  // the row's sites, all in the low B bits of each byte
-  const uint32_t negm = (c.y_mode != kYPbc) ? valid : 0u;
-#pragma unroll
-  for (uint32_t j = 0; j < R; j++) {
-    const uint32_t ky = ky0 + j;
-    Fetched f;
-    fetch_word(c, kx, ky, 0, f);
-    const uint32_t X = (kx + ky + 1 + c.colour) & 1u;
-    const uint32_t zs = z_shifted<false>(c, f, X, true) & valid;
-    const uint32_t sh = j * B;
-    p.S |= f.S << sh;
-    p.xm |= f.xm << sh;
-    p.xp |= f.xp << sh;
-    p.ym |= (f.ym ^ (ky > 1 ? 0u : negm)) << sh;
-    p.yp |= (f.yp ^ (ky < c.Ly ? 0u : negm)) << sh;
-    p.z0 |= f.z0 << sh;
-    p.Zs |= zs << sh;
+// The words of word w of row (kx, ky).
+__device__ __forceinline__ void fetch_row(const FilmCtx& c, uint32_t kx, uint32_t ky, uint32_t w, Hood& f) {
+  const uint32_t Lx = c.Lx, Ly = c.Ly, W = c.W;
+  const uint32_t row = (kx - 1) * Ly + (ky - 1);
+  const uint32_t X = (kx + ky + 1 + c.colour) & 1u;
+  const uint32_t* __restrict__ P = X ? c.plane1 : c.plane0;
+  const uint32_t* __restrict__ Q = X ? c.plane0 : c.plane1;
+  const uint32_t rbase = row * W;  // planes hold < 2^31 words
+  const uint32_t base = rbase + w;
+  const uint32_t LyW = Ly * W;
+  const uint32_t gkx = (c.y_mode == kYGapbc) ? (Lx - kx) : (kx - 1);  // 0-based layer of the wrap row
+  const uint32_t lim = c.plane_words;
+  f.S = ISG_LD(P, base, lim, 1);
+  f.xm = (kx > 1) ? ISG_LD(P, base - LyW, lim, 2)
+                  : (c.x_pbc ? ISG_LD(P, base + (Lx - 1) * LyW, lim, 3) : 0u);
+  f.xp = (kx < Lx) ? ISG_LD(P, base + LyW, lim, 4)
+                   : (c.x_pbc ? ISG_LD(P, base - (Lx - 1) * LyW, lim, 5) : 0u);
+  f.ym = (ky > 1) ? ISG_LD(P, base - W, lim, 6) : (ISG_LD(P, (gkx * Ly + (Ly - 1)) * W + w, lim, 7) ^ c.neg);
+  f.yp = (ky < Ly) ? ISG_LD(P, base + W, lim, 8) : (ISG_LD(P, gkx * LyW + w, lim, 9) ^ c.neg);
+  f.z0 = ISG_LD(Q, base, lim, 10);
+  // the second z neighbour: site j of array 0 meets site j - 1 of array 1,
+  // site j of array 1 meets site j + 1 of array 0, the row's ends joined
+  if (W == 1) {
+    f.zs = X ? packed_next(f.z0, 1u, c.pos) : packed_prev(f.z0, 1u, c.pos);
+  } else if (X == 0) {
+    const uint32_t pw = (w > 0) ? ISG_LD(Q, base - 1, lim, 11) >> 31 : (ISG_LD(Q, rbase + W - 1, lim, 12) >> c.pos) & 1u;
+    f.zs = shift_prev(f.z0, pw << 31);
+  } else {
+    const bool last = w + 1 == W;
+    const uint32_t nw = last ? ISG_LD(Q, rbase, lim, 14) : ISG_LD(Q, base + 1, lim, 13);
+    f.zs = shift_next(f.z0, 0u) | ((nw & 1u) << (last ? c.pos : 31u));
   }
 }
 
-// The word of each of the R rows back into its own array.
-template <uint32_t R>
-__device__ __forceinline__ void store_packed(const FilmCtx& c, const Packed& p, uint32_t v) {
-  constexpr uint32_t B = 8 / R;
+// The same for R rows (kx, ky .. ky+R-1) of one-word rows, packed.
+//
+// Thin films: a film whose rows hold one partial word per parity array
+// (W = 1) with at most 8 sites (R = 4) or 16 sites (R = 2) per array would
+// spend the per-word work on a quarter or a half of a word's 32 sites.  Row
+// j's bits, which sit in the low B = 8/R bits of each byte, move up by j*B
+// bits into one register: packed bit j*B + q + 8*i is row j's site 4q + i,
+// served by that row's Philox call q.  Consecutive rows update opposite
+// arrays, and none reads an array another updates in the same half-sweep.
+template <int R>
+__device__ __forceinline__ void fetch_rows(const FilmCtx& c, uint32_t kx, uint32_t ky, uint32_t w, Hood& p) {
+  if constexpr (R == 1) {
+    fetch_row(c, kx, ky, w, p);
+  } else {
+    constexpr uint32_t B = 8 / R;
+    p = Hood{0, 0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (uint32_t j = 0; j < R; j++) {
+      Hood f;
+      fetch_row(c, kx, ky + j, 0, f);
+      const uint32_t sh = j * B, valid = c.last_mask;
+      p.S |= f.S << sh;
+      p.xm |= f.xm << sh;
+      p.xp |= f.xp << sh;
+      p.ym |= (f.ym & valid) << sh;
+      p.yp |= (f.yp & valid) << sh;
+      p.z0 |= f.z0 << sh;
+      p.zs |= (f.zs & valid) << sh;
+    }
+  }
+}
+
+template <int R>
+__device__ __forceinline__ void store_rows(const FilmCtx& c, uint32_t kx, uint32_t ky, uint32_t w, uint32_t v) {
 #pragma unroll
   for (uint32_t j = 0; j < R; j++) {
-    const uint32_t ky = p.ky0 + j;
-    const uint32_t row = (p.kx - 1) * c.Ly + (ky - 1);
-    const uint32_t X = (p.kx + ky + 1 + c.colour) & 1u;
+    const uint32_t row = (kx - 1) * c.Ly + (ky + j - 1);
+    const uint32_t X = (kx + ky + j + 1 + c.colour) & 1u;
     uint32_t* __restrict__ P = X ? c.plane1 : c.plane0;
-    ISG_ST(P, row * c.Wp, c.plane_words, 17, (v >> (j * B)) & slot_mask<R>());
+    ISG_ST(P, row * c.W + w, c.plane_words, 16, R == 1 ? v : (v >> (j * (8 / R))) & slot_mask<R>());
   }
 }
 
-// Metropolis decisions of the packed word: the flip mask (packed).
-template <uint32_t R, bool FAST>
-__device__ __forceinline__ uint32_t decide_packed(const FilmCtx& c, const Packed& p,
-                                                  const uint32_t* __restrict__ s_thr,
-                                                  const uint32_t* __restrict__ s_alw) {
-  constexpr uint32_t B = 8 / R;
-  const uint32_t Lx = c.Lx, kx = p.kx;
-  const uint32_t S = p.S;
-  const uint32_t xm_on = (kx > 1 || c.x_pbc) ? 0xFFFFFFFFu : 0u;
-  const uint32_t xp_on = (kx < Lx || c.x_pbc) ? 0xFFFFFFFFu : 0u;
-  const uint32_t a0 = ~(S ^ p.xm) & xm_on;
-  const uint32_t a1 = ~(S ^ p.xp) & xp_on;
-  const uint32_t a2 = ~(S ^ p.ym);
-  const uint32_t a3 = ~(S ^ p.yp);
-  const uint32_t a4 = ~(S ^ p.z0);
-  const uint32_t a5 = ~(S ^ p.Zs);
-  const uint32_t s1 = a0 ^ a1 ^ a2, k1 = maj3(a0, a1, a2);
-  const uint32_t s2 = a3 ^ a4 ^ a5, k2 = maj3(a3, a4, a5);
-  const uint32_t c0 = s1 ^ s2, k3 = s1 & s2;
-  const uint32_t c1 = k1 ^ k2 ^ k3, c2 = maj3(k1, k2, k3);
-
-  const uint32_t cls = row_class(kx, Lx);
-  uint32_t alw = 0;
-  if (!FAST) {
-    const uint4* m4 = reinterpret_cast<const uint4*>(s_alw + cls * 16);
-    const uint4 ma = m4[0], mb = m4[1], mc = m4[2], md = m4[3];
-    const uint32_t v0 = (S & ma.y) | (~S & ma.x);
-    const uint32_t v1 = (S & ma.w) | (~S & ma.z);
-    const uint32_t v2 = (S & mb.y) | (~S & mb.x);
-    const uint32_t v3 = (S & mb.w) | (~S & mb.z);
-    const uint32_t v4 = (S & mc.y) | (~S & mc.x);
-    const uint32_t v5 = (S & mc.w) | (~S & mc.z);
-    const uint32_t v6 = (S & md.y) | (~S & md.x);
-    const uint32_t v7 = (S & md.w) | (~S & md.z);
-    const uint32_t w0 = (c0 & v1) | (~c0 & v0);
-    const uint32_t w1 = (c0 & v3) | (~c0 & v2);
-    const uint32_t w2 = (c0 & v5) | (~c0 & v4);
-    const uint32_t w3 = (c0 & v7) | (~c0 & v6);
-    const uint32_t x0 = (c1 & w1) | (~c1 & w0);
-    const uint32_t x1 = (c1 & w3) | (~c1 & w2);
-    alw = (c2 & x1) | (~c2 & x0);
-  }
-  const uint32_t T0 = (S & 0x55555555u) | ((c0 & 0x55555555u) << 1);
-  const uint32_t T1 = ((S >> 1) & 0x55555555u) | (c0 & 0xAAAAAAAAu);
-  const uint32_t T2 = (c1 & 0x55555555u) | ((c2 & 0x55555555u) << 1);
-  const uint32_t T3 = ((c1 >> 1) & 0x55555555u) | (c2 & 0xAAAAAAAAu);
-  uint32_t U[4];
-  U[0] = (T0 & 0x33333333u) | ((T2 & 0x33333333u) << 2);
-  U[1] = (T1 & 0x33333333u) | ((T3 & 0x33333333u) << 2);
-  U[2] = ((T0 >> 2) & 0x33333333u) | (T2 & 0xCCCCCCCCu);
-  U[3] = ((T1 >> 2) & 0x33333333u) | (T3 & 0xCCCCCCCCu);
-
-  const uint32_t clsb = (cls * 64u) * 0x01010101u;
-  const char* tb = reinterpret_cast<const char*>(s_thr);
-  const uint32_t ncalls = c.last_calls;  // calls of one row (q < ncalls)
-  const uint32_t rowb = (kx - 1) * c.Ly + (p.ky0 - 1);
-  uint32_t lt = 0;
-  // call Q (0..7) of the packed word: row Q / B's call Q % B, whose sites sit
-  // at bits Q + 8 I; their table indices are nibbles of U[Q & 3] (the low or
-  // high nibble of each byte for Q < 4 or Q >= 4)
-  auto call = [&](auto qc) {
-    constexpr uint32_t Q = decltype(qc)::value;
-    constexpr uint32_t j = Q / B, q = Q % B;
-    if (q < ncalls) {
-      const uint32_t X = (kx + p.ky0 + j + 1 + c.colour) & 1u;
-      uint32_t u[4];
-      PhiloxRow(rowb + j, c.sweep, X, c.rk0, c.rk1).draw(q, u);
-      const uint32_t Uq = U[Q & 3];
-      const uint32_t Y = (Q < 4 ? ((Uq << 2) & 0x3C3C3C3Cu) : ((Uq >> 2) & 0x3C3C3C3Cu)) | clsb;
-      site_one<FAST, Q, 0>(lt, tb, Y, u[0]);
-      site_one<FAST, Q, 1>(lt, tb, Y, u[1]);
-      site_one<FAST, Q, 2>(lt, tb, Y, u[2]);
-      site_one<FAST, Q, 3>(lt, tb, Y, u[3]);
-    }
-  };
-  call(std::integral_constant<uint32_t, 0>{});
-  call(std::integral_constant<uint32_t, 4>{});
-  call(std::integral_constant<uint32_t, 1>{});
-  call(std::integral_constant<uint32_t, 5>{});
-  call(std::integral_constant<uint32_t, 2>{});
-  call(std::integral_constant<uint32_t, 6>{});
-  call(std::integral_constant<uint32_t, 3>{});
-  call(std::integral_constant<uint32_t, 7>{});
-  uint32_t valid = 0;
-#pragma unroll
-  for (uint32_t j = 0; j < R; j++) valid |= c.last_mask << (j * B);
-  return (lt | alw) & valid;
+// A word of array X at an offset from a word of it, for columns.
+__device__ __forceinline__ uint32_t col_ld(const FilmCtx& c, const uint32_t* p, ptrdiff_t off, uint32_t X,
+                                           uint32_t site) {
+#ifdef ISING_CHECKED
+  const uint32_t* base = X ? c.plane1 : c.plane0;
+  return ISG_LD(base, (uint64_t)(p + off - base), c.plane_words, site);
+#else
+  return p[off];
+#endif
+}
+__device__ __forceinline__ void col_st(const FilmCtx& c, const uint32_t* p, uint32_t X, uint32_t v) {
+  uint32_t* base = X ? c.plane1 : c.plane0;
+#ifdef ISING_CHECKED
+  ISG_ST(base, (uint64_t)(p - base), c.plane_words, 16, v);
+#else
+  (void)base;
+  *const_cast<uint32_t*>(p) = v;
+#endif
 }
 
-// The R rows of a group, and, for the group holding ky = 1, then the group
-// holding ky = Ly of the wrap partner layer (fetched after the first group is
-// stored, as update_fetched does with single rows).  Plain launches only: the
-// summing launches take a group's rows one at a time (sweep_block_rows).
-template <uint32_t R, bool FAST>
-__device__ __forceinline__ void update_packed(const FilmCtx& c, const Packed& p, const uint32_t* s_thr,
-                                              const uint32_t* s_alw) {
-  const uint32_t fl = decide_packed<R, FAST>(c, p, s_thr, s_alw);
-  store_packed<R>(c, p, p.S ^ fl);
-  if (p.ky0 != 1) return;
-  const uint32_t kx2 = (c.y_mode == kYGapbc) ? (c.Lx + 1 - p.kx) : p.kx;
-  Packed g;
-  fetch_packed<R>(c, kx2, c.Ly - R + 1, g);
-  const uint32_t fl2 = decide_packed<R, FAST>(c, g, s_thr, s_alw);
-  store_packed<R>(c, g, g.S ^ fl2);
+// Bond slots of a site of layer kx.
+__device__ __forceinline__ int bond_slots(uint32_t kx, uint32_t Lx, uint32_t x_pbc) {
+  return 4 + ((kx > 1 || x_pbc) ? 1 : 0) + ((kx < Lx || x_pbc) ? 1 : 0);
 }
 
-// Group of packed update item `item`: the first Lx items are the groups
-// holding ky = 1 (whose threads then update the wrap partner's last group),
-// the others the middle groups of each layer.  (dm, dl) divide by
-// Ly / R - 2 (by 1 when that is 0).
-template <uint32_t R>
-__device__ __forceinline__ void item_group(const FilmCtx& c, uint32_t item, uint32_t dm, uint32_t dl, uint32_t& kx,
-                                           uint32_t& ky0) {
-  const bool pair = item < c.Lx;
-  const uint32_t r = pair ? 0u : item - c.Lx;
-  const uint32_t q = fastdiv(r, dm, dl);
-  kx = (pair ? item : q) + 1;
-  ky0 = pair ? 1u : (r - q * (c.Ly / R - 2) + 1) * R + 1;
+// Record sums of half-sweep 1.  Every neighbour word a thread loaded is final
+// after it -- it holds the other colour -- except the -y word of a ky = 1 row
+// when the seam joins one colour: that is its wrap partner, which the same
+// thread updates right after it.  So each thread adds up, for its word, the
+// magnetisation of the row's two words and sum sigma_b S_i S_j over the bonds
+// from the word's sites to their neighbours (an empty x slot is no bond), and
+// every bond of the film is counted once.
+__device__ __forceinline__ LayerSums word_sums(uint32_t kx, const Count& k, uint32_t v, uint32_t z0, uint32_t valid,
+                                               int D) {
+  LayerSums r;
+  r.layer = kx - 1;
+  r.b = word_bond_sum(k, v, valid, D);
+  r.m = 2 * (__popc(v) + __popc(z0)) - 2 * __popc(valid);
+  return r;
 }
 
-// The packed items of one block (as sweep_block's word items) in a plain
-// launch.
-template <uint32_t R, bool FAST>
-__device__ __forceinline__ void sweep_block_packed(const FilmCtx& c, uint32_t first, uint32_t items, uint32_t dm,
-                                                   uint32_t dl, const uint32_t* __restrict__ s_thr,
-                                                   const uint32_t* __restrict__ s_alw) {
-  const uint32_t item = first + threadIdx.x;
-  if (item >= items) return;
-  uint32_t kx, ky0;
-  item_group<R>(c, item, dm, dl, kx, ky0);
-  Packed p;
-  fetch_packed<R>(c, kx, ky0, p);
-  update_packed<R, FAST>(c, p, s_thr, s_alw);
+// Seam correction of a ky = 1 word (new value v, other word z0) and its
+// partner word (old value S2, other word z2; the partner row is its slot at
+// bit shift sh) when the seam joins one colour: the first word's -y count used
+// the partner's old word, so it comes out again (the partner counts that bond
+// from its +y side with both final words), and the seam bonds between the two
+// rows' other arrays, which no one else holds, go in.
+__device__ __forceinline__ int seam_adjust(uint32_t v, uint32_t z0, uint32_t S2, uint32_t z2, uint32_t sh,
+                                           uint32_t neg, uint32_t valid) {
+  const int nv = __popc(valid);
+  const int stale = 2 * __popc(~(v ^ (S2 >> sh) ^ neg) & valid) - nv;
+  const int other = nv - 2 * __popc((z0 ^ (z2 >> sh)) & valid);
+  return (neg ? -other : other) - stale;
 }
 
-// The packed items of one block, each group's rows decided one at a time
-// with the single-row body (update_fetched): rows ky0 .. ky0+R-1 of layer
-// kx, and for the group holding ky = 1 (whose row 1 then updates its wrap
-// partner, row Ly of layer kx') the other rows of the partner's group.  The
-// record sums of a group's rows (one layer) and of the partner's rows
-// (another) are added up in registers and then added like a single word's.
-template <bool FAST, bool MEAS, bool PATHS4, typename AccOf>
-__device__ __forceinline__ void sweep_block_rows(const FilmCtx& c, uint32_t first, uint32_t items, uint32_t dm,
-                                                 uint32_t dl, const uint32_t* __restrict__ s_thr,
-                                                 const uint32_t* __restrict__ s_alw, bool meas, AccOf acc_of,
-                                                 uint32_t* stash) {
-  const uint32_t R = c.pack;
-  const uint32_t item = first + threadIdx.x;
-  const bool mine = item < items;
-  LayerSums g1, g2;
-  if (mine) {
-    uint32_t kx, ky0;
-    const uint32_t G2 = c.Ly / R - 2;
-    const bool pair = item < c.Lx;
-    const uint32_t r = pair ? 0u : item - c.Lx;
-    const uint32_t q = fastdiv(r, dm, dl);
-    kx = (pair ? item : q) + 1;
-    ky0 = pair ? 1u : (r - q * G2 + 1) * R + 1;
-    const uint32_t kx2 = (c.y_mode == kYGapbc) ? (c.Lx + 1 - kx) : kx;
-    if (MEAS) {
-      g1.layer = kx - 1;
-      if (pair) g2.layer = kx2 - 1;
-    }
-    const uint32_t nrows = pair ? 2 * R - 1 : R;  // the partner row itself comes with row 1
+// The pair of a ky = 1 word (group 0 of layer kx) and its wrap partner's, row Ly
+// of layer kx' (= Lx + 1 - kx under Eq. 11, else kx), in this order.
+template <int R, bool MEAS, class Wait, class AccOf>
+__device__ __forceinline__ void update_pair(const FilmCtx& c, uint32_t kx, uint32_t w, uint32_t calls, uint32_t valid,
+                                            uint32_t valid1, bool meas, AccOf acc_of, Wait wait) {
+  constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  const uint32_t kx2 = (c.y_mode == kYGapbc) ? c.Lx + 1 - kx : kx, ky2 = c.Ly - R + 1;
+  const uint32_t c1 = row_class(kx, c.Lx), c2 = row_class(kx2, c.Lx);
+  const bool any7 = !c.cls[c1].sym || !c.cls[c2].sym;
+  Drawn a[2];
 #pragma unroll 1
-    for (uint32_t i = 0; i < nrows; i++) {
-      const bool own = i < R;
-      const uint32_t rkx = own ? kx : kx2, rky = own ? ky0 + i : c.Ly - R + 1 + (i - R);
-      Fetched f;
-      fetch_word(c, rkx, rky, 0, f);
+  for (uint32_t n = 0; n < 2; n++) {
+    const uint32_t k = n ? kx2 : kx, ky = n ? ky2 : 1u;
+    Drawn x;
+    draw_any<R>(x, any7, c.cls[n ? c2 : c1], (k - 1) * c.Ly + ky - 1, (k + ky + 1 + c.colour) & 1u, w, calls,
+                    c.last_mask == 0xFFFFFFFFu, c.W > 1, c.sweep, c.rk0, c.rk1);
+    if (n == 0) a[0] = x;
+    else a[1] = x;
+  }
+  wait();
+  Hood h, g;
+  fetch_rows<R>(c, kx, 1, w, h);
+  fetch_rows<R>(c, kx2, ky2, w, g);
+  const Count k = count_up(h);
+  const uint32_t v = h.S ^ (decide(h, k, any7, a[0], c.cls[c1]) & valid);
+  store_rows<R>(c, kx, 1, w, v);
+  // the partner's wrap neighbour is the word just decided where the seam joins
+  // one colour
+  if (c.seam_same) g.yp = (g.yp & ~(valid1 << kSeam)) | (((v ^ c.neg) & valid1) << kSeam);
+  const Count k2 = count_up(g);
+  const uint32_t v2 = g.S ^ (decide(g, k2, any7, a[1], c.cls[c2]) & valid);
+  store_rows<R>(c, kx2, ky2, w, v2);
+  if (MEAS && meas) {
+    add_lane_sums(acc_of(), word_sums(kx, k, v, h.z0, valid, bond_slots(kx, c.Lx, c.x_pbc)));
+    LayerSums q = word_sums(kx2, k2, v2, g.z0, valid, bond_slots(kx2, c.Lx, c.x_pbc));
+    if (c.seam_same) q.b += seam_adjust(v, h.z0, g.S, g.z0, kSeam, c.neg, valid1);
+    add_lane_sums(acc_of(), q);
+  }
+}
+
+// One word (of R packed rows) per thread, or a pair: the shortest launch, for
+// films and film sets that do not fill the GPU for long.  The masks need
+// nothing of the lattice, so they are drawn before wait() -- while the previous
+// launch of the stream still runs -- and what follows it is the loads, some
+// forty operations and the store.
+template <int R, bool MEAS, class Wait, class AccOf>
+__device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep,
+                                            uint32_t at, bool meas, AccOf acc_of, Wait wait) {
+  constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  const uint32_t W = d.W, cols = d.cols[1];
+  const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
+  const uint32_t w = R == 1 ? at - rp * W : 0u;
+  const bool pair = rp < d.Lx;
+  const uint32_t rq = pair ? 0u : rp - d.Lx, q = fastdiv(rq, d.divc_m[1], d.divc_l[1]);
+  const bool on = pair || rq < d.Lx * cols;
+  const uint32_t kx = on ? (pair ? rp : q) + 1 : 1u, ky = pair || !on ? 1u : (rq - q * cols + 1) * R + 1;
+  const uint32_t kx2 = (d.y_mode == kYGapbc) ? (d.Lx + 1 - kx) : kx, ky2 = d.Ly - R + 1;
+  const bool any7 = __any_sync(0xFFFFFFFFu, on && (!d.cls[row_class(kx, d.Lx)].sym ||
+                                                   (pair && !d.cls[row_class(kx2, d.Lx)].sym)));
+  const uint32_t calls = w + 1 == W ? d.last_calls : 8u;
+  Drawn a{{0, 0, 0, 0, 0, 0, 0}}, b{{0, 0, 0, 0, 0, 0, 0}};
+#pragma unroll 1
+  for (uint32_t r = 0; r < 2; r++) {
+    if (r ? !pair : !on) continue;
+    const uint32_t k = r ? kx2 : kx, y = r ? ky2 : ky;
+    Drawn x;
+    draw_any<R, true>(x, any7, d.cls[row_class(k, d.Lx)], (k - 1) * d.Ly + y - 1, (k + y + 1 + colour) & 1u, w, calls,
+                      d.last_mask == 0xFFFFFFFFu, W > 1, sweep, d.rk0, d.rk1);
+    if (r) b = x;
+    else a = x;
+  }
+  wait();
+  // what the draws do not need is read from the descriptor only now
+  FilmCtx c;
+  film_ctx(c, d, pool, colour, sweep);
+  LayerSums r1, r2;
+  if (on) {
+    const ClassDraw &cl = d.cls[row_class(kx, c.Lx)], &cl2 = d.cls[row_class(kx2, c.Lx)];
+    const uint32_t valid1 = w + 1 == W ? c.last_mask : 0xFFFFFFFFu;  // one row's sites
+    uint32_t valid = valid1;
+    if (R > 1) {
+      valid = 0;
+#pragma unroll
+      for (uint32_t j = 0; j < R; j++) valid |= c.last_mask << (j * B);
+    }
+    Hood h, g;
+    fetch_rows<R>(c, kx, ky, w, h);
+    if (pair) fetch_rows<R>(c, kx2, ky2, w, g);
+    const Count k = count_up(h);
+    const uint32_t v = h.S ^ (decide(h, k, any7, a, cl) & valid);
+    store_rows<R>(c, kx, ky, w, v);
+    if (MEAS && meas) r1 = word_sums(kx, k, v, h.z0, valid, bond_slots(kx, c.Lx, c.x_pbc));
+    if (pair) {
+      // the partner's wrap neighbour is the word just decided where the seam
+      // joins one colour
+      if (c.seam_same) g.yp = (g.yp & ~(valid1 << kSeam)) | (((v ^ c.neg) & valid1) << kSeam);
+      const Count k2 = count_up(g);
+      const uint32_t v2 = g.S ^ (decide(g, k2, any7, b, cl2) & valid);
+      store_rows<R>(c, kx2, ky2, w, v2);
       if (MEAS && meas) {
-        LayerSums a, b;
-        update_fetched<FAST, true, PATHS4>(c, f, s_thr, s_alw, stash, &a, &b);
-        LayerSums& g = own ? g1 : g2;
-        g.m += a.m;
-        g.b += a.b;
-        if (b.layer != 0xFFFFFFFFu) {  // the partner row of row 1
-          g2.m += b.m;
-          g2.b += b.b;
-        }
-      } else {
-        update_fetched<FAST, false, PATHS4>(c, f, s_thr, s_alw);
+        r2 = word_sums(kx2, k2, v2, g.z0, valid, bond_slots(kx2, c.Lx, c.x_pbc));
+        if (c.seam_same) r2.b += seam_adjust(v, h.z0, g.S, g.z0, kSeam, c.neg, valid1);
       }
     }
   }
   if (MEAS && meas) {
-    add_layer_sums(acc_of(), g1);
-    add_lane_sums(acc_of(), g2);
+    add_layer_sums(acc_of(), r1);
+    add_lane_sums(acc_of(), r2);
   }
+}
+
+// The columns of a film's launch: thread `at` has word w of the rows ky, ky + 1, ...
+// of a layer (packed: of groups of R rows), and decides one after another.
+// Rows next to each other update opposite arrays and read each other's other
+// array, so a step loads five words where a lone row loads seven, the
+// addresses move by a row, and what depends on the layer is set up once.  The
+// first Lx * W columns are the pairs (update_pair); kept together, they fill
+// whole warps.
+//
+// A step's masks need nothing of the lattice, so the first step's are drawn
+// before wait() -- while the previous launch of the stream still runs.
+template <int R, bool MEAS, class Wait, class AccOf>
+__device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx& c, uint32_t at, uint32_t items,
+                                               bool meas, AccOf acc_of, Wait wait) {
+  constexpr uint32_t B = 8 / R;
+  const uint32_t W = c.W, cols = d.cols[items];
+  const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
+  const uint32_t w = R == 1 ? at - rp * W : 0u;
+  const uint32_t calls = w + 1 == W ? c.last_calls : 8u;
+  const uint32_t valid1 = w + 1 == W ? c.last_mask : 0xFFFFFFFFu;  // one row's sites
+  uint32_t valid = valid1;
+  if (R > 1) {
+    valid = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < R; j++) valid |= c.last_mask << (j * B);
+  }
+  // the column: groups g .. g1 - 1 of layer kx (none for a pair's thread)
+  const uint32_t rq = rp < c.Lx ? 0u : rp - c.Lx;
+  const uint32_t q = fastdiv(rq, d.divc_m[items], d.divc_l[items]);
+  const bool mine = rp >= c.Lx && rq < c.Lx * cols;
+  const uint32_t kx = mine ? q + 1 : 1u, len = column_len(items);
+  // an idle thread's range is empty, the drawing-only step included
+  const uint32_t g = mine ? 1 + (rq - q * cols) * len : 1u, g1 = mine ? min(g + len, c.Ly / R - 1) : 0u;
+  const ClassDraw& cl = c.cls[row_class(kx, c.Lx)];
+  const bool any7 = __any_sync(0xFFFFFFFFu, mine && !cl.sym);
+  if (rp < c.Lx) {
+    update_pair<R, MEAS>(c, rp + 1, w, calls, valid, valid1, meas, acc_of, wait);
+    if (!MEAS) return;
+  }
+  LayerSums sum;
+  // R = 1: pA is row ky's word in the array it updates, pB in the other; om and
+  // o0 are the words of row ky - 1 (array of pA) and of pB
+  uint32_t X = (kx + g * R + 2 + c.colour) & 1u;
+  const uint32_t base = ((kx - 1) * c.Ly + g * R) * W + w;
+  const uint32_t* pA = (X ? c.plane1 : c.plane0) + base;
+  const uint32_t* pB = (X ? c.plane0 : c.plane1) + base;
+  const ptrdiff_t dL = (ptrdiff_t)c.Ly * W;
+  const ptrdiff_t dxm = kx > 1 ? -dL : (ptrdiff_t)(c.Lx - 1) * dL, dxp = kx < c.Lx ? dL : -(ptrdiff_t)(c.Lx - 1) * dL;
+  const bool xm = kx > 1 || c.x_pbc, xp = kx < c.Lx || c.x_pbc;
+  // z: array 0 meets the word before, array 1 the word after, the row's ends joined
+  const int zp = w > 0 ? -1 : (int)W - 1, zn = w + 1 < W ? 1 : 1 - (int)W;
+  const uint32_t sp = w > 0 ? 31u : c.pos, sn = w + 1 < W ? 31u : c.pos;
+  uint32_t row = (kx - 1) * c.Ly + g * R;
+  uint32_t om = 0, o0 = 0;
+  auto walk = [&](auto general) {
+    constexpr bool k7 = decltype(general)::value;
+    Drawn a;
+    // step n loads row n's words, draws row n + 1's masks behind the loads, and
+    // decides row n; step g - 1 only draws
+#pragma unroll 1
+    for (uint32_t n = g - 1; n < g1; n++) {
+      const bool first = n == g - 1;
+      Hood h;
+      uint32_t e = 0;
+      if (!first) {
+        if constexpr (R > 1) {
+          fetch_rows<R>(c, kx, n * R + 1, w, h);
+        } else {
+          h.S = col_ld(c, pA, 0, X, 3);
+          h.ym = om;
+          h.z0 = o0;
+          h.yp = col_ld(c, pA, W, X, 4);
+          h.xm = xm ? col_ld(c, pA, dxm, X, 5) : 0u;
+          h.xp = xp ? col_ld(c, pA, dxp, X, 6) : 0u;
+          if (W > 1) e = col_ld(c, pB, X ? zn : zp, X ^ 1u, 7);
+        }
+      }
+      Drawn b;
+      if (n + 1 != g1) {
+        draw_any<R>(b, k7, cl, row, R == 1 && !first ? X ^ 1u : X, w, calls, c.last_mask == 0xFFFFFFFFu, W > 1,
+                        c.sweep, c.rk0, c.rk1);
+        row += R;
+      }
+      if (first) {
+        wait();
+        if (R == 1) {
+          om = col_ld(c, pA, -(ptrdiff_t)W, X, 1);
+          o0 = col_ld(c, pB, 0, X ^ 1u, 2);
+        }
+      } else {
+        if constexpr (R == 1) {
+          if (W == 1) h.zs = X ? packed_next(o0, 1u, c.pos) : packed_prev(o0, 1u, c.pos);
+          else h.zs = X ? shift_next(o0, 0u) | ((e & 1u) << sn) : shift_prev(o0, (e >> sp) << 31);
+        }
+        const Count k = count_up(h);
+        const uint32_t v = h.S ^ (decide(h, k, k7, a, cl) & valid);
+        if (MEAS && meas) {
+          const LayerSums r = word_sums(kx, k, v, h.z0, valid, bond_slots(kx, c.Lx, c.x_pbc));
+          sum.layer = r.layer;
+          sum.m += r.m;
+          sum.b += r.b;
+        }
+        if constexpr (R > 1) {
+          store_rows<R>(c, kx, n * R + 1, w, v);
+        } else {
+          col_st(c, pA, X, v);
+          const uint32_t* p = pA + W;
+          pA = pB + W;
+          pB = p;
+          om = o0;
+          o0 = h.yp;
+          X ^= 1u;
+        }
+      }
+      a = b;
+    }
+  };
+  if (any7) walk(std::true_type{});
+  else walk(std::false_type{});
+  if (MEAS && meas) {
+    __syncwarp();
+    add_layer_sums(acc_of(), sum);
+  }
+  wait();  // a thread without a word too: the launch must not end before its predecessor
 }
 
 }  // namespace
 
-// The words of one block of words_per_block(ITEMS) consecutive words: each
-// thread fetches its ITEMS words (kFilmThreads apart) before deciding any;
-// ITEMS = 0: four lanes per word (kFilmThreads / 4 words).  MEAS and meas
-// (half-sweep 1 of a sweep after which the film records): the words' record
-// sums go into the film's per-layer accumulators acc_of() (a pointer made
-// where it is used, not kept across the draws); s_stash holds kStashSlots
-// words per thread.
-template <bool FAST, uint32_t ITEMS, bool MEAS, bool PATHS4, bool H3, bool PK, typename AccOf>
-__device__ __forceinline__ void sweep_block(const FilmCtx& c, uint32_t first, uint32_t items, uint32_t dwm,
-                                            uint32_t dwl, uint32_t dym, uint32_t dyl,
-                                            const uint32_t* __restrict__ s_thr, const uint32_t* __restrict__ s_alw,
-                                            bool meas, AccOf acc_of, uint32_t* s_stash) {
-  uint32_t* stash = s_stash + threadIdx.x * kStashSlots;
-  if (ITEMS == 0) {
-    const uint32_t item = first + (threadIdx.x >> 2);
-    const bool on = item < items;
-    const uint32_t gmask = __ballot_sync(0xFFFFFFFFu, on);
-    Fetched f;
-    if (on) {
-      uint32_t kx, ky, w;
-      item_word(c, item, dwm, dwl, dym, dyl, kx, ky, w);
-      fetch_word(c, kx, ky, w, f);
-    }
-    LayerSums r1, r2;
-    if (MEAS && meas) {
-      update_fetched_quarter<FAST, true>(c, f, on, threadIdx.x & 3u, gmask, s_thr, s_alw, stash, r1, r2);
-      add_layer_sums(acc_of(), r1);
-      add_lane_sums(acc_of(), r2);
-    } else {
-      update_fetched_quarter<FAST, false>(c, f, on, threadIdx.x & 3u, gmask, s_thr, s_alw, stash, r1, r2);
-    }
-    return;
-  }
-  constexpr uint32_t NI = ITEMS == 0 ? 1 : ITEMS;
-  if (PK && ITEMS == 1 && c.pack > 1) {  // the same for the whole film (the block)
-    // fast-table plain launches decide a group's rows at once; the summing
-    // and exact-table launches, whose registers have no room for the packed
-    // body, take the group's rows one after another
-    if (FAST && !MEAS) {
-      if (c.pack == 4) sweep_block_packed<4, FAST>(c, first, items, dym, dyl, s_thr, s_alw);
-      else sweep_block_packed<2, FAST>(c, first, items, dym, dyl, s_thr, s_alw);
-    } else {
-      sweep_block_rows<FAST, MEAS, PATHS4>(c, first, items, dym, dyl, s_thr, s_alw, meas, acc_of, stash);
-    }
-    return;
-  }
-  Fetched fw[NI];
-  bool mine[NI];
-#pragma unroll
-  for (uint32_t it = 0; it < NI; it++) {
-    const uint32_t item = first + threadIdx.x + it * kFilmThreads;
-    mine[it] = item < items;
-    if (mine[it]) {
-      uint32_t kx, ky, w;
-      item_word(c, item, dwm, dwl, dym, dyl, kx, ky, w);
-      fetch_word(c, kx, ky, w, fw[it]);
-    }
-  }
-  if (MEAS && meas) {
-#pragma unroll
-    for (uint32_t it = 0; it < NI; it++) {
-      LayerSums r1, r2;
-      if (mine[it]) update_fetched<FAST, true, PATHS4, H3>(c, fw[it], s_thr, s_alw, stash, &r1, &r2);
-      add_layer_sums(acc_of(), r1);
-      add_lane_sums(acc_of(), r2);
-    }
-    return;
-  }
-#pragma unroll
-  for (uint32_t it = 0; it < NI; it++)
-    if (mine[it]) update_fetched<FAST, false, PATHS4, H3>(c, fw[it], s_thr, s_alw);
-}
-
-// Half-sweep of every film of a launch: block b handles words_per_block(ITEMS)
-// words of film owner[b], whose descriptor is staged in shared memory.  FAST:
-// no film of the launch has a reachable thr = 0 entry (the compare-only
-// table); otherwise every film takes the exact variant (which, at two words
-// per thread, needs the registers of one block per SM fewer, and so does its
-// recording form at one word).  At one word per thread the plain and
-// record-writing forms fit one block per SM more (kMultiMinBlocks1), so that a
-// small film set's half-sweep is one wave where it would spill into a second.
-// MODE kUpdAccumulate: the half-sweep 1 launch
-// of a sweep after which some film records; those films add their record
-// sums into their accumulators in `part`.  MODE kUpdWriteRecord: a half-sweep
-// 0 launch right after such a sweep; the last block of each film that
-// recorded after `rec_done` sweeps writes that record (write_record) before
-// its update, so the write overlaps the launch's other blocks.  The last
-// block holds the film's ragged end, so it has the fewest words; the first
-// ones hold the pair items, whose threads also update the wrap partner.
+// Half-sweep of every film of a launch: block b handles kFilmThreads columns of
+// film owner[b], whose descriptor is staged in shared memory.  MODE kUpdAccumulate: the half-sweep 1 launch of a sweep
+// after which some film records; those films add their record sums into their
+// accumulators in `part`.  MODE kUpdWriteRecord: a half-sweep 0 launch right
+// after such a sweep; the last block of each film that recorded after
+// `rec_done` sweeps writes that record (write_record) before its update, so
+// the write overlaps the launch's other blocks.  The last block holds the
+// film's ragged end, so it has the fewest words; the first ones hold the pair
+// items, whose threads also update the wrap partner.
+//
+// The masks are drawn before pdl_wait, from the film's sweep counter.  Only
+// advance_kernel writes that, between chunks: the first launch of a chunk
+// (`first`) waits before it reads the counter and lets its successor start
+// only then, so every later launch of the chunk starts after the write.
 enum : uint32_t { kUpdPlain = 0, kUpdAccumulate = 1, kUpdWriteRecord = 2 };
 
-template <uint32_t ITEMS>
-__device__ __forceinline__ uint32_t last_update_block(const FilmDesc& d) {
-  return d.upd_block_begin + (grid_items(d, ITEMS) + words_per_block(ITEMS) - 1) / words_per_block(ITEMS) - 1;
+__device__ __forceinline__ uint32_t last_update_block(const FilmDesc& d, uint32_t items) {
+  return d.upd_block_begin + update_blocks(d, items) - 1;
 }
 
-template <bool FAST, uint32_t ITEMS, uint32_t MODE, bool PK = false>
-__global__ void __launch_bounds__(kFilmThreads, PK ? (MODE == kUpdAccumulate ? (FAST ? kMultiMinBlocks - 1
-                                                                                    : kMultiMinBlocks - 2)
-                                                                           : kMultiMinBlocks)
-                                                : (ITEMS == 1 && MODE != kUpdAccumulate) ? kMultiMinBlocks1
-                                                : (FAST || (ITEMS < 2 && MODE != kUpdAccumulate))
-                                                    ? kMultiMinBlocks : kMultiMinBlocks - 1)
+template <uint32_t MODE, bool PK, bool ONE>
+__global__ void __launch_bounds__(kFilmThreads, multi_min_blocks(ONE, MODE == kUpdAccumulate, PK))
 update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ owner,
               const LaunchHdr* __restrict__ hdr, uint32_t* __restrict__ pool, uint32_t colour, uint32_t k,
-              int64_t* __restrict__ part, int64_t* __restrict__ records, uint32_t rec_done) {
+              uint32_t items, int64_t* __restrict__ part, int64_t* __restrict__ records, uint32_t rec_done,
+              uint32_t first) {
   constexpr bool MEAS = MODE == kUpdAccumulate;
   constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
   static_assert(sizeof(FilmDesc) % 16 == 0, "descriptor copied as uint4");
   __shared__ __align__(16) FilmDesc s_d;
-  __shared__ __align__(16) uint32_t s_alw[FAST ? 1 : 64];
-  __shared__ __align__(16) uint32_t s_lo[64];
-  __shared__ uint32_t s_stash[MEAS ? kStashSlots * kFilmThreads : 1];
   __shared__ int64_t s_red[MODE == kUpdWriteRecord ? kFilmThreads / 32 : 1];
   __shared__ uint32_t s_slot;
+  if (first) pdl_wait();
   pdl_trigger();
-  const uint32_t nvb = hdr->upd_blocks;
-  for (uint32_t vb = blockIdx.x; vb < nvb; vb += gridDim.x) {
-    const uint32_t f = owner[vb];  // the same for every thread of the block
-    __syncthreads();
-    const uint4* src = reinterpret_cast<const uint4*>(films + f);
-    uint4* dst = reinterpret_cast<uint4*>(&s_d);
-    for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
-    __syncthreads();
-    for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) {
-      const bool a = (s_d.always[i >> 4] >> (i & 15)) & 1u;
-      if (!FAST) s_alw[i] = a ? 0xFFFFFFFFu : 0u;
-      s_lo[i] = FAST ? (a ? 0xFFFFFFFFu : s_d.thr[i >> 4][i & 15] - 1u) : s_d.thr[i >> 4][i & 15];
-    }
-    __syncthreads();
-    if (!s_d.active) continue;
-    // The owner table, the descriptor and the table above are written by the
-    // host before the launch; the lattice and the film's sweep counter may
-    // still be written by the previous kernel of the stream (its blocks run
-    // while these stage).  Wait for it (a no-op after the first time), then
-    // read the counter again, around L1 (the staged copy may predate the
-    // wait).
+  // owner table and descriptor are written by the host before the launch
+  const uint32_t vb = blockIdx.x;
+  const uint32_t f = owner[vb];  // the same for every thread of the block
+  const uint4* src = reinterpret_cast<const uint4*>(films + f);
+  uint4* dst = reinterpret_cast<uint4*>(&s_d);
+  for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
+  __syncthreads();
+  if (threadIdx.x == 0) s_d.sweep = __ldcg(&films[f].sweep);  // around L1: an earlier chunk's line may be there
+  __syncthreads();
+  const uint32_t t = s_d.sweep + k;
+  if (!s_d.active || t > s_d.sweep_end || (MODE != kUpdWriteRecord && t >= s_d.sweep_end)) {
+    pdl_wait();  // the launch must not end before its predecessor has
+    return;
+  }
+  FilmCtx c;
+  film_ctx(c, s_d, pool, colour, t);
+  const bool meas = MEAS && measured_now(s_d, k + 1, 0);
+  const FilmDesc* sd = &s_d;
+  auto acc_of = [part, sd]() { return reinterpret_cast<unsigned long long*>(part + acc_offset(*sd)); };
+  auto wait = [&]() { pdl_wait(); };
+  if (MODE == kUpdWriteRecord && vb == last_update_block(s_d, items) && records_after(s_d, s_d.sweep, rec_done)) {
     pdl_wait();
-    if (threadIdx.x == 0) s_d.sweep = __ldcg(&films[f].sweep);
-    __syncthreads();
-    if (MODE == kUpdWriteRecord && vb == last_update_block<ITEMS>(s_d) && records_after(s_d, s_d.sweep, rec_done))
-      write_record(const_cast<FilmDesc*>(films + f), s_d, s_d.sweep, part, records, rec_done, s_red, &s_slot);
-    if (s_d.sweep + k >= s_d.sweep_end) continue;
-    FilmCtx c;
-    c.Lx = s_d.Lx; c.Ly = s_d.Ly; c.n = s_d.n; c.W = s_d.W; c.Wp = s_d.Wp;
-    c.plane_words = s_d.Lx * s_d.Ly * s_d.Wp;
-    c.y_mode = s_d.y_mode; c.x_pbc = s_d.x_pbc; c.rk0 = s_d.rk0; c.rk1 = s_d.rk1;
-    c.last_mask = s_d.last_mask; c.last_calls = s_d.last_calls;
-    c.colour = colour; c.sweep = s_d.sweep + k;
-    c.plane0 = pool + s_d.spin_off;
-    c.plane1 = c.plane0 + (size_t)c.Lx * c.Ly * c.Wp;
-    c.seam_same = seam_joins_one_colour(c.Lx, c.Ly, c.y_mode);
-    const bool meas = MEAS && colour == 1 && measured_now(s_d, k + 1, 0);
-    const FilmDesc* sd = &s_d;
-    auto acc_of = [part, sd]() { return reinterpret_cast<unsigned long long*>(part + acc_offset(*sd)); };
-    const uint32_t first = (vb - s_d.upd_block_begin) * words_per_block(ITEMS);
-    // two words per thread, and the exact table: the register budget keeps
-    // the two-path decision
-    // packed thin films: group items and their divisor
-    c.pack = PK ? s_d.pack : 1u;
-    const bool pk = c.pack > 1;
-    sweep_block<FAST, ITEMS, MEAS, FAST && ITEMS != 2, false, PK>(
-        c, first, pk ? s_d.pk_items : s_d.upd_items, s_d.divw_m, s_d.divw_l, pk ? s_d.pk_divm : s_d.divy_m,
-        pk ? s_d.pk_divl : s_d.divy_l, s_lo, s_alw, meas, acc_of, s_stash);
+    write_record(const_cast<FilmDesc*>(films + f), s_d, s_d.sweep, part, records, rec_done, s_red, &s_slot);
+  }
+  if (MODE == kUpdWriteRecord && t >= s_d.sweep_end) {
+    pdl_wait();
+    return;
+  }
+  const uint32_t at = (vb - s_d.upd_block_begin) * kFilmThreads + threadIdx.x;
+  if (ONE) {
+    if (PK && s_d.pack == 4) update_word<4, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_word<2, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
+    else update_word<1, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
+  } else {
+    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    else update_columns<1, MEAS>(s_d, c, at, items, meas, acc_of, wait);
   }
 }
 
 // Single-film half-sweep.  The descriptor is a __grid_constant__ kernel
 // parameter, so every per-film constant (round keys included) is read straight
-// from the constant bank; block b updates words b * words_per_block(ITEMS)
-// onwards.  MEAS: half-sweep 1 before a record, whose sums go into the
-// film's accumulators acc.
-template <bool FAST, uint32_t ITEMS, bool MEAS, bool PK = false>
-__global__ void __launch_bounds__(kFilmThreads, PK && MEAS ? kFilmMinBlocks - 1 : kFilmMinBlocks)
+// from the constant bank, and the sweep is known before pdl_wait.  MEAS:
+// half-sweep 1 before a record, whose sums go into the film's accumulators
+// acc.
+template <int R, bool MEAS, bool ONE>
+__global__ void __launch_bounds__(kFilmThreads, film_min_blocks(R, MEAS, ONE))
 update_film_kernel(const __grid_constant__ FilmDesc d, uint32_t* __restrict__ pool, uint32_t colour,
-                   uint32_t sweep, int64_t* __restrict__ acc) {
+                   uint32_t sweep, uint32_t items, int64_t* __restrict__ acc) {
   pdl_trigger();
-  __shared__ __align__(16) uint32_t s_thr[64];
-  __shared__ __align__(16) uint32_t s_alw[64];
-  __shared__ uint32_t s_stash[MEAS ? kStashSlots * kFilmThreads : 1];
-  for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) {
-    const bool a = (d.always[i >> 4] >> (i & 15)) & 1u;
-    s_thr[i] = FAST ? (a ? 0xFFFFFFFFu : d.thr[i >> 4][i & 15] - 1u) : d.thr[i >> 4][i & 15];
-    s_alw[i] = a ? 0xFFFFFFFFu : 0u;
-  }
-  __syncthreads();
-  pdl_wait();  // the table above needs nothing from the previous grid
   FilmCtx c;
-  c.Lx = d.Lx; c.Ly = d.Ly; c.n = d.n; c.W = d.W; c.Wp = d.Wp;
-  c.plane_words = d.Lx * d.Ly * d.Wp;
-  c.y_mode = d.y_mode; c.x_pbc = d.x_pbc; c.rk0 = d.rk0; c.rk1 = d.rk1;
-  c.last_mask = d.last_mask; c.last_calls = d.last_calls;
-  c.colour = colour; c.sweep = sweep;
-  c.plane0 = pool + d.spin_off;
-  c.plane1 = c.plane0 + (size_t)d.Lx * d.Ly * d.Wp;
-  c.seam_same = seam_joins_one_colour(d.Lx, d.Ly, d.y_mode);
+  film_ctx(c, d, pool, colour, sweep);
   auto acc_of = [acc]() { return reinterpret_cast<unsigned long long*>(acc); };
-  // the Philox head with round 3's product hoisted (PhiloxRow3) wherever the
-  // registers allow it: not in the recording launch
-  c.pack = PK ? d.pack : 1u;
-  const bool pk = c.pack > 1;
-  sweep_block<FAST, ITEMS, MEAS, true, !MEAS, PK>(c, blockIdx.x * words_per_block(ITEMS), pk ? d.pk_items : d.upd_items,
-                                              d.divw_m, d.divw_l, pk ? d.pk_divm : d.divy_m,
-                                              pk ? d.pk_divl : d.divy_l, s_thr, s_alw, MEAS, acc_of, s_stash);
+  auto wait = [&]() { pdl_wait(); };
+  const uint32_t at = blockIdx.x * kFilmThreads + threadIdx.x;
+  if (ONE) update_word<R, MEAS>(d, pool, colour, sweep, at, MEAS, acc_of, wait);
+  else update_columns<R, MEAS>(d, c, at, items, MEAS, acc_of, wait);
 }
 
 // ------------------------------------------------------------ measurement
@@ -1259,438 +870,821 @@ __global__ void advance_kernel(FilmDesc* __restrict__ films, const LaunchHdr* __
   }
 }
 
-// ------------------------------------------------------------ resident path
+// ------------------------------------------------------------- slab path
 
-// All sweeps of a run for one small film per block.  The planes are copied
-// into shared memory once (row stride W), each half-sweep is the same block
-// body as the grid kernels followed by a block barrier (the next colour reads
-// what this one wrote), the records of the run go straight into the film's
-// ring, and the planes, sweep and rec_next are written back at the end.
-template <bool FAST>
-__global__ void __launch_bounds__(kResidentThreads, 1)
-resident_kernel(FilmDesc* __restrict__ films, uint32_t* __restrict__ pool, int64_t* __restrict__ records,
-                uint32_t n_sweeps) {
-  extern __shared__ __align__(16) uint32_t s_planes[];
-  constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
-  __shared__ __align__(16) FilmDesc s_d;
-  __shared__ __align__(16) uint32_t s_thr[64];
-  __shared__ __align__(16) uint32_t s_alw[64];
-  __shared__ uint32_t s_stash[kStashSlots * kResidentThreads];
-  __shared__ int s_tot[2];  // B and M of the record being summed
-  pdl_trigger();
-  pdl_wait();
-  FilmDesc* Fg = films + blockIdx.x;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(Fg);
-    uint4* dst = reinterpret_cast<uint4*>(&s_d);
-    for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
-  }
-  __syncthreads();
-  for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) {
-    const bool a = (s_d.always[i >> 4] >> (i & 15)) & 1u;
-    s_thr[i] = FAST ? (a ? 0xFFFFFFFFu : s_d.thr[i >> 4][i & 15] - 1u) : s_d.thr[i >> 4][i & 15];
-    s_alw[i] = a ? 0xFFFFFFFFu : 0u;
-  }
-  if (!s_d.active) return;  // the same for the whole block
-  const uint32_t Lx = s_d.Lx, Ly = s_d.Ly, W = s_d.W, Wp = s_d.Wp;
-  const uint32_t words = Lx * Ly * W;  // one plane in shared memory
-  int* s_m = reinterpret_cast<int*>(s_planes + 2 * words);
-  uint32_t* g0 = pool + s_d.spin_off;
-  uint32_t* g1 = g0 + (size_t)Lx * Ly * Wp;
-  for (uint32_t i = threadIdx.x; i < 2 * words; i += blockDim.x) {
-    const uint32_t X = i >= words ? 1u : 0u;
-    const uint32_t rw = i - X * words, r = rw / W, w = rw - r * W;
-    s_planes[i] = ISG_LD(X ? g1 : g0, (size_t)r * Wp + w, (size_t)Lx * Ly * Wp, 41);
-  }
-  for (uint32_t kx = threadIdx.x; kx < Lx; kx += blockDim.x) s_m[kx] = 0;
-  if (threadIdx.x < 2) s_tot[threadIdx.x] = 0;
-  __syncthreads();
-  FilmCtx c;
-  c.Lx = Lx; c.Ly = Ly; c.n = s_d.n; c.W = W; c.Wp = W;
-  c.plane_words = words;
-  c.y_mode = s_d.y_mode; c.x_pbc = s_d.x_pbc; c.rk0 = s_d.rk0; c.rk1 = s_d.rk1;
-  c.last_mask = s_d.last_mask; c.last_calls = s_d.last_calls;
-  c.plane0 = s_planes;
-  c.plane1 = s_planes + words;
-  c.seam_same = seam_joins_one_colour(Lx, Ly, s_d.y_mode);
-  c.pack = 1;  // the resident kernel updates single rows
-  const uint32_t items = s_d.upd_items;
-  const uint32_t m_every = s_d.measure_every;
-  uint32_t rec_next = s_d.rec_next;
-  uint32_t done = 0;
-  for (uint32_t k = 0; k < n_sweeps; k++) {
-    const uint32_t t = s_d.sweep + k;
-    if (t >= s_d.sweep_end) break;
-    c.sweep = t;
-    // half-sweep 1 of a sweep after which the film records also sums the
-    // record (as the grid kernels do) into s_m and s_tot
-    const bool rec_now = m_every != 0 && (t + 1) % m_every == 0;
-    for (uint32_t colour = 0; colour < 2; colour++) {
-      c.colour = colour;
-      if (colour == 1 && rec_now) {
-        uint32_t* stash = s_stash + threadIdx.x * kStashSlots;
-        for (uint32_t base = 0; base < items; base += blockDim.x) {
-          const uint32_t item = base + threadIdx.x;
-          LayerSums r1, r2;
-          if (item < items) {
-            uint32_t kx, ky, w;
-            item_word(c, item, s_d.divw_m, s_d.divw_l, s_d.divy_m, s_d.divy_l, kx, ky, w);
-            Fetched f;
-            fetch_word(c, kx, ky, w, f);
-            update_fetched<FAST, true>(c, f, s_thr, s_alw, stash, &r1, &r2);
-          }
-          add_layer_sums_shared(s_m, s_tot, r1);
-          add_layer_sums_shared(s_m, s_tot, r2);
-        }
-      } else {
-        for (uint32_t item = threadIdx.x; item < items; item += blockDim.x) {
-          uint32_t kx, ky, w;
-          item_word(c, item, s_d.divw_m, s_d.divw_l, s_d.divy_m, s_d.divy_l, kx, ky, w);
-          Fetched f;
-          fetch_word(c, kx, ky, w, f);
-          update_fetched<FAST>(c, f, s_thr, s_alw);
-        }
-      }
-      __syncthreads();
-    }
-    done = k + 1;
-    if (!rec_now) continue;
-    // record of sweep t + 1; every thread clears what it read, and the next
-    // sweep's first barrier orders that before the next sums
-    const uint32_t slot = s_d.rec_cap ? rec_next % s_d.rec_cap : 0u;
-    int64_t* rec = records + s_d.rec_off + (size_t)slot * (5 + Lx);
-    for (uint32_t kx = threadIdx.x; kx < Lx; kx += blockDim.x) {
-      const int v = s_m[kx];
-      s_m[kx] = 0;
-      rec[5 + kx] = v;
-      if (kx == 0) rec[3] = v;
-      if (kx == Lx - 1) rec[4] = v;
-    }
-    if (threadIdx.x == 0) {
-      rec[0] = (int64_t)t + 1;
-      rec[1] = s_tot[0];
-      rec[2] = s_tot[1];
-      s_tot[0] = 0;
-      s_tot[1] = 0;
-    }
-    rec_next++;
-  }
-  for (uint32_t i = threadIdx.x; i < 2 * words; i += blockDim.x) {
-    const uint32_t X = i >= words ? 1u : 0u;
-    const uint32_t rw = i - X * words, r = rw / W, w = rw - r * W;
-    ISG_ST(X ? g1 : g0, (size_t)r * Wp + w, (size_t)Lx * Ly * Wp, 42, s_planes[i]);
-  }
-  if (threadIdx.x == 0) {
-    Fg->sweep = s_d.sweep + done;
-    Fg->rec_next = rec_next;
-  }
+// Films held in shared memory for every sweep of a call: one CTA holds a film
+// (C = 1), or a thread-block cluster of C CTAs holds it in distributed shared
+// memory, CTA r layers kx - 1 in [r Lx / C, (r + 1) Lx / C).  Only a film's own
+// CTAs meet between its half-sweeps, at a block or cluster barrier; films
+// never wait for one another and no launch boundary falls between them.
+//
+// Layout.  In shared memory the two arrays of a row are sorted by colour, not
+// by z parity: plane c holds what half-sweep c updates, so a word's six
+// neighbour words all sit in the other plane (the wrap bonds of a same-colour
+// seam apart), and rows of thin films are packed R to a word (fetch_rows'
+// bit order).  A layer is G = Ly / R groups of W words.
+//
+// A word's masks are drawn between the barrier's arrival and the wait for it
+// (one CTA: before the block barrier), so that the barrier hides behind the
+// draws of the next half-sweep, and what follows it is loads from shared
+// memory and bit logic.
+//
+// Within a half-sweep no word is read that another thread writes (the
+// checkerboard; a partner row's wrap neighbour comes from the register of the
+// thread that has just decided it), so plain loads suffice, and the
+// barrier's release/acquire orders one half-sweep's stores before the next
+// one's loads.
+namespace {
+
+template <bool CL>
+__device__ __forceinline__ uint32_t sld(uint32_t addr) {
+  uint32_t v;
+  if (CL) asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  else asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
 }
-
-// ------------------------------------------------------------- cluster-resident path
-
-// Films held in distributed shared memory.  One thread-block cluster of C
-// CTAs keeps one film for every sweep of a call: CTA r holds layers
-// kx - 1 in [r Lx / C, (r + 1) Lx / C) of both planes (row stride W), and
-// the cluster barrier between half-sweeps is the only synchronisation, so
-// films never wait for one another and no launch boundary falls between
-// half-sweeps.  A word's x-neighbour layer across a slab boundary, and the
-// mirrored layer of an Eq. 11 partner row, sit in a peer CTA: every access
-// goes through a table of the generic addresses of all layers of the film
-// (the own CTA's shared window, or a peer's mapped into the cluster window),
-// so such a word is a distributed-shared-memory load, and the partner's
-// update a remote store.  Within a half-sweep no word is read that another
-// thread writes (the checkerboard; the partner row reads the ky = 1 word its
-// own thread has just written), so plain loads suffice, and the barrier's
-// release/acquire orders one half-sweep's stores before the next one's loads.
-
-// The words of fetch_word for word w of row (kx, ky), from the layer table
-// lp[X * Lx + kx - 1] (plane X, 0-based layer kx - 1).
-__device__ __forceinline__ void fetch_word_cl(const FilmCtx& c, uint32_t* const* lp, uint32_t kx, uint32_t ky,
-                                              uint32_t w, Fetched& f) {
-  const uint32_t Lx = c.Lx, Ly = c.Ly, W = c.W;
-  const uint32_t X = (kx + ky + 1 + c.colour) & 1u;
-  uint32_t* const* LP = lp + X * Lx;
-  uint32_t* const* LQ = lp + (X ^ 1u) * Lx;
-  const uint32_t rbase = (ky - 1) * W, base = rbase + w;
-  const uint32_t lim = Ly * W;  // words of one layer
-  const uint32_t* P = LP[kx - 1];
-  const uint32_t* Q = LQ[kx - 1];
-  const uint32_t gkx = (c.y_mode == kYGapbc) ? (Lx - kx) : (kx - 1);  // 0-based layer of the wrap row
-  f.kx = kx; f.ky = ky; f.w = w;
-  f.S = ISG_LD(P, base, lim, 61);
-  f.xm = (kx > 1) ? ISG_LD(LP[kx - 2], base, lim, 62) : (c.x_pbc ? ISG_LD(LP[Lx - 1], base, lim, 63) : 0u);
-  f.xp = (kx < Lx) ? ISG_LD(LP[kx], base, lim, 64) : (c.x_pbc ? ISG_LD(LP[0], base, lim, 65) : 0u);
-  f.ym = (ky > 1) ? ISG_LD(P, base - W, lim, 66) : ISG_LD(LP[gkx], (Ly - 1) * W + w, lim, 67);
-  f.yp = (ky < Ly) ? ISG_LD(P, base + W, lim, 68) : ISG_LD(LP[gkx], w, lim, 69);
-  f.z0 = ISG_LD(Q, base, lim, 70);
-  if (X == 0)  // previous word, or the row's last
-    f.za = (w > 0) ? ISG_LD(Q, base - 1, lim, 71) : ISG_LD(Q, rbase + W - 1, lim, 72);
-  else  // next word, or the row's first
-    f.za = (w + 1 < W) ? ISG_LD(Q, base + 1, lim, 73) : ISG_LD(Q, rbase, lim, 74);
-  f.zf = ISG_LD(Q, rbase, lim, 75);
+template <bool CL>
+__device__ __forceinline__ void sst(uint32_t addr, uint32_t v) {
+  if (CL) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+  else asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-
-__device__ __forceinline__ void store_word_cl(const FilmCtx& c, uint32_t* const* lp, const Fetched& f, uint32_t v) {
-  const uint32_t X = (f.kx + f.ky + 1 + c.colour) & 1u;
-  ISG_ST(lp[X * c.Lx + f.kx - 1], (f.ky - 1) * c.W + f.w, c.Ly * c.W, 76, v);
+template <bool CL>
+__device__ __forceinline__ void sadd(uint32_t addr, int v) {
+  if (CL) asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+  else asm volatile("red.relaxed.cta.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-
-// update_fetched over the layer table.
-template <bool FAST, bool MEAS>
-__device__ __forceinline__ void update_fetched_cl(const FilmCtx& c, uint32_t* const* lp, const Fetched& f,
-                                                  const uint32_t* s_thr, const uint32_t* s_alw,
-                                                  uint32_t* stash = nullptr, LayerSums* r1 = nullptr,
-                                                  LayerSums* r2 = nullptr) {
-  const uint32_t fl = decide_any<FAST, false, MEAS, true>(c, f, s_thr, s_alw, 0, stash);
-  const uint32_t v = f.S ^ fl;
-  store_word_cl(c, lp, f, v);
-  if (MEAS) *r1 = word_sums(c, f.kx, f.w, fl, v, stash);
-  if (f.ky == 1) {
-    const uint32_t kx2 = (c.y_mode == kYGapbc) ? (c.Lx + 1 - f.kx) : f.kx;
-    Fetched g;
-    fetch_word_cl(c, lp, kx2, c.Ly, f.w, g);
-    if (MEAS) stash[4] = c.seam_same ? (uint32_t)seam_adjust(c, f.w, v, stash[3], g) : 0u;
-    const uint32_t fl2 = decide_any<FAST, false, MEAS, true>(c, g, s_thr, s_alw, 0, stash);
-    const uint32_t v2 = g.S ^ fl2;
-    store_word_cl(c, lp, g, v2);
-    if (MEAS) {
-      *r2 = word_sums(c, kx2, g.w, fl2, v2, stash);
-      r2->b += (int)stash[4];
-    }
-  }
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t v;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(v) : "r"(addr), "r"(rank));
+  return v;
 }
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Word of the CTA's update item `item`: its nl layers from layer a + 1 on,
-// the ky = 1 words first (their threads also update the wrap partner), then
-// rows ky = 2 .. Ly-1 layer by layer (item_word on a slab of layers).
-__device__ __forceinline__ void slab_item_word(const FilmDesc& d, uint32_t a, uint32_t nl, uint32_t item,
-                                               uint32_t& kx, uint32_t& ky, uint32_t& w) {
-  const uint32_t rp = fastdiv(item, d.divw_m, d.divw_l);
-  w = item - rp * d.W;
-  const bool pair = rp < nl;
-  const uint32_t rq = pair ? 0u : rp - nl;
-  const uint32_t q = fastdiv(rq, d.divy_m, d.divy_l);
-  kx = a + (pair ? rp : q) + 1;
-  ky = pair ? 1u : rq - q * (d.Ly - 2) + 2;
+#ifdef ISING_CHECKED
+__device__ __forceinline__ uint32_t in_layer(uint32_t idx, uint32_t lim, uint32_t site) {
+  return oob(idx, lim, site) ? 0u : idx;
 }
+#else
+__device__ __forceinline__ uint32_t in_layer(uint32_t idx, uint32_t, uint32_t) { return idx; }
+#endif
 
-// Rounds of a CTA's half-sweep: a pair item (a ky = 1 word and its wrap
-// partner) is two words of work, so its thread spends two rounds on it and
-// takes one regular item fewer, and no warp runs a round longer than the
-// others.  With P = q T + s pair items over T threads, thread t draws pair
-// items t, t + T, ... (q + [t < s] of them) in rounds 0, 2, ..., and the
-// P' regular items fill the remaining (thread, round) slots round by round:
-// R = max(2 ceil(P / T), ceil((P' + 2 P) / T)) rounds hold them all.
-struct SlabRounds {
-  uint32_t P, q, s, R;
+// A film on its CTA; kept in shared memory, where it costs no registers.
+struct Slab {
+  uint32_t Lx, Ly, W, G, lw, pw;  // lw = G W words of a layer; pw: words of a local plane
+  uint32_t a, nl;                 // first own layer (0-based), own layers
+  uint32_t planes;                // shared address of the own planes
+  const uint32_t* lp;             // address of layer k's plane 0 in its CTA (cluster window)
+  const uint32_t* lm;             // address of layer k's sum in its CTA
+  uint32_t y_mode, x_pbc, last_mask, last_calls, pos, neg, seam_same;
+  uint32_t len, cols, turns;      // slab_columns: words of a column, columns, columns per thread
 };
 
-__device__ __forceinline__ SlabRounds slab_rounds(uint32_t P, uint32_t P2, uint32_t T) {
-  SlabRounds o;
-  o.P = P;
-  o.q = P / T;
-  o.s = P - o.q * T;
-  const uint32_t rp = 2 * ((P + T - 1) / T), rw = (P2 + 2 * P + T - 1) / T;
-  o.R = rp > rw ? rp : rw;
+// The packed word of R rows from the words of plane p, group g (index i in the
+// layer) and, for the wrapped slot, `wrap`.
+// Own item (kx, group g, word w): every word but the x neighbours is in the
+// own planes.  CL: the x neighbours through the layer table.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_fetch(const Slab& s, uint32_t c, bool own, uint32_t kx, uint32_t g, uint32_t w, Hood& h) {
+  constexpr uint32_t B = 8 / R, kLow = slot_mask<R>(), kTop = kLow << (8 - B), kFirst = first_bits<R>();
+  const uint32_t o = c ^ 1u, k = kx - 1, lim = s.lw;
+  const uint32_t X = (kx + g * R + 2 + c) & 1u;  // parity array of the group's first row (ky = g R + 1)
+  const uint32_t pb = 4 * s.pw;                    // plane stride in bytes
+  const uint32_t i = in_layer(g * s.W + w, lim, 61);
+  const uint32_t base = CL && !own ? s.lp[k] : s.planes + 4 * (k - s.a) * s.lw;
+  const uint32_t bS = base + c * pb, bO = base + o * pb;
+  auto ld = [&](uint32_t at) { return CL && !own ? sld<true>(at) : sld<false>(at); };
+  h.S = ld(bS + 4 * i);
+  h.z0 = ld(bO + 4 * i);
+  const uint32_t km = k > 0 ? k - 1 : s.Lx - 1, kp = k + 1 < s.Lx ? k + 1 : 0u;
+  const uint32_t xo = o * pb + 4 * i;
+  if (CL) {
+    h.xm = (k > 0 || s.x_pbc) ? sld<true>(s.lp[km] + xo) : 0u;
+    h.xp = (k + 1 < s.Lx || s.x_pbc) ? sld<true>(s.lp[kp] + xo) : 0u;
+  } else {
+    h.xm = (k > 0 || s.x_pbc) ? sld<false>(s.planes + 4 * km * s.lw + xo) : 0u;
+    h.xp = (k + 1 < s.Lx || s.x_pbc) ? sld<false>(s.planes + 4 * kp * s.lw + xo) : 0u;
+  }
+  // y neighbours: rows inside the packed word are its own other array's
+  // (plane o), one slot over; the wrap row is array X of the mirrored layer
+  const uint32_t gk = (s.y_mode == kYGapbc) ? (s.Lx - 1 - k) : k;
+  const uint32_t gbase = CL ? s.lp[gk] : s.planes + 4 * gk * s.lw;
+  uint32_t ym, yp;
+  if (g > 0) ym = ld(bO + 4 * in_layer(i - s.W, lim, 62));
+  else ym = sld<CL>(gbase + ((X + gk + s.Ly) & 1u) * pb + 4 * in_layer((s.G - 1) * s.W + w, lim, 63)) ^ s.neg;
+  if (g + 1 < s.G) yp = ld(bO + 4 * in_layer(i + s.W, lim, 64));
+  else yp = sld<CL>(gbase + ((X + (R - 1) + gk + 1) & 1u) * pb + 4 * in_layer(w, lim, 65)) ^ s.neg;
+  if constexpr (R > 1) {
+    ym = ((h.z0 << B) & ~kLow) | ((ym >> (8 - B)) & kLow);
+    yp = ((h.z0 >> B) & ~kTop) | ((yp << (8 - B)) & kTop);
+  }
+  h.ym = ym;
+  h.yp = yp;
+  if (R > 1 || s.W == 1) {
+    const uint32_t pr = packed_prev(h.z0, kFirst, s.pos), nx = packed_next(h.z0, kFirst, s.pos);
+    // rows alternate between the arrays
+    constexpr uint32_t kEven = R == 1 ? 0xFFFFFFFFu : R == 2 ? kLow : kLow | (kLow << 4);
+    const uint32_t e = X ? ~kEven : kEven;  // slots whose row updates array 0
+    h.zs = R == 1 ? (X ? nx : pr) : (pr & e) | (nx & ~e);
+  } else if (X == 0) {
+    const uint32_t pw = w > 0 ? ld(bO + 4 * in_layer(i - 1, lim, 66)) >> 31
+                              : (ld(bO + 4 * in_layer(i + s.W - 1, lim, 67)) >> s.pos) & 1u;
+    h.zs = shift_prev(h.z0, pw << 31);
+  } else {
+    const bool last = w + 1 == s.W;
+    const uint32_t nw = ld(bO + 4 * in_layer(last ? i - w : i + 1, lim, 68));
+    h.zs = shift_next(h.z0, 0u) | ((nw & 1u) << (last ? s.pos : 31u));
+  }
+}
+
+__device__ __forceinline__ uint32_t slab_mirror(const Slab& s, uint32_t kx) {
+  return s.y_mode == kYGapbc ? s.Lx + 1 - kx : kx;
+}
+
+// A thread's column: word w of the groups that the steps v0 .. v1 - 1 of layer kx
+// name.  A layer's G steps are: the first group, its wrap partner (the last
+// group of layer kx'), the groups 1 .. G - 2; a column is `len` steps, so that
+// a first group and its partner are one thread's, in this order.  Columns that
+// start with a first group come first, so that they share warps.
+struct Column {
+  uint32_t kx, w, v0, v1;
+};
+
+__device__ __forceinline__ Column slab_column(const Slab& s, uint32_t at) {
+  Column o{s.a + 1, 0, 0, 0};
+  if (at >= s.cols) return o;
+  const uint32_t per = s.nl * s.W;
+  uint32_t l, q = 0;
+  if (at < per) {
+    l = at / s.W;
+    o.w = at - l * s.W;
+  } else {
+    // the others layer by layer, so that few warps hold a wall's layer
+    const uint32_t r = at - per, n = s.cols / per - 1, m = r / s.W;
+    o.w = r - m * s.W;
+    l = m / n;
+    q = m - l * n + 1;
+  }
+  o.kx = s.a + l + 1;
+  o.v0 = q * s.len;
+  o.v1 = min(o.v0 + s.len, s.G);
   return o;
 }
 
-// Item of thread t in round j: the pair item's index (< P) at the round that
-// starts it, 0xFFFFFFFF at the round its partner takes, else P + the regular
-// item's index (which may be >= P + P': nothing to do).
-__device__ __forceinline__ uint32_t slab_round_item(const SlabRounds& r, uint32_t t, uint32_t j, uint32_t T) {
-  const uint32_t kt = r.q + (t < r.s ? 1u : 0u);  // this thread's pair items
-  if (j < 2 * kt) return (j & 1u) ? 0xFFFFFFFFu : t + (j >> 1) * T;
-  const uint32_t j0 = 2 * r.q;
-  const uint32_t reg = (j < j0 + 2) ? (j - j0) * (T - r.s) + (t - r.s) : 2 * (T - r.s) + (j - j0 - 2) * T + t;
-  return r.P + reg;
+// The words of interior group g of own layer kx.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_fetch_in(const Slab& s, uint32_t c, uint32_t kx, uint32_t g, uint32_t w, Hood& h) {
+  constexpr uint32_t B = 8 / R, kLow = slot_mask<R>(), kTop = kLow << (8 - B), kFirst = first_bits<R>();
+  const uint32_t k = kx - 1, W = s.W, pb = 4 * s.pw, o = (c ^ 1u) * pb;
+  const uint32_t X = (kx + g * R + 2 + c) & 1u;  // array of the group's first row
+  const uint32_t i = 4 * in_layer(g * W + w, s.lw, 61);
+  const uint32_t own = s.planes + 4 * (k - s.a) * s.lw + i;
+  const uint32_t at = own + o;  // its other plane's word
+  h.S = sld<false>(own + c * pb);
+  h.z0 = sld<false>(at);
+  const uint32_t ym = sld<false>(at - 4 * W), yp = sld<false>(at + 4 * W);
+  const uint32_t km = k > 0 ? k - 1 : s.Lx - 1, kp = k + 1 < s.Lx ? k + 1 : 0u;
+  h.xm = (k > 0 || s.x_pbc) ? sld<CL>(o + i + (CL ? s.lp[km] : s.planes + 4 * km * s.lw)) : 0u;
+  h.xp = (k + 1 < s.Lx || s.x_pbc) ? sld<CL>(o + i + (CL ? s.lp[kp] : s.planes + 4 * kp * s.lw)) : 0u;
+  if constexpr (R == 1) {
+    h.ym = ym;
+    h.yp = yp;
+    if (W == 1) {
+      h.zs = X ? packed_next(h.z0, 1u, s.pos) : packed_prev(h.z0, 1u, s.pos);
+    } else if (X == 0) {
+      const uint32_t e = sld<false>(w > 0 ? at - 4 : at + 4 * (W - 1));
+      h.zs = shift_prev(h.z0, (e >> (w > 0 ? 31u : s.pos)) << 31);
+    } else {
+      const bool last = w + 1 == W;
+      const uint32_t e = sld<false>(last ? at - 4 * w : at + 4);
+      h.zs = shift_next(h.z0, 0u) | ((e & 1u) << (last ? s.pos : 31u));
+    }
+  } else {
+    h.ym = ((h.z0 << B) & ~kLow) | ((ym >> (8 - B)) & kLow);
+    h.yp = ((h.z0 >> B) & ~kTop) | ((yp << (8 - B)) & kTop);
+    constexpr uint32_t kEven = R == 2 ? kLow : kLow | (kLow << 4);
+    const uint32_t e = X ? ~kEven : kEven;  // slots whose row updates array 0
+    h.zs = (packed_prev(h.z0, kFirst, s.pos) & e) | (packed_next(h.z0, kFirst, s.pos) & ~e);
+  }
 }
 
-// The record of sweep t (records-ring slot `slot`) from the layer sums the
-// cluster's CTAs left in buffer `buf`: this CTA writes m(kx) of its own
-// layers [a, b), rank 0 the totals.
-__device__ __forceinline__ void cluster_record(cg::cluster_group& cl, const FilmDesc& d, int64_t* records, int* s_m,
-                                               int (*s_tot)[2], uint32_t buf, uint32_t a, uint32_t b, uint32_t C,
-                                               uint32_t t, uint32_t slot) {
-  const uint32_t Lx = d.Lx;
-  int64_t* rec = records + d.rec_off + (size_t)slot * (5 + Lx);
-  for (uint32_t kx = a + threadIdx.x; kx < b; kx += blockDim.x) {
-    int v = 0;
-    for (uint32_t q = 0; q < C; q++) v += cl.map_shared_rank(s_m + buf * Lx, q)[kx];
+// The record of `t` completed sweeps: this CTA writes m(kx) of its own layers,
+// rank 0 the totals; both are cleared for the next record (whose sums come
+// after the next barrier).
+__device__ __forceinline__ void slab_record(const Slab& s, const FilmDesc& d, int64_t* records, int* s_m, int* s_tot,
+                                            bool rank0, uint32_t t) {
+  const uint32_t i0 = blockDim.x - 1 - threadIdx.x;  // from the threads with the fewest items on
+  if (i0 >= s.nl && i0 != 0) return;
+  // the ring slot: this call's records before this one, from where the ring stood
+  const uint32_t nth = d.rec_next + (t / d.measure_every - d.sweep / d.measure_every) - 1;
+  int64_t* rec = records + d.rec_off + (size_t)(d.rec_cap ? nth % d.rec_cap : 0u) * (5 + s.Lx);
+  for (uint32_t kx = s.a + i0; kx < s.a + s.nl; kx += blockDim.x) {
+    const int v = s_m[kx];
+    s_m[kx] = 0;
     rec[5 + kx] = v;
     if (kx == 0) rec[3] = v;
-    if (kx == Lx - 1) rec[4] = v;
+    if (kx == s.Lx - 1) rec[4] = v;
   }
-  if (cl.block_rank() == 0 && threadIdx.x == 0) {
-    int B = 0, M = 0;
-    for (uint32_t q = 0; q < C; q++) {
-      const int* p = cl.map_shared_rank(&s_tot[buf][0], q);
-      B += p[0];
-      M += p[1];
-    }
+  if (rank0 && i0 == 0) {
     rec[0] = (int64_t)t;
-    rec[1] = B;
-    rec[2] = M;
+    rec[1] = s_tot[0];
+    rec[2] = s_tot[1];
+    s_tot[0] = 0;
+    s_tot[1] = 0;
   }
 }
 
-// n_sweeps sweeps of film Fg on this cluster (C = its size), records into
-// its ring, sweep and rec_next advanced at the end.  Dynamic shared memory
-// s_dyn: planes [2][ceil(Lx / C)][Ly][W] words, the layer table (2 Lx
-// generic addresses), and two buffers of Lx layer sums.  Ends with a cluster
-// barrier, after which the CTA's shared memory is free for the next film.
-template <bool FAST>
-__device__ __forceinline__ void cluster_film(cg::cluster_group& cl, FilmDesc* Fg, uint32_t* __restrict__ pool,
-                                             int64_t* __restrict__ records, uint32_t n_sweeps, FilmDesc& s_d,
-                                             uint32_t* s_thr, uint32_t* s_alw, uint32_t* s_stash, int (*s_tot)[2],
-                                             uint32_t* s_dyn) {
-  constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
-  const uint32_t C = cl.num_blocks();
-  const uint32_t r = cl.block_rank();
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(Fg);
-    uint4* dst = reinterpret_cast<uint4*>(&s_d);
-    for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
+template <bool CL>
+__device__ __forceinline__ void slab_arrive() {
+  if (CL) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+}
+template <bool CL>
+__device__ __forceinline__ void slab_wait() {
+  if (CL) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+  else asm volatile("barrier.sync 0;" ::: "memory");
+}
+
+// Sets up the slab of film d (staged in shared memory): geometry, the planes
+// sorted by colour and packed R rows to a word, the layer tables, zero sums.
+// Every CTA's part is in place once the cluster's next barrier has passed.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_load(const FilmDesc& d, const uint32_t* __restrict__ pool, int* s_tot,
+                                          uint32_t* s_dyn, Slab& s, uint32_t C, uint32_t rank) {
+  constexpr uint32_t B = 8 / R;
+  if (threadIdx.x == 0) {
+    s.Lx = d.Lx; s.Ly = d.Ly; s.W = d.W; s.G = d.Ly / R; s.lw = s.G * s.W;
+    s.a = rank * d.Lx / C;
+    s.nl = (rank + 1) * d.Lx / C - s.a;
+    s.pw = (d.Lx + C - 1) / C * s.lw;
+    s.y_mode = d.y_mode; s.x_pbc = d.x_pbc; s.last_mask = d.last_mask; s.last_calls = d.last_calls;
+    s.pos = bitpos((d.n - 1) & 31u);
+    s.neg = d.y_mode != kYPbc ? 0xFFFFFFFFu : 0u;
+    s.seam_same = seam_joins_one_colour(d.Lx, d.Ly, d.y_mode);
+    s.planes = smem_addr(s_dyn);
+    s.lp = s_dyn + 2 * s.pw;
+    s.lm = s.lp + s.Lx;
+    const SlabShape sh = slab_shape(d, C, blockDim.x);
+    s.len = sh.len;
+    s.cols = s.nl * s.W * ((s.G + sh.len - 1) / sh.len);
+    s.turns = sh.turns;
   }
   __syncthreads();
-  for (uint32_t i = threadIdx.x; i < 64; i += blockDim.x) {
-    const bool al = (s_d.always[i >> 4] >> (i & 15)) & 1u;
-    s_thr[i] = FAST ? (al ? 0xFFFFFFFFu : s_d.thr[i >> 4][i & 15] - 1u) : s_d.thr[i >> 4][i & 15];
-    s_alw[i] = al ? 0xFFFFFFFFu : 0u;
+  uint32_t* planes = s_dyn;
+  uint32_t* lp = s_dyn + 2 * s.pw;
+  uint32_t* lm = lp + s.Lx;
+  int* s_m = reinterpret_cast<int*>(lm + s.Lx);
+  const uint32_t* g0 = pool + d.spin_off;
+  const size_t gpl = (size_t)d.Lx * d.Ly * d.W;
+  for (uint32_t i = threadIdx.x; i < 2 * s.nl * s.lw; i += blockDim.x) {
+    const uint32_t c = i >= s.nl * s.lw ? 1u : 0u, r = i - c * s.nl * s.lw;
+    const uint32_t l = r / s.lw, q = r - l * s.lw, g = q / s.W, w = q - g * s.W;
+    uint32_t v = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < R; j++) {
+      const uint32_t row = (s.a + l) * s.Ly + g * R + j;             // kx - 1 = a + l, ky - 1 = g R + j
+      const uint32_t X = (s.a + l + g * R + j + 1 + c) & 1u;         // (kx + ky + 1 + c) & 1
+      v |= ISG_LD(g0, X * gpl + (size_t)row * s.W + w, 2 * gpl, 77) << (j * B);
+    }
+    planes[c * s.pw + r] = v;
   }
-  if (!s_d.active) return;  // the same for the whole cluster
-  const uint32_t Lx = s_d.Lx, Ly = s_d.Ly, W = s_d.W;
-  const uint32_t a = r * Lx / C, b = (r + 1) * Lx / C, nl = b - a;
-  const uint32_t lw = Ly * W;                    // words of one layer
-  const uint32_t pw = (Lx + C - 1) / C * lw;     // words of one local plane
-  uint32_t* s_planes = s_dyn;
-  uint32_t** s_lp = reinterpret_cast<uint32_t**>(s_dyn + 2 * pw);  // 8-byte aligned: 2 pw is even
-  int* s_m = reinterpret_cast<int*>(s_lp + 2 * Lx);
-  const size_t gpl = (size_t)Lx * lw;  // words of one plane in the pool (row stride W)
-  uint32_t* g = pool + s_d.spin_off;
-  for (uint32_t i = threadIdx.x; i < 2 * nl * lw; i += blockDim.x) {
-    const uint32_t X = i >= nl * lw ? 1u : 0u;
-    const uint32_t j = i - X * nl * lw;
-    s_planes[X * pw + j] = ISG_LD(g, X * gpl + (size_t)a * lw + j, 2 * gpl, 77);
-  }
-  for (uint32_t i = threadIdx.x; i < 2 * Lx; i += blockDim.x) {
-    const uint32_t X = i >= Lx ? 1u : 0u, k = i - X * Lx;
+  for (uint32_t k = threadIdx.x; k < s.Lx; k += blockDim.x) {
     uint32_t q = 0;
-    while (q + 1 < C && (q + 1) * Lx / C <= k) q++;
-    uint32_t* base = q == r ? s_planes : cl.map_shared_rank(s_planes, q);
-    s_lp[i] = base + X * pw + (k - q * Lx / C) * lw;
-    s_m[i] = 0;
+    while (q + 1 < C && (q + 1) * s.Lx / C <= k) q++;
+    const uint32_t at = s.planes + 4 * (k - q * s.Lx / C) * s.lw, am = smem_addr(s_m + k);
+    lp[k] = CL ? mapa(at, q) : at;
+    lm[k] = CL ? mapa(am, q) : am;
+    s_m[k] = 0;
   }
-  if (threadIdx.x < 4) s_tot[threadIdx.x >> 1][threadIdx.x & 1] = 0;
-  FilmCtx c;
-  c.Lx = Lx; c.Ly = Ly; c.n = s_d.n; c.W = W; c.Wp = W;
-  c.plane_words = lw;
-  c.y_mode = s_d.y_mode; c.x_pbc = s_d.x_pbc; c.rk0 = s_d.rk0; c.rk1 = s_d.rk1;
-  c.last_mask = s_d.last_mask; c.last_calls = s_d.last_calls;
-  c.plane0 = nullptr;
-  c.plane1 = nullptr;
-  c.seam_same = seam_joins_one_colour(Lx, Ly, s_d.y_mode);
-  c.pack = 1;
-  const uint32_t items = nl * (Ly - 1) * W;
-  const SlabRounds rounds = slab_rounds(nl * W, nl * (Ly - 2) * W, blockDim.x);
-  const uint32_t m_every = s_d.measure_every;
-  uint32_t rec_next = s_d.rec_next, nrec = 0, done = 0;
-  // a record's sums are read in the half-sweep after the one that took them
-  // and cleared in the next; two buffers alternate between records
-  int read_buf = -1, clear_buf = -1;
-  uint32_t read_t = 0, read_slot = 0;
-  cl.sync();  // every CTA's planes are in place
-  for (uint32_t k = 0; k < n_sweeps; k++) {
-    const uint32_t t = s_d.sweep + k;
-    if (t >= s_d.sweep_end) break;
-    c.sweep = t;
-    const bool rec_now = m_every != 0 && (t + 1) % m_every == 0;
-    for (uint32_t colour = 0; colour < 2; colour++) {
-      c.colour = colour;
-      if (clear_buf >= 0) {
-        for (uint32_t i = threadIdx.x; i < Lx; i += blockDim.x) s_m[clear_buf * Lx + i] = 0;
-        if (threadIdx.x < 2) s_tot[clear_buf][threadIdx.x] = 0;
-        clear_buf = -1;
-      }
-      if (read_buf >= 0) {
-        cluster_record(cl, s_d, records, s_m, s_tot, (uint32_t)read_buf, a, b, C, read_t, read_slot);
-        clear_buf = read_buf;
-        read_buf = -1;
-      }
-      if (colour == 1 && rec_now) {
-        int* sm = s_m + (nrec & 1u) * Lx;
-        int* st = s_tot[nrec & 1u];
-        uint32_t* stash = s_stash + threadIdx.x * kStashSlots;
-        for (uint32_t j = 0; j < rounds.R; j++) {  // the same count for every thread (warp-wide sums)
-          const uint32_t item = slab_round_item(rounds, threadIdx.x, j, blockDim.x);
-          LayerSums r1, r2;
-          if (item < items) {
-            uint32_t kx, ky, w;
-            slab_item_word(s_d, a, nl, item, kx, ky, w);
-            Fetched f;
-            fetch_word_cl(c, s_lp, kx, ky, w, f);
-            update_fetched_cl<FAST, true>(c, s_lp, f, s_thr, s_alw, stash, &r1, &r2);
-          }
-          add_layer_sums_shared(sm, st, r1);
-          add_layer_sums_shared(sm, st, r2);
-        }
-      } else {
-        for (uint32_t j = 0; j < rounds.R; j++) {
-          const uint32_t item = slab_round_item(rounds, threadIdx.x, j, blockDim.x);
-          if (item >= items) continue;
-          uint32_t kx, ky, w;
-          slab_item_word(s_d, a, nl, item, kx, ky, w);
-          Fetched f;
-          fetch_word_cl(c, s_lp, kx, ky, w, f);
-          update_fetched_cl<FAST, false>(c, s_lp, f, s_thr, s_alw);
-        }
-      }
-      cl.sync();
-    }
-    done = k + 1;
-    if (rec_now) {
-      read_buf = (int)(nrec & 1u);
-      read_t = t + 1;
-      read_slot = s_d.rec_cap ? rec_next % s_d.rec_cap : 0u;
-      rec_next++;
-      nrec++;
-    }
-  }
-  if (read_buf >= 0) cluster_record(cl, s_d, records, s_m, s_tot, (uint32_t)read_buf, a, b, C, read_t, read_slot);
-  for (uint32_t i = threadIdx.x; i < 2 * nl * lw; i += blockDim.x) {
-    const uint32_t X = i >= nl * lw ? 1u : 0u;
-    const uint32_t j = i - X * nl * lw;
-    ISG_ST(g, X * gpl + (size_t)a * lw + j, 2 * gpl, 78, s_planes[X * pw + j]);
-  }
-  if (r == 0 && threadIdx.x == 0) {
-    Fg->sweep = s_d.sweep + done;
-    Fg->rec_next = rec_next;
-  }
-  cl.sync();  // peers may still be reading this CTA's layer sums
+  if (threadIdx.x < 2) s_tot[threadIdx.x] = 0;
 }
 
-// Clusters of C CTAs, cluster i sweeping films list[n_clusters + 1 + j] for j
-// in [list[i], list[i + 1]) one after another (all n_sweeps sweeps of one,
-// then the next): films never wait for one another, and the host packs them
-// so that the clusters' loads are about equal.
-template <bool FAST>
-__global__ void __launch_bounds__(cluster_max_threads(!FAST), 1)
-cluster_kernel(FilmDesc* __restrict__ films, const uint32_t* __restrict__ list, uint32_t n_clusters,
-               uint32_t* __restrict__ pool, int64_t* __restrict__ records, uint32_t n_sweeps) {
+// Writes the planes back, advances the film's counters to t1, and leaves the
+// shared memory free for the next film once every peer is done.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_store(FilmDesc* Fg, const FilmDesc& d, uint32_t* __restrict__ pool,
+                                           const uint32_t* planes, const Slab& s, uint32_t rank, uint32_t t1) {
+  constexpr uint32_t B = 8 / R;
+  uint32_t* g0 = pool + d.spin_off;
+  const size_t gpl = (size_t)d.Lx * d.Ly * d.W;
+  for (uint32_t i = threadIdx.x; i < 2 * s.nl * s.lw; i += blockDim.x) {
+    const uint32_t c = i >= s.nl * s.lw ? 1u : 0u, r = i - c * s.nl * s.lw;
+    const uint32_t l = r / s.lw, q = r - l * s.lw, g = q / s.W, w = q - g * s.W;
+    const uint32_t v = planes[c * s.pw + r];
+#pragma unroll
+    for (uint32_t j = 0; j < R; j++) {
+      const uint32_t row = (s.a + l) * s.Ly + g * R + j;
+      const uint32_t X = (s.a + l + g * R + j + 1 + c) & 1u;
+      ISG_ST(g0, X * gpl + (size_t)row * s.W + w, 2 * gpl, 78, R == 1 ? v : (v >> (j * B)) & slot_mask<R>());
+    }
+  }
+  if (rank == 0 && threadIdx.x == 0) {
+    Fg->sweep = t1;
+    if (d.measure_every) Fg->rec_next = d.rec_next + (t1 / d.measure_every - d.sweep / d.measure_every);
+  }
+  // the CTA's shared memory is free for its next film once every peer is done
+  slab_arrive<CL>();
+  slab_wait<CL>();
+}
+
+
+// The sweep this call ends before.
+__device__ __forceinline__ uint32_t slab_end(const FilmDesc& d, uint32_t n_sweeps) {
+  return (d.sweep_end - d.sweep < n_sweeps) ? max(d.sweep_end, d.sweep) : d.sweep + n_sweeps;
+}
+
+// n_sweeps sweeps of the film of descriptor d (staged from Fg) on this CTA or
+// cluster, rows packed R to a word.  Thread i has columns i, i + T, ...; one
+// loop runs all steps of all half-sweeps, each step deciding a word and then
+// drawing the thread's next one, the first of the next half-sweep included:
+// between the barrier's arrival and the wait for it.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint32_t* __restrict__ pool,
+                                          int64_t* __restrict__ records, uint32_t n_sweeps, int* s_tot,
+                                          uint32_t* s_dyn, Slab& s, uint32_t C, uint32_t rank) {
+  constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  slab_load<CL, R>(d, pool, s_tot, s_dyn, s, C, rank);
+  int* s_m = reinterpret_cast<int*>(s_dyn + 2 * s.pw + 2 * s.Lx);
+  const uint32_t tot = CL ? mapa(smem_addr(s_tot), 0) : smem_addr(s_tot);
+  const uint32_t t0 = d.sweep, t1 = slab_end(d, n_sweeps);
+  const uint32_t m_every = d.measure_every;
+  uint32_t m_left = m_every ? m_every - t0 % m_every : 0u;  // sweeps until the next record
+  bool pending = false;  // a record's sums are complete, not yet written
+  uint32_t c = 0, t = t0, turn = 0;
+  Column col = slab_column(s, threadIdx.x);
+  uint32_t v = col.v0;
+  bool on = col.v0 < col.v1, any7 = false;
+  Drawn a{{0, 0, 0, 0, 0, 0, 0}};
+  // what a first group leaves for its partner: its new word and its row's other array
+  uint32_t pv = 0, pz = 0;
+  int tb = 0, tm = 0;
+  slab_arrive<CL>();
+#pragma unroll 1
+  for (bool go = false, more = false;;) {
+    if (go) {
+      // decide step v of the column
+      const bool meas = c == 1 && m_left == 1;
+      if (on) {
+        const bool partner = v == 1;
+        const uint32_t kx = partner ? slab_mirror(s, col.kx) : col.kx;
+        const uint32_t g = v == 0 ? 0u : partner ? s.G - 1 : v - 1;
+        const uint32_t valid1 = col.w + 1 == s.W ? s.last_mask : 0xFFFFFFFFu;  // one row's sites
+        uint32_t valid = valid1;
+        if (R > 1) {
+          valid = 0;
+#pragma unroll
+          for (uint32_t j = 0; j < R; j++) valid |= s.last_mask << (j * B);
+        }
+        Hood h;
+        if (v >= 2) slab_fetch_in<CL, R>(s, c, kx, g, col.w, h);
+        else slab_fetch<CL, R>(s, c, !partner, kx, g, col.w, h);
+        // the partner's wrap neighbour is the word just decided where the seam
+        // joins one colour
+        const bool seam = partner && s.seam_same;
+        if (seam) h.yp = (h.yp & ~(valid1 << kSeam)) | (((pv ^ s.neg) & valid1) << kSeam);
+        const Count k = count_up(h);
+        const uint32_t nv = h.S ^ (decide(h, k, any7, a, d.cls[row_class(kx, s.Lx)]) & valid);
+        const uint32_t off = 4 * (c * s.pw + in_layer(g * s.W + col.w, s.lw, 70));
+        if (CL && partner) sst<true>(s.lp[kx - 1] + off, nv);
+        else sst<false>(s.planes + 4 * (kx - 1 - s.a) * s.lw + off, nv);
+        if (meas) {
+          LayerSums r = word_sums(kx, k, nv, h.z0, valid, bond_slots(kx, s.Lx, s.x_pbc));
+          if (seam) r.b += seam_adjust(pv, pz, h.S, h.z0, kSeam, s.neg, valid1);
+          tb += r.b;
+          tm += r.m;
+          if (CL && partner) sadd<true>(s.lm[kx - 1], r.m);
+          else sadd<false>(smem_addr(s_m + kx - 1), r.m);
+        }
+        pv = nv;
+        pz = h.z0;
+      }
+      // the next step: of this column, of the thread's next one, or of the next half-sweep
+      v++;
+      more = v - col.v0 < s.len;
+      if (!more && turn + 1 < s.turns) {
+        turn++;
+        col = slab_column(s, threadIdx.x + turn * blockDim.x);
+        v = col.v0;
+        more = true;
+      }
+      if (!more) {
+        if (meas) {
+          tb = __reduce_add_sync(0xFFFFFFFFu, tb);
+          tm = __reduce_add_sync(0xFFFFFFFFu, tm);
+          if ((threadIdx.x & 31u) == 0) {
+            sadd<CL>(tot, tb);
+            sadd<CL>(tot + 4, tm);
+          }
+          tb = tm = 0;
+          pending = true;
+        }
+        slab_arrive<CL>();
+        if (turn) {
+          turn = 0;
+          col = slab_column(s, threadIdx.x);
+        }
+        v = col.v0;
+        if (c) {
+          m_left = m_every ? (m_left == 1 ? m_every : m_left - 1) : 0u;
+          t++;
+        }
+        c ^= 1u;
+      }
+      on = v < col.v1;
+    }
+    if (t < t1) {
+      const bool partner = v == 1;
+      const uint32_t kx = partner ? slab_mirror(s, col.kx) : col.kx;
+      const uint32_t g = v == 0 ? 0u : partner ? s.G - 1 : v - 1;
+      const ClassDraw& cl = d.cls[row_class(kx, s.Lx)];
+      any7 = __any_sync(0xFFFFFFFFu, on && !cl.sym);
+      if (on)
+        draw_any<R>(a, any7, cl, (kx - 1) * s.Ly + g * R, (kx + g * R + 2 + c) & 1u, col.w,
+                          col.w + 1 == s.W ? s.last_calls : 8u, s.last_mask == 0xFFFFFFFFu, s.W > 1, t, d.rk0, d.rk1);
+    }
+    if (!more) {
+      slab_wait<CL>();  // the first time: every CTA's planes and tables are in place
+      if (pending && c == 0) {
+        slab_record(s, d, records, s_m, s_tot, rank == 0, t);
+        pending = false;
+      }
+      if (t >= t1) break;
+      go = true;
+    }
+  }
+  slab_store<CL, R>(Fg, d, pool, s_dyn, s, rank, t1);
+}
+
+// ---- tasks: the draws of a half-sweep spread evenly over the threads
+//
+// Films of few words per CTA are bound by latency: one warp takes some 2000
+// cycles for a word's eight Philox calls however idle the SM is, and a thread
+// with a pair (a first group and its wrap partner's) or a warp on a wall's layer
+// takes twice that while the others wait at the barrier.  So drawing and
+// deciding are separate here.  Four lanes draw a word, two calls each, and
+// leave its masks in shared memory, the words of a half-sweep dealt out over
+// all threads; deciding reads them and is short.  The masks drawn between two
+// barriers are the next half-sweep's, in a second buffer.
+
+// What a decision needs to know of its word; plane 0 addresses.  The plane an
+// address lies in changes with the colour for every word a decision reads:
+// plane = phase ^ c.
+struct SlabWord {
+  uint32_t own, xm, xp, ym, yp;  // the word, its x and y neighbours
+  uint32_t f;                    // kW* bits; 8, 9: row class; 16..: layer
+  uint32_t row;                  // index of its first row, | w << 16
+  uint32_t pad;
+};
+// X in half-sweep 0, the phases of ym and yp, the first group (ym wraps), the
+// word is its row's first, last, it has an x neighbour below, above; the last
+// group (yp wraps; bit 10)
+enum : uint32_t { kWX = 1, kWYm = 2, kWYp = 4, kWTop = 8, kWFirst = 16, kWLast = 32, kWXm = 64, kWXp = 128, kWEnd = 1024 };
+
+template <bool CL, int R>
+__device__ __forceinline__ SlabWord slab_word(const Slab& s, uint32_t kx, uint32_t g, uint32_t w) {
+  SlabWord o;
+  const uint32_t k = kx - 1, W = s.W, lim = s.lw;
+  auto layer = [&](uint32_t l) { return CL ? s.lp[l] : s.planes + 4 * l * s.lw; };
+  const uint32_t i = in_layer(g * W + w, lim, 61), X = (kx + g * R + 2) & 1u;
+  const uint32_t base = layer(k), gk = (s.y_mode == kYGapbc) ? (s.Lx - 1 - k) : k;
+  o.own = base + 4 * i;
+  o.xm = layer(k > 0 ? k - 1 : s.Lx - 1) + 4 * i;
+  o.xp = layer(k + 1 < s.Lx ? k + 1 : 0u) + 4 * i;
+  o.ym = g > 0 ? base + 4 * in_layer(i - W, lim, 62) : layer(gk) + 4 * in_layer((s.G - 1) * W + w, lim, 63);
+  o.yp = g + 1 < s.G ? base + 4 * in_layer(i + W, lim, 64) : layer(gk) + 4 * in_layer(w, lim, 65);
+  o.row = (k * s.Ly + g * R) | w << 16;
+  // plane of the wrapped neighbour: the one that holds array X of its row
+  const uint32_t pm = g > 0 ? 1u : (X + gk + s.Ly) & 1u, pp = g + 1 < s.G ? 1u : (X + (R - 1) + gk + 1) & 1u;
+  o.f = X * kWX | pm * kWYm | pp * kWYp | (g == 0 ? kWTop : 0u) | (g + 1 == s.G ? kWEnd : 0u) |
+        (w == 0 ? kWFirst : 0u) | (w + 1 == W ? kWLast : 0u) | row_class(kx, s.Lx) << 8 | k << 16;
+  if (k > 0 || s.x_pbc) o.f |= kWXm;
+  if (k + 1 < s.Lx || s.x_pbc) o.f |= kWXp;
+  o.pad = 0;
+  return o;
+}
+
+// The words of a decision.  ANY: the word itself may be a peer CTA's.
+template <bool CL, bool ANY, int R>
+__device__ __forceinline__ void slab_read(const Slab& s, const SlabWord& a, uint32_t c, uint32_t pb, Hood& h) {
+  constexpr uint32_t B = 8 / R, kLow = slot_mask<R>(), kTop = kLow << (8 - B), kFirst = first_bits<R>();
+  const uint32_t S = c * pb, O = pb - S, X = (a.f ^ c) & kWX;
+  h.S = sld<CL && ANY>(a.own + S);
+  h.z0 = sld<CL && ANY>(a.own + O);
+  h.xm = (a.f & kWXm) ? sld<CL>(a.xm + O) : 0u;
+  h.xp = (a.f & kWXp) ? sld<CL>(a.xp + O) : 0u;
+  h.ym = sld<CL>(a.ym + ((a.f & kWYm) ? O : S));
+  h.yp = sld<CL>(a.yp + ((a.f & kWYp) ? O : S));
+  if constexpr (R == 1) {
+    if (s.W == 1) {
+      h.zs = X ? packed_next(h.z0, 1u, s.pos) : packed_prev(h.z0, 1u, s.pos);
+    } else if (X) {
+      const bool last = a.f & kWLast;
+      const uint32_t e = sld<CL && ANY>(a.own + O + (last ? 4 - 4 * s.W : 4));
+      h.zs = shift_next(h.z0, 0u) | ((e & 1u) << (last ? s.pos : 31u));
+    } else {
+      const bool first = a.f & kWFirst;
+      const uint32_t e = sld<CL && ANY>(a.own + O + (first ? 4 * s.W - 4 : -4));
+      h.zs = shift_prev(h.z0, (e >> (first ? s.pos : 31u)) << 31);
+    }
+  } else {
+    constexpr uint32_t kEven = R == 2 ? kLow : kLow | (kLow << 4);
+    const uint32_t e = X ? ~kEven : kEven;  // slots whose row updates array 0
+    h.zs = (packed_prev(h.z0, kFirst, s.pos) & e) | (packed_next(h.z0, kFirst, s.pos) & ~e);
+  }
+  // wrap signs, and (R > 1) the rows inside the packed word
+  if (a.f & kWTop) h.ym ^= s.neg;
+  if (a.f & kWEnd) h.yp ^= s.neg;
+  if constexpr (R > 1) {
+    h.ym = ((h.z0 << B) & ~kLow) | ((h.ym >> (8 - B)) & kLow);
+    h.yp = ((h.z0 >> B) & ~kTop) | ((h.yp << (8 - B)) & kTop);
+  }
+}
+
+// One lane's part of a word's masks, call number c1 on: bits 8 i for call c1,
+// 8 i + D for the second call.
+template <int K, int D>
+__device__ __forceinline__ void draw_part(Masks<K>& a, const uint32_t (&t)[K], const PhiloxRow3& p, uint32_t ca,
+                                          uint32_t cb, bool second) {
+  masks_zero(a);
+  uint32_t u[4], v[4];
+  if (second) {
+    p.draw2(ca, cb, u, v);
+    put_call<0>(a, t, u);
+    put_call<D>(a, t, v);
+  } else {
+    p.draw(ca, u);
+    put_call<0>(a, t, u);
+  }
+}
+
+// The draws of half-sweep (c, t) into mask buffer m: three words per three-mask
+// word, then seven per general one.  Words that fill two turns of the threads
+// are drawn by one lane each (no shuffles, the row's products once per word);
+// fewer by four lanes, task i being part i & 3 of word i >> 2.  me: the thread's
+// first task.
+template <int R>
+__device__ __forceinline__ void slab_tasks(const Slab& s, const FilmDesc& d, const SlabWord* words, uint32_t n_words,
+                                           uint32_t n3, uint32_t* m, uint32_t c, uint32_t t, uint32_t me) {
+  constexpr uint32_t B = 8 / R;
+  constexpr int D = R == 1 ? 4 : 1;
+  if (2 * n_words > blockDim.x) {
+    for (uint32_t i = me; i < (n_words + 31u & ~31u); i += blockDim.x) {  // whole warps
+      const uint32_t n = min(i, n_words - 1), f = words[n].f, rw = words[n].row;
+      const bool any7 = __any_sync(0xFFFFFFFFu, n >= n3);
+      Drawn a;
+      draw_any<R>(a, any7, d.cls[(f >> 8) & 3u], rw & 0xFFFFu, (f ^ c) & kWX, rw >> 16,
+                  R == 1 && !(f & kWLast) ? 8u : s.last_calls, s.last_mask == 0xFFFFFFFFu, s.W > 1, t, d.rk0, d.rk1);
+      if (i >= n_words) continue;
+      if (n < n3) {
+#pragma unroll
+        for (int k = 0; k < 3; k++) m[3 * n + k] = a.m[4 + k];
+      } else {
+        uint32_t* o = m + 3 * n3 + 7 * (n - n3);
+#pragma unroll
+        for (int k = 0; k < 7; k++) o[k] = a.m[k];
+      }
+    }
+    return;
+  }
+  const uint32_t tasks = 4 * n_words, j = threadIdx.x & 3u;
+  for (uint32_t i = me; i < (tasks + 31u & ~31u); i += blockDim.x) {  // whole warps
+    const uint32_t n = min(i >> 2, n_words - 1);
+    const uint32_t f = words[n].f, rw = words[n].row, w = rw >> 16;
+    const uint32_t ncalls = R == 1 && !(f & kWLast) ? 8u : s.last_calls;
+    const uint32_t rj = R == 1 ? 0u : R == 2 ? j >> 1 : j, q = R == 1 ? j : R == 2 ? 2 * (j & 1u) : 0u;
+    const bool on = q < ncalls, second = q + D < ncalls;
+    const ClassDraw& cl = d.cls[(f >> 8) & 3u];
+    const bool any7 = __any_sync(0xFFFFFFFFu, n >= n3);
+    const PhiloxRow3 p((rw & 0xFFFFu) + rj, t, ((f ^ c) & kWX) ^ (rj & 1u), d.rk0, d.rk1);
+    const uint32_t sh = rj * B + q;
+    auto share = [&](uint32_t v) {
+      v = on ? v << sh : 0u;
+      v |= __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+      return v | __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+    };
+    if (!any7) {
+      Masks<3> a;
+      masks_zero(a);
+      const uint32_t th[3] = {cl.t[4], cl.t[5], cl.t[6]};
+      if (on) draw_part<3, D>(a, th, p, 8u * w + q, 8u * w + q + D, second);
+      uint32_t v = 0;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        const uint32_t x = share(a.m[k]) | ((cl.alw >> (4 + k)) & 1u ? 0xFFFFFFFFu : 0u);
+        if (j == k) v = x;
+      }
+      if (j < 3 && (i >> 2) < n_words) m[3 * n + j] = v;
+    } else {
+      Masks<7> a;
+      masks_zero(a);
+      if (on) draw_part<7, D>(a, cl.t, p, 8u * w + q, 8u * w + q + D, second);
+      uint32_t lo = 0, hi = 0;
+#pragma unroll
+      for (int k = 0; k < 7; k++) {
+        const uint32_t x = share(a.m[k]) | ((cl.alw >> k) & 1u ? 0xFFFFFFFFu : 0u);
+        if (j == (k & 3)) (k < 4 ? lo : hi) = x;
+      }
+      if ((i >> 2) < n_words) {
+        if (n >= n3) {  // general words have seven masks
+          uint32_t* o = m + 3 * n3 + 7 * (n - n3);
+          o[j] = lo;
+          if (j < 3) o[4 + j] = hi;
+        } else if (j < 3) {  // a three-mask word in such a warp
+          m[3 * n + j] = hi;
+        }
+      }
+    }
+  }
+}
+
+// The sweeps of a film by tasks.  Shared memory behind the layer sums: the words
+// (three-mask words, then general ones), two mask buffers, the pair list.
+template <bool CL, int R>
+__device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d, uint32_t* __restrict__ pool,
+                                                int64_t* __restrict__ records, uint32_t n_sweeps, int* s_tot,
+                                                uint32_t* s_dyn, Slab& s, uint32_t C, uint32_t rank) {
+  constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  slab_load<CL, R>(d, pool, s_tot, s_dyn, s, C, rank);
+  int* s_m = reinterpret_cast<int*>(s_dyn + 2 * s.pw + 2 * s.Lx);
+  const uint32_t tot = CL ? mapa(smem_addr(s_tot), 0) : smem_addr(s_tot);
+  const uint32_t per = s.nl * s.W, n_words = per * s.G;
+  // 16-byte aligned: s_dyn is, and the planes and tables before are rounded up
+  SlabWord* words = reinterpret_cast<SlabWord*>(s_dyn + ((2 * s.pw + 3 * s.Lx + 3) & ~3u));
+  uint16_t* job = reinterpret_cast<uint16_t*>(words + n_words);  // word of (layer, group, w), the pairs' partners included
+  uint32_t* masks = reinterpret_cast<uint32_t*>(job + ((n_words + 1) & ~1u));
+  slab_arrive<CL>();
+  slab_wait<CL>();  // every CTA's planes and tables are in place
+  // Words in order of (group, own layer, w); the last group of a pair is its
+  // partner's, in layer kx'.  The general ones go to the end: a word's place is
+  // the number of words of its kind before it.
+  const bool sym0 = d.cls[0].sym;
+  auto general = [&](uint32_t kx) { return !d.cls[row_class(kx, s.Lx)].sym; };
+  auto layer_of = [&](uint32_t g, uint32_t l) {
+    const uint32_t kx = s.a + l + 1;
+    return g + 1 == s.G ? slab_mirror(s, kx) : kx;
+  };
+  (void)sym0;
+  uint32_t n3 = 0;
+  {
+    uint32_t gen_in = 0, gen_end = 0;  // general layers among the own ones, and among their mirrors
+    for (uint32_t l = 0; l < s.nl; l++) {
+      gen_in += general(s.a + l + 1) ? 1u : 0u;
+      gen_end += general(layer_of(s.G - 1, l)) ? 1u : 0u;
+    }
+    n3 = n_words - (gen_in * (s.G - 1) + gen_end) * s.W;
+    for (uint32_t i = threadIdx.x; i < n_words; i += blockDim.x) {
+      const uint32_t g = i / per, r = i - g * per, l = r / s.W, w = r - l * s.W;
+      uint32_t before = 0;  // general layers before l in this group
+      for (uint32_t q = 0; q < l; q++) before += general(layer_of(g, q)) ? 1u : 0u;
+      const uint32_t gen_g = g + 1 == s.G ? gen_end : gen_in;
+      const uint32_t kx = layer_of(g, l);
+      const uint32_t at = general(kx) ? n3 + (g * gen_in + before) * s.W + w
+                                      : (g * (s.nl - gen_in) + l - before) * s.W + w;
+      (void)gen_g;
+      words[at] = slab_word<CL, R>(s, kx, g, w);
+      job[i] = (uint16_t)at;
+    }
+  }
+  const uint32_t mw = 3 * n3 + 7 * (n_words - n3);  // words of a mask buffer
+  __syncthreads();
+  const uint32_t t0 = d.sweep, t1 = slab_end(d, n_sweeps);
+  const uint32_t m_every = d.measure_every;
+  uint32_t m_left = m_every ? m_every - t0 % m_every : 0u;  // sweeps until the next record
+  const uint32_t pb = 4 * s.pw, jobs = n_words - per;       // a pair is one job
+  bool pending = false;  // a record's sums are complete, not yet written
+  // The first warps decide, so the tasks start at the warp behind them: where
+  // there are threads enough, deciding one half-sweep and drawing the next go on
+  // side by side.
+  const uint32_t busy = ((jobs + 31u) & ~31u) % blockDim.x;
+  const uint32_t me = threadIdx.x >= busy ? threadIdx.x - busy : threadIdx.x + blockDim.x - busy;
+  if (t0 < t1) slab_tasks<R>(s, d, words, n_words, n3, masks, 0, t0, me);
+  __syncthreads();
+  uint32_t c = 0, t = t0;
+#pragma unroll 1
+  while (t < t1) {
+    const uint32_t* m = masks + c * mw;
+    const bool meas = c == 1 && m_left == 1;
+    int tb = 0, tm = 0;
+    for (uint32_t i = threadIdx.x; i < jobs; i += blockDim.x) {
+      const bool pair = i < per;
+      uint32_t v0 = 0, z0 = 0, valid0 = 0;
+#pragma unroll 1
+      for (uint32_t r = 0; r < (pair ? 2u : 1u); r++) {
+        const uint32_t n = job[r ? i + per * (s.G - 1) : i];
+        const SlabWord a = words[n];
+        Hood h;
+        if (r) slab_read<CL, true, R>(s, a, c, pb, h);
+        else slab_read<CL, false, R>(s, a, c, pb, h);
+        const uint32_t valid1 = (a.f & kWLast) ? s.last_mask : 0xFFFFFFFFu;  // one row's sites
+        uint32_t valid = valid1;
+        if (R > 1) {
+          valid = 0;
+#pragma unroll
+          for (uint32_t j = 0; j < R; j++) valid |= s.last_mask << (j * B);
+        }
+        // the partner's wrap neighbour is the word just decided where the seam
+        // joins one colour
+        const bool seam = r && s.seam_same;
+        if (seam) h.yp = (h.yp & ~(valid1 << kSeam)) | (((v0 ^ s.neg) & valid1) << kSeam);
+        const Count k = count_up(h);
+        uint32_t fl;
+        if (n < n3) {
+          const uint32_t* q = m + 3 * n;
+          fl = flips3(h.S, k, q[0], q[1], q[2]);
+        } else {
+          const uint32_t* q = m + 3 * n3 + 7 * (n - n3);
+          const ClassDraw& cl = d.cls[(a.f >> 8) & 3u];
+          const uint32_t mm[7] = {q[0], q[1], q[2], q[3], q[4], q[5], q[6]};
+          fl = flips7(h.S, k, mm, cl.up, cl.frz);
+        }
+        const uint32_t v = h.S ^ (fl & valid);
+        if (r) sst<CL>(a.own + c * pb, v);
+        else sst<false>(a.own + c * pb, v);
+        if (meas) {
+          const uint32_t kx = (a.f >> 16) + 1;
+          LayerSums x = word_sums(kx, k, v, h.z0, valid, bond_slots(kx, s.Lx, s.x_pbc));
+          if (seam) x.b += seam_adjust(v0, z0, h.S, h.z0, kSeam, s.neg, valid1);
+          tb += x.b;
+          tm += x.m;
+          if (r) sadd<CL>(s.lm[kx - 1], x.m);
+          else sadd<false>(smem_addr(s_m + kx - 1), x.m);
+        }
+        v0 = v;
+        z0 = h.z0;
+      }
+      (void)valid0;
+    }
+    if (meas) {
+      __syncwarp();
+      tb = __reduce_add_sync(0xFFFFFFFFu, tb);
+      tm = __reduce_add_sync(0xFFFFFFFFu, tm);
+      if ((threadIdx.x & 31u) == 0) {
+        sadd<CL>(tot, tb);
+        sadd<CL>(tot + 4, tm);
+      }
+      pending = true;
+    }
+    if (c) {
+      m_left = m_every ? (m_left == 1 ? m_every : m_left - 1) : 0u;
+      t++;
+    }
+    c ^= 1u;
+    __syncwarp();
+    if (t < t1) slab_tasks<R>(s, d, words, n_words, n3, masks + c * mw, c, t, me);
+    slab_arrive<CL>();
+    slab_wait<CL>();
+    if (pending && c == 0) {
+      slab_record(s, d, records, s_m, s_tot, rank == 0, t);
+      pending = false;
+    }
+  }
+  slab_store<CL, R>(Fg, d, pool, s_dyn, s, rank, t1);
+}
+
+}  // namespace
+
+// Clusters of C CTAs (CL; else C = 1: single CTAs), cluster i sweeping films
+// list[n_clusters + 1 + j] for j in [list[i], list[i + 1]) one after another
+// (all n_sweeps sweeps of one, then the next); list = null: cluster i sweeps
+// film i.
+template <bool CL, bool TASKS>
+__global__ void __launch_bounds__(TASKS ? kTaskThreads : kSlabThreads, 1)
+slab_kernel(FilmDesc* __restrict__ films, const uint32_t* __restrict__ list, uint32_t n_clusters,
+            uint32_t* __restrict__ pool, int64_t* __restrict__ records, uint32_t n_sweeps) {
   extern __shared__ __align__(16) uint32_t s_dyn[];
+  constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
   __shared__ __align__(16) FilmDesc s_d;
-  __shared__ __align__(16) uint32_t s_thr[64];
-  __shared__ __align__(16) uint32_t s_alw[64];
-  __shared__ uint32_t s_stash[kStashSlots * kClusterThreads];
-  __shared__ int s_tot[2][2];  // {B, M} of the record being summed, two buffers
-  cg::cluster_group cl = cg::this_cluster();
-  const uint32_t ci = blockIdx.x / cl.num_blocks();
+  __shared__ int s_tot[2];  // {B, M} of the record being summed (rank 0's)
+  __shared__ Slab s_s;
+  pdl_trigger();
+  pdl_wait();
+  uint32_t C = 1, rank = 0;
+  if (CL) {
+    cg::cluster_group cl = cg::this_cluster();
+    C = cl.num_blocks();
+    rank = cl.block_rank();
+  }
+  const uint32_t ci = blockIdx.x / C;
   if (ci >= n_clusters) return;  // the same for the whole cluster
-  const uint32_t j1 = list[ci + 1];
-  for (uint32_t j = list[ci]; j < j1; j++) {
+  const uint32_t j0 = list ? list[ci] : 0u, j1 = list ? list[ci + 1] : 1u;
+  for (uint32_t j = j0; j < j1; j++) {
     __syncthreads();  // every thread is done with the previous film's descriptor
-    cluster_film<FAST>(cl, films + list[n_clusters + 1 + j], pool, records, n_sweeps, s_d, s_thr, s_alw, s_stash,
-                       s_tot, s_dyn);
+    FilmDesc* Fg = films + (list ? list[n_clusters + 1 + j] : ci);
+    {
+      const uint4* src = reinterpret_cast<const uint4*>(Fg);
+      uint4* dst = reinterpret_cast<uint4*>(&s_d);
+      for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = __ldcg(src + i);
+    }
+    __syncthreads();
+    if (!s_d.active) continue;  // the same for the whole cluster
+    const uint32_t R = slab_rows(s_d, C);
+    if (TASKS) {
+      if (R == 4) slab_film_tasks<CL, 4>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+      else if (R == 2) slab_film_tasks<CL, 2>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+      else slab_film_tasks<CL, 1>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+    } else {
+      if (R == 4) slab_film<CL, 4>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+      else if (R == 2) slab_film<CL, 2>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+      else slab_film<CL, 1>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+    }
   }
 }
 
@@ -1787,48 +1781,37 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, 
 
 namespace {
 
-// pk: one item per thread and some film of the launch packs rows
-template <uint32_t MODE>
-auto update_variant(bool exact, uint32_t items, bool pk) {
-  if (pk) return exact ? update_kernel<false, 1, MODE, true> : update_kernel<true, 1, MODE, true>;
-  return exact ? (items == 2 ? update_kernel<false, 2, MODE>
-                             : items == 1 ? update_kernel<false, 1, MODE> : update_kernel<false, 0, MODE>)
-               : (items == 2 ? update_kernel<true, 2, MODE>
-                             : items == 1 ? update_kernel<true, 1, MODE> : update_kernel<true, 0, MODE>);
+template <bool ONE>
+auto update_variant(uint32_t mode, bool pack) {
+  return mode == kUpdAccumulate    ? (pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>)
+         : mode == kUpdWriteRecord ? (pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>)
+                                   : (pack ? update_kernel<kUpdPlain, true, ONE> : update_kernel<kUpdPlain, false, ONE>);
 }
 
-template <bool MEAS>
-auto update_film_variant(bool exact, uint32_t items, bool pk) {
-  if (pk) return exact ? update_film_kernel<false, 1, MEAS, true> : update_film_kernel<true, 1, MEAS, true>;
-  return exact ? (items == 2 ? update_film_kernel<false, 2, MEAS>
-                             : items == 1 ? update_film_kernel<false, 1, MEAS> : update_film_kernel<false, 0, MEAS>)
-               : (items == 2 ? update_film_kernel<true, 2, MEAS>
-                             : items == 1 ? update_film_kernel<true, 1, MEAS> : update_film_kernel<true, 0, MEAS>);
+template <bool MEAS, bool ONE>
+auto update_film_variant(uint32_t pack) {
+  return pack == 4 ? update_film_kernel<4, MEAS, ONE>
+                   : pack == 2 ? update_film_kernel<2, MEAS, ONE> : update_film_kernel<1, MEAS, ONE>;
 }
 
 }  // namespace
 
-cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k, bool exact,
+cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
                           uint32_t items, bool pack, int64_t* part, int64_t* records, bool accumulate,
-                          uint32_t rec_done, cudaStream_t st) {
+                          uint32_t rec_done, bool first, cudaStream_t st) {
   if (grid == 0) return cudaSuccess;
-  const bool pk = pack && items == 1;
-  auto* kern = (accumulate && colour == 1) ? update_variant<kUpdAccumulate>(exact, items, pk)
-               : (rec_done && colour == 0) ? update_variant<kUpdWriteRecord>(exact, items, pk)
-                                           : update_variant<kUpdPlain>(exact, items, pk);
+  const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
+  auto* kern = items == 1 ? update_variant<true>(mode, pack) : update_variant<false>(mode, pack);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, (const FilmDesc*)L.films, (const uint32_t*)L.owner_upd,
-                    (const LaunchHdr*)L.hdr, pool, colour, k, part, records, rec_done);
+                    (const LaunchHdr*)L.hdr, pool, colour, k, items, part, records, rec_done, first ? 1u : 0u);
 }
 
 cudaError_t launch_update_film(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep, uint32_t items,
                                int64_t* acc, cudaStream_t st) {
-  const uint32_t ipb = words_per_block(items);
-  const uint32_t grid = (grid_items(d, items) + ipb - 1) / ipb;
-  if (grid == 0) return cudaSuccess;
-  const bool exact = d.has_never != 0;
-  const bool pk = items == 1 && d.pack > 1;
-  auto* kern = acc ? update_film_variant<true>(exact, items, pk) : update_film_variant<false>(exact, items, pk);
-  return launch_pdl(kern, grid, kFilmThreads, 0, st, d, pool, colour, sweep, acc);
+  const uint32_t grid = update_blocks(d, items);
+  auto* kern = items == 1 ? (acc ? update_film_variant<true, true>(d.pack) : update_film_variant<false, true>(d.pack))
+                          : (acc ? update_film_variant<true, false>(d.pack) : update_film_variant<false, false>(d.pack));
+  return launch_pdl(kern, grid, kFilmThreads, 0, st, d, pool, colour, sweep, items, acc);
 }
 
 cudaError_t launch_record(const LaunchSet& L, uint32_t grid, int64_t* part, int64_t* records, uint32_t done,
@@ -1877,21 +1860,27 @@ uint32_t resident_smem_bytes(const FilmDesc& d) {
   const uint64_t sites = (uint64_t)d.Lx * d.Ly * d.Lz;
   const uint64_t bytes = 4ull * (2ull * d.Lx * d.Ly * d.W + d.Lx);
   if (sites > kResidentMaxSites || bytes > kResidentMaxSmem) return 0;
-  return (uint32_t)bytes;
+  return (uint32_t)(bytes + 8ull * d.Lx);  // the layer tables beside the planes and sums
 }
 
-uint32_t resident_threads(const FilmDesc& d) {
-  const uint32_t t = ((d.upd_items + 31u) / 32u) * 32u;
-  return t < 32u ? 32u : (t > kResidentThreads ? kResidentThreads : t);
+// Dynamic shared memory of the task form: planes, tables, words, mask buffers.
+static uint64_t slab_task_bytes(const FilmDesc& d, uint32_t C) {
+  const uint64_t nlm = (d.Lx + C - 1) / C, words = nlm * (d.Ly / slab_rows(d, C)) * d.W;
+  bool all7 = !d.cls[0].sym;
+  // a CTA's general words: its share of the walls' layers and of their mirrors
+  const uint64_t gen = all7 ? words : std::min<uint64_t>(words, 2 * (words / nlm) + 2 * d.W);
+  return 8ull * words + 12ull * d.Lx + 16 + words * sizeof(uint32_t) * 8 + 2 * ((words + 1) & ~1ull) +
+         2 * 4ull * (3 * (words - gen) + 7 * gen) + 16;
 }
 
-cudaError_t launch_resident(FilmDesc* films, uint32_t n_films, uint32_t smem_bytes, uint32_t threads, bool exact,
-                            uint32_t* pool, int64_t* records, uint32_t n_sweeps, cudaStream_t st) {
-  if (n_films == 0 || n_sweeps == 0) return cudaSuccess;
-  if (smem_bytes > kResidentMaxSmem || threads == 0 || threads > kResidentThreads || threads % 32u)
-    return cudaErrorInvalidValue;
-  auto* kern = exact ? resident_kernel<false> : resident_kernel<true>;
-  return launch_pdl(kern, n_films, threads, smem_bytes, st, films, pool, records, n_sweeps);
+bool slab_tasks_fit(const FilmDesc& d, uint32_t C) {
+  const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * (d.Ly / slab_rows(d, C)) * d.W;
+  return words <= 0xFFFFu && (uint64_t)d.Lx * d.Ly <= 0xFFFFu && d.W <= 0xFFFFu &&
+         slab_task_bytes(d, C) <= kClusterMaxSmem;
+}
+
+uint32_t slab_dyn_bytes(const FilmDesc& d, uint32_t C, bool tasks) {
+  return tasks ? (uint32_t)slab_task_bytes(d, C) : cluster_smem_bytes(d, C);
 }
 
 uint32_t cluster_smem_bytes(const FilmDesc& d, uint32_t C) {
@@ -1902,14 +1891,16 @@ uint32_t cluster_smem_bytes(const FilmDesc& d, uint32_t C) {
   return (uint32_t)bytes;
 }
 
-uint32_t cluster_threads(const FilmDesc& d, uint32_t C, bool exact, uint32_t per_sm) {
-  // a pair item (ky = 1 word and its wrap partner) is two words of work
-  const uint64_t tmax = std::max<uint64_t>(32, cluster_max_threads(exact) / std::max<uint32_t>(per_sm, 1) / 32 * 32);
-  const uint64_t nlm = (d.Lx + C - 1) / C;
-  const uint64_t work = nlm * d.Ly * d.W;
-  const uint64_t rounds = std::max<uint64_t>(1, (work + tmax - 1) / tmax);
-  const uint64_t t = ((work + rounds - 1) / rounds + 31) / 32 * 32;
-  return (uint32_t)std::min<uint64_t>(std::max<uint64_t>(t, 32), tmax);
+uint32_t cluster_threads(const FilmDesc& d, uint32_t C, uint32_t per_sm, bool tasks) {
+  const uint32_t per = std::max<uint32_t>(per_sm, 1);
+  if (!tasks) return slab_shape(d, C, kSlabThreads / per / 32 * 32).threads;
+  const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * (d.Ly / slab_rows(d, C)) * d.W, tmax = kTaskThreads / per / 32 * 32;
+  // four lanes per word and a thread per decision, if there is room for both
+  const uint64_t t = (words + 31) / 32 * 32;
+  if (5 * t <= tmax) return (uint32_t)(5 * t);
+  if (2 * t <= tmax) return (uint32_t)tmax;
+  const uint64_t turns = (words + tmax - 1) / tmax;  // one lane per word, in equal turns
+  return (uint32_t)std::min<uint64_t>(((words + turns - 1) / turns + 31) / 32 * 32, tmax);
 }
 
 namespace {
@@ -1935,13 +1926,22 @@ cudaError_t cluster_launch_smem(K kern, uint32_t needed, uint32_t per_sm, uint32
   return cudaSuccess;
 }
 
-template <typename K>
-cudaLaunchConfig_t cluster_config(K kern, uint32_t grid, uint32_t C, uint32_t smem, uint32_t threads,
-                                  cudaStream_t st, cudaLaunchAttribute* attr, cudaError_t* e) {
-  *e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterMaxSmem);
+using SlabKernel = void (*)(FilmDesc*, const uint32_t*, uint32_t, uint32_t*, int64_t*, uint32_t);
+SlabKernel slab_variant(uint32_t C, bool tasks) {
+  return C > 1 ? (tasks ? slab_kernel<true, true> : slab_kernel<true, false>)
+               : (tasks ? slab_kernel<false, true> : slab_kernel<false, false>);
+}
+
+cudaError_t slab_attributes(SlabKernel kern) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kClusterMaxSmem);
   // the whole unified L1 as shared memory, so that per_sm padded CTAs fit
-  if (*e == cudaSuccess)
-    *e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
+  return e;
+}
+
+cudaLaunchConfig_t cluster_config(uint32_t grid, uint32_t C, uint32_t smem, uint32_t threads, cudaStream_t st,
+                                  cudaLaunchAttribute* attr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
@@ -1956,38 +1956,38 @@ cudaLaunchConfig_t cluster_config(K kern, uint32_t grid, uint32_t C, uint32_t sm
   return cfg;
 }
 
+bool slab_launch_ok(uint32_t C, uint32_t per_sm, uint32_t smem_bytes, uint32_t threads, bool tasks) {
+  return C >= 1 && C <= kClusterMaxSize && per_sm >= 1 && per_sm <= kClusterMaxPerSm && smem_bytes <= kClusterMaxSmem &&
+         threads && threads % 32u == 0 && threads <= (tasks ? kTaskThreads : kSlabThreads);
+}
+
 }  // namespace
 
-int cluster_capacity(uint32_t C, uint32_t per_sm, uint32_t smem_bytes, uint32_t threads, bool exact) {
-  if (C == 0 || C > kClusterMaxSize || per_sm == 0 || per_sm > kClusterMaxPerSm || smem_bytes > kClusterMaxSmem ||
-      threads == 0 || threads > cluster_max_threads(exact) || threads % 32u)
-    return 0;
-  auto* kern = exact ? cluster_kernel<false> : cluster_kernel<true>;
+int cluster_capacity(uint32_t C, uint32_t per_sm, uint32_t smem_bytes, uint32_t threads, bool tasks,
+                     uint32_t* smem_launch) {
+  if (!slab_launch_ok(C, per_sm, smem_bytes, threads, tasks)) return 0;
+  const SlabKernel kern = slab_variant(C, tasks);
   uint32_t smem = 0;
-  if (cluster_launch_smem(kern, smem_bytes, per_sm, &smem) != cudaSuccess) return -1;
+  if (slab_attributes(kern) != cudaSuccess || cluster_launch_smem(kern, smem_bytes, per_sm, &smem) != cudaSuccess)
+    return -1;
+  *smem_launch = smem;
   cudaLaunchAttribute attr[1];
-  cudaError_t e;
-  cudaLaunchConfig_t cfg = cluster_config(kern, C, C, smem, threads, nullptr, attr, &e);
-  if (e != cudaSuccess) return -1;
+  cudaLaunchConfig_t cfg = cluster_config(C, C, smem, threads, nullptr, attr);
   int n = 0;
   if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) return -1;
   return n;
 }
 
-cudaError_t launch_cluster(FilmDesc* films, const uint32_t* list, uint32_t n_clusters, uint32_t C, uint32_t per_sm,
-                           uint32_t smem_bytes, uint32_t threads, bool exact, uint32_t* pool, int64_t* records,
+cudaError_t launch_cluster(FilmDesc* films, const uint32_t* list, uint32_t n_clusters, uint32_t C,
+                           uint32_t smem_launch, uint32_t threads, bool tasks, uint32_t* pool, int64_t* records,
                            uint32_t n_sweeps, cudaStream_t st) {
   if (n_clusters == 0 || n_sweeps == 0) return cudaSuccess;
-  if (C == 0 || C > kClusterMaxSize || per_sm == 0 || per_sm > kClusterMaxPerSm || smem_bytes > kClusterMaxSmem ||
-      threads == 0 || threads > cluster_max_threads(exact) || threads % 32u)
-    return cudaErrorInvalidValue;
-  auto* kern = exact ? cluster_kernel<false> : cluster_kernel<true>;
-  uint32_t smem = 0;
-  cudaError_t e = cluster_launch_smem(kern, smem_bytes, per_sm, &smem);
-  if (e != cudaSuccess) return e;
+  if (!slab_launch_ok(C, 1, smem_launch, threads, tasks)) return cudaErrorInvalidValue;
+  const SlabKernel kern = slab_variant(C, tasks);
+  if (C == 1)
+    return launch_pdl(kern, n_clusters, threads, smem_launch, st, films, list, n_clusters, pool, records, n_sweeps);
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = cluster_config(kern, n_clusters * C, C, smem, threads, st, attr, &e);
-  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = cluster_config(n_clusters * C, C, smem_launch, threads, st, attr);
   return cudaLaunchKernelEx(&cfg, kern, films, list, n_clusters, pool, records, n_sweeps);
 }
 
@@ -2005,7 +2005,7 @@ int read_oob_counters(unsigned long long* count, unsigned long long* first) {
 
 int update_blocks_per_sm() {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, update_kernel<true, 1, kUpdPlain>, kFilmThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, update_kernel<kUpdPlain, false, true>, kFilmThreads, 0) !=
       cudaSuccess)
     return 0;
   return nb;

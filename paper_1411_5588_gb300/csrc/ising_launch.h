@@ -8,20 +8,18 @@
 
 namespace isg {
 
-// Grid update kernels: threads per block and blocks per SM.  A block updates
-// items * kFilmThreads consecutive words of one film, items (words per
-// thread, 1 or 2) being the launch shape the autotuner picks per film or
-// film set: one word per thread halves the dependency chain of a launch
-// (small and medium films are latency bound), two let each thread overlap
-// the loads of its second word with the first word's arithmetic.
+// Grid update kernels: threads per block and blocks per SM.  A thread has a
+// column of column_len(items) words, items being the launch shape: GRID_1 (1)
+// one, GRID_Q (0) two, GRID_2 (2) four.
 constexpr uint32_t kFilmThreads = 128;
-constexpr int kFilmMinBlocks = 6;
-constexpr int kMultiMinBlocks = 6;
-constexpr int kMultiMinBlocks1 = 7;  // multi-film kernel, one word per thread, not summing records
-// items = 0 is the quarter shape: four lanes share each word (they split its
-// eight Philox calls), so a block covers kFilmThreads / 4 words.
-__host__ __device__ constexpr uint32_t words_per_block(uint32_t items) {
-  return items == 0 ? kFilmThreads / 4 : kFilmThreads * items;
+constexpr int film_min_blocks(int rows, bool meas, bool one) {
+  return one ? (rows == 4 ? 5 : meas ? 7 : 8) : rows > 1 || meas ? 5 : 6;
+}
+constexpr int multi_min_blocks(bool one, bool meas, bool pack) {
+  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 4 : 5;
+}
+__host__ __device__ constexpr uint32_t column_len(uint32_t items) {
+  return items == 1 ? 1 : items == 2 ? 4 : 2;
 }
 constexpr int kMeasureBlock = 256;
 
@@ -41,10 +39,13 @@ __host__ __device__ inline uint64_t acc_offset(const FilmDesc& d) {
 // (fill_geometry); four rows pack at any size.
 constexpr uint32_t kPack2Rows = 8192;
 
-// Items of a film in the grid update kernels with `items` words per thread:
-// thin films pack rows at one item per thread only.
+// Columns of a film in the grid update kernels (of words, or of packed words of
+// `pack` rows): the pairs, then the rows between the first and the last.
 __host__ __device__ inline uint32_t grid_items(const FilmDesc& d, uint32_t items) {
-  return (items == 1 && d.pack > 1) ? d.pk_items : d.upd_items;
+  return d.Lx * d.W * (1 + d.cols[items]);
+}
+__host__ __device__ inline uint32_t update_blocks(const FilmDesc& d, uint32_t items) {
+  return (grid_items(d, items) + kFilmThreads - 1) / kFilmThreads;
 }
 
 // Measurement blocks of one film.
@@ -52,32 +53,57 @@ inline uint32_t meas_units(const FilmDesc& d) {
   return d.meas_lpu > 1 ? (d.Lx + d.meas_lpu - 1) / d.meas_lpu : d.Lx * d.meas_bpl;
 }
 
-// Resident path: one block per film holds the film's packed planes in shared
-// memory (row stride W) for a whole run of sweeps, records included.  Films
-// up to kResidentMaxSites spins whose planes and layer sums fit in
+// Resident path: one CTA holds the film in shared memory for a whole run of
+// sweeps, records included (the slab kernel with C = 1).  Films up to
+// kResidentMaxSites spins whose planes and layer sums fit in
 // kResidentMaxSmem bytes qualify; larger ones use the per-half-sweep grid.
-// Chosen automatically up to kResidentAutoSites: beyond that one SM's issue
-// rate loses to the grid kernels (about 16 us per sweep there without
-// records, 27 us with one every sweep).
-constexpr uint32_t kResidentThreads = 512;
+// Chosen automatically, without a measurement, up to kResidentAutoSites; the
+// cluster path from there up to kClusterAutoSites.  Per sweep on GB300, a record
+// every sweep, resident / cluster of 8 / best grid: 8^3 2.3 / 2.6 / 8.4 us,
+// 16x48x32 5.7 / 3.3 / 8.4, 32^3 7.8 / 3.6 / 7.6, 32x64x64 - / 5.6 / 8.9; without
+// records the grid draws level at 32x96x64 (6.0 / 6.0 us).
 constexpr uint64_t kResidentMaxSites = 1ull << 16;
-constexpr uint64_t kResidentAutoSites = 1ull << 15;
+constexpr uint64_t kResidentAutoSites = 1ull << 10;
+constexpr uint64_t kClusterAutoSites = 3ull << 15;
+constexpr uint64_t kResidentOnlySites = 1ull << 15;
 constexpr uint32_t kResidentMaxSmem = 48u * 1024u;
 
-// Cluster-resident path: a thread-block cluster of C CTAs (C <= kClusterMaxSize)
-// holds one film in distributed shared memory for a whole call of sweeps,
-// each CTA a slab of ceil(Lx / C) layers or one fewer.  kClusterThreads is the
-// most threads a CTA runs (one CTA per SM at the update body's registers);
-// kClusterMaxSmem the most dynamic shared memory a CTA takes.  The exact-table
-// variant (a strict compare and a mux tree per site) needs more registers, so
-// it runs at most kClusterThreadsExact.
-constexpr uint32_t kClusterThreads = 704;
-constexpr uint32_t kClusterThreadsExact = 512;
-__host__ __device__ constexpr uint32_t cluster_max_threads(bool exact) {
-  return exact ? kClusterThreadsExact : kClusterThreads;
-}
+// Slab path: a thread-block cluster of C CTAs (C <= kClusterMaxSize) holds one
+// film in distributed shared memory for a whole call of sweeps, each CTA a
+// slab of ceil(Lx / C) layers or one fewer.  kSlabThreads is the most threads
+// a CTA runs on columns, kTaskThreads the most on tasks (slab_tasks_fit);
+// kClusterMaxSmem the most dynamic shared memory it takes.
+constexpr uint32_t kSlabThreads = 640;
+constexpr uint32_t kTaskThreads = 640;
 constexpr uint32_t kClusterMaxSize = 8;
 constexpr uint32_t kClusterMaxSmem = 200u * 1024u;
+
+// Rows per word of film d on clusters of C CTAs: thin films pack (sl_pack)
+// unless the words, one row each, already fit one turn of a CTA's threads.
+__host__ __device__ inline uint32_t slab_rows(const FilmDesc& d, uint32_t C) {
+  const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * d.Ly * d.W;
+  return words <= 128 ? 1u : d.sl_pack;
+}
+// Columns of a slab (the largest of the cluster's) over at most tmax threads:
+// each layer's G groups (words, W of them per group) in equal columns of
+// `len` >= 2 steps, as short as one turn of the threads allows; with more than
+// tmax columns of whole layers, threads take several in turn.
+struct SlabShape {
+  uint32_t len, turns, threads;
+};
+__host__ __device__ inline SlabShape slab_shape(const FilmDesc& d, uint32_t C, uint32_t tmax) {
+  const uint32_t G = d.Ly / slab_rows(d, C), per = (d.Lx + C - 1) / C * d.W;
+  uint32_t n = tmax / per;  // columns per layer and word
+  if (n < 1) n = 1;
+  SlabShape o;
+  o.len = (G + n - 1) / n;
+  if (o.len < 2) o.len = 2;
+  const uint32_t cols = per * ((G + o.len - 1) / o.len);
+  o.turns = (cols + tmax - 1) / tmax;
+  o.threads = ((cols + o.turns - 1) / o.turns + 31) / 32 * 32;
+  if (o.threads > tmax) o.threads = tmax;
+  return o;
+}
 
 // Device arrays describing the films of a launch.
 struct LaunchSet {
@@ -87,18 +113,17 @@ struct LaunchSet {
   LaunchHdr* hdr = nullptr;          // sizes
 };
 
-// exact: some film of the launch has a reachable thr = 0 entry (has_never);
-// items: words per thread (1 or 2, or 0 for four lanes per word), matching the
-// owner table's block size.  Records: with accumulate (colour 1) the films
-// that record after sweep k add their record sums into their accumulators in
-// part; with rec_done > 0 (colour 0) the films that recorded after rec_done
-// sweeps have that record written into their rings in records by this
-// launch (the chunk's last record goes through launch_record instead).
-// pack: some film of the launch packs rows (FilmDesc::pack > 1; with items
-// 1 its owner table counts groups of rows, grid_items).
-cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k, bool exact,
+// items: the launch shape, matching the owner table's block size.  Records:
+// with accumulate (colour 1) the films that record after sweep k add their
+// record sums into their accumulators in part; with rec_done > 0 (colour 0) the
+// films that recorded after rec_done sweeps have that record written into
+// their rings in records by this launch (the chunk's last record goes through
+// launch_record instead).  pack: some film of the launch packs rows
+// (FilmDesc::pack > 1).  first: the chunk's first launch, whose predecessor may
+// still be advancing the films' sweep counters.
+cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
                           uint32_t items, bool pack, int64_t* part, int64_t* records, bool accumulate,
-                          uint32_t rec_done, cudaStream_t st);
+                          uint32_t rec_done, bool first, cudaStream_t st);
 // One half-sweep of a single film whose descriptor (with `sweep` absolute) is
 // passed by value; acc (colour 1 of a recorded sweep, else null): the film's
 // accumulators.
@@ -118,39 +143,37 @@ cudaError_t launch_pack(const FilmDesc& f, uint32_t* pool, const int8_t* s, cuda
 cudaError_t launch_unpack(const FilmDesc& f, const uint32_t* pool, int8_t* s, cudaStream_t st);
 // Dynamic shared memory of a film on the resident path, 0 if it does not qualify.
 uint32_t resident_smem_bytes(const FilmDesc& d);
-// Threads per block for a film on the resident path (a multiple of 32).
-uint32_t resident_threads(const FilmDesc& d);
-// n_sweeps sweeps (with their records) of films[0..n_films) on the resident
-// path, one block each; every film must qualify, smem_bytes and threads cover
-// the largest.  The kernel advances each descriptor's sweep and rec_next.
-cudaError_t launch_resident(FilmDesc* films, uint32_t n_films, uint32_t smem_bytes, uint32_t threads, bool exact,
-                            uint32_t* pool, int64_t* records, uint32_t n_sweeps, cudaStream_t st);
 // Dynamic shared memory of a CTA of film d on the cluster-resident path with
 // clusters of C CTAs, 0 if the film does not qualify (C out of range, fewer
 // layers than C, or too large).
 uint32_t cluster_smem_bytes(const FilmDesc& d, uint32_t C);
-// CTAs of the cluster path that share one SM (1..kClusterMaxPerSm): a CTA's
-// half-sweep ends at a cluster barrier where its warps wait for the slowest,
-// and CTAs of other films on the same SM fill that wait.  per_sm divides the
-// threads a CTA may run, and the launch pads each CTA's shared memory so
-// that no more than per_sm CTAs fit on an SM.
-constexpr uint32_t kClusterMaxPerSm = 3;
+// CTAs of the cluster path that share one SM (1..kClusterMaxPerSm): the launch
+// pads each CTA's shared memory so that no more than per_sm fit on an SM.
+constexpr uint32_t kClusterMaxPerSm = 2;
 // Threads per CTA for film d with clusters of C CTAs, per_sm CTAs per SM: the
-// slab's update items spread over as few full rounds as
-// cluster_max_threads(exact) / per_sm allows (a multiple of 32).
-uint32_t cluster_threads(const FilmDesc& d, uint32_t C, bool exact, uint32_t per_sm);
+// slab's columns (slab_shape) over at most kSlabThreads / per_sm threads, or its
+// draw tasks over at most kTaskThreads / per_sm (a multiple of 32).
+uint32_t cluster_threads(const FilmDesc& d, uint32_t C, uint32_t per_sm, bool tasks);
+// Whether the task form's words and masks fit a CTA's shared memory, and the
+// dynamic shared memory of either form.
+bool slab_tasks_fit(const FilmDesc& d, uint32_t C);
+uint32_t slab_dyn_bytes(const FilmDesc& d, uint32_t C, bool tasks);
 // Clusters of C CTAs (smem_bytes of dynamic shared memory needed and threads
 // each, per_sm of them per SM) that one GPU can hold at once (0: such a
-// launch cannot run), or -1 on a CUDA error.
-int cluster_capacity(uint32_t C, uint32_t per_sm, uint32_t smem_bytes, uint32_t threads, bool exact);
+// launch cannot run), or -1 on a CUDA error.  Sets the kernel's attributes and
+// *smem_launch, the padded shared memory to launch with: a launch needs no
+// further queries (six calls, some 5 us of host time).
+int cluster_capacity(uint32_t C, uint32_t per_sm, uint32_t smem_bytes, uint32_t threads, bool tasks,
+                     uint32_t* smem_launch);
 // n_sweeps sweeps (with their records) of films on the cluster path:
-// n_clusters clusters of C CTAs, per_sm CTAs per SM, cluster i sweeping the
-// films list[n_clusters + 1 + j], j in [list[i], list[i + 1]), one after
-// another (list: device memory).  Every listed film must qualify for C, and
-// smem_bytes and threads cover the largest.  The kernel advances each
-// descriptor's sweep and rec_next.
-cudaError_t launch_cluster(FilmDesc* films, const uint32_t* list, uint32_t n_clusters, uint32_t C, uint32_t per_sm,
-                           uint32_t smem_bytes, uint32_t threads, bool exact, uint32_t* pool, int64_t* records,
+// n_clusters clusters of C CTAs, cluster i sweeping the films list[n_clusters +
+// 1 + j], j in [list[i], list[i + 1]), one after another (list: device memory;
+// null: cluster i sweeps film i).  Every listed film must qualify for C (tasks:
+// for slab_tasks_fit), threads cover the largest, and smem_launch is
+// cluster_capacity's for these.  The kernel advances each descriptor's sweep
+// and rec_next.
+cudaError_t launch_cluster(FilmDesc* films, const uint32_t* list, uint32_t n_clusters, uint32_t C,
+                           uint32_t smem_launch, uint32_t threads, bool tasks, uint32_t* pool, int64_t* records,
                            uint32_t n_sweeps, cudaStream_t st);
 // Checked builds: the out-of-range access counters (returns 1); other
 // builds return 0 with both zero; -1 on a CUDA error.
