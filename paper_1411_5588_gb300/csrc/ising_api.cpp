@@ -261,7 +261,9 @@ int wait_stream(cudaStream_t st, double timeout_s) {
     if (e != cudaErrorNotReady) return fail(ISING_ECUDA, "stream: %s", cudaGetErrorString(e));
     const double dt = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (dt > timeout_s) return fail(ISING_ETIMEOUT, "wait timed out after %.3f s", dt);
-    std::this_thread::sleep_for(std::chrono::microseconds(50));
+    // most waits end within a few launches: a sleep (50 us and the wake-up)
+    // would be the longest part of them
+    if (dt > 200e-6) std::this_thread::sleep_for(std::chrono::microseconds(50));
   }
 }
 
