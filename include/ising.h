@@ -78,11 +78,10 @@ enum { ISING_INIT_RANDOM = 0, ISING_INIT_SLAB_Y = 1, ISING_INIT_ALL_UP = 2 };
  * GRID_1    two grid launches per sweep, one 32-site word per thread: the
  *           shortest launch latency.  A recorded sweep's second launch also
  *           sums the record, and a small kernel writes it;
- * GRID_2    the same with two words per thread, which overlaps one word's
- *           loads with the other's arithmetic;
- * GRID_Q    the same with four threads per word, each drawing two of its
- *           eight Philox calls: four times the threads for the same work,
- *           for films too small to fill the GPU otherwise.
+ * GRID_2    the same with a column of four words per thread, which share
+ *           loads and address arithmetic: the least work per word;
+ * GRID_Q    the same with columns of two words, between the two: for films
+ *           whose columns of four are too few to fill the GPU.
  * CLUSTER   a thread-block cluster of C CTAs keeps a film in distributed
  *           shared memory for all sweeps of an ising_sweep or
  *           ising_batch_sweep call, CTA r holding layers [r Lx / C,
@@ -96,8 +95,10 @@ enum { ISING_INIT_RANDOM = 0, ISING_INIT_SLAB_Y = 1, ISING_INIT_ALL_UP = 2 };
  *           falls between half-sweeps (the Appendix's many independent
  *           films, each on its own few SMs).
  * AUTO      the autotuner's measurement for this film shape and record
- *           interval if there is one, else RESIDENT up to 32768 spins and
- *           GRID_1 above. */
+ *           interval if there is one, else RESIDENT up to 1024 spins,
+ *           CLUSTER up to 98304 (a film that qualifies for no cluster of two
+ *           or more: RESIDENT up to 32768), GRID_1 above, and GRID_Q from
+ *           2^18 words per half-sweep up. */
 enum { ISING_SHAPE_AUTO = 0, ISING_SHAPE_RESIDENT = 1, ISING_SHAPE_GRID_1 = 2, ISING_SHAPE_GRID_2 = 3,
        ISING_SHAPE_GRID_Q = 4, ISING_SHAPE_CLUSTER = 5 };
 
@@ -171,8 +172,8 @@ int ising_get_shape(ising *h, uint32_t measure_every, int *shape);
  * shape) on a scratch film of the same shape and parameters, with a record
  * every measure_every sweeps, so this handle's chain is not touched.  The
  * fastest goes into a process-wide table keyed by (Lx, Ly, Lz, boundary
- * modes, table variant, record interval up to 16) that every AUTO handle of
- * that key then uses; *shape (may be NULL) receives it.  Shapes are tried
+ * modes, record interval up to 16) that every AUTO handle of that key then
+ * uses; *shape (may be NULL) receives it.  Shapes are tried
  * in the order RESIDENT, GRID_1, GRID_2, GRID_Q, CLUSTER, and a later one must be at least 2%
  * faster to win.  Synchronises. */
 int ising_autotune(ising *h, uint32_t measure_every, int *shape);
@@ -267,7 +268,8 @@ int ising_batch_sweep(ising_batch *b, uint64_t n_sweeps, int use_graph);
 int ising_batch_reserve_records(ising_batch *b, uint64_t n_records);
 
 /* Launch shape of the batch: GRID_1, GRID_2, GRID_Q, CLUSTER, or AUTO (the
- * autotuner's choice once ising_batch_autotune has run, else GRID_1).
+ * autotuner's choice once ising_batch_autotune has run, else GRID_1, or GRID_2
+ * where the lanes have more than 2^18 words each on average).
  * CLUSTER takes the pinned cluster size (ising_batch_set_cluster_size), else
  * the largest C <= 8 for which every film qualifies and the n films' n C CTAs
  * fit on the GPU's SMs (C = 1 when the films outnumber the SMs); a film

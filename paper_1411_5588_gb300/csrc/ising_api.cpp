@@ -348,8 +348,9 @@ uint32_t handle_cluster_size(ising* h) {
 // The launch shape of an ising_sweep call: the pinned one, else the
 // autotuner's choice for this film shape and record interval, else the
 // resident kernel up to kResidentAutoSites spins, a cluster up to
-// kClusterAutoSites, and one word per thread above; a film that no cluster
-// takes (one layer) is resident up to kResidentOnlySites.
+// kClusterAutoSites, one word per thread above up to kOneWordAutoWords, and
+// columns of two; a film that no cluster takes (one layer) is resident up to
+// kResidentOnlySites.
 int resolve_shape(ising* h, uint32_t measure_every) {
   const FilmDesc& d = h->d();
   if (h->shape != ISING_SHAPE_AUTO) return h->shape;
@@ -360,7 +361,8 @@ int resolve_shape(ising* h, uint32_t measure_every) {
   const uint64_t sites = (uint64_t)d.Lx * d.Ly * d.Lz;
   if (sites <= kResidentAutoSites && resident_smem_bytes(d)) return ISING_SHAPE_RESIDENT;
   if (sites <= kClusterAutoSites && handle_cluster_size(h) > 1) return ISING_SHAPE_CLUSTER;
-  return (sites <= kResidentOnlySites && resident_smem_bytes(d)) ? ISING_SHAPE_RESIDENT : ISING_SHAPE_GRID_1;
+  if (sites <= kResidentOnlySites && resident_smem_bytes(d)) return ISING_SHAPE_RESIDENT;
+  return launch_words(d) <= kOneWordAutoWords ? ISING_SHAPE_GRID_1 : ISING_SHAPE_GRID_Q;
 }
 
 int sync_desc(ising* h) {

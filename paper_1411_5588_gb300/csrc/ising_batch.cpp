@@ -34,7 +34,7 @@ struct Lane {
   std::map<uint32_t, cudaGraphExec_t> graphs;  // chunk length -> executable graph
   cudaEvent_t ev_done = nullptr;               // the lane's last sweep call has finished
   // cluster-resident path (CTAs per film; 0: the grid kernels), with the
-  // launch's shared memory and threads per CTA and its table variant
+  // launch's shared memory and threads per CTA
   uint32_t cl_size = 0, cl_smem = 0, cl_threads = 0;
   bool cl_tasks = false;           // the task form (slab_tasks_fit)
   uint32_t cl_clusters = 0;        // clusters of the lane's launch
@@ -414,6 +414,14 @@ struct ising_batch {
 
 namespace {
 
+// Without a measurement: columns of four when the lanes' launches are large.
+uint32_t batch_auto_items(const ising_batch* b) {
+  uint64_t words = 0;
+  for (const Lane* l : b->lanes)
+    for (const FilmDesc& d : l->fs.h) words += launch_words(d);
+  return words <= kOneWordAutoWords * b->lanes.size() ? 1u : 2u;
+}
+
 int batch_apply_items(ising_batch* b, uint32_t items) {
   for (Lane* l : b->lanes) {
     int rc = lane_apply_cluster(l, 0, 0);
@@ -496,6 +504,7 @@ int batch_create(const ising_job* jobs, size_t n, uint32_t lanes, ising_batch** 
     rc = fail(ISING_ECUDA, "event creation failed");
   }
   if (!rc) b->device = b->lanes[0]->fs.device;
+  if (!rc) rc = batch_apply_items(b, batch_auto_items(b));
   if (rc) {
     ising_batch_destroy(b);
     return rc;
@@ -592,7 +601,7 @@ int ising_batch_set_shape(ising_batch* b, int shape) {
   }
   b->shape = shape;
   if (shape == ISING_SHAPE_AUTO && b->tuned_shape == ISING_SHAPE_CLUSTER) return batch_apply_cluster(b, b->tuned_cl);
-  const uint32_t items = shape == ISING_SHAPE_AUTO ? (b->tuned_shape ? shape_items(b->tuned_shape) : 1u)
+  const uint32_t items = shape == ISING_SHAPE_AUTO ? (b->tuned_shape ? shape_items(b->tuned_shape) : batch_auto_items(b))
                                                    : shape_items(shape);
   return batch_apply_items(b, items);
 }

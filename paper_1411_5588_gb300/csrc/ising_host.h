@@ -70,7 +70,7 @@ struct FilmSet {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int n_sm = 0, upd_per_sm = 0, meas_per_sm = 0;
-  uint32_t items = 1;  // words per thread of the grid update kernel (1, 2; 0 = four threads per word)
+  uint32_t items = 1;  // launch shape of the grid update kernels (column_len: 1 one word per thread, 0 two, 2 four)
 
   std::vector<FilmDesc> h;  // host mirror (counters tracked on the host too)
   LaunchHdr hh{};
@@ -104,11 +104,11 @@ struct FilmSet {
 
 // A candidate launch shape replaces the autotuner's current best only when it
 // is this much faster (candidates are tried in the order RESIDENT, GRID_1,
-// GRID_2, GRID_Q), so that shapes within timing noise of each other resolve
+// GRID_2, GRID_Q, CLUSTER), so that shapes within timing noise of each other resolve
 // the same way on every run.
 constexpr float kTuneMargin = 0.98f;
 
-// Grid kernel words-per-thread code of a grid shape, and back.
+// The grid kernels' code of a grid shape (column_len), and back.
 inline uint32_t shape_items(int shape) {
   return shape == ISING_SHAPE_GRID_2 ? 2u : shape == ISING_SHAPE_GRID_Q ? 0u : 1u;
 }

@@ -1,15 +1,21 @@
 // CUDA kernels of the Ising-film sweep for sm_103a.
 //
-//  - update_kernel: one half-sweep (colour c) of every film of a launch.  The
-//    four phases of a sweep (Appendix checkerboard, split by the Eq. 11 wrap
-//    rows) run as two launches: a thread updates one word of row (kx, ky<Ly)
-//    and, when ky = 1, then the word of row (kx', Ly) whose wrap neighbour is
-//    (kx, 1) -- kx' = Lx+1-kx for the Eq. 11 rule, kx' = kx otherwise.  That
-//    row depends on nothing else updated in the half-sweep, so the thread-local
-//    order reproduces "all of {c, ky<Ly}, then all of {c, ky=Ly}" exactly.
-//    The half-sweep 1 launch of a sweep after which films record also sums
-//    their int64 record quantities B, M, M1, Mn and m(kx) (Eqs. 1, 7, 9, 17,
-//    19) from the words it holds in registers, into per-layer accumulators.
+//  - update_kernel, update_film_kernel: one half-sweep (colour c) of every film
+//    of a launch, of one film.  The four phases of a sweep (Appendix
+//    checkerboard, split by the Eq. 11 wrap rows) run as two launches: the
+//    thread that decides a word of row (kx, 1) decides the word of row (kx', Ly)
+//    whose wrap neighbour it is right after it -- kx' = Lx+1-kx for the Eq. 11
+//    rule, kx' = kx otherwise.  That row depends on nothing else updated in the
+//    half-sweep, so the thread-local order reproduces "all of {c, ky<Ly}, then
+//    all of {c, ky=Ly}" exactly.  The half-sweep 1 launch of a sweep after which
+//    films record also sums their int64 record quantities B, M, M1, Mn and
+//    m(kx) (Eqs. 1, 7, 9, 17, 19) from the words it holds in registers, into
+//    per-layer accumulators.
+//  - slab_kernel: every sweep of a call with the film in shared memory, of one
+//    CTA (the resident path) or of a cluster's CTAs.
+//  In both a word's random numbers are drawn and compared before its lattice
+//  neighbourhood is known (ising_draw.cuh), so the wait for the previous
+//  half-sweep -- a launch or a barrier -- hides behind the draws.
 //  - record_kernel: writes those records and clears the accumulators.
 //  - measure_partial_kernel / measure_finalize_kernel: the same sums from the
 //    lattice alone (an on-demand measurement), per-block partials in a
@@ -201,9 +207,10 @@ struct Drawn {
 };
 
 // Masks of one word of R rows from row `row` (parity array X) of class cl;
-// any7: the warp takes the general form (ROLL: as a
-// loop over the calls, in fewer registers).  calls: the word's (R > 1: a row's)
-// Philox calls; full: every word of the film has eight.
+// any7: the warp takes the general form (ROLL: as a loop over the calls, in
+// fewer registers: the general form of one word per thread then keeps to the 64
+// of eight blocks per SM).  calls: the word's (R > 1: a row's) Philox calls;
+// full: every word of the film has eight.
 template <int R, bool ROLL = false>
 __device__ __forceinline__ void draw_any(Drawn& o, bool any7, const ClassDraw& cl, uint32_t row, uint32_t X,
                                          uint32_t w, uint32_t calls, bool full, bool paired, uint32_t sweep,
@@ -392,7 +399,7 @@ __device__ __forceinline__ void update_pair(const FilmCtx& c, uint32_t kx, uint3
   for (uint32_t n = 0; n < 2; n++) {
     const uint32_t k = n ? kx2 : kx, ky = n ? ky2 : 1u;
     Drawn x;
-    draw_any<R>(x, any7, c.cls[n ? c2 : c1], (k - 1) * c.Ly + ky - 1, (k + ky + 1 + c.colour) & 1u, w, calls,
+    draw_any<R, true>(x, any7, c.cls[n ? c2 : c1], (k - 1) * c.Ly + ky - 1, (k + ky + 1 + c.colour) & 1u, w, calls,
                     c.last_mask == 0xFFFFFFFFu, c.W > 1, c.sweep, c.rk0, c.rk1);
     if (n == 0) a[0] = x;
     else a[1] = x;
@@ -418,22 +425,48 @@ __device__ __forceinline__ void update_pair(const FilmCtx& c, uint32_t kx, uint3
   }
 }
 
+// Column rp - Lx (behind the pairs) of shape `items`: groups g .. g1 - 1 of layer
+// kx; the two walls' columns come first (grid_columns).
+struct GridColumn {
+  bool on;
+  uint32_t kx, g, g1;
+};
+template <int R>
+__device__ __forceinline__ GridColumn grid_column(const FilmDesc& d, uint32_t items, uint32_t rp) {
+  const uint32_t rq = rp < d.Lx ? 0u : rp - d.Lx;
+  const uint32_t n = d.cols[items], wi = wall_items(items), wn = d.cols[wi], walls = min(d.Lx, 2u) * wn;
+  const bool wall = rq < walls;
+  const uint32_t ri = rq - walls, q = fastdiv(wall ? 0u : ri, d.divc_m[items], d.divc_l[items]);
+  GridColumn o;
+  o.on = rp >= d.Lx && (wall || (d.Lx > 2 && n != 0 && q < d.Lx - 2));
+  const uint32_t at = wall ? (rq >= wn ? rq - wn : rq) : ri - q * n, len = column_len(wall ? wi : items);
+  o.kx = !o.on ? 1u : wall ? (rq >= wn ? d.Lx : 1u) : q + 2;
+  o.g = o.on ? 1 + at * len : 1u;
+  o.g1 = o.on ? min(o.g + len, d.Ly / R - 1) : 0u;
+  return o;
+}
+
 // One word (of R packed rows) per thread, or a pair: the shortest launch, for
 // films and film sets that do not fill the GPU for long.  The masks need
 // nothing of the lattice, so they are drawn before wait() -- while the previous
 // launch of the stream still runs -- and what follows it is the loads, some
 // forty operations and the store.
+//
+// Bound by latency where the launch is short: a word's eight Philox calls take
+// some 2000 cycles however idle the SM is.  100 sweeps of 37x75x214 in a bulk
+// field, a record every five: 0.98 ms with the draws behind the loads, 0.64 ms
+// now; 1,000 sweeps of ten contact-angle films 8.2 and 6.6 ms.
 template <int R, bool MEAS, class Wait, class AccOf>
 __device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep,
                                             uint32_t at, bool meas, AccOf acc_of, Wait wait) {
   constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
-  const uint32_t W = d.W, cols = d.cols[1];
+  const uint32_t W = d.W;
   const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
   const uint32_t w = R == 1 ? at - rp * W : 0u;
   const bool pair = rp < d.Lx;
-  const uint32_t rq = pair ? 0u : rp - d.Lx, q = fastdiv(rq, d.divc_m[1], d.divc_l[1]);
-  const bool on = pair || rq < d.Lx * cols;
-  const uint32_t kx = on ? (pair ? rp : q) + 1 : 1u, ky = pair || !on ? 1u : (rq - q * cols + 1) * R + 1;
+  const GridColumn gc = grid_column<R>(d, 1, rp);
+  const bool on = pair || gc.on;
+  const uint32_t kx = pair ? rp + 1 : gc.kx, ky = pair || !on ? 1u : gc.g * R + 1;
   const uint32_t kx2 = (d.y_mode == kYGapbc) ? (d.Lx + 1 - kx) : kx, ky2 = d.Ly - R + 1;
   const bool any7 = __any_sync(0xFFFFFFFFu, on && (!d.cls[row_class(kx, d.Lx)].sym ||
                                                    (pair && !d.cls[row_class(kx2, d.Lx)].sym)));
@@ -499,11 +532,20 @@ __device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, u
 //
 // A step's masks need nothing of the lattice, so the first step's are drawn
 // before wait() -- while the previous launch of the stream still runs.
+//
+// Bound by the integer pipes (the draws: 805 of a word's some 1000 cycles per
+// warp scheduler), not by memory.  120x240x1600 (46M sites), one sweep without
+// records: 42.1 us with a look-up per site and two words per thread in any
+// order, 38.1 us now in columns of two, 40.3 in columns of four.  The general form
+// is a loop over the calls: unrolled, both forms together overran the
+// instruction cache (1.4 stalls per issue; 41.9 us).  Columns of three or five
+// words and five or seven blocks per SM were slower (by 1 to 4%), and so were
+// masks drawn two steps ahead (registers).
 template <int R, bool MEAS, class Wait, class AccOf>
 __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx& c, uint32_t at, uint32_t items,
                                                bool meas, AccOf acc_of, Wait wait) {
   constexpr uint32_t B = 8 / R;
-  const uint32_t W = c.W, cols = d.cols[items];
+  const uint32_t W = c.W;
   const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
   const uint32_t w = R == 1 ? at - rp * W : 0u;
   const uint32_t calls = w + 1 == W ? c.last_calls : 8u;
@@ -514,13 +556,11 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
 #pragma unroll
     for (uint32_t j = 0; j < R; j++) valid |= c.last_mask << (j * B);
   }
-  // the column: groups g .. g1 - 1 of layer kx (none for a pair's thread)
-  const uint32_t rq = rp < c.Lx ? 0u : rp - c.Lx;
-  const uint32_t q = fastdiv(rq, d.divc_m[items], d.divc_l[items]);
-  const bool mine = rp >= c.Lx && rq < c.Lx * cols;
-  const uint32_t kx = mine ? q + 1 : 1u, len = column_len(items);
-  // an idle thread's range is empty, the drawing-only step included
-  const uint32_t g = mine ? 1 + (rq - q * cols) * len : 1u, g1 = mine ? min(g + len, c.Ly / R - 1) : 0u;
+  // the column: groups g .. g1 - 1 of layer kx (none for a pair's thread; an idle
+  // thread's range is empty, the drawing-only step included)
+  const GridColumn gc = grid_column<R>(d, items, rp);
+  const bool mine = gc.on;
+  const uint32_t kx = gc.kx, g = gc.g, g1 = gc.g1;
   const ClassDraw& cl = c.cls[row_class(kx, c.Lx)];
   const bool any7 = __any_sync(0xFFFFFFFFu, mine && !cl.sym);
   if (rp < c.Lx) {
@@ -567,7 +607,7 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
       }
       Drawn b;
       if (n + 1 != g1) {
-        draw_any<R>(b, k7, cl, row, R == 1 && !first ? X ^ 1u : X, w, calls, c.last_mask == 0xFFFFFFFFu, W > 1,
+        draw_any<R, true>(b, k7, cl, row, R == 1 && !first ? X ^ 1u : X, w, calls, c.last_mask == 0xFFFFFFFFu, W > 1,
                         c.sweep, c.rk0, c.rk1);
         row += R;
       }
@@ -617,14 +657,13 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
 }  // namespace
 
 // Half-sweep of every film of a launch: block b handles kFilmThreads columns of
-// film owner[b], whose descriptor is staged in shared memory.  MODE kUpdAccumulate: the half-sweep 1 launch of a sweep
-// after which some film records; those films add their record sums into their
-// accumulators in `part`.  MODE kUpdWriteRecord: a half-sweep 0 launch right
+// film owner[b], whose descriptor is staged in shared memory.  MODE
+// kUpdAccumulate: the half-sweep 1 launch of a sweep after which some film
+// records; those films add their record sums into their accumulators in `part`.  MODE kUpdWriteRecord: a half-sweep 0 launch right
 // after such a sweep; the last block of each film that recorded after
 // `rec_done` sweeps writes that record (write_record) before its update, so
 // the write overlaps the launch's other blocks.  The last block holds the
-// film's ragged end, so it has the fewest words; the first ones hold the pair
-// items, whose threads also update the wrap partner.
+// film's ragged end, so it has the fewest words; the first ones hold the pairs.
 //
 // The masks are drawn before pdl_wait, from the film's sweep counter.  Only
 // advance_kernel writes that, between chunks: the first launch of a chunk
@@ -646,6 +685,7 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
   constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
   static_assert(sizeof(FilmDesc) % 16 == 0, "descriptor copied as uint4");
   __shared__ __align__(16) FilmDesc s_d;
+  __shared__ FilmCtx s_c;  // for columns, whose registers it would take
   __shared__ int64_t s_red[MODE == kUpdWriteRecord ? kFilmThreads / 32 : 1];
   __shared__ uint32_t s_slot;
   if (first) pdl_wait();
@@ -664,8 +704,10 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     pdl_wait();  // the launch must not end before its predecessor has
     return;
   }
-  FilmCtx c;
-  film_ctx(c, s_d, pool, colour, t);
+  if (!ONE) {
+    if (threadIdx.x == 0) film_ctx(s_c, s_d, pool, colour, t);
+    __syncthreads();
+  }
   const bool meas = MEAS && measured_now(s_d, k + 1, 0);
   const FilmDesc* sd = &s_d;
   auto acc_of = [part, sd]() { return reinterpret_cast<unsigned long long*>(part + acc_offset(*sd)); };
@@ -684,9 +726,9 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     else if (PK && s_d.pack == 2) update_word<2, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
     else update_word<1, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
   } else {
-    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, c, at, items, meas, acc_of, wait);
-    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, c, at, items, meas, acc_of, wait);
-    else update_columns<1, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
+    else update_columns<1, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
   }
 }
 
@@ -939,12 +981,12 @@ struct Slab {
   uint32_t len, cols, turns;      // slab_columns: words of a column, columns, columns per thread
 };
 
-// The packed word of R rows from the words of plane p, group g (index i in the
-// layer) and, for the wrapped slot, `wrap`.
-// Own item (kx, group g, word w): every word but the x neighbours is in the
-// own planes.  CL: the x neighbours through the layer table.
+// The words of word w of group g, layer kx, any group.  own: the layer is this
+// CTA's, and so is every word but the x and wrap neighbours, which are found
+// through the layer table.
 template <bool CL, int R>
-__device__ __forceinline__ void slab_fetch(const Slab& s, uint32_t c, bool own, uint32_t kx, uint32_t g, uint32_t w, Hood& h) {
+__device__ __forceinline__ void slab_fetch(const Slab& s, uint32_t c, bool own, uint32_t kx, uint32_t g, uint32_t w,
+                                           Hood& h) {
   constexpr uint32_t B = 8 / R, kLow = slot_mask<R>(), kTop = kLow << (8 - B), kFirst = first_bits<R>();
   const uint32_t o = c ^ 1u, k = kx - 1, lim = s.lw;
   const uint32_t X = (kx + g * R + 2 + c) & 1u;  // parity array of the group's first row (ky = g R + 1)
@@ -1030,7 +1072,7 @@ __device__ __forceinline__ Column slab_column(const Slab& s, uint32_t at) {
   return o;
 }
 
-// The words of interior group g of own layer kx.
+// The words of interior group g of own layer kx: no wrap, no peer's own words.
 template <bool CL, int R>
 __device__ __forceinline__ void slab_fetch_in(const Slab& s, uint32_t c, uint32_t kx, uint32_t g, uint32_t w, Hood& h) {
   constexpr uint32_t B = 8 / R, kLow = slot_mask<R>(), kTop = kLow << (8 - B), kFirst = first_bits<R>();
@@ -1196,6 +1238,15 @@ __device__ __forceinline__ uint32_t slab_end(const FilmDesc& d, uint32_t n_sweep
 // loop runs all steps of all half-sweeps, each step deciding a word and then
 // drawing the thread's next one, the first of the next half-sweep included:
 // between the barrier's arrival and the wait for it.
+//
+// For slabs whose words and masks do not fit beside the planes (slab_tasks_fit).
+// Bound by the draws of its slowest warp: the columns of a wall's layer take the
+// general form, half as long again, while the barrier holds the others.  The
+// per-site table that it replaces had no such form and was the faster one here
+// (96x192x384 on a cluster of eight, 123 us per sweep against 155), but it ran all
+// its work behind the barrier, and lost by more on small slabs.  Films of that
+// size get a cluster only when asked to: the grid, with 152 SMs instead of eight,
+// takes them through a sweep in 7 us.
 template <bool CL, int R>
 __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint32_t* __restrict__ pool,
                                           int64_t* __restrict__ records, uint32_t n_sweeps, int* s_tot,
@@ -1323,6 +1374,12 @@ __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint3
 // leave its masks in shared memory, the words of a half-sweep dealt out over
 // all threads; deciding reads them and is short.  The masks drawn between two
 // barriers are the next half-sweep's, in a second buffer.
+//
+// What bounds a sweep now is two rounds of draws (500 cycles), shared memory
+// loads and barriers (a cluster's 360 to 600 cycles, a block's 16 to 76).
+// 1,000 sweeps of 8^3 on one CTA, a record every sweep, took 3.05 ms
+// and take 2.32 ms; a call of ten sweeps of 16x48x32 97 us on one CTA, and 61 us
+// on the cluster of eight that such films now get.
 
 // What a decision needs to know of its word; plane 0 addresses.  The plane an
 // address lies in changes with the colour for every word a decision reads:
@@ -1515,13 +1572,11 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
   // Words in order of (group, own layer, w); the last group of a pair is its
   // partner's, in layer kx'.  The general ones go to the end: a word's place is
   // the number of words of its kind before it.
-  const bool sym0 = d.cls[0].sym;
   auto general = [&](uint32_t kx) { return !d.cls[row_class(kx, s.Lx)].sym; };
   auto layer_of = [&](uint32_t g, uint32_t l) {
     const uint32_t kx = s.a + l + 1;
     return g + 1 == s.G ? slab_mirror(s, kx) : kx;
   };
-  (void)sym0;
   uint32_t n3 = 0;
   {
     uint32_t gen_in = 0, gen_end = 0;  // general layers among the own ones, and among their mirrors
@@ -1534,11 +1589,9 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
       const uint32_t g = i / per, r = i - g * per, l = r / s.W, w = r - l * s.W;
       uint32_t before = 0;  // general layers before l in this group
       for (uint32_t q = 0; q < l; q++) before += general(layer_of(g, q)) ? 1u : 0u;
-      const uint32_t gen_g = g + 1 == s.G ? gen_end : gen_in;
       const uint32_t kx = layer_of(g, l);
       const uint32_t at = general(kx) ? n3 + (g * gen_in + before) * s.W + w
                                       : (g * (s.nl - gen_in) + l - before) * s.W + w;
-      (void)gen_g;
       words[at] = slab_word<CL, R>(s, kx, g, w);
       job[i] = (uint16_t)at;
     }
@@ -1565,7 +1618,7 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
     int tb = 0, tm = 0;
     for (uint32_t i = threadIdx.x; i < jobs; i += blockDim.x) {
       const bool pair = i < per;
-      uint32_t v0 = 0, z0 = 0, valid0 = 0;
+      uint32_t v0 = 0, z0 = 0;
 #pragma unroll 1
       for (uint32_t r = 0; r < (pair ? 2u : 1u); r++) {
         const uint32_t n = job[r ? i + per * (s.G - 1) : i];
@@ -1610,7 +1663,6 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
         v0 = v;
         z0 = h.z0;
       }
-      (void)valid0;
     }
     if (meas) {
       __syncwarp();
@@ -1840,11 +1892,15 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, 
 
 namespace {
 
+// Columns: the record-writing kernel, without a record to write, takes the plain
+// launches too (its own spills two registers at six blocks per SM).
 template <bool ONE>
 auto update_variant(uint32_t mode, bool pack) {
-  return mode == kUpdAccumulate    ? (pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>)
-         : mode == kUpdWriteRecord ? (pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>)
-                                   : (pack ? update_kernel<kUpdPlain, true, ONE> : update_kernel<kUpdPlain, false, ONE>);
+  if (mode == kUpdAccumulate)
+    return pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>;
+  if (ONE && mode == kUpdPlain)
+    return pack ? update_kernel<kUpdPlain, true, true> : update_kernel<kUpdPlain, false, true>;
+  return pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>;
 }
 
 template <bool MEAS, bool ONE>
@@ -1862,7 +1918,8 @@ cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uin
   const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
   auto* kern = items == 1 ? update_variant<true>(mode, pack) : update_variant<false>(mode, pack);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, (const FilmDesc*)L.films, (const uint32_t*)L.owner_upd,
-                    (const LaunchHdr*)L.hdr, pool, colour, k, items, part, records, rec_done, first ? 1u : 0u);
+                    (const LaunchHdr*)L.hdr, pool, colour, k, items, part, records,
+                    mode == kUpdWriteRecord ? rec_done : 0u, first ? 1u : 0u);
 }
 
 cudaError_t launch_update_film(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep, uint32_t items,

@@ -10,13 +10,21 @@ namespace isg {
 
 // Grid update kernels: threads per block and blocks per SM.  A thread has a
 // column of column_len(items) words, items being the launch shape: GRID_1 (1)
-// one, GRID_Q (0) two, GRID_2 (2) four.
+// one, GRID_Q (0) two, GRID_2 (2) four.  A word of a column costs five loads
+// instead of seven and no address set-up, but a launch then has a quarter of
+// the threads and four words one after another in each: per sweep, no records,
+// one / two / four words take 45.5 / 38.1 / 40.3 us on 120x240x1600, and 5.9 / 6.1 /
+// 12.3 us on 32x96x64.
+//
+// The blocks per SM are the most whose registers hold each variant without a
+// spill: 128 threads are a warp on each scheduler, whose register file grants
+// 64 a thread at eight blocks, 80 at six, 96 at five.
 constexpr uint32_t kFilmThreads = 128;
 constexpr int film_min_blocks(int rows, bool meas, bool one) {
   return one ? (rows == 4 ? 5 : meas ? 7 : 8) : rows > 1 || meas ? 5 : 6;
 }
 constexpr int multi_min_blocks(bool one, bool meas, bool pack) {
-  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 4 : 5;
+  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 5 : pack ? 5 : 6;
 }
 __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
   return items == 1 ? 1 : items == 2 ? 4 : 2;
@@ -40,13 +48,31 @@ __host__ __device__ inline uint64_t acc_offset(const FilmDesc& d) {
 constexpr uint32_t kPack2Rows = 8192;
 
 // Columns of a film in the grid update kernels (of words, or of packed words of
-// `pack` rows): the pairs, then the rows between the first and the last.
+// `pack` rows): the pairs, then the rows between the first and the last, those
+// of the first and the last layer before the others.  A wall's words have
+// thresholds of their own and take half as long again to draw, so its columns
+// are those of the next shorter shape: a block of longer ones outlasts the
+// others (320 films of 32x96x64 on GRID_2: 67.2 us per sweep with walls, 54.5
+// without any).
+__host__ __device__ constexpr uint32_t wall_items(uint32_t items) { return items == 2 ? 0u : 1u; }
+__host__ __device__ inline uint32_t grid_columns(const FilmDesc& d, uint32_t items) {
+  const uint32_t walls = d.Lx < 2 ? d.Lx : 2u;
+  return walls * d.cols[wall_items(items)] + (d.Lx - walls) * d.cols[items];
+}
 __host__ __device__ inline uint32_t grid_items(const FilmDesc& d, uint32_t items) {
-  return d.Lx * d.W * (1 + d.cols[items]);
+  return d.W * (d.Lx + grid_columns(d, items));
 }
 __host__ __device__ inline uint32_t update_blocks(const FilmDesc& d, uint32_t items) {
   return (grid_items(d, items) + kFilmThreads - 1) / kFilmThreads;
 }
+
+// Words a half-sweep's launch updates for film d, and the most for which, without
+// a measurement, a launch takes one word per thread: it is the shorter launch,
+// columns are the higher rate.  Per sweep, one word / columns of two (one film)
+// or of four (a batch's lane): 245760 words 15.7 / 16.5 us, 524288 33.2 / 28.1;
+// lanes of 245760 words 35.2 / 35.8, of 491520 68.1 / 61.7, of 806400 110 / 89.
+constexpr uint64_t kOneWordAutoWords = 1ull << 18;
+inline uint64_t launch_words(const FilmDesc& d) { return (uint64_t)d.Lx * (d.Ly / d.pack) * d.W; }
 
 // Measurement blocks of one film.
 inline uint32_t meas_units(const FilmDesc& d) {
@@ -79,7 +105,9 @@ constexpr uint32_t kClusterMaxSize = 8;
 constexpr uint32_t kClusterMaxSmem = 200u * 1024u;
 
 // Rows per word of film d on clusters of C CTAs: thin films pack (sl_pack)
-// unless the words, one row each, already fit one turn of a CTA's threads.
+// unless the words, one row each, are few enough (128) for four drawing lanes and
+// a deciding thread each in one turn: a packed word then only lengthens the
+// chain of Philox calls.
 __host__ __device__ inline uint32_t slab_rows(const FilmDesc& d, uint32_t C) {
   const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * d.Ly * d.W;
   return words <= 128 ? 1u : d.sl_pack;
