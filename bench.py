@@ -37,8 +37,8 @@ def alu_frac(attempts_per_ns):
     return attempts_per_ns * OPS_PER_ATTEMPT / (N_SM * LANES_PER_SM * SM_MAX_GHZ)
 
 
-SHAPE_NAMES = {0: "auto", 1: "resident", 2: "grid, 1 word/thread", 3: "grid, 2 words/thread",
-               4: "grid, 4 threads/word", 5: "cluster-resident"}
+SHAPE_NAMES = {0: "auto", 1: "resident", 2: "grid, 1 word/thread", 3: "grid, 4 words/thread",
+               4: "grid, 2 words/thread", 5: "cluster-resident"}
 SHAPE_FLAGS = {1: "resident", 2: "grid1", 3: "grid2", 4: "gridq", 5: "cluster"}
 METRIC = "spin-flip attempts/ns on 1 GB300, batched vs plain, % roofline; p99 latency"
 UNIT = "attempts/ns"
@@ -52,6 +52,7 @@ OPS_PER_ATTEMPT = 30
 N_SM, LANES_PER_SM, SM_MAX_GHZ = 152, 128, 2.07
 PROFILE = os.path.join(ROOT, "profiles", "update_film_kernel_film46m.md")
 KERNEL_SOURCES = ["paper_1411_5588_gb300/csrc/ising_kernels.cu", "paper_1411_5588_gb300/csrc/ising_device.cuh",
+                  "paper_1411_5588_gb300/csrc/ising_draw.cuh",
                   "paper_1411_5588_gb300/csrc/ising_launch.h"]
 
 
