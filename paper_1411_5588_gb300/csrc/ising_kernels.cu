@@ -685,7 +685,6 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
   constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
   static_assert(sizeof(FilmDesc) % 16 == 0, "descriptor copied as uint4");
   __shared__ __align__(16) FilmDesc s_d;
-  __shared__ FilmCtx s_c;  // for columns, whose registers it would take
   __shared__ int64_t s_red[MODE == kUpdWriteRecord ? kFilmThreads / 32 : 1];
   __shared__ uint32_t s_slot;
   if (first) pdl_wait();
@@ -704,10 +703,8 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     pdl_wait();  // the launch must not end before its predecessor has
     return;
   }
-  if (!ONE) {
-    if (threadIdx.x == 0) film_ctx(s_c, s_d, pool, colour, t);
-    __syncthreads();
-  }
+  FilmCtx c;
+  film_ctx(c, s_d, pool, colour, t);
   const bool meas = MEAS && measured_now(s_d, k + 1, 0);
   const FilmDesc* sd = &s_d;
   auto acc_of = [part, sd]() { return reinterpret_cast<unsigned long long*>(part + acc_offset(*sd)); };
@@ -726,9 +723,9 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     else if (PK && s_d.pack == 2) update_word<2, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
     else update_word<1, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
   } else {
-    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
-    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
-    else update_columns<1, MEAS>(s_d, s_c, at, items, meas, acc_of, wait);
+    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    else update_columns<1, MEAS>(s_d, c, at, items, meas, acc_of, wait);
   }
 }
 
@@ -1892,15 +1889,11 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, 
 
 namespace {
 
-// Columns: the record-writing kernel, without a record to write, takes the plain
-// launches too (its own spills two registers at six blocks per SM).
 template <bool ONE>
 auto update_variant(uint32_t mode, bool pack) {
-  if (mode == kUpdAccumulate)
-    return pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>;
-  if (ONE && mode == kUpdPlain)
-    return pack ? update_kernel<kUpdPlain, true, true> : update_kernel<kUpdPlain, false, true>;
-  return pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>;
+  return mode == kUpdAccumulate    ? (pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>)
+         : mode == kUpdWriteRecord ? (pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>)
+                                   : (pack ? update_kernel<kUpdPlain, true, ONE> : update_kernel<kUpdPlain, false, ONE>);
 }
 
 template <bool MEAS, bool ONE>

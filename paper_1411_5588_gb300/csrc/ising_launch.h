@@ -24,7 +24,7 @@ constexpr int film_min_blocks(int rows, bool meas, bool one) {
   return one ? (rows == 4 ? 5 : meas ? 7 : 8) : rows > 1 || meas ? 5 : 6;
 }
 constexpr int multi_min_blocks(bool one, bool meas, bool pack) {
-  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 5 : pack ? 5 : 6;
+  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 4 : 5;
 }
 __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
   return items == 1 ? 1 : items == 2 ? 4 : 2;
