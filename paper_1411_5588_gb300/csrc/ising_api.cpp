@@ -293,10 +293,12 @@ struct ising {
   int8_t* d_stage = nullptr;
   bool dirty = true;
   int shape = ISING_SHAPE_AUTO;
-  // launch parameters of the cluster and the resident path, looked up once (the
-  // geometry of a handle never changes): cl_size -1 and resident.C 0, not yet
+  // launch parameters of the cluster and the resident path, looked up once per
+  // form of the tables (slab_form; the geometry of a handle never changes):
+  // cl_size -1 and resident.C 0, not yet
   int cl_size = -1;
   SlabLaunch cluster, resident;
+  uint32_t slab_for = 0;  // the slab_form they were looked up for
   // asynchronous record copies (ising_read_series_async): records
   // [inflight_lo, inflight_hi) of the ring counters are still being copied
   // on copy_stream until ev_copied
@@ -339,10 +341,41 @@ uint32_t film_cluster_size(const FilmDesc& d, SlabLaunch* o) {
                  cluster_capacity(1, 1, slab_dyn_bytes(d, 1, o->tasks), o->threads, o->tasks, &o->smem) > 0 ? 1u : 0u;
 }
 
-// film_cluster_size of the handle's film, looked up once.
+// Drops the handle's slab launch parameters if the tables' form has changed:
+// new parameters can need more shared memory, or another form of the kernel.
+void slab_refresh(ising* h) {
+  const uint32_t form = slab_form(h->d());
+  if (form == h->slab_for) return;
+  h->slab_for = form;
+  h->cl_size = -1;
+  h->resident = SlabLaunch();
+}
+
+// film_cluster_size of the handle's film, looked up once per table form.
 uint32_t handle_cluster_size(ising* h) {
+  slab_refresh(h);
   if (h->cl_size < 0) h->cl_size = (int)film_cluster_size(h->d(), &h->cluster);
   return (uint32_t)h->cl_size;
+}
+
+// The resident path's launch parameters of the handle's film, likewise.
+bool handle_resident(ising* h) {
+  slab_refresh(h);
+  if (!h->resident.C && !film_slab(h->d(), 1, &h->resident)) h->resident = SlabLaunch();
+  return h->resident.C != 0;
+}
+
+// n sweeps of the handle's film on the slab path, at most `step` per launch.
+int sweep_slab(ising* h, const SlabLaunch& l, uint64_t n, uint64_t step) {
+  if (slab_dyn_bytes(h->d(), l.C, l.tasks) > l.smem)  // the kernel lays out its buffers from the descriptor
+    return fail(ISING_EINVAL, "slab launch of %u bytes, the film needs %u", l.smem, slab_dyn_bytes(h->d(), l.C, l.tasks));
+  for (uint64_t done = 0; done < n;) {
+    const uint32_t k = (uint32_t)std::min<uint64_t>(n - done, step);
+    ISG_CK(launch_cluster(h->fs.L.films, nullptr, 1, l.C, l.smem, l.threads, l.tasks, h->fs.pool, h->fs.rec, k,
+                          h->fs.stream));
+    done += k;
+  }
+  return ISING_OK;
 }
 
 // The launch shape of an ising_sweep call: the pinned one, else the
@@ -704,30 +737,14 @@ int ising_sweep(ising* h, uint64_t n, uint32_t measure_every) {
   rc = sync_desc(h);
   if (rc) return rc;
   const int shape = resolve_shape(h, measure_every);
-  if (shape == ISING_SHAPE_CLUSTER) {
-    // every sweep of the call in one launch: one cluster holds the film in
-    // distributed shared memory
-    const uint32_t C = handle_cluster_size(h);
-    if (C == 0) return fail(ISING_EINVAL, "film too large for the cluster kernel");
-    for (uint64_t done = 0; done < n;) {
-      const uint32_t k = (uint32_t)std::min<uint64_t>(n - done, 4096);
-      ISG_CK(launch_cluster(h->fs.L.films, nullptr, 1, C, h->cluster.smem, h->cluster.threads, h->cluster.tasks,
-                            h->fs.pool, h->fs.rec, k, h->fs.stream));
-      done += k;
-    }
-    d.sweep = (uint32_t)(s0 + n);
-    d.rec_next += (uint32_t)nrec;
-    h->rec_written += nrec;
-    return ISING_OK;
-  }
-  if (shape == ISING_SHAPE_RESIDENT) {
-    // small film: every sweep of the call in one launch, planes in shared memory
-    if (!h->resident.C && !film_slab(d, 1, &h->resident)) {
-      h->resident.C = 0;
-      return fail(ISING_EINVAL, "film too large for the resident kernel");
-    }
-    ISG_CK(launch_cluster(h->fs.L.films, nullptr, 1, 1, h->resident.smem, h->resident.threads, h->resident.tasks,
-                          h->fs.pool, h->fs.rec, (uint32_t)n, h->fs.stream));
+  if (shape == ISING_SHAPE_CLUSTER || shape == ISING_SHAPE_RESIDENT) {
+    // every sweep of the call in one launch, the film in the shared memory of
+    // one cluster or one CTA
+    const bool cl = shape == ISING_SHAPE_CLUSTER;
+    if (cl ? !handle_cluster_size(h) : !handle_resident(h))
+      return fail(ISING_EINVAL, "film too large for the %s kernel", cl ? "cluster" : "resident");
+    rc = sweep_slab(h, cl ? h->cluster : h->resident, n, cl ? 4096 : n);
+    if (rc) return rc;
     d.sweep = (uint32_t)(s0 + n);
     d.rec_next += (uint32_t)nrec;
     h->rec_written += nrec;

@@ -184,6 +184,9 @@ constexpr uint32_t kClusterMaxPerSm = 2;
 uint32_t cluster_threads(const FilmDesc& d, uint32_t C, uint32_t per_sm, bool tasks);
 // Whether the task form's words and masks fit a CTA's shared memory, and the
 // dynamic shared memory of either form.
+// Both depend on the film's geometry and on slab_form of its tables: words of a
+// class without the three-mask form hold seven masks.
+inline uint32_t slab_form(const FilmDesc& d) { return d.cls[0].sym; }
 bool slab_tasks_fit(const FilmDesc& d, uint32_t C);
 uint32_t slab_dyn_bytes(const FilmDesc& d, uint32_t C, bool tasks);
 // Clusters of C CTAs (smem_bytes of dynamic shared memory needed and threads

@@ -1,0 +1,94 @@
+// The slab launches of a handle whose parameters change between sweeps, as the
+// host code issues them: the library's own objects, linked with a CUDA runtime
+// that keeps device memory on the heap and records each launch.  Prints one
+// line per slab launch: its CTAs per cluster, form, shared memory and threads,
+// and what the descriptor it would read needs.
+#include <cstdio>
+#include <cstdlib>
+#include <cstring>
+#include <map>
+#include <string>
+
+#include "ising_host.h"
+
+namespace {
+std::map<const void*, std::string> g_names;
+}
+
+extern "C" {
+void __cudaRegisterFunction(void**, const char* host, char*, const char* name, int, void*, void*, void*, void*, int*) {
+  g_names[host] = name;
+}
+void** __cudaRegisterFatBinary(void*) { static void* h[4]; return h; }
+cudaError_t cudaMalloc(void** p, size_t n) { *p = calloc(n, 1); return cudaSuccess; }
+cudaError_t cudaMallocHost(void** p, size_t n) { return cudaMalloc(p, n); }
+cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaMemset(void* p, int v, size_t n) { memset(p, v, n); return cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t) {
+  memcpy(d, s, n);
+  return cudaSuccess;
+}
+const char* cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {  // a GB300's
+  *v = a == cudaDevAttrMaxSharedMemoryPerMultiprocessor ? 228 * 1024 : a == cudaDevAttrReservedSharedMemoryPerBlock ? 1024 : 152;
+  return cudaSuccess;
+}
+cudaError_t cudaFuncGetAttributes(cudaFuncAttributes* a, const void*) {
+  memset(a, 0, sizeof *a);
+  a->sharedSizeBytes = 1024;
+  return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int* n, const void*, int, size_t, unsigned) {
+  *n = 4;
+  return cudaSuccess;
+}
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {
+  *n = 10;
+  return cudaSuccess;
+}
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
+  const std::string& name = g_names[f];
+  const size_t at = name.find("slab_kernelILb");
+  if (at == std::string::npos) return cudaSuccess;
+  const bool tasks = name[at + strlen("slab_kernelILb1ELb")] == '1';
+  uint32_t C = 1;
+  for (unsigned i = 0; i < c->numAttrs; i++)
+    if (c->attrs[i].id == cudaLaunchAttributeClusterDimension) C = c->attrs[i].val.clusterDim.x;
+  const isg::FilmDesc& d = **static_cast<isg::FilmDesc**>(args[0]);
+  printf("C %u tasks %d fit %d smem %zu need %u threads %u want %u\n", C, tasks, isg::slab_tasks_fit(d, C),
+         (size_t)c->dynamicSmemBytes, isg::slab_dyn_bytes(d, C, tasks), c->blockDim.x,
+         isg::cluster_threads(d, C, 1, tasks));
+  return cudaSuccess;
+}
+// calls that need do nothing here
+#define NOTHING(name)              \
+  int nothing_##name() asm(#name); \
+  int nothing_##name() { return 0; }
+NOTHING(__cudaGetKernel) NOTHING(__cudaLaunchKernel) NOTHING(__cudaPopCallConfiguration)
+NOTHING(__cudaPushCallConfiguration) NOTHING(__cudaRegisterFatBinaryEnd) NOTHING(__cudaRegisterVar)
+NOTHING(__cudaUnregisterFatBinary) NOTHING(cudaEventCreate) NOTHING(cudaEventCreateWithFlags) NOTHING(cudaEventDestroy)
+NOTHING(cudaEventElapsedTime) NOTHING(cudaEventQuery) NOTHING(cudaEventRecord) NOTHING(cudaEventSynchronize)
+NOTHING(cudaFreeHost) NOTHING(cudaFuncSetAttribute) NOTHING(cudaGetLastError) NOTHING(cudaGetSymbolAddress)
+NOTHING(cudaMemcpy) NOTHING(cudaMemcpyFromSymbol) NOTHING(cudaSetDevice) NOTHING(cudaStreamCreateWithFlags)
+NOTHING(cudaStreamDestroy) NOTHING(cudaStreamQuery) NOTHING(cudaStreamSynchronize) NOTHING(cudaStreamWaitEvent)
+}
+
+// Lx Ly Lz shape: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
+int main(int, char** a) {
+  ising* h = nullptr;
+  auto ok = [](int rc) { if (rc) { printf("status %d: %s\n", rc, ising_last_error()); exit(1); } };
+  ok(ising_create(atoi(a[1]), atoi(a[2]), atoi(a[3]), 1.0, 0.5, 3.0, 1, &h));
+  ok(ising_set_shape(h, atoi(a[4])));
+  ok(ising_sweep(h, 2, 1));
+  ok(ising_set_params(h, -1.0, 0.5, 3.0));
+  ok(ising_sweep(h, 2, 1));
+  ok(ising_set_params(h, 1.0, 0.5, 3.0));
+  ok(ising_sweep(h, 2, 1));
+  ok(ising_set_options(h, ISING_Y_GAPBC, ISING_X_FREE, 0.3, 0));
+  ok(ising_sweep(h, 2, 1));
+  ok(ising_set_options(h, ISING_Y_GAPBC, ISING_X_FREE, 0.0, 0));
+  ok(ising_sweep(h, 2, 1));
+  ok(ising_destroy(h));
+  return 0;
+}

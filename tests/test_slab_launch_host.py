@@ -1,0 +1,43 @@
+"""Slab launches (a film in the shared memory of one CTA or one cluster) of a
+handle whose couplings or bulk field change between sweeps: each launch must
+allocate what the present descriptor needs, in the form that fits it.  Runs the
+library's host code against a CUDA runtime without a device."""
+import os
+import subprocess
+
+import pytest
+
+from paper_1411_5588_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    B.build()
+    exe = str(tmp_path_factory.mktemp("slab") / "slab_launches")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
+    objs = [os.path.join(B.BUILD, o) for o in ("ising_api.o", "ising_kernels.o", "ising_noalloc.o", "ising_tune.o")]
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", cuda, "-I", B.INCLUDE, "-I", B.CSRC,
+                    os.path.join(HERE, "host", "slab_launches.cpp")] + objs + ["-lpthread", "-o", exe], check=True)
+    return exe
+
+
+AUTO, RESIDENT, CLUSTER = 0, 1, 5
+
+
+# Sizes whose need differs between the three- and the seven-mask tables, by less
+# and by more than the launch's padding, and where the task form stops fitting.
+@pytest.mark.parametrize("Lx,Ly,Lz,shape", [
+    (8, 8, 8, AUTO), (24, 601, 4, AUTO), (64, 768, 2, AUTO), (64, 153, 10, AUTO), (41, 47, 34, RESIDENT),
+    (64, 128, 128, CLUSTER), (96, 192, 64, CLUSTER), (16, 150, 130, CLUSTER), (96, 192, 384, CLUSTER)])
+def test_launch_holds_the_present_tables(harness, Lx, Ly, Lz, shape):
+    out = subprocess.run([harness, str(Lx), str(Ly), str(Lz), str(shape)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    lines = [dict(zip(l.split()[::2], map(int, l.split()[1::2]))) for l in out.stdout.splitlines()]
+    assert len(lines) == 5, out.stdout
+    for n, l in enumerate(lines):
+        assert l["smem"] >= l["need"], (n, l)
+        assert l["tasks"] == l["fit"] and l["threads"] == l["want"], (n, l)
+    # the same tables, the same launch
+    assert lines[0] == lines[2] == lines[4] and lines[1] == lines[3]
