@@ -947,10 +947,12 @@ __device__ __forceinline__ void sst(uint32_t addr, uint32_t v) {
   if (CL) asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
   else asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
-template <bool CL>
+// Adds to a sum: of the CTA's own, or (PEER) one that CTAs of the cluster share,
+// which every add then reaches at cluster scope.
+template <bool PEER>
 __device__ __forceinline__ void sadd(uint32_t addr, int v) {
-  if (CL) asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
-  else asm volatile("red.relaxed.cta.shared.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+  if (PEER) asm volatile("red.relaxed.cluster.shared::cluster.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+  else asm volatile("red.relaxed.cta.shared::cta.add.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   uint32_t v;
@@ -973,7 +975,7 @@ struct Slab {
   uint32_t a, nl;                 // first own layer (0-based), own layers
   uint32_t planes;                // shared address of the own planes
   const uint32_t* lp;             // address of layer k's plane 0 in its CTA (cluster window)
-  const uint32_t* lm;             // address of layer k's sum in its CTA
+  const uint32_t* lm;             // address of layer k's sum in its CTA (a cluster: of the partner words' sum)
   uint32_t y_mode, x_pbc, last_mask, last_calls, pos, neg, seam_same;
   uint32_t len, cols, turns;      // slab_columns: words of a column, columns, columns per thread
 };
@@ -1108,7 +1110,11 @@ __device__ __forceinline__ void slab_fetch_in(const Slab& s, uint32_t c, uint32_
 
 // The record of `t` completed sweeps: this CTA writes m(kx) of its own layers,
 // rank 0 the totals; both are cleared for the next record (whose sums come
-// after the next barrier).
+// after the next barrier).  On a cluster a layer's partner words, which any CTA
+// may hold, have a sum of their own (s_m[Lx ..]): adds to one address from
+// several CTAs have cluster scope, those of the CTA alone need not, and the two
+// must not meet at one address.
+template <bool CL>
 __device__ __forceinline__ void slab_record(const Slab& s, const FilmDesc& d, int64_t* records, int* s_m, int* s_tot,
                                             bool rank0, uint32_t t) {
   const uint32_t i0 = blockDim.x - 1 - threadIdx.x;  // from the threads with the fewest items on
@@ -1117,8 +1123,12 @@ __device__ __forceinline__ void slab_record(const Slab& s, const FilmDesc& d, in
   const uint32_t nth = d.rec_next + (t / d.measure_every - d.sweep / d.measure_every) - 1;
   int64_t* rec = records + d.rec_off + (size_t)(d.rec_cap ? nth % d.rec_cap : 0u) * (5 + s.Lx);
   for (uint32_t kx = s.a + i0; kx < s.a + s.nl; kx += blockDim.x) {
-    const int v = s_m[kx];
+    int v = s_m[kx];
     s_m[kx] = 0;
+    if (CL) {
+      v += s_m[s.Lx + kx];
+      s_m[s.Lx + kx] = 0;
+    }
     rec[5 + kx] = v;
     if (kx == 0) rec[3] = v;
     if (kx == s.Lx - 1) rec[4] = v;
@@ -1188,10 +1198,11 @@ __device__ __forceinline__ void slab_load(const FilmDesc& d, const uint32_t* __r
   for (uint32_t k = threadIdx.x; k < s.Lx; k += blockDim.x) {
     uint32_t q = 0;
     while (q + 1 < C && (q + 1) * s.Lx / C <= k) q++;
-    const uint32_t at = s.planes + 4 * (k - q * s.Lx / C) * s.lw, am = smem_addr(s_m + k);
+    const uint32_t at = s.planes + 4 * (k - q * s.Lx / C) * s.lw, am = smem_addr(s_m + (CL ? s.Lx + k : k));
     lp[k] = CL ? mapa(at, q) : at;
     lm[k] = CL ? mapa(am, q) : am;
     s_m[k] = 0;
+    if (CL) s_m[s.Lx + k] = 0;
   }
   if (threadIdx.x < 2) s_tot[threadIdx.x] = 0;
 }
@@ -1351,7 +1362,7 @@ __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint3
     if (!more) {
       slab_wait<CL>();  // the first time: every CTA's planes and tables are in place
       if (pending && c == 0) {
-        slab_record(s, d, records, s_m, s_tot, rank == 0, t);
+        slab_record<CL>(s, d, records, s_m, s_tot, rank == 0, t);
         pending = false;
       }
       if (t >= t1) break;
@@ -1561,7 +1572,7 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
   const uint32_t tot = CL ? mapa(smem_addr(s_tot), 0) : smem_addr(s_tot);
   const uint32_t per = s.nl * s.W, n_words = per * s.G;
   // 16-byte aligned: s_dyn is, and the planes and tables before are rounded up
-  SlabWord* words = reinterpret_cast<SlabWord*>(s_dyn + ((2 * s.pw + 3 * s.Lx + 3) & ~3u));
+  SlabWord* words = reinterpret_cast<SlabWord*>(s_dyn + ((2 * s.pw + (CL ? 4 : 3) * s.Lx + 3) & ~3u));
   uint16_t* job = reinterpret_cast<uint16_t*>(words + n_words);  // word of (layer, group, w), the pairs' partners included
   uint32_t* masks = reinterpret_cast<uint32_t*>(job + ((n_words + 1) & ~1u));
   slab_arrive<CL>();
@@ -1681,7 +1692,7 @@ __device__ __forceinline__ void slab_film_tasks(FilmDesc* Fg, const FilmDesc& d,
     slab_arrive<CL>();
     slab_wait<CL>();
     if (pending && c == 0) {
-      slab_record(s, d, records, s_m, s_tot, rank == 0, t);
+      slab_record<CL>(s, d, records, s_m, s_tot, rank == 0, t);
       pending = false;
     }
   }
@@ -1994,7 +2005,7 @@ static uint64_t slab_task_bytes(const FilmDesc& d, uint32_t C) {
   bool all7 = !d.cls[0].sym;
   // a CTA's general words: its share of the walls' layers and of their mirrors
   const uint64_t gen = all7 ? words : std::min<uint64_t>(words, 2 * (words / nlm) + 2 * d.W);
-  return 8ull * words + 12ull * d.Lx + 16 + words * sizeof(uint32_t) * 8 + 2 * ((words + 1) & ~1ull) +
+  return 8ull * words + (C > 1 ? 16ull : 12ull) * d.Lx + 16 + words * sizeof(uint32_t) * 8 + 2 * ((words + 1) & ~1ull) +
          2 * 4ull * (3 * (words - gen) + 7 * gen) + 16;
 }
 

@@ -3,6 +3,7 @@ handle whose couplings or bulk field change between sweeps: each launch must
 allocate what the present descriptor needs, in the form that fits it.  Runs the
 library's host code against a CUDA runtime without a device."""
 import os
+import re
 import subprocess
 
 import pytest
@@ -41,3 +42,21 @@ def test_launch_holds_the_present_tables(harness, Lx, Ly, Lz, shape):
         assert l["tasks"] == l["fit"] and l["threads"] == l["want"], (n, l)
     # the same tables, the same launch
     assert lines[0] == lines[2] == lines[4] and lines[1] == lines[3]
+
+
+def test_adds_to_one_sum_have_one_scope():
+    """In a cluster a layer's magnetisation gets adds from its own CTA and, in the
+    same half-sweep, from the peer that holds the layer's wrap partner.  PTX:
+    atomics on one address race unless each one's scope includes the other's
+    thread.  So adds of CTA scope go to the CTA's own sums and nothing else does;
+    what peers reach (through the table of shared addresses, or rank 0's
+    totals) gets cluster scope from everyone."""
+    with open(os.path.join(B.CSRC, "ising_kernels.cu")) as f:
+        src = f.read()
+    slab = src[src.index("slab path"):src.index("set-up")]
+    own = set(re.findall(r"sadd<false>\((.*?), ", slab))
+    assert own == {"smem_addr(s_m + kx - 1)"}
+    shared = re.findall(r"sadd<(?:CL|true)>\((.*?), ", slab)
+    assert sorted(set(shared)) == ["s.lm[kx - 1]", "tot", "tot + 4"]
+    # the shared table's sums are not the CTA's own
+    assert re.search(r"am = smem_addr\(s_m \+ \(CL \? s\.Lx \+ k : k\)\)", slab)
