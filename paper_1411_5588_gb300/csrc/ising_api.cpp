@@ -145,9 +145,8 @@ void build_tables(FilmDesc& d, double J, double H, double H1, double T) {
 int FilmSet::init_device() {
   ISG_CK(cudaGetDevice(&device));
   ISG_CK(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device));
-  upd_per_sm = update_blocks_per_sm();
   meas_per_sm = measure_blocks_per_sm();
-  if (upd_per_sm <= 0 || meas_per_sm <= 0) return fail(ISING_ECUDA, "occupancy query failed (no sm_103a device?)");
+  if (update_blocks_per_sm() <= 0 || meas_per_sm <= 0) return fail(ISING_ECUDA, "occupancy query failed (no sm_103a device?)");
   if (!stream) {
     ISG_CK(cudaStreamCreateWithFlags(&stream, cudaStreamNonBlocking));
     own_stream = true;
@@ -212,21 +211,19 @@ uint32_t FilmSet::upd_grid() const { return hh.upd_blocks; }
 uint32_t FilmSet::meas_grid() const { return std::min<uint32_t>(hh.meas_blocks, meas_grid_max()); }
 uint32_t FilmSet::fin_grid() const { return std::min<uint32_t>(hh.n_films, (uint32_t)(2 * n_sm)); }
 
-int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n, bool all_meas, bool fixed_grid) {
-  const uint32_t ug = fixed_grid ? upd_grid_max() : upd_grid();
-  const uint32_t fg = fixed_grid ? (uint32_t)(2 * n_sm) : fin_grid();
+int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
+  const uint32_t ug = upd_grid(), fg = fin_grid();
   bool pack = false;
   for (const auto& d : h) pack = pack || d.pack > 1;
   bool prev_meas = false;
   for (uint32_t k = k0; k < k0 + n; k++) {
-    bool meas = all_meas;
-    if (!meas)
-      for (const auto& d : h)
-        if (d.active && d.measure_every && (uint64_t)(d.sweep + k + 1) % d.measure_every == 0 &&
-            (uint64_t)d.sweep + k + 1 <= d.sweep_end) {
-          meas = true;
-          break;
-        }
+    bool meas = false;
+    for (const auto& d : h)
+      if (d.active && d.measure_every && (uint64_t)(d.sweep + k + 1) % d.measure_every == 0 &&
+          (uint64_t)d.sweep + k + 1 <= d.sweep_end) {
+        meas = true;
+        break;
+      }
     // records: half-sweep 1 accumulates the sums; the next half-sweep 0
     // writes them, or, after the last sweep of the call, a small kernel
     ISG_CK(launch_update(L, ug, pool, 0, k, items, pack, part, rec, false, prev_meas ? k : 0, k == k0, stream));

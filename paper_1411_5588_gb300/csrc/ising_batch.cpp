@@ -230,7 +230,7 @@ int lane_cluster_sweeps(Lane* b, uint64_t n) {
 int lane_direct_sweeps(Lane* b, uint32_t n) {
   if (n == 0) return ISING_OK;
   FilmSet& fs = b->fs;
-  int rc = fs.enqueue_sweeps(0, n, false, false);
+  int rc = fs.enqueue_sweeps(0, n);
   if (rc) return rc;
   ISG_CK(launch_advance(fs.L, (fs.hh.n_films + 127) / 128, n, fs.stream));
   for (auto& d : fs.h) d.sweep += n;
@@ -345,7 +345,7 @@ int lane_sweep(Lane* b, uint64_t n, int use_graph) {
     if (!rc && left >= G && !b->graphs.count(g)) {
       cudaGraph_t graph = nullptr;
       ISG_CK(cudaStreamBeginCapture(fs.stream, cudaStreamCaptureModeThreadLocal));
-      int crc = fs.enqueue_sweeps(0, g, false, false);
+      int crc = fs.enqueue_sweeps(0, g);
       if (!crc && launch_advance(fs.L, (fs.hh.n_films + 127) / 128, g, fs.stream) != cudaSuccess)
         crc = fail(ISING_ECUDA, "advance launch failed");
       cudaError_t e = cudaStreamEndCapture(fs.stream, &graph);

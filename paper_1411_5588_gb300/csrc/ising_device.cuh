@@ -86,7 +86,7 @@ inline void fastdiv_magic(uint32_t d, uint32_t* m, uint32_t* l) {
 // captured chunk can be replayed while films come and go.
 struct LaunchHdr {
   uint32_t n_films;
-  uint32_t upd_blocks;   // virtual update blocks (owner table length)
+  uint32_t upd_blocks;   // update blocks (owner table length, the grid of a half-sweep)
   uint32_t meas_blocks;  // virtual measurement blocks
   uint32_t pad;
 };

@@ -69,7 +69,7 @@ struct FilmSet {
   int device = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  int n_sm = 0, upd_per_sm = 0, meas_per_sm = 0;
+  int n_sm = 0, meas_per_sm = 0;
   uint32_t items = 1;  // launch shape of the grid update kernels (column_len: 1 one word per thread, 0 two, 2 four)
 
   std::vector<FilmDesc> h;  // host mirror (counters tracked on the host too)
@@ -89,15 +89,13 @@ struct FilmSet {
   int init_device();          // device, stream, occupancy
   void layout(bool assign_part = true);  // block ranges, owner tables, partial offsets
   int upload();               // copies hdr/films/owners to the device (synchronous)
-  uint32_t upd_grid() const;  // grid of a direct launch
+  uint32_t upd_grid() const;  // grid of a half-sweep: a block per entry of the owner table
   uint32_t meas_grid() const;
   uint32_t fin_grid() const;
-  uint32_t upd_grid_max() const { return (uint32_t)(n_sm * upd_per_sm); }
   uint32_t meas_grid_max() const { return (uint32_t)(n_sm * meas_per_sm); }
-  // Kernels of sweeps k0..k0+n-1 of the current chunk, with measurements
-  // where some film's measure_every divides (sweep + k + 1) (all_meas: after
-  // every sweep, films decide on the device).
-  int enqueue_sweeps(uint32_t k0, uint32_t n, bool all_meas, bool fixed_grid);
+  // Kernels of sweeps k0..k0+n-1 of the current chunk, with records where some
+  // film's measure_every divides (sweep + k + 1).
+  int enqueue_sweeps(uint32_t k0, uint32_t n);
   int release();
   ~FilmSet() { release(); }
 };

@@ -657,7 +657,7 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
 }  // namespace
 
 // Half-sweep of every film of a launch: block b handles kFilmThreads columns of
-// film owner[b], whose descriptor is staged in shared memory.  MODE
+// film owner[b] (the grid has a block per entry of that table), whose descriptor is staged in shared memory.  MODE
 // kUpdAccumulate: the half-sweep 1 launch of a sweep after which some film
 // records; those films add their record sums into their accumulators in `part`.  MODE kUpdWriteRecord: a half-sweep 0 launch right
 // after such a sweep; the last block of each film that recorded after
@@ -678,9 +678,8 @@ __device__ __forceinline__ uint32_t last_update_block(const FilmDesc& d, uint32_
 template <uint32_t MODE, bool PK, bool ONE>
 __global__ void __launch_bounds__(kFilmThreads, multi_min_blocks(ONE, MODE == kUpdAccumulate, PK))
 update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ owner,
-              const LaunchHdr* __restrict__ hdr, uint32_t* __restrict__ pool, uint32_t colour, uint32_t k,
-              uint32_t items, int64_t* __restrict__ part, int64_t* __restrict__ records, uint32_t rec_done,
-              uint32_t first) {
+              uint32_t* __restrict__ pool, uint32_t colour, uint32_t k, uint32_t items,
+              int64_t* __restrict__ part, int64_t* __restrict__ records, uint32_t rec_done, uint32_t first) {
   constexpr bool MEAS = MODE == kUpdAccumulate;
   constexpr uint32_t kDescWords = sizeof(FilmDesc) / 4;
   static_assert(sizeof(FilmDesc) % 16 == 0, "descriptor copied as uint4");
@@ -1922,7 +1921,7 @@ cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uin
   const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
   auto* kern = items == 1 ? update_variant<true>(mode, pack) : update_variant<false>(mode, pack);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, (const FilmDesc*)L.films, (const uint32_t*)L.owner_upd,
-                    (const LaunchHdr*)L.hdr, pool, colour, k, items, part, records,
+                    pool, colour, k, items, part, records,
                     mode == kUpdWriteRecord ? rec_done : 0u, first ? 1u : 0u);
 }
 

@@ -155,7 +155,7 @@ struct ising_server {
   Slot slot[2];
   uint32_t cap_films = 0, cap_upd = 0, cap_meas = 0;
   size_t meta_bytes = 0;  // one lane's share of a slot's descriptor buffer
-  uint32_t grid_upd = 0, grid_meas = 0, grid_fin = 0, grid_adv = 0;
+  uint32_t grid_adv = 0;
 
   double now() const { return std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count(); }
   void loop();
@@ -408,13 +408,13 @@ void ising_server::loop() {
       rc = fail(ISING_ECUDA, "lane fork failed");
     if (!rc) {
       fs.L = S.L;
-      rc = fs.enqueue_sweeps(0, chunk, false, false);
+      rc = fs.enqueue_sweeps(0, chunk);
       if (!rc && launch_advance(S.L, grid_adv, chunk, fs.stream) != cudaSuccess)
         rc = fail(ISING_ECUDA, "advance launch failed");
     }
     if (!rc && two) {
       fs2.L = S.L2;
-      rc = fs2.enqueue_sweeps(0, chunk, false, false);
+      rc = fs2.enqueue_sweeps(0, chunk);
       if (!rc && launch_advance(S.L2, grid_adv, chunk, fs2.stream) != cudaSuccess)
         rc = fail(ISING_ECUDA, "advance launch failed");
       if (!rc && (cudaEventRecord(ev_join, fs2.stream) != cudaSuccess ||
@@ -513,9 +513,6 @@ int ising_server_create(size_t hbm_budget_bytes, uint32_t chunk_sweeps, ising_se
     f->rec = reinterpret_cast<int64_t*>(s->arena_dev);
     f->part = reinterpret_cast<int64_t*>(s->arena_dev);
   }
-  s->grid_upd = s->fs.upd_grid_max();
-  s->grid_meas = s->fs.meas_grid_max();
-  s->grid_fin = (uint32_t)(2 * s->fs.n_sm);
   s->grid_adv = 64;
   for (Slot& sl : s->slot)
     if (!rc && cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming) != cudaSuccess)

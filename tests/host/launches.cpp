@@ -1,8 +1,11 @@
-// The slab launches of a handle whose parameters change between sweeps, as the
-// host code issues them: the library's own objects, linked with a CUDA runtime
-// that keeps device memory on the heap and records each launch.  Prints one
-// line per slab launch: its CTAs per cluster, form, shared memory and threads,
-// and what the descriptor it would read needs.
+// Launches as the host code issues them: the library's own objects, linked with a
+// CUDA runtime that keeps device memory on the heap and records each launch.
+//   slab Lx Ly Lz shape  a handle whose parameters change between sweeps; a line
+//                        per slab launch: its CTAs per cluster, form, shared
+//                        memory and threads, and what the descriptor it would
+//                        read needs
+//   grid items           half-sweeps of a film set; a line per launch: its grid,
+//                        and the entries of the owner table
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -13,6 +16,7 @@
 
 namespace {
 std::map<const void*, std::string> g_names;
+uint32_t g_blocks = 0;  // owner table entries of the film set in use
 }
 
 extern "C" {
@@ -49,6 +53,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   const std::string& name = g_names[f];
+  if (name.find("update_kernelI") != std::string::npos) printf("grid %u blocks %u\n", c->gridDim.x, g_blocks);
   const size_t at = name.find("slab_kernelILb");
   if (at == std::string::npos) return cudaSuccess;
   const bool tasks = name[at + strlen("slab_kernelILb1ELb")] == '1';
@@ -74,10 +79,37 @@ NOTHING(cudaMemcpy) NOTHING(cudaMemcpyFromSymbol) NOTHING(cudaSetDevice) NOTHING
 NOTHING(cudaStreamDestroy) NOTHING(cudaStreamQuery) NOTHING(cudaStreamSynchronize) NOTHING(cudaStreamWaitEvent)
 }
 
-// Lx Ly Lz shape: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
+namespace {
+void ok(int rc) {
+  if (rc) { printf("status %d: %s\n", rc, ising_last_error()); exit(1); }
+}
+
+// a small, a medium and a large film: more blocks than the GPU holds at once
+void grids(uint32_t items) {
+  isg::FilmSet fs;
+  fs.items = items;
+  fs.h.resize(3);
+  const int L[3][3] = {{4, 6, 8}, {24, 30, 96}, {120, 240, 1600}};
+  for (int i = 0; i < 3; i++) {
+    memset(&fs.h[i], 0, sizeof fs.h[i]);
+    isg::fill_geometry(fs.h[i], L[i][0], L[i][1], L[i][2], ISING_Y_GAPBC, ISING_X_FREE, 1, i);
+    isg::build_tables(fs.h[i], 1.0, 0.0, 0.5, 3.0);
+  }
+  ok(fs.init_device());
+  fs.layout();
+  ok(fs.upload());
+  g_blocks = fs.hh.upd_blocks;
+  ok(fs.enqueue_sweeps(0, 2));
+}
+}  // namespace
+
+// slab: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
 int main(int, char** a) {
+  if (!strcmp(*++a, "grid")) {
+    grids((uint32_t)atoi(a[1]));
+    return 0;
+  }
   ising* h = nullptr;
-  auto ok = [](int rc) { if (rc) { printf("status %d: %s\n", rc, ising_last_error()); exit(1); } };
   ok(ising_create(atoi(a[1]), atoi(a[2]), atoi(a[3]), 1.0, 0.5, 3.0, 1, &h));
   ok(ising_set_shape(h, atoi(a[4])));
   ok(ising_sweep(h, 2, 1));

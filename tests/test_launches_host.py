@@ -1,7 +1,9 @@
-"""Slab launches (a film in the shared memory of one CTA or one cluster) of a
-handle whose couplings or bulk field change between sweeps: each launch must
-allocate what the present descriptor needs, in the form that fits it.  Runs the
-library's host code against a CUDA runtime without a device."""
+"""Launches of the host code, run against a CUDA runtime without a device.
+
+Slab launches (a film in the shared memory of one CTA or one cluster) of a
+handle whose couplings or bulk field change between sweeps must allocate what
+the present descriptor needs, in the form that fits it; a film set's launches
+have a block per entry of the owner table."""
 import os
 import re
 import subprocess
@@ -16,11 +18,11 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 @pytest.fixture(scope="module")
 def harness(tmp_path_factory):
     B.build()
-    exe = str(tmp_path_factory.mktemp("slab") / "slab_launches")
+    exe = str(tmp_path_factory.mktemp("slab") / "launches")
     cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B.nvcc()))), "include")
     objs = [os.path.join(B.BUILD, o) for o in ("ising_api.o", "ising_kernels.o", "ising_noalloc.o", "ising_tune.o")]
     subprocess.run(["g++", "-std=c++17", "-O1", "-I", cuda, "-I", B.INCLUDE, "-I", B.CSRC,
-                    os.path.join(HERE, "host", "slab_launches.cpp")] + objs + ["-lpthread", "-o", exe], check=True)
+                    os.path.join(HERE, "host", "launches.cpp")] + objs + ["-lpthread", "-o", exe], check=True)
     return exe
 
 
@@ -33,7 +35,7 @@ AUTO, RESIDENT, CLUSTER = 0, 1, 5
     (8, 8, 8, AUTO), (24, 601, 4, AUTO), (64, 768, 2, AUTO), (64, 153, 10, AUTO), (41, 47, 34, RESIDENT),
     (64, 128, 128, CLUSTER), (96, 192, 64, CLUSTER), (16, 150, 130, CLUSTER), (96, 192, 384, CLUSTER)])
 def test_launch_holds_the_present_tables(harness, Lx, Ly, Lz, shape):
-    out = subprocess.run([harness, str(Lx), str(Ly), str(Lz), str(shape)], capture_output=True, text=True)
+    out = subprocess.run([harness, "slab", str(Lx), str(Ly), str(Lz), str(shape)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     lines = [dict(zip(l.split()[::2], map(int, l.split()[1::2]))) for l in out.stdout.splitlines()]
     assert len(lines) == 5, out.stdout
@@ -60,3 +62,13 @@ def test_adds_to_one_sum_have_one_scope():
     assert sorted(set(shared)) == ["s.lm[kx - 1]", "tot", "tot + 4"]
     # the shared table's sums are not the CTA's own
     assert re.search(r"am = smem_addr\(s_m \+ \(CL \? s\.Lx \+ k : k\)\)", slab)
+
+
+@pytest.mark.parametrize("items", [0, 1, 2])
+def test_a_block_per_owner_entry(harness, items):
+    """update_kernel takes the film of its block from the owner table and makes
+    no second turn: every launch of a film set has a block per entry."""
+    out = subprocess.run([harness, "grid", str(items)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    lines = [l.split() for l in out.stdout.splitlines()]
+    assert len(lines) == 4 and all(l[1] == l[3] and int(l[3]) > 152 * 8 for l in lines), out.stdout
