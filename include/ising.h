@@ -172,8 +172,8 @@ int ising_get_shape(ising *h, uint32_t measure_every, int *shape);
  * shape) on a scratch film of the same shape and parameters, with a record
  * every measure_every sweeps, so this handle's chain is not touched.  The
  * fastest goes into a process-wide table keyed by (Lx, Ly, Lz, boundary
- * modes, record interval up to 16) that every AUTO handle of that key then
- * uses; *shape (may be NULL) receives it.  Shapes are tried
+ * modes, whether H = 0 and J >= 0, record interval up to 16) that every AUTO
+ * handle of that key then uses; *shape (may be NULL) receives it.  Shapes are tried
  * in the order RESIDENT, GRID_1, GRID_2, GRID_Q, CLUSTER, and a later one must be at least 2%
  * faster to win.  Synchronises. */
 int ising_autotune(ising *h, uint32_t measure_every, int *shape);

@@ -291,11 +291,11 @@ struct ising {
   bool dirty = true;
   int shape = ISING_SHAPE_AUTO;
   // launch parameters of the cluster and the resident path, looked up once per
-  // form of the tables (slab_form; the geometry of a handle never changes):
+  // form of the tables (table_form; the geometry of a handle never changes):
   // cl_size -1 and resident.C 0, not yet
   int cl_size = -1;
   SlabLaunch cluster, resident;
-  uint32_t slab_for = 0;  // the slab_form they were looked up for
+  uint32_t slab_for = 0;  // the table_form they were looked up for
   // asynchronous record copies (ising_read_series_async): records
   // [inflight_lo, inflight_hi) of the ring counters are still being copied
   // on copy_stream until ev_copied
@@ -341,7 +341,7 @@ uint32_t film_cluster_size(const FilmDesc& d, SlabLaunch* o) {
 // Drops the handle's slab launch parameters if the tables' form has changed:
 // new parameters can need more shared memory, or another form of the kernel.
 void slab_refresh(ising* h) {
-  const uint32_t form = slab_form(h->d());
+  const uint32_t form = table_form(h->d());
   if (form == h->slab_for) return;
   h->slab_for = form;
   h->cl_size = -1;

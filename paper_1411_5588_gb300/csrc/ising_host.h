@@ -127,10 +127,10 @@ struct DeviceGuard {
 };
 
 // Autotuner cache, shared by every handle of the process: the fastest launch
-// shape (ISING_SHAPE_*) measured for a film shape, boundary, table variant
-// and record interval.
+// shape (ISING_SHAPE_*) measured for a film shape, boundary, table form
+// (table_form) and record interval.
 struct TuneKey {
-  uint32_t Lx, Ly, Lz, y_mode, x_pbc, m_class;
+  uint32_t Lx, Ly, Lz, y_mode, x_pbc, form, m_class;
   bool operator<(const TuneKey& o) const;
 };
 TuneKey tune_key(const FilmDesc& d, uint32_t measure_every);

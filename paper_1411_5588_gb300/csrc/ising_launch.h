@@ -79,6 +79,10 @@ inline uint32_t meas_units(const FilmDesc& d) {
   return d.meas_lpu > 1 ? (d.Lx + d.meas_lpu - 1) / d.meas_lpu : d.Lx * d.meas_bpl;
 }
 
+// The form of a film's tables that its cost and its slab's size depend on: 1 where
+// the inner layers take three masks, 0 where they take seven.
+inline uint32_t table_form(const FilmDesc& d) { return d.cls[0].sym; }
+
 // Resident path: one CTA holds the film in shared memory for a whole run of
 // sweeps, records included (the slab kernel with C = 1).  Films up to
 // kResidentMaxSites spins whose planes and layer sums fit in
@@ -184,9 +188,7 @@ constexpr uint32_t kClusterMaxPerSm = 2;
 uint32_t cluster_threads(const FilmDesc& d, uint32_t C, uint32_t per_sm, bool tasks);
 // Whether the task form's words and masks fit a CTA's shared memory, and the
 // dynamic shared memory of either form.
-// Both depend on the film's geometry and on slab_form of its tables: words of a
-// class without the three-mask form hold seven masks.
-inline uint32_t slab_form(const FilmDesc& d) { return d.cls[0].sym; }
+// Both depend on the film's geometry and on table_form.
 bool slab_tasks_fit(const FilmDesc& d, uint32_t C);
 uint32_t slab_dyn_bytes(const FilmDesc& d, uint32_t C, bool tasks);
 // Clusters of C CTAs (smem_bytes of dynamic shared memory needed and threads

@@ -4,6 +4,9 @@
 //                        per slab launch: its CTAs per cluster, form, shared
 //                        memory and threads, and what the descriptor it would
 //                        read needs
+//   tune Lx Ly Lz        the shapes AUTO takes: untuned, tuned (every candidate
+//                        taking no time, so that the first one wins), with a bulk
+//                        field, and without it again
 //   grid items           half-sweeps of a film set; a line per launch: its grid,
 //                        and the entries of the owner table
 #include <cstdio>
@@ -16,6 +19,7 @@
 
 namespace {
 std::map<const void*, std::string> g_names;
+bool g_quiet = false;
 uint32_t g_blocks = 0;  // owner table entries of the film set in use
 }
 
@@ -52,6 +56,7 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
   return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
+  if (g_quiet) return cudaSuccess;
   const std::string& name = g_names[f];
   if (name.find("update_kernelI") != std::string::npos) printf("grid %u blocks %u\n", c->gridDim.x, g_blocks);
   const size_t at = name.find("slab_kernelILb");
@@ -101,6 +106,22 @@ void grids(uint32_t items) {
   g_blocks = fs.hh.upd_blocks;
   ok(fs.enqueue_sweeps(0, 2));
 }
+
+void tune(ising* h) {
+  auto show = [h] {
+    int s = 0;
+    ok(ising_get_shape(h, 1, &s));
+    printf("shape %d\n", s);
+  };
+  show();
+  ok(ising_autotune(h, 1, nullptr));
+  show();
+  ok(ising_set_options(h, ISING_Y_GAPBC, ISING_X_FREE, 0.3, 0));
+  show();
+  ok(ising_set_options(h, ISING_Y_GAPBC, ISING_X_FREE, 0.0, 0));
+  show();
+  ok(ising_destroy(h));
+}
 }  // namespace
 
 // slab: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
@@ -111,6 +132,11 @@ int main(int, char** a) {
   }
   ising* h = nullptr;
   ok(ising_create(atoi(a[1]), atoi(a[2]), atoi(a[3]), 1.0, 0.5, 3.0, 1, &h));
+  if (!strcmp(a[0], "tune")) {
+    g_quiet = true;
+    tune(h);
+    return 0;
+  }
   ok(ising_set_shape(h, atoi(a[4])));
   ok(ising_sweep(h, 2, 1));
   ok(ising_set_params(h, -1.0, 0.5, 3.0));

@@ -72,3 +72,12 @@ def test_a_block_per_owner_entry(harness, items):
     assert out.returncode == 0, out.stdout + out.stderr
     lines = [l.split() for l in out.stdout.splitlines()]
     assert len(lines) == 4 and all(l[1] == l[3] and int(l[3]) > 152 * 8 for l in lines), out.stdout
+
+
+def test_a_measured_shape_is_for_its_table_form(harness):
+    """A film in a bulk field draws seven masks per word where it draws three
+    without one: the autotuner's choice for one is not taken for the other."""
+    out = subprocess.run([harness, "tune", "41", "47", "34"], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    shapes = [int(l.split()[1]) for l in out.stdout.splitlines()]
+    assert shapes == [CLUSTER, RESIDENT, CLUSTER, RESIDENT]
