@@ -131,6 +131,9 @@ void build_tables(FilmDesc& d, double J, double H, double H1, double T) {
         c.t[k] = thr[0];
       }
     }
+    // no site has more than D up neighbours: their bit of `up` continues D's, so
+    // that the usual classes share two values
+    for (int k = D + 1; k <= 6; k++) c.up |= ((c.up >> D) & 1u) << k;
     bool sym = D == 6 && (c.alw & 8u) && !c.frz;
     for (int k = 0; k < 3 && sym; k++) {
       const bool a = (c.alw >> k) & 1u, b = (c.alw >> (6 - k)) & 1u;
@@ -214,7 +217,13 @@ uint32_t FilmSet::fin_grid() const { return std::min<uint32_t>(hh.n_films, (uint
 int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
   const uint32_t ug = upd_grid(), fg = fin_grid();
   bool pack = false;
-  for (const auto& d : h) pack = pack || d.pack > 1;
+  uint64_t words = 0, general = 0;
+  for (const auto& d : h) {
+    pack = pack || d.pack > 1;
+    words += launch_words(d);
+    if (!table_form(d)) general += launch_words(d);
+  }
+  const bool look = 2 * general > words;
   bool prev_meas = false;
   for (uint32_t k = k0; k < k0 + n; k++) {
     bool meas = false;
@@ -226,8 +235,8 @@ int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
       }
     // records: half-sweep 1 accumulates the sums; the next half-sweep 0
     // writes them, or, after the last sweep of the call, a small kernel
-    ISG_CK(launch_update(L, ug, pool, 0, k, items, pack, part, rec, false, prev_meas ? k : 0, k == k0, stream));
-    ISG_CK(launch_update(L, ug, pool, 1, k, items, pack, part, rec, meas, 0, false, stream));
+    ISG_CK(launch_update(L, ug, pool, 0, k, items, pack, look, part, rec, false, prev_meas ? k : 0, k == k0, stream));
+    ISG_CK(launch_update(L, ug, pool, 1, k, items, pack, look, part, rec, meas, 0, false, stream));
     if (meas && k + 1 == k0 + n) ISG_CK(launch_record(L, fg, part, rec, k + 1, stream));
     prev_meas = meas;
   }
@@ -307,6 +316,13 @@ struct ising {
 };
 
 namespace {
+
+// The tables of the handle's film, and what of its geometry depends on them.
+void set_tables(ising* h) {
+  FilmDesc& d = h->d();
+  build_tables(d, h->J, h->H, h->H1, h->T);
+  d.wall_short = table_form(d);
+}
 
 int ensure_stage(ising* h) {
   if (!h->d_stage && dev_alloc(&h->d_stage, (size_t)h->d().Lx * h->d().Ly * h->d().Lz) != cudaSuccess)
@@ -462,7 +478,7 @@ int ising_create(int Lx, int Ly, int Lz, double J, double H1, double T, uint64_t
   FilmDesc& d = h->fs.h[0];
   std::memset(&d, 0, sizeof d);
   fill_geometry(d, Lx, Ly, Lz, ISING_Y_GAPBC, ISING_X_FREE, seed, 0);
-  build_tables(d, J, 0.0, H1, T);
+  set_tables(h);
   rc = h->fs.init_device();
   if (rc) { delete h; return rc; }
   h->fs.layout();
@@ -500,7 +516,7 @@ int ising_set_options(ising* h, int y_mode, int x_mode, double H, uint32_t repli
   d.x_pbc = x_mode == ISING_X_PBC;
   d.key1 = replica;
   for (int r = 0; r < 10; r++) d.rk1[r] = replica + (uint32_t)r * kWeyl1;
-  build_tables(d, h->J, H, h->H1, h->T);
+  set_tables(h);
   h->dirty = true;
   return ISING_OK;
 }
@@ -512,7 +528,7 @@ int ising_set_params(ising* h, double J, double H1, double T) {
   h->J = J;
   h->H1 = H1;
   h->T = T;
-  build_tables(h->d(), J, h->H, H1, T);
+  set_tables(h);
   h->dirty = true;
   return ISING_OK;
 }

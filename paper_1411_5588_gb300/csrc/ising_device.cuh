@@ -70,7 +70,8 @@ struct FilmDesc {
   uint32_t cols[3];            // columns of a layer without its pairs, by launch shape (column_len)
   uint32_t divc_m[3], divc_l[3];  // division by them (by 1 when there are none)
   uint32_t sl_pack;            // the most rows a packed word holds on the slab path (1, 2, 4)
-  uint32_t pad[2];
+  uint32_t wall_short;         // the walls' columns are those of the next shorter shape (grid_columns)
+  uint32_t pad[1];
 };
 
 // Division by a runtime constant d < 2^31 for numerators n < 2^31 (round-up

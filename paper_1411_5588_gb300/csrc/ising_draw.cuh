@@ -14,13 +14,17 @@
 //
 // Without a field on the layer (every inner layer when H = 0), M_k = M_{6-k}
 // and k = 3 always flips: three masks.  The walls' layers and films in a bulk
-// field take the general seven.
+// field take seven, which is half as long again.  Where a launch is bound by the
+// integer pipes and not by its chain, those are drawn the other way round: once
+// the lattice is known, a site's t_k is looked up in shared memory and its
+// word compared with that one (draw_looked_up).
 //
 // Measured on GB300, register-only loops, cycles per 32-site word and warp
-// scheduler: 16 products per Philox call alone 600; three masks 805; the
-// former 16-entry table of (S, aligned neighbours), one look-up in shared
-// memory per site, 830.  So the masks cost no throughput, and move the draws
-// out of the dependent chain.
+// scheduler: 16 products per Philox call alone 600; three masks 805; a table
+// in shared memory, one look-up per site, 830.  So three masks cost no
+// throughput, and move the draws out of the dependent chain.  120x240x1600 in a
+// bulk field, per sweep: seven masks 63.1 us, look-ups 40.7 (without the field,
+// three masks, 38.2).
 #pragma once
 #include <type_traits>
 
@@ -186,6 +190,118 @@ __device__ __forceinline__ uint32_t flips7(uint32_t S, const Count& c, const uin
                                            uint32_t frz) {
   uint32_t fl = mux7(c, m) | (S ^ bits7(c, up));
   if (frz) fl &= ~bits7(c, frz);
+  return fl;
+}
+
+// Thresholds of the four row classes for look-ups by k, t[k] of class c at 8 c + k:
+// 32 words in as many banks of shared memory, so that no two sites conflict.
+constexpr uint32_t kLookWords = 32;
+
+// The thresholds of the four sites of one call: byte i of `at` is site i's byte
+// offset in the table.
+__device__ __forceinline__ void look_up(uint32_t (&t)[4], const uint32_t* look, uint32_t at) {
+#pragma unroll
+  for (uint32_t i = 0; i < 4; i++)
+    t[i] = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(look) + __byte_perm(at, 0u, 0x4440u + i));
+}
+
+// The mask [u < t_k] of a word whose counts k are known, class cl: one comparison
+// per site with a looked-up threshold, where the general form compares each site
+// with all seven.  The arguments are draw_masks'; FULL (R = 1): eight calls,
+// straight-line code, so that one pair's look-ups pass under another's draws.
+template <int R, bool FULL>
+__device__ __forceinline__ uint32_t draw_looked_up(const Count& k, const uint32_t* look, uint32_t cl, uint32_t row,
+                                                   uint32_t X, uint32_t c1, uint32_t ncalls, uint32_t sweep,
+                                                   const uint32_t* rk0, const uint32_t* rk1) {
+  const uint32_t base = cl * 0x20202020u;  // the class's part of the offsets
+  uint32_t acc = 0;
+  uint32_t u[4], v[4], tu[4], tv[4];
+  auto put = [](uint32_t& s, auto at, const uint32_t (&x)[4], const uint32_t (&t)[4]) {
+    constexpr uint32_t A = decltype(at)::value;
+    put_if_lt<1u << A>(s, x[0], t[0]);
+    put_if_lt<1u << (A + 8)>(s, x[1], t[1]);
+    put_if_lt<1u << (A + 16)>(s, x[2], t[2]);
+    put_if_lt<1u << (A + 24)>(s, x[3], t[3]);
+  };
+  using I0 = std::integral_constant<uint32_t, 0>;
+  using I1 = std::integral_constant<uint32_t, 1>;
+  using I2 = std::integral_constant<uint32_t, 2>;
+  using I3 = std::integral_constant<uint32_t, 3>;
+  using I4 = std::integral_constant<uint32_t, 4>;
+  // y[q]: the counts of the sites at bits q and q + 4 of each byte, in its low and
+  // its high nibble
+  const uint32_t p0 = (k.c0 & 0x55555555u) | ((k.c1 << 1) & 0xAAAAAAAAu);
+  const uint32_t p1 = ((k.c0 >> 1) & 0x55555555u) | (k.c1 & 0xAAAAAAAAu);
+  const uint32_t y0 = (p0 & 0x33333333u) | ((k.c2 << 2) & 0x44444444u);
+  const uint32_t y1 = (p1 & 0x33333333u) | ((k.c2 << 1) & 0x44444444u);
+  const uint32_t y2 = ((p0 >> 2) & 0x33333333u) | (k.c2 & 0x44444444u);
+  const uint32_t y3 = ((p1 >> 2) & 0x33333333u) | ((k.c2 >> 1) & 0x44444444u);
+  if constexpr (R == 1 && FULL) {
+    // calls q and q + 4 side by side
+    const PhiloxRow3 p(row, sweep, X, rk0, rk1);
+    auto two = [&](auto qc, uint32_t y) {
+      constexpr uint32_t q = decltype(qc)::value;
+      look_up(tu, look, ((y << 2) & 0x3C3C3C3Cu) | base);
+      look_up(tv, look, ((y >> 2) & 0x3C3C3C3Cu) | base);
+      p.draw2(c1 + q, c1 + q + 4, u, v);
+      put(acc, qc, u, tu);
+      put(acc, std::integral_constant<uint32_t, q + 4>{}, v, tv);
+    };
+    two(I0{}, y0);
+    two(I1{}, y1);
+    two(I2{}, y2);
+    two(I3{}, y3);
+  } else if constexpr (R == 1) {
+    // the same, for a row's only word with fewer than eight calls
+    const PhiloxRow3 p(row, sweep, X, rk0, rk1);
+#pragma unroll 1
+    for (uint32_t q = 0; q < 4 && q < ncalls; q++) {
+      const uint32_t y = q == 0 ? y0 : q == 1 ? y1 : q == 2 ? y2 : y3;
+      uint32_t s = 0;
+      look_up(tu, look, ((y << 2) & 0x3C3C3C3Cu) | base);
+      if (q + 4 < ncalls) {
+        look_up(tv, look, ((y >> 2) & 0x3C3C3C3Cu) | base);
+        p.draw2(c1 + q, c1 + q + 4, u, v);
+        put(s, I4{}, v, tv);
+      } else {
+        p.draw(c1 + q, u);
+      }
+      put(s, I0{}, u, tu);
+      acc |= s << q;
+    }
+  } else {
+    // row j's calls q and q + 1 side by side: bits b and b + 1 of a byte
+    constexpr uint32_t B = 8 / R;
+#pragma unroll 1
+    for (uint32_t b = 0; b < 8; b += 2) {
+      const uint32_t j = b / B, q = b % B;
+      if (q >= ncalls) continue;
+      const uint32_t ya = ((b & 2u) ? y2 : y0) >> (b & 4u), yb = ((b & 2u) ? y3 : y1) >> (b & 4u);
+      const PhiloxRow3 p(row + j, sweep, X ^ (j & 1u), rk0, rk1);
+      uint32_t s = 0;
+      look_up(tu, look, ((ya << 2) & 0x3C3C3C3Cu) | base);
+      if (q + 1 < ncalls) {
+        look_up(tv, look, ((yb << 2) & 0x3C3C3C3Cu) | base);
+        p.draw2(c1 + q, c1 + q + 1, u, v);
+        put(s, I1{}, v, tv);
+      } else {
+        p.draw(c1 + q, u);
+      }
+      put(s, I0{}, u, tu);
+      acc |= s << b;
+    }
+  }
+  return acc;
+}
+
+// Sites that flip, mask m = [u < t_k].
+__device__ __forceinline__ uint32_t flips_looked_up(uint32_t S, const Count& c, uint32_t m, const ClassDraw& cl) {
+  // the usual orders of k: with a small field, or none, the costly move starts
+  // from an up spin for k >= 4 or k >= 3
+  const uint32_t up = cl.up == 0x70u ? c.c2 : cl.up == 0x78u ? c.c2 | (c.c0 & c.c1) : bits7(c, cl.up);
+  uint32_t fl = m | (S ^ up);
+  if (cl.alw) fl |= bits7(c, cl.alw);
+  if (cl.frz) fl &= ~bits7(c, cl.frz);
   return fl;
 }
 

@@ -13,9 +13,10 @@
 //    per-layer accumulators.
 //  - slab_kernel: every sweep of a call with the film in shared memory, of one
 //    CTA (the resident path) or of a cluster's CTAs.
-//  In both a word's random numbers are drawn and compared before its lattice
-//  neighbourhood is known (ising_draw.cuh), so the wait for the previous
-//  half-sweep -- a launch or a barrier -- hides behind the draws.
+//  Where a half-sweep is bound by its chain, a word's random numbers are drawn
+//  and compared before its lattice neighbourhood is known (ising_draw.cuh), so
+//  the wait for the previous half-sweep -- a launch or a barrier -- hides behind
+//  the draws.
 //  - record_kernel: writes those records and clears the accumulators.
 //  - measure_partial_kernel / measure_finalize_kernel: the same sums from the
 //    lattice alone (an on-demand measurement), per-block partials in a
@@ -201,6 +202,14 @@ __device__ __forceinline__ void film_ctx(FilmCtx& c, const FilmDesc& d, uint32_t
   c.plane1 = c.plane0 + (size_t)d.Lx * d.Ly * d.W;
 }
 
+// Fills the block's threshold table for look-ups (the caller synchronises).
+__device__ __forceinline__ void fill_look(uint32_t* look, const ClassDraw* cls) {
+  if (threadIdx.x < kLookWords) {
+    const uint32_t k = threadIdx.x & 7u;
+    look[threadIdx.x] = k < 7 ? cls[threadIdx.x >> 3].t[k] : 0u;
+  }
+}
+
 // The masks of a word drawn ahead: the three-mask form fills m[4..6].
 struct Drawn {
   uint32_t m[7];
@@ -234,6 +243,21 @@ __device__ __forceinline__ void draw_any(Drawn& o, bool any7, const ClassDraw& c
 #pragma unroll
     for (int k = 0; k < 7; k++) o.m[k] = (cl.alw >> k) & 1u ? 0xFFFFFFFFu : a.m[k];
   }
+}
+
+// The sites of a word that flip, by look-ups.  eight: most words of the film have
+// eight calls, and all then take the straight-line form (a warp with one
+// row's partial last word has full ones too, and what is drawn beyond the
+// row's end is not valid).
+template <int R>
+__device__ __forceinline__ uint32_t look_and_decide(const Hood& h, const Count& k, const uint32_t* look, uint32_t ci,
+                                                    const ClassDraw& cl, uint32_t row, uint32_t X, uint32_t w,
+                                                    uint32_t calls, bool eight, uint32_t sweep, const uint32_t* rk0,
+                                                    const uint32_t* rk1) {
+  uint32_t m;
+  if (R == 1 && eight) m = draw_looked_up<R, true>(k, look, ci, row, X, 8u * w, 8u, sweep, rk0, rk1);
+  else m = draw_looked_up<R, false>(k, look, ci, row, X, 8u * w, calls, sweep, rk0, rk1);
+  return flips_looked_up(h.S, k, m, cl);
 }
 
 __device__ __forceinline__ uint32_t decide(const Hood& h, const Count& k, bool any7, const Drawn& a,
@@ -385,6 +409,44 @@ __device__ __forceinline__ int seam_adjust(uint32_t v, uint32_t z0, uint32_t S2,
   return (neg ? -other : other) - stale;
 }
 
+// The word of group (kx, ky) and, for a pair, its wrap partner's after it, by
+// look-ups, once the previous launch is complete: nothing is drawn ahead, but a
+// general word is drawn in two thirds of the masks' time.
+template <int R, bool MEAS>
+__device__ __forceinline__ void update_looked_up(const FilmCtx& c, const uint32_t* look, uint32_t kx, uint32_t ky,
+                                                 uint32_t w, bool pair, uint32_t calls, uint32_t valid, uint32_t valid1,
+                                                 bool meas, LayerSums& r1, LayerSums& r2) {
+  constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  const uint32_t kx2 = (c.y_mode == kYGapbc) ? c.Lx + 1 - kx : kx, ky2 = c.Ly - R + 1;
+  Hood h, g;
+  fetch_rows<R>(c, kx, ky, w, h);
+  if (pair) fetch_rows<R>(c, kx2, ky2, w, g);
+  uint32_t v1 = 0, z1 = 0;
+#pragma unroll 1
+  for (uint32_t r = 0; r < (pair ? 2u : 1u); r++) {
+    const uint32_t x = r ? kx2 : kx, y = r ? ky2 : ky, cl = row_class(x, c.Lx);
+    if (r) {
+      // the partner's wrap neighbour is the word just decided where the seam
+      // joins one colour
+      if (c.seam_same) g.yp = (g.yp & ~(valid1 << kSeam)) | (((v1 ^ c.neg) & valid1) << kSeam);
+      h = g;
+    }
+    const Count k = count_up(h);
+    const uint32_t v =
+        h.S ^ (look_and_decide<R>(h, k, look, cl, c.cls[cl], (x - 1) * c.Ly + y - 1, (x + y + 1 + c.colour) & 1u, w,
+                                            calls, c.W > 1 || c.last_mask == 0xFFFFFFFFu, c.sweep, c.rk0, c.rk1) & valid);
+    store_rows<R>(c, x, y, w, v);
+    if (MEAS && meas) {
+      LayerSums q = word_sums(x, k, v, h.z0, valid, bond_slots(x, c.Lx, c.x_pbc));
+      if (r && c.seam_same) q.b += seam_adjust(v1, z1, h.S, h.z0, kSeam, c.neg, valid1);
+      if (r) r2 = q;
+      else r1 = q;
+    }
+    v1 = v;
+    z1 = h.z0;
+  }
+}
+
 // The pair of a ky = 1 word (group 0 of layer kx) and its wrap partner's, row Ly
 // of layer kx' (= Lx + 1 - kx under Eq. 11, else kx), in this order.
 template <int R, bool MEAS, class Wait, class AccOf>
@@ -400,7 +462,7 @@ __device__ __forceinline__ void update_pair(const FilmCtx& c, uint32_t kx, uint3
     const uint32_t k = n ? kx2 : kx, ky = n ? ky2 : 1u;
     Drawn x;
     draw_any<R, true>(x, any7, c.cls[n ? c2 : c1], (k - 1) * c.Ly + ky - 1, (k + ky + 1 + c.colour) & 1u, w, calls,
-                    c.last_mask == 0xFFFFFFFFu, c.W > 1, c.sweep, c.rk0, c.rk1);
+                      c.last_mask == 0xFFFFFFFFu, c.W > 1, c.sweep, c.rk0, c.rk1);
     if (n == 0) a[0] = x;
     else a[1] = x;
   }
@@ -434,7 +496,7 @@ struct GridColumn {
 template <int R>
 __device__ __forceinline__ GridColumn grid_column(const FilmDesc& d, uint32_t items, uint32_t rp) {
   const uint32_t rq = rp < d.Lx ? 0u : rp - d.Lx;
-  const uint32_t n = d.cols[items], wi = wall_items(items), wn = d.cols[wi], walls = min(d.Lx, 2u) * wn;
+  const uint32_t n = d.cols[items], wi = wall_items(d, items), wn = d.cols[wi], walls = min(d.Lx, 2u) * wn;
   const bool wall = rq < walls;
   const uint32_t ri = rq - walls, q = fastdiv(wall ? 0u : ri, d.divc_m[items], d.divc_l[items]);
   GridColumn o;
@@ -455,10 +517,11 @@ __device__ __forceinline__ GridColumn grid_column(const FilmDesc& d, uint32_t it
 // Bound by latency where the launch is short: a word's eight Philox calls take
 // some 2000 cycles however idle the SM is.  100 sweeps of 37x75x214 in a bulk
 // field, a record every five: 0.98 ms with the draws behind the loads, 0.64 ms
-// now; 1,000 sweeps of ten contact-angle films 8.2 and 6.6 ms.
-template <int R, bool MEAS, class Wait, class AccOf>
-__device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep,
-                                            uint32_t at, bool meas, AccOf acc_of, Wait wait) {
+// now; 1,000 sweeps of ten contact-angle films 8.2 and 6.6 ms.  LOOK: launches
+// past kLookBlocks, where the arithmetic counts.
+template <int R, bool MEAS, bool LOOK, class Wait, class AccOf>
+__device__ __forceinline__ void update_word(const FilmDesc& d, const uint32_t* look, uint32_t* pool, uint32_t colour,
+                                            uint32_t sweep, uint32_t at, bool meas, AccOf acc_of, Wait wait) {
   constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
   const uint32_t W = d.W;
   const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
@@ -471,6 +534,26 @@ __device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, u
   const bool any7 = __any_sync(0xFFFFFFFFu, on && (!d.cls[row_class(kx, d.Lx)].sym ||
                                                    (pair && !d.cls[row_class(kx2, d.Lx)].sym)));
   const uint32_t calls = w + 1 == W ? d.last_calls : 8u;
+  if (LOOK) {
+    wait();
+    FilmCtx c;
+    film_ctx(c, d, pool, colour, sweep);
+    LayerSums r1, r2;
+    const uint32_t valid1 = w + 1 == W ? c.last_mask : 0xFFFFFFFFu;
+    uint32_t valid = valid1;
+    if (R > 1) {
+      valid = 0;
+#pragma unroll
+      for (uint32_t j = 0; j < R; j++) valid |= c.last_mask << (j * B);
+    }
+    if (on) update_looked_up<R, MEAS>(c, look, kx, ky, w, pair, calls, valid, valid1, meas, r1, r2);
+    if (MEAS && meas) {
+      __syncwarp();
+      add_layer_sums(acc_of(), r1);
+      add_lane_sums(acc_of(), r2);
+    }
+    return;
+  }
   Drawn a{{0, 0, 0, 0, 0, 0, 0}}, b{{0, 0, 0, 0, 0, 0, 0}};
 #pragma unroll 1
   for (uint32_t r = 0; r < 2; r++) {
@@ -530,20 +613,24 @@ __device__ __forceinline__ void update_word(const FilmDesc& d, uint32_t* pool, u
 // first Lx * W columns are the pairs (update_pair); kept together, they fill
 // whole warps.
 //
-// A step's masks need nothing of the lattice, so the first step's are drawn
-// before wait() -- while the previous launch of the stream still runs.
+// By masks: a step's need nothing of the lattice, so the first step's are drawn
+// before wait() -- while the previous launch of the stream still runs.  LOOK: by
+// look-ups, every word of whatever class at one comparison per site.
 //
 // Bound by the integer pipes (the draws: 805 of a word's some 1000 cycles per
 // warp scheduler), not by memory.  120x240x1600 (46M sites), one sweep without
 // records: 42.1 us with a look-up per site and two words per thread in any
-// order, 38.1 us now in columns of two, 40.3 in columns of four.  The general form
-// is a loop over the calls: unrolled, both forms together overran the
-// instruction cache (1.4 stalls per issue; 41.9 us).  Columns of three or five
-// words and five or seven blocks per SM were slower (by 1 to 4%), and so were
-// masks drawn two steps ahead (registers).
-template <int R, bool MEAS, class Wait, class AccOf>
-__device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx& c, uint32_t at, uint32_t items,
-                                               bool meas, AccOf acc_of, Wait wait) {
+// order; by masks 38.2 us in columns of two, 40.4 in columns of four; in a bulk
+// field by look-ups 40.7 and 41.4 (by seven masks 63.1).  The seven masks of the
+// walls are a loop over the calls: unrolled, both mask forms together overran the
+// instruction cache (1.4 stalls per issue; 41.9 us), and masks beside look-ups
+// for the walls alone were slower too (39.9).  The look-ups of a full word are
+// straight-line code: as a loop 48.1 us.  Columns of three or five words and
+// five or seven blocks per SM were slower (by 1 to 4%; by look-ups seven blocks
+// are 1% faster), and so were masks drawn two steps ahead (registers).
+template <int R, bool MEAS, bool LOOK, class Wait, class AccOf>
+__device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx& c, const uint32_t* look, uint32_t at,
+                                               uint32_t items, bool meas, AccOf acc_of, Wait wait) {
   constexpr uint32_t B = 8 / R;
   const uint32_t W = c.W;
   const uint32_t rp = R == 1 ? fastdiv(at, d.divw_m, d.divw_l) : at;
@@ -561,10 +648,21 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
   const GridColumn gc = grid_column<R>(d, items, rp);
   const bool mine = gc.on;
   const uint32_t kx = gc.kx, g = gc.g, g1 = gc.g1;
-  const ClassDraw& cl = c.cls[row_class(kx, c.Lx)];
-  const bool any7 = __any_sync(0xFFFFFFFFu, mine && !cl.sym);
+  const uint32_t ci = row_class(kx, c.Lx);
+  const ClassDraw& cl = c.cls[ci];
+  const bool any7 = !LOOK && __any_sync(0xFFFFFFFFu, mine && !cl.sym);
   if (rp < c.Lx) {
-    update_pair<R, MEAS>(c, rp + 1, w, calls, valid, valid1, meas, acc_of, wait);
+    if (LOOK) {
+      LayerSums r1, r2;
+      wait();
+      update_looked_up<R, MEAS>(c, look, rp + 1, 1, w, true, calls, valid, valid1, meas, r1, r2);
+      if (MEAS && meas) {
+        add_lane_sums(acc_of(), r1);
+        add_lane_sums(acc_of(), r2);
+      }
+    } else {
+      update_pair<R, MEAS>(c, rp + 1, w, calls, valid, valid1, meas, acc_of, wait);
+    }
     if (!MEAS) return;
   }
   LayerSums sum;
@@ -582,7 +680,40 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
   const uint32_t sp = w > 0 ? 31u : c.pos, sn = w + 1 < W ? 31u : c.pos;
   uint32_t row = (kx - 1) * c.Ly + g * R;
   uint32_t om = 0, o0 = 0;
-  auto walk = [&](auto general) {
+  // row ky's words but the second z neighbour; om and o0 the row before has held
+  auto load = [&](Hood& h, uint32_t& e) {
+    h.S = col_ld(c, pA, 0, X, 3);
+    h.ym = om;
+    h.z0 = o0;
+    h.yp = col_ld(c, pA, W, X, 4);
+    h.xm = xm ? col_ld(c, pA, dxm, X, 5) : 0u;
+    h.xp = xp ? col_ld(c, pA, dxp, X, 6) : 0u;
+    if (W > 1) e = col_ld(c, pB, X ? zn : zp, X ^ 1u, 7);
+  };
+  auto z_side = [&](Hood& h, uint32_t e) {
+    if (W == 1) h.zs = X ? packed_next(o0, 1u, c.pos) : packed_prev(o0, 1u, c.pos);
+    else h.zs = X ? shift_next(o0, 0u) | ((e & 1u) << sn) : shift_prev(o0, (e >> sp) << 31);
+  };
+  auto settle = [&](uint32_t n, const Hood& h, const Count& k, uint32_t v) {
+    if (MEAS && meas) {
+      const LayerSums r = word_sums(kx, k, v, h.z0, valid, bond_slots(kx, c.Lx, c.x_pbc));
+      sum.layer = r.layer;
+      sum.m += r.m;
+      sum.b += r.b;
+    }
+    if constexpr (R > 1) {
+      store_rows<R>(c, kx, n * R + 1, w, v);
+    } else {
+      col_st(c, pA, X, v);
+      const uint32_t* p = pA + W;
+      pA = pB + W;
+      pB = p;
+      om = o0;
+      o0 = h.yp;
+      X ^= 1u;
+    }
+  };
+  auto by_masks = [&](auto general) {
     constexpr bool k7 = decltype(general)::value;
     Drawn a;
     // step n loads row n's words, draws row n + 1's masks behind the loads, and
@@ -593,22 +724,13 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
       Hood h;
       uint32_t e = 0;
       if (!first) {
-        if constexpr (R > 1) {
-          fetch_rows<R>(c, kx, n * R + 1, w, h);
-        } else {
-          h.S = col_ld(c, pA, 0, X, 3);
-          h.ym = om;
-          h.z0 = o0;
-          h.yp = col_ld(c, pA, W, X, 4);
-          h.xm = xm ? col_ld(c, pA, dxm, X, 5) : 0u;
-          h.xp = xp ? col_ld(c, pA, dxp, X, 6) : 0u;
-          if (W > 1) e = col_ld(c, pB, X ? zn : zp, X ^ 1u, 7);
-        }
+        if constexpr (R > 1) fetch_rows<R>(c, kx, n * R + 1, w, h);
+        else load(h, e);
       }
       Drawn b;
       if (n + 1 != g1) {
         draw_any<R, true>(b, k7, cl, row, R == 1 && !first ? X ^ 1u : X, w, calls, c.last_mask == 0xFFFFFFFFu, W > 1,
-                        c.sweep, c.rk0, c.rk1);
+                          c.sweep, c.rk0, c.rk1);
         row += R;
       }
       if (first) {
@@ -618,35 +740,42 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
           o0 = col_ld(c, pB, 0, X ^ 1u, 2);
         }
       } else {
-        if constexpr (R == 1) {
-          if (W == 1) h.zs = X ? packed_next(o0, 1u, c.pos) : packed_prev(o0, 1u, c.pos);
-          else h.zs = X ? shift_next(o0, 0u) | ((e & 1u) << sn) : shift_prev(o0, (e >> sp) << 31);
-        }
+        if constexpr (R == 1) z_side(h, e);
         const Count k = count_up(h);
-        const uint32_t v = h.S ^ (decide(h, k, k7, a, cl) & valid);
-        if (MEAS && meas) {
-          const LayerSums r = word_sums(kx, k, v, h.z0, valid, bond_slots(kx, c.Lx, c.x_pbc));
-          sum.layer = r.layer;
-          sum.m += r.m;
-          sum.b += r.b;
-        }
-        if constexpr (R > 1) {
-          store_rows<R>(c, kx, n * R + 1, w, v);
-        } else {
-          col_st(c, pA, X, v);
-          const uint32_t* p = pA + W;
-          pA = pB + W;
-          pB = p;
-          om = o0;
-          o0 = h.yp;
-          X ^= 1u;
-        }
+        settle(n, h, k, h.S ^ (decide(h, k, k7, a, cl) & valid));
       }
       a = b;
     }
   };
-  if (any7) walk(std::true_type{});
-  else walk(std::false_type{});
+  auto by_look = [&]() {
+    wait();
+    if (R == 1 && g < g1) {
+      om = col_ld(c, pA, -(ptrdiff_t)W, X, 1);
+      o0 = col_ld(c, pB, 0, X ^ 1u, 2);
+    }
+#pragma unroll 1
+    for (uint32_t n = g; n < g1; n++) {
+      Hood h;
+      uint32_t e = 0;
+      if constexpr (R > 1) {
+        fetch_rows<R>(c, kx, n * R + 1, w, h);
+      } else {
+        load(h, e);
+        z_side(h, e);
+      }
+      const Count k = count_up(h);
+      const uint32_t fl = look_and_decide<R>(h, k, look, ci, cl, row, (kx + n * R + 2 + c.colour) & 1u, w, calls,
+                                                            W > 1 || c.last_mask == 0xFFFFFFFFu, c.sweep, c.rk0, c.rk1);
+      row += R;
+      settle(n, h, k, h.S ^ (fl & valid));
+    }
+  };
+  if constexpr (LOOK) {
+    by_look();
+  } else {
+    if (any7) by_masks(std::true_type{});
+    else by_masks(std::false_type{});
+  }
   if (MEAS && meas) {
     __syncwarp();
     add_layer_sums(acc_of(), sum);
@@ -675,8 +804,8 @@ __device__ __forceinline__ uint32_t last_update_block(const FilmDesc& d, uint32_
   return d.upd_block_begin + update_blocks(d, items) - 1;
 }
 
-template <uint32_t MODE, bool PK, bool ONE>
-__global__ void __launch_bounds__(kFilmThreads, multi_min_blocks(ONE, MODE == kUpdAccumulate, PK))
+template <uint32_t MODE, bool PK, uint32_t FORM>
+__global__ void __launch_bounds__(kFilmThreads, multi_min_blocks(FORM, MODE == kUpdAccumulate, PK))
 update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ owner,
               uint32_t* __restrict__ pool, uint32_t colour, uint32_t k, uint32_t items,
               int64_t* __restrict__ part, int64_t* __restrict__ records, uint32_t rec_done, uint32_t first) {
@@ -686,6 +815,7 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
   __shared__ __align__(16) FilmDesc s_d;
   __shared__ int64_t s_red[MODE == kUpdWriteRecord ? kFilmThreads / 32 : 1];
   __shared__ uint32_t s_slot;
+  __shared__ uint32_t s_look[kLookWords];
   if (first) pdl_wait();
   pdl_trigger();
   // owner table and descriptor are written by the host before the launch
@@ -696,6 +826,7 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
   for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
   __syncthreads();
   if (threadIdx.x == 0) s_d.sweep = __ldcg(&films[f].sweep);  // around L1: an earlier chunk's line may be there
+  if (FORM != kFormWord) fill_look(s_look, s_d.cls);
   __syncthreads();
   const uint32_t t = s_d.sweep + k;
   if (!s_d.active || t > s_d.sweep_end || (MODE != kUpdWriteRecord && t >= s_d.sweep_end)) {
@@ -717,14 +848,15 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     return;
   }
   const uint32_t at = (vb - s_d.upd_block_begin) * kFilmThreads + threadIdx.x;
-  if (ONE) {
-    if (PK && s_d.pack == 4) update_word<4, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
-    else if (PK && s_d.pack == 2) update_word<2, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
-    else update_word<1, MEAS>(s_d, pool, colour, t, at, meas, acc_of, wait);
+  if (FORM == kFormWord || FORM == kFormWordLook) {
+    constexpr bool LOOK = FORM == kFormWordLook;
+    if (PK && s_d.pack == 4) update_word<4, MEAS, LOOK>(s_d, s_look, pool, colour, t, at, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_word<2, MEAS, LOOK>(s_d, s_look, pool, colour, t, at, meas, acc_of, wait);
+    else update_word<1, MEAS, LOOK>(s_d, s_look, pool, colour, t, at, meas, acc_of, wait);
   } else {
-    if (PK && s_d.pack == 4) update_columns<4, MEAS>(s_d, c, at, items, meas, acc_of, wait);
-    else if (PK && s_d.pack == 2) update_columns<2, MEAS>(s_d, c, at, items, meas, acc_of, wait);
-    else update_columns<1, MEAS>(s_d, c, at, items, meas, acc_of, wait);
+    if (PK && s_d.pack == 4) update_columns<4, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_columns<2, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
+    else update_columns<1, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
   }
 }
 
@@ -733,18 +865,24 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
 // from the constant bank, and the sweep is known before pdl_wait.  MEAS:
 // half-sweep 1 before a record, whose sums go into the film's accumulators
 // acc.
-template <int R, bool MEAS, bool ONE>
-__global__ void __launch_bounds__(kFilmThreads, film_min_blocks(R, MEAS, ONE))
+template <int R, bool MEAS, uint32_t FORM>
+__global__ void __launch_bounds__(kFilmThreads, film_min_blocks(R, MEAS, FORM))
 update_film_kernel(const __grid_constant__ FilmDesc d, uint32_t* __restrict__ pool, uint32_t colour,
                    uint32_t sweep, uint32_t items, int64_t* __restrict__ acc) {
+  __shared__ uint32_t s_look[kLookWords];
   pdl_trigger();
+  if (FORM == kFormWordLook || FORM == kFormColumnsLook) {
+    fill_look(s_look, d.cls);
+    __syncthreads();
+  }
   FilmCtx c;
   film_ctx(c, d, pool, colour, sweep);
   auto acc_of = [acc]() { return reinterpret_cast<unsigned long long*>(acc); };
   auto wait = [&]() { pdl_wait(); };
   const uint32_t at = blockIdx.x * kFilmThreads + threadIdx.x;
-  if (ONE) update_word<R, MEAS>(d, pool, colour, sweep, at, MEAS, acc_of, wait);
-  else update_columns<R, MEAS>(d, c, at, items, MEAS, acc_of, wait);
+  if (FORM == kFormWord || FORM == kFormWordLook)
+    update_word<R, MEAS, FORM == kFormWordLook>(d, s_look, pool, colour, sweep, at, MEAS, acc_of, wait);
+  else update_columns<R, MEAS, FORM == kFormColumnsLook>(d, c, s_look, at, items, MEAS, acc_of, wait);
 }
 
 // ------------------------------------------------------------ measurement
@@ -922,10 +1060,10 @@ __global__ void advance_kernel(FilmDesc* __restrict__ films, const LaunchHdr* __
 // seam apart), and rows of thin films are packed R to a word (fetch_rows'
 // bit order).  A layer is G = Ly / R groups of W words.
 //
-// A word's masks are drawn between the barrier's arrival and the wait for it
-// (one CTA: before the block barrier), so that the barrier hides behind the
-// draws of the next half-sweep, and what follows it is loads from shared
-// memory and bit logic.
+// In small slabs a word's masks are drawn before the barrier (slab_film_tasks),
+// which then hides behind the draws of the next half-sweep, and what follows it
+// is loads from shared memory and bit logic; large ones (slab_film) draw behind
+// it.
 //
 // Within a half-sweep no word is read that another thread writes (the
 // checkerboard; a partner row's wrap neighbour comes from the register of the
@@ -976,7 +1114,7 @@ struct Slab {
   const uint32_t* lp;             // address of layer k's plane 0 in its CTA (cluster window)
   const uint32_t* lm;             // address of layer k's sum in its CTA (a cluster: of the partner words' sum)
   uint32_t y_mode, x_pbc, last_mask, last_calls, pos, neg, seam_same;
-  uint32_t len, cols, turns;      // slab_columns: words of a column, columns, columns per thread
+  uint32_t len, cols;             // slab_column: words of a column, columns
 };
 
 // The words of word w of group g, layer kx, any group.  own: the layer is this
@@ -1173,7 +1311,6 @@ __device__ __forceinline__ void slab_load(const FilmDesc& d, const uint32_t* __r
     const SlabShape sh = slab_shape(d, C, blockDim.x);
     s.len = sh.len;
     s.cols = s.nl * s.W * ((s.G + sh.len - 1) / sh.len);
-    s.turns = sh.turns;
   }
   __syncthreads();
   uint32_t* planes = s_dyn;
@@ -1241,56 +1378,50 @@ __device__ __forceinline__ uint32_t slab_end(const FilmDesc& d, uint32_t n_sweep
 }
 
 // n_sweeps sweeps of the film of descriptor d (staged from Fg) on this CTA or
-// cluster, rows packed R to a word.  Thread i has columns i, i + T, ...; one
-// loop runs all steps of all half-sweeps, each step deciding a word and then
-// drawing the thread's next one, the first of the next half-sweep included:
-// between the barrier's arrival and the wait for it.
+// cluster, rows packed R to a word.  Thread i has columns i, i + T, ..., each word
+// decided by look-ups.
 //
-// For slabs whose words and masks do not fit beside the planes (slab_tasks_fit).
-// Bound by the draws of its slowest warp: the columns of a wall's layer take the
-// general form, half as long again, while the barrier holds the others.  The
-// per-site table that it replaces had no such form and was the faster one here
-// (96x192x384 on a cluster of eight, 123 us per sweep against 155), but it ran all
-// its work behind the barrier, and lost by more on small slabs.  Films of that
-// size get a cluster only when asked to: the grid, with 152 SMs instead of eight,
-// takes them through a sweep in 7 us.
+// For slabs of more words than threads, whose draws fill the SM by themselves
+// (slab_tasks_fit), so there is no wait to hide: bound by the integer pipes at
+// five warps per scheduler.  96x192x384 on a cluster of eight, per sweep: 126 us,
+// in a bulk field 125; with a word's masks drawn ahead of the barrier 155 and
+// 177.
 template <bool CL, int R>
 __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint32_t* __restrict__ pool,
-                                          int64_t* __restrict__ records, uint32_t n_sweeps, int* s_tot,
+                                          int64_t* __restrict__ records, uint32_t n_sweeps, int* s_tot, uint32_t* look,
                                           uint32_t* s_dyn, Slab& s, uint32_t C, uint32_t rank) {
   constexpr uint32_t B = 8 / R, kSeam = (R - 1) * B;  // the partner row's slot: the last of its group
+  fill_look(look, d.cls);  // in place once slab_load has synchronised
   slab_load<CL, R>(d, pool, s_tot, s_dyn, s, C, rank);
   int* s_m = reinterpret_cast<int*>(s_dyn + 2 * s.pw + 2 * s.Lx);
   const uint32_t tot = CL ? mapa(smem_addr(s_tot), 0) : smem_addr(s_tot);
   const uint32_t t0 = d.sweep, t1 = slab_end(d, n_sweeps);
   const uint32_t m_every = d.measure_every;
   uint32_t m_left = m_every ? m_every - t0 % m_every : 0u;  // sweeps until the next record
-  bool pending = false;  // a record's sums are complete, not yet written
-  uint32_t c = 0, t = t0, turn = 0;
-  Column col = slab_column(s, threadIdx.x);
-  uint32_t v = col.v0;
-  bool on = col.v0 < col.v1, any7 = false;
-  Drawn a{{0, 0, 0, 0, 0, 0, 0}};
-  // what a first group leaves for its partner: its new word and its row's other array
-  uint32_t pv = 0, pz = 0;
-  int tb = 0, tm = 0;
   slab_arrive<CL>();
+  slab_wait<CL>();  // every CTA's planes and tables are in place
+  uint32_t c = 0, t = t0;
 #pragma unroll 1
-  for (bool go = false, more = false;;) {
-    if (go) {
-      // decide step v of the column
-      const bool meas = c == 1 && m_left == 1;
-      if (on) {
+  while (t < t1) {
+    const bool meas = c == 1 && m_left == 1;
+    int tb = 0, tm = 0;
+#pragma unroll 1
+    for (uint32_t at = threadIdx.x; at < s.cols; at += blockDim.x) {
+      const Column col = slab_column(s, at);
+      const uint32_t valid1 = col.w + 1 == s.W ? s.last_mask : 0xFFFFFFFFu;  // one row's sites
+      uint32_t valid = valid1;
+      if (R > 1) {
+        valid = 0;
+#pragma unroll
+        for (uint32_t j = 0; j < R; j++) valid |= s.last_mask << (j * B);
+      }
+      // what a first group leaves for its partner: its new word and its row's other array
+      uint32_t pv = 0, pz = 0;
+#pragma unroll 1
+      for (uint32_t v = col.v0; v < col.v1; v++) {
         const bool partner = v == 1;
         const uint32_t kx = partner ? slab_mirror(s, col.kx) : col.kx;
         const uint32_t g = v == 0 ? 0u : partner ? s.G - 1 : v - 1;
-        const uint32_t valid1 = col.w + 1 == s.W ? s.last_mask : 0xFFFFFFFFu;  // one row's sites
-        uint32_t valid = valid1;
-        if (R > 1) {
-          valid = 0;
-#pragma unroll
-          for (uint32_t j = 0; j < R; j++) valid |= s.last_mask << (j * B);
-        }
         Hood h;
         if (v >= 2) slab_fetch_in<CL, R>(s, c, kx, g, col.w, h);
         else slab_fetch<CL, R>(s, c, !partner, kx, g, col.w, h);
@@ -1299,7 +1430,11 @@ __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint3
         const bool seam = partner && s.seam_same;
         if (seam) h.yp = (h.yp & ~(valid1 << kSeam)) | (((pv ^ s.neg) & valid1) << kSeam);
         const Count k = count_up(h);
-        const uint32_t nv = h.S ^ (decide(h, k, any7, a, d.cls[row_class(kx, s.Lx)]) & valid);
+        const uint32_t ci = row_class(kx, s.Lx);
+        const uint32_t fl = look_and_decide<R>(h, k, look, ci, d.cls[ci], (kx - 1) * s.Ly + g * R,
+                                                     (kx + g * R + 2 + c) & 1u, col.w, col.w + 1 == s.W ? s.last_calls : 8u,
+                                                     s.W > 1 || s.last_mask == 0xFFFFFFFFu, t, d.rk0, d.rk1);
+        const uint32_t nv = h.S ^ (fl & valid);
         const uint32_t off = 4 * (c * s.pw + in_layer(g * s.W + col.w, s.lw, 70));
         if (CL && partner) sst<true>(s.lp[kx - 1] + off, nv);
         else sst<false>(s.planes + 4 * (kx - 1 - s.a) * s.lw + off, nv);
@@ -1314,59 +1449,24 @@ __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint3
         pv = nv;
         pz = h.z0;
       }
-      // the next step: of this column, of the thread's next one, or of the next half-sweep
-      v++;
-      more = v - col.v0 < s.len;
-      if (!more && turn + 1 < s.turns) {
-        turn++;
-        col = slab_column(s, threadIdx.x + turn * blockDim.x);
-        v = col.v0;
-        more = true;
-      }
-      if (!more) {
-        if (meas) {
-          tb = __reduce_add_sync(0xFFFFFFFFu, tb);
-          tm = __reduce_add_sync(0xFFFFFFFFu, tm);
-          if ((threadIdx.x & 31u) == 0) {
-            sadd<CL>(tot, tb);
-            sadd<CL>(tot + 4, tm);
-          }
-          tb = tm = 0;
-          pending = true;
-        }
-        slab_arrive<CL>();
-        if (turn) {
-          turn = 0;
-          col = slab_column(s, threadIdx.x);
-        }
-        v = col.v0;
-        if (c) {
-          m_left = m_every ? (m_left == 1 ? m_every : m_left - 1) : 0u;
-          t++;
-        }
-        c ^= 1u;
-      }
-      on = v < col.v1;
     }
-    if (t < t1) {
-      const bool partner = v == 1;
-      const uint32_t kx = partner ? slab_mirror(s, col.kx) : col.kx;
-      const uint32_t g = v == 0 ? 0u : partner ? s.G - 1 : v - 1;
-      const ClassDraw& cl = d.cls[row_class(kx, s.Lx)];
-      any7 = __any_sync(0xFFFFFFFFu, on && !cl.sym);
-      if (on)
-        draw_any<R>(a, any7, cl, (kx - 1) * s.Ly + g * R, (kx + g * R + 2 + c) & 1u, col.w,
-                          col.w + 1 == s.W ? s.last_calls : 8u, s.last_mask == 0xFFFFFFFFu, s.W > 1, t, d.rk0, d.rk1);
-    }
-    if (!more) {
-      slab_wait<CL>();  // the first time: every CTA's planes and tables are in place
-      if (pending && c == 0) {
-        slab_record<CL>(s, d, records, s_m, s_tot, rank == 0, t);
-        pending = false;
+    if (meas) {
+      __syncwarp();
+      tb = __reduce_add_sync(0xFFFFFFFFu, tb);
+      tm = __reduce_add_sync(0xFFFFFFFFu, tm);
+      if ((threadIdx.x & 31u) == 0) {
+        sadd<CL>(tot, tb);
+        sadd<CL>(tot + 4, tm);
       }
-      if (t >= t1) break;
-      go = true;
     }
+    slab_arrive<CL>();
+    if (c) {
+      m_left = m_every ? (m_left == 1 ? m_every : m_left - 1) : 0u;
+      t++;
+    }
+    c ^= 1u;
+    slab_wait<CL>();
+    if (meas) slab_record<CL>(s, d, records, s_m, s_tot, rank == 0, t);
   }
   slab_store<CL, R>(Fg, d, pool, s_dyn, s, rank, t1);
 }
@@ -1713,6 +1813,7 @@ slab_kernel(FilmDesc* __restrict__ films, const uint32_t* __restrict__ list, uin
   __shared__ __align__(16) FilmDesc s_d;
   __shared__ int s_tot[2];  // {B, M} of the record being summed (rank 0's)
   __shared__ Slab s_s;
+  __shared__ uint32_t s_look[TASKS ? 1 : kLookWords];
   pdl_trigger();
   pdl_wait();
   uint32_t C = 1, rank = 0;
@@ -1740,9 +1841,9 @@ slab_kernel(FilmDesc* __restrict__ films, const uint32_t* __restrict__ list, uin
       else if (R == 2) slab_film_tasks<CL, 2>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
       else slab_film_tasks<CL, 1>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
     } else {
-      if (R == 4) slab_film<CL, 4>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
-      else if (R == 2) slab_film<CL, 2>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
-      else slab_film<CL, 1>(Fg, s_d, pool, records, n_sweeps, s_tot, s_dyn, s_s, C, rank);
+      if (R == 4) slab_film<CL, 4>(Fg, s_d, pool, records, n_sweeps, s_tot, s_look, s_dyn, s_s, C, rank);
+      else if (R == 2) slab_film<CL, 2>(Fg, s_d, pool, records, n_sweeps, s_tot, s_look, s_dyn, s_s, C, rank);
+      else slab_film<CL, 1>(Fg, s_d, pool, records, n_sweeps, s_tot, s_look, s_dyn, s_s, C, rank);
     }
   }
 }
@@ -1899,27 +2000,34 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), uint32_t grid, uint32_t block, 
 
 namespace {
 
-template <bool ONE>
+template <uint32_t FORM>
 auto update_variant(uint32_t mode, bool pack) {
-  return mode == kUpdAccumulate    ? (pack ? update_kernel<kUpdAccumulate, true, ONE> : update_kernel<kUpdAccumulate, false, ONE>)
-         : mode == kUpdWriteRecord ? (pack ? update_kernel<kUpdWriteRecord, true, ONE> : update_kernel<kUpdWriteRecord, false, ONE>)
-                                   : (pack ? update_kernel<kUpdPlain, true, ONE> : update_kernel<kUpdPlain, false, ONE>);
+  return mode == kUpdAccumulate    ? (pack ? update_kernel<kUpdAccumulate, true, FORM> : update_kernel<kUpdAccumulate, false, FORM>)
+         : mode == kUpdWriteRecord ? (pack ? update_kernel<kUpdWriteRecord, true, FORM> : update_kernel<kUpdWriteRecord, false, FORM>)
+                                   : (pack ? update_kernel<kUpdPlain, true, FORM> : update_kernel<kUpdPlain, false, FORM>);
 }
 
-template <bool MEAS, bool ONE>
+template <bool MEAS, uint32_t FORM>
 auto update_film_variant(uint32_t pack) {
-  return pack == 4 ? update_film_kernel<4, MEAS, ONE>
-                   : pack == 2 ? update_film_kernel<2, MEAS, ONE> : update_film_kernel<1, MEAS, ONE>;
+  return pack == 4 ? update_film_kernel<4, MEAS, FORM>
+                   : pack == 2 ? update_film_kernel<2, MEAS, FORM> : update_film_kernel<1, MEAS, FORM>;
+}
+
+template <uint32_t FORM>
+auto update_film_variant(uint32_t pack, bool meas) {
+  return meas ? update_film_variant<true, FORM>(pack) : update_film_variant<false, FORM>(pack);
 }
 
 }  // namespace
 
 cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
-                          uint32_t items, bool pack, int64_t* part, int64_t* records, bool accumulate,
+                          uint32_t items, bool pack, bool general, int64_t* part, int64_t* records, bool accumulate,
                           uint32_t rec_done, bool first, cudaStream_t st) {
   if (grid == 0) return cudaSuccess;
   const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
-  auto* kern = items == 1 ? update_variant<true>(mode, pack) : update_variant<false>(mode, pack);
+  auto* kern = items != 1                         ? update_variant<kFormColumnsLook>(mode, pack)
+               : general && grid >= kLookBlocks ? update_variant<kFormWordLook>(mode, pack)
+                                                : update_variant<kFormWord>(mode, pack);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, (const FilmDesc*)L.films, (const uint32_t*)L.owner_upd,
                     pool, colour, k, items, part, records,
                     mode == kUpdWriteRecord ? rec_done : 0u, first ? 1u : 0u);
@@ -1928,8 +2036,11 @@ cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uin
 cudaError_t launch_update_film(const FilmDesc& d, uint32_t* pool, uint32_t colour, uint32_t sweep, uint32_t items,
                                int64_t* acc, cudaStream_t st) {
   const uint32_t grid = update_blocks(d, items);
-  auto* kern = items == 1 ? (acc ? update_film_variant<true, true>(d.pack) : update_film_variant<false, true>(d.pack))
-                          : (acc ? update_film_variant<true, false>(d.pack) : update_film_variant<false, false>(d.pack));
+  const bool general = !table_form(d), meas = acc != nullptr;
+  auto* kern = items != 1 ? (general ? update_film_variant<kFormColumnsLook>(d.pack, meas)
+                                     : update_film_variant<kFormColumns>(d.pack, meas))
+               : general && grid >= kLookBlocks ? update_film_variant<kFormWordLook>(d.pack, meas)
+                                                : update_film_variant<kFormWord>(d.pack, meas);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, d, pool, colour, sweep, items, acc);
 }
 
@@ -2140,7 +2251,7 @@ int read_oob_counters(unsigned long long* count, unsigned long long* first) {
 
 int update_blocks_per_sm() {
   int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, update_kernel<kUpdPlain, false, true>, kFilmThreads, 0) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, update_kernel<kUpdPlain, false, kFormWord>, kFilmThreads, 0) !=
       cudaSuccess)
     return 0;
   return nb;

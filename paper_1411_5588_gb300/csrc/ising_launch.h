@@ -16,19 +16,36 @@ namespace isg {
 // one / two / four words take 45.5 / 38.1 / 40.3 us on 120x240x1600, and 5.9 / 6.1 /
 // 12.3 us on 32x96x64.
 //
+// Forms: columns by masks (single films without a bulk field), columns by
+// look-ups (single films in one, and film sets, whose walls would otherwise take
+// seven masks: 320 films of 32x96x64 60.1 us per sweep by masks, 53.7 by look-ups,
+// in a field 85.7 and 52.8), one word by masks drawn ahead, and one word by
+// look-ups (kLookBlocks).
+//
 // The blocks per SM are the most whose registers hold each variant without a
 // spill: 128 threads are a warp on each scheduler, whose register file grants
-// 64 a thread at eight blocks, 80 at six, 96 at five.
+// 64 a thread at eight blocks, 72 at seven, 80 at six, 96 at five.
 constexpr uint32_t kFilmThreads = 128;
-constexpr int film_min_blocks(int rows, bool meas, bool one) {
-  return one ? (rows == 4 ? 5 : meas ? 7 : 8) : rows > 1 || meas ? 5 : 6;
+enum : uint32_t { kFormColumns = 0, kFormColumnsLook = 1, kFormWord = 2, kFormWordLook = 3 };
+constexpr int film_min_blocks(int rows, bool meas, uint32_t form) {
+  return form == kFormWord || form == kFormWordLook ? (rows == 4 ? 5 : meas ? 7 : 8)
+         : form == kFormColumnsLook                 ? (meas ? 6 : 7)
+                                                    : rows > 1 || meas ? 5 : 6;
 }
-constexpr int multi_min_blocks(bool one, bool meas, bool pack) {
-  return one ? (pack ? (meas ? 5 : 6) : 8) : meas ? 4 : 5;
+constexpr int multi_min_blocks(uint32_t form, bool meas, bool pack) {
+  return form == kFormWord       ? (pack ? (meas ? 5 : 6) : 8)
+         : form == kFormWordLook ? (meas ? 5 : 6)
+                                 : meas ? 4 : 5;
 }
 __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
   return items == 1 ? 1 : items == 2 ? 4 : 2;
 }
+// Blocks from which a launch of one word per thread is made by look-ups where
+// most of its words are general: more than a wave (152 SMs, eight blocks each).
+// Below it the chain counts, and seven masks drawn ahead are no slower.  Films
+// in a bulk field, per sweep, masks / look-ups: 864 blocks 10.7 / 12.2 us, 1024
+// blocks 12.7 / 12.7, 5625 blocks 68.1 / 45.6.
+constexpr uint32_t kLookBlocks = 8 * 152 + 1;
 constexpr int kMeasureBlock = 256;
 
 // Items a measurement block covers per layer before another block is added;
@@ -49,15 +66,17 @@ constexpr uint32_t kPack2Rows = 8192;
 
 // Columns of a film in the grid update kernels (of words, or of packed words of
 // `pack` rows): the pairs, then the rows between the first and the last, those
-// of the first and the last layer before the others.  A wall's words have
-// thresholds of their own and take half as long again to draw, so its columns
-// are those of the next shorter shape: a block of longer ones outlasts the
-// others (320 films of 32x96x64 on GRID_2: 67.2 us per sweep with walls, 54.5
-// without any).
-__host__ __device__ constexpr uint32_t wall_items(uint32_t items) { return items == 2 ? 0u : 1u; }
+// of the first and the last layer before the others.  By masks a wall's words
+// take half as long again to draw, and a block of them outlasts the others, so
+// its columns are those of the next shorter shape (wall_short; 96x192x384 on
+// GRID_Q: 9.9 us per sweep without, 8.5 with).  By look-ups all words cost alike
+// (320 films of 32x96x64 on GRID_2: 53.7 us, 55.2 with shorter ones).
+__host__ __device__ inline uint32_t wall_items(const FilmDesc& d, uint32_t items) {
+  return !d.wall_short ? items : items == 2 ? 0u : 1u;
+}
 __host__ __device__ inline uint32_t grid_columns(const FilmDesc& d, uint32_t items) {
   const uint32_t walls = d.Lx < 2 ? d.Lx : 2u;
-  return walls * d.cols[wall_items(items)] + (d.Lx - walls) * d.cols[items];
+  return walls * d.cols[wall_items(d, items)] + (d.Lx - walls) * d.cols[items];
 }
 __host__ __device__ inline uint32_t grid_items(const FilmDesc& d, uint32_t items) {
   return d.W * (d.Lx + grid_columns(d, items));
@@ -154,7 +173,7 @@ struct LaunchSet {
 // (FilmDesc::pack > 1).  first: the chunk's first launch, whose predecessor may
 // still be advancing the films' sweep counters.
 cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
-                          uint32_t items, bool pack, int64_t* part, int64_t* records, bool accumulate,
+                          uint32_t items, bool pack, bool general, int64_t* part, int64_t* records, bool accumulate,
                           uint32_t rec_done, bool first, cudaStream_t st);
 // One half-sweep of a single film whose descriptor (with `sweep` absolute) is
 // passed by value; acc (colour 1 of a recorded sweep, else null): the film's

@@ -7,8 +7,10 @@
 //   tune Lx Ly Lz        the shapes AUTO takes: untuned, tuned (every candidate
 //                        taking no time, so that the first one wins), with a bulk
 //                        field, and without it again
-//   grid items           half-sweeps of a film set; a line per launch: its grid,
-//                        and the entries of the owner table
+//   film Lx Ly Lz shape H  a sweep of a handle; a line per launch: its form
+//   grid items H0 H1 H2  half-sweeps of a set of a small, a medium and a large film
+//                        in those bulk fields; a line per launch: its grid, the
+//                        entries of the owner table, and its form
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -58,7 +60,13 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   if (g_quiet) return cudaSuccess;
   const std::string& name = g_names[f];
-  if (name.find("update_kernelI") != std::string::npos) printf("grid %u blocks %u\n", c->gridDim.x, g_blocks);
+  // the last template argument of either update kernel
+  auto form = [&name](const char* kernel) {
+    const size_t k = name.find(kernel);
+    return k == std::string::npos ? -1 : atoi(name.c_str() + name.find("EE", k) - 1);
+  };
+  if (form("update_kernelI") >= 0) printf("grid %u blocks %u form %d\n", c->gridDim.x, g_blocks, form("update_kernelI"));
+  if (form("update_film_kernelI") >= 0) printf("form %d\n", form("update_film_kernelI"));
   const size_t at = name.find("slab_kernelILb");
   if (at == std::string::npos) return cudaSuccess;
   const bool tasks = name[at + strlen("slab_kernelILb1ELb")] == '1';
@@ -90,7 +98,7 @@ void ok(int rc) {
 }
 
 // a small, a medium and a large film: more blocks than the GPU holds at once
-void grids(uint32_t items) {
+void grids(uint32_t items, char** H) {
   isg::FilmSet fs;
   fs.items = items;
   fs.h.resize(3);
@@ -98,7 +106,7 @@ void grids(uint32_t items) {
   for (int i = 0; i < 3; i++) {
     memset(&fs.h[i], 0, sizeof fs.h[i]);
     isg::fill_geometry(fs.h[i], L[i][0], L[i][1], L[i][2], ISING_Y_GAPBC, ISING_X_FREE, 1, i);
-    isg::build_tables(fs.h[i], 1.0, 0.0, 0.5, 3.0);
+    isg::build_tables(fs.h[i], 1.0, atof(H[i]), 0.5, 3.0);
   }
   ok(fs.init_device());
   fs.layout();
@@ -127,7 +135,7 @@ void tune(ising* h) {
 // slab: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
 int main(int, char** a) {
   if (!strcmp(*++a, "grid")) {
-    grids((uint32_t)atoi(a[1]));
+    grids((uint32_t)atoi(a[1]), a + 2);
     return 0;
   }
   ising* h = nullptr;
@@ -138,6 +146,12 @@ int main(int, char** a) {
     return 0;
   }
   ok(ising_set_shape(h, atoi(a[4])));
+  if (!strcmp(a[0], "film")) {
+    ok(ising_set_options(h, ISING_Y_GAPBC, ISING_X_FREE, atof(a[5]), 0));
+    ok(ising_sweep(h, 1, 1));
+    ok(ising_destroy(h));
+    return 0;
+  }
   ok(ising_sweep(h, 2, 1));
   ok(ising_set_params(h, -1.0, 0.5, 3.0));
   ok(ising_sweep(h, 2, 1));

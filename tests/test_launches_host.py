@@ -68,7 +68,7 @@ def test_adds_to_one_sum_have_one_scope():
 def test_a_block_per_owner_entry(harness, items):
     """update_kernel takes the film of its block from the owner table and makes
     no second turn: every launch of a film set has a block per entry."""
-    out = subprocess.run([harness, "grid", str(items)], capture_output=True, text=True)
+    out = subprocess.run([harness, "grid", str(items), "0", "0", "0"], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     lines = [l.split() for l in out.stdout.splitlines()]
     assert len(lines) == 4 and all(l[1] == l[3] and int(l[3]) > 152 * 8 for l in lines), out.stdout
@@ -81,3 +81,31 @@ def test_a_measured_shape_is_for_its_table_form(harness):
     assert out.returncode == 0, out.stdout + out.stderr
     shapes = [int(l.split()[1]) for l in out.stdout.splitlines()]
     assert shapes == [CLUSTER, RESIDENT, CLUSTER, RESIDENT]
+
+
+# kFormColumns, kFormColumnsLook, kFormWord, kFormWordLook
+MASKS, COLUMNS_LOOK, WORD, WORD_LOOK = range(4)
+
+
+@pytest.mark.parametrize("Lx,Ly,Lz,shape,H,form", [
+    (120, 240, 1600, 4, 0.0, MASKS), (120, 240, 1600, 3, 0.0, MASKS), (120, 240, 1600, 4, 0.05, COLUMNS_LOOK),
+    (120, 240, 1600, 3, -0.3, COLUMNS_LOOK), (32, 96, 64, 4, 0.05, COLUMNS_LOOK), (120, 240, 1600, 2, 0.0, WORD),
+    (120, 240, 1600, 2, 0.05, WORD_LOOK), (64, 256, 512, 2, 0.05, WORD), (32, 96, 64, 2, 0.05, WORD)])
+def test_films_in_a_field_look_thresholds_up(harness, Lx, Ly, Lz, shape, H, form):
+    """Where a launch is bound by the integer pipes, a film in a bulk field
+    compares each site with one looked-up threshold, not with seven."""
+    out = subprocess.run([harness, "film", str(Lx), str(Ly), str(Lz), str(shape), str(H)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    forms = [int(l.split()[1]) for l in out.stdout.splitlines()]
+    assert forms == [form, form], out.stdout
+
+
+@pytest.mark.parametrize("items,H,form", [
+    (0, (0, 0, 0), COLUMNS_LOOK), (2, (0, 0, 0.1), COLUMNS_LOOK), (1, (0, 0, 0), WORD), (1, (0.1, 0.1, 0), WORD),
+    (1, (0, 0, 0.1), WORD_LOOK)])
+def test_sets_look_thresholds_up(harness, items, H, form):
+    """Sets of films: in columns always, at one word per thread where most words
+    of a large launch are in a bulk field."""
+    out = subprocess.run([harness, "grid", str(items)] + [str(h) for h in H], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    assert [int(l.split()[5]) for l in out.stdout.splitlines()] == [form] * 4, out.stdout
