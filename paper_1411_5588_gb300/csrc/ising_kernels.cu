@@ -1580,16 +1580,18 @@ __device__ __forceinline__ void draw_part(Masks<K>& a, const uint32_t (&t)[K], c
 }
 
 // The draws of half-sweep (c, t) into mask buffer m: three words per three-mask
-// word, then seven per general one.  Words that fill two turns of the threads
-// are drawn by one lane each (no shuffles, the row's products once per word);
-// fewer by four lanes, task i being part i & 3 of word i >> 2.  me: the thread's
-// first task.
+// word, then seven per general one.  Words whose four parts take
+// one turn of the threads are drawn by four lanes, task i being part i & 3 of
+// word i >> 2; more by one lane each (no shuffles, the row's products once per
+// word): a second turn of parts falls on threads that decide as well (288 packed
+// words, 24x48x20 on two CTAs: 6.7 us per sweep in two turns of parts, 4.7).  me:
+// the thread's first task.
 template <int R>
 __device__ __forceinline__ void slab_tasks(const Slab& s, const FilmDesc& d, const SlabWord* words, uint32_t n_words,
                                            uint32_t n3, uint32_t* m, uint32_t c, uint32_t t, uint32_t me) {
   constexpr uint32_t B = 8 / R;
   constexpr int D = R == 1 ? 4 : 1;
-  if (2 * n_words > blockDim.x) {
+  if (4 * n_words > blockDim.x) {
     for (uint32_t i = me; i < (n_words + 31u & ~31u); i += blockDim.x) {  // whole warps
       const uint32_t n = min(i, n_words - 1), f = words[n].f, rw = words[n].row;
       const bool any7 = __any_sync(0xFFFFFFFFu, n >= n3);
@@ -2121,7 +2123,13 @@ static uint64_t slab_task_bytes(const FilmDesc& d, uint32_t C) {
 
 bool slab_tasks_fit(const FilmDesc& d, uint32_t C) {
   const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * (d.Ly / slab_rows(d, C)) * d.W;
-  return words <= 0xFFFFu && (uint64_t)d.Lx * d.Ly <= 0xFFFFu && d.W <= 0xFFFFu &&
+  // More words than one turn of drawing threads go to columns, whose draws then
+  // fill the SM anyway and need no masks in shared memory.  Per sweep, tasks /
+  // columns: 576 words per CTA (48x96x64 on eight) 8.0 / 9.1 us, 768 (32x96x64 on
+  // four) 9.9 / 9.1, 1536 (on two) 19.3 / 15.3; 1224 words of two calls (64x153x10
+  // on eight) 7.5 / 8.3.
+  const uint64_t calls = d.W == 1 && slab_rows(d, C) == 1 ? d.last_calls : 8;  // of a word
+  return words * calls <= 8 * kTaskThreads && words <= 0xFFFFu && (uint64_t)d.Lx * d.Ly <= 0xFFFFu && d.W <= 0xFFFFu &&
          slab_task_bytes(d, C) <= kClusterMaxSmem;
 }
 

@@ -205,8 +205,8 @@ constexpr uint32_t kClusterMaxPerSm = 2;
 // slab's columns (slab_shape) over at most kSlabThreads / per_sm threads, or its
 // draw tasks over at most kTaskThreads / per_sm (a multiple of 32).
 uint32_t cluster_threads(const FilmDesc& d, uint32_t C, uint32_t per_sm, bool tasks);
-// Whether the task form's words and masks fit a CTA's shared memory, and the
-// dynamic shared memory of either form.
+// Whether the film takes the task form (its words few enough, and they and the
+// masks fit a CTA's shared memory), and the dynamic shared memory of either form.
 // Both depend on the film's geometry and on table_form.
 bool slab_tasks_fit(const FilmDesc& d, uint32_t C);
 uint32_t slab_dyn_bytes(const FilmDesc& d, uint32_t C, bool tasks);

@@ -46,6 +46,16 @@ def test_launch_holds_the_present_tables(harness, Lx, Ly, Lz, shape):
     assert lines[0] == lines[2] == lines[4] and lines[1] == lines[3]
 
 
+# Words per CTA on both sides of one turn of drawing threads: 576, 768 and 1728 of
+# eight calls, 1224 of two.
+@pytest.mark.parametrize("Lx,Ly,Lz,tasks", [(48, 96, 64, 1), (64, 96, 64, 0), (48, 96, 192, 0), (64, 153, 10, 1)])
+def test_slabs_of_many_words_are_columns(harness, Lx, Ly, Lz, tasks):
+    out = subprocess.run([harness, "slab", str(Lx), str(Ly), str(Lz), str(CLUSTER)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    lines = [dict(zip(l.split()[::2], map(int, l.split()[1::2]))) for l in out.stdout.splitlines()]
+    assert lines and all(l["C"] == 8 and l["tasks"] == tasks for l in lines), out.stdout
+
+
 def test_adds_to_one_sum_have_one_scope():
     """In a cluster a layer's magnetisation gets adds from its own CTA and, in the
     same half-sweep, from the peer that holds the layer's wrap partner.  PTX:
