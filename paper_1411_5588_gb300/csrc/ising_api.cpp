@@ -78,19 +78,19 @@ void fill_geometry(FilmDesc& d, int Lx, int Ly, int Lz, int y_mode, int x_mode, 
   d.active = 1;
   d.sweep_end = 0xFFFFFFFFu;
   fastdiv_magic(d.W, &d.divw_m, &d.divw_l);
-  // thin films: a word of the grid kernels holds 4 (at most 8 sites per array)
-  // or 2 (at most 16) rows; the first and the last group of a layer must
-  // differ.  Two rows pay only on films of at least kPack2Rows rows: packing
-  // halves a film's threads and doubles each one's chain of Philox calls,
-  // which a small film's few waves cannot hide (measured on GB300: the
-  // beta-integration set's films of 1200-3000 rows lose 6%, the line-tension
-  // set's of 13824 rows gain).  On the slab path films pack whenever they can
-  // (slab_rows decides).
+  // thin films: a word of R = 4 (at most 8 sites per array) or 2 (at most 16)
+  // rows; the first and the last group of a layer must differ.  On the slab path
+  // films pack whenever they can (slab_rows decides), in the grid kernels by the
+  // launch they are part of (grid_pack)
   d.sl_pack = 1;
   if (d.W == 1 && d.n <= 8 && d.Ly % 4 == 0 && d.Ly >= 8) d.sl_pack = 4;
   else if (d.W == 1 && d.n <= 16 && d.Ly % 2 == 0 && d.Ly >= 4) d.sl_pack = 2;
-  d.pack = (d.sl_pack == 2 && d.Lx * d.Ly < kPack2Rows) ? 1 : d.sl_pack;
-  const uint32_t groups = d.Ly / d.pack;
+  set_pack(d, d.sl_pack);
+}
+
+void set_pack(FilmDesc& d, uint32_t rows) {
+  d.pack = rows;
+  const uint32_t groups = d.Ly / rows;
   for (uint32_t i = 0; i < 3; i++) {
     const uint32_t len = column_len(i);
     d.cols[i] = (groups - 2 + len - 1) / len;
@@ -160,7 +160,10 @@ int FilmSet::init_device() {
 void FilmSet::layout(bool assign_part) {
   uint32_t ub = 0, mb = 0;
   size_t po = 0;
+  uint64_t words = 0;  // of the lanes' launches, a row each in thin films
+  for (const auto& d : h) words += (uint64_t)d.Lx * d.Ly * d.W * lanes;
   for (auto& d : h) {
+    set_pack(d, grid_pack(d, words));
     d.upd_block_begin = ub;
     d.meas_block_begin = mb;
     if (assign_part) d.part_off = po;

@@ -240,9 +240,9 @@ int lane_direct_sweeps(Lane* b, uint32_t n) {
 
 void lane_destroy(Lane* b);
 
-// A lane of the given films (caller's order within the lane), initial
-// states drawn, descriptors uploaded.
-int lane_create(const std::vector<ising_job>& jobs, Lane** out) {
+// A lane of the given films (caller's order within the lane), one of `lanes`,
+// initial states drawn, descriptors uploaded.
+int lane_create(const std::vector<ising_job>& jobs, uint32_t lanes, Lane** out) {
   *out = nullptr;
   const size_t n = jobs.size();
   Lane* b = new (std::nothrow) Lane();
@@ -251,6 +251,7 @@ int lane_create(const std::vector<ising_job>& jobs, Lane** out) {
   b->rec_written.assign(n, 0);
   b->rec_read.assign(n, 0);
   FilmSet& fs = b->fs;
+  fs.lanes = lanes;
   fs.h.resize(n);
   size_t words = 0, stage = 0;
   for (size_t i = 0; i < n; i++) {
@@ -496,7 +497,7 @@ int batch_create(const ising_job* jobs, size_t n, uint32_t lanes, ising_batch** 
   int rc = ISING_OK;
   for (uint32_t l = 0; !rc && l < lanes; l++) {
     Lane* ln = nullptr;
-    rc = lane_create(per[l], &ln);
+    rc = lane_create(per[l], lanes, &ln);
     if (!rc) b->lanes.push_back(ln);
   }
   if (!rc && cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess) {

@@ -54,6 +54,10 @@ int check_film(int Lx, int Ly, int Lz, double T, int y_mode, int x_mode);
 // Geometry, key and work sizes of a descriptor (no offsets, no tables).
 void fill_geometry(FilmDesc& d, int Lx, int Ly, int Lz, int y_mode, int x_mode, uint64_t seed, uint32_t replica);
 
+// Rows per packed word of the film in the grid kernels (1, 2, 4), and the columns
+// that follow from it.
+void set_pack(FilmDesc& d, uint32_t rows);
+
 // Metropolis thresholds of Eq. 1 for the four row classes (binary64, libm exp).
 void build_tables(FilmDesc& d, double J, double H, double H1, double T);
 
@@ -70,6 +74,7 @@ struct FilmSet {
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   int n_sm = 0, meas_per_sm = 0;
+  uint32_t lanes = 1;  // film sets that run side by side, this one included
   uint32_t items = 1;  // launch shape of the grid update kernels (column_len: 1 one word per thread, 0 two, 2 four)
 
   std::vector<FilmDesc> h;  // host mirror (counters tracked on the host too)

@@ -45,7 +45,8 @@ __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
 // Below it the chain counts, and seven masks drawn ahead are no slower.  Films
 // in a bulk field, per sweep, masks / look-ups: 864 blocks 10.7 / 12.2 us, 1024
 // blocks 12.7 / 12.7, 5625 blocks 68.1 / 45.6.
-constexpr uint32_t kLookBlocks = 8 * 152 + 1;
+constexpr uint32_t kWaveWords = 8 * 152 * kFilmThreads;
+constexpr uint32_t kLookBlocks = kWaveWords / kFilmThreads + 1;
 constexpr int kMeasureBlock = 256;
 
 // Items a measurement block covers per layer before another block is added;
@@ -60,9 +61,23 @@ __host__ __device__ inline uint64_t acc_offset(const FilmDesc& d) {
   return d.part_off + 2ull * d.Lx * d.meas_bpl;
 }
 
-// Films of at least this many rows pack two rows per word when they qualify
-// (fill_geometry); four rows pack at any size.
+// Rows that a thin film packs to a word in launches of `words` words with a row
+// each, side by side.  Packed words are fewer instructions per site, but a chain of all their
+// rows' Philox calls in a fraction of the threads: they pay once the rows fill
+// the GPU for longer than a wave (two and a half for four rows, whose calls are
+// two each), those of the launches beside it included.  Per sweep, a word per row
+// / packed: four rows 65536 rows (128x512x16) 6.3 / 12.4 us, 262144 (256x1024x16)
+// 10.6 / 14.1, 327680 12.0 / 14.4, 524288 17.0 / 14.4, 16 and 32 films of 64x256x16
+// (262144 and 524288) 10.4 / 12.9 and 20.0 / 17.3; two rows 65536 (128x512x32)
+// 6.1 / 9.4, 153600 7.3 / 10.1, 196608 9.0 / 9.2, 262144 12.2 / 10.0.  Two rows only in films of at least
+// kPack2Rows: a set of small ones is bound by its chains (the beta-integration
+// set's films of 1200-3000 rows lose 6% packed, the line-tension set's of 13824
+// gain).
 constexpr uint32_t kPack2Rows = 8192;
+inline uint32_t grid_pack(const FilmDesc& d, uint64_t words) {
+  if (d.sl_pack == 4) return 2 * words > 5 * kWaveWords ? 4u : 1u;
+  return d.sl_pack == 2 && d.Lx * d.Ly >= kPack2Rows && words > kWaveWords ? 2u : 1u;
+}
 
 // Columns of a film in the grid update kernels (of words, or of packed words of
 // `pack` rows): the pairs, then the rows between the first and the last, those

@@ -330,6 +330,7 @@ void ising_server::loop() {
       if (jobs[t].d.sweep_end - jobs[t].d.sweep <= chunk) S.finishing.push_back(t);
     lk.unlock();
     fs2.items = fs.items;
+    fs.lanes = fs2.lanes = fs2.h.empty() ? 1u : 2u;
     fs.layout(false);  // partial sums stay in each job's own arena area
     fs2.layout(false);
     int rc = ensure_capacity(std::max(fs.hh.n_films, fs2.hh.n_films), std::max(fs.hh.upd_blocks, fs2.hh.upd_blocks),

@@ -7,7 +7,8 @@
 //   tune Lx Ly Lz        the shapes AUTO takes: untuned, tuned (every candidate
 //                        taking no time, so that the first one wins), with a bulk
 //                        field, and without it again
-//   film Lx Ly Lz shape H  a sweep of a handle; a line per launch: its form
+//   film Lx Ly Lz shape H  a sweep of a handle; a line per launch: its form, and the
+//                        rows of a packed word
 //   grid items H0 H1 H2  half-sweeps of a set of a small, a medium and a large film
 //                        in those bulk fields; a line per launch: its grid, the
 //                        entries of the owner table, and its form
@@ -66,7 +67,9 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
     return k == std::string::npos ? -1 : atoi(name.c_str() + name.find("EE", k) - 1);
   };
   if (form("update_kernelI") >= 0) printf("grid %u blocks %u form %d\n", c->gridDim.x, g_blocks, form("update_kernelI"));
-  if (form("update_film_kernelI") >= 0) printf("form %d\n", form("update_film_kernelI"));
+  const size_t film = name.find("update_film_kernelILi");
+  if (film != std::string::npos)
+    printf("form %d rows %d\n", form("update_film_kernelI"), atoi(name.c_str() + film + strlen("update_film_kernelILi")));
   const size_t at = name.find("slab_kernelILb");
   if (at == std::string::npos) return cudaSuccess;
   const bool tasks = name[at + strlen("slab_kernelILb1ELb")] == '1';

@@ -119,3 +119,13 @@ def test_sets_look_thresholds_up(harness, items, H, form):
     out = subprocess.run([harness, "grid", str(items)] + [str(h) for h in H], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     assert [int(l.split()[5]) for l in out.stdout.splitlines()] == [form] * 4, out.stdout
+
+
+@pytest.mark.parametrize("Lx,Ly,Lz,rows", [
+    (128, 512, 16, 1), (256, 512, 8, 1), (64, 128, 12, 1), (256, 1024, 16, 1), (512, 1024, 16, 4), (128, 512, 32, 1),
+    (64, 256, 20, 1), (256, 1024, 32, 2), (512, 1024, 24, 2), (512, 1022, 16, 2), (512, 1024, 34, 1)])
+@pytest.mark.parametrize("shape", [2, 3, 4])
+def test_thin_films_pack_where_they_fill_the_gpu(harness, Lx, Ly, Lz, rows, shape):
+    out = subprocess.run([harness, "film", str(Lx), str(Ly), str(Lz), str(shape), "0"], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    assert [int(l.split()[3]) for l in out.stdout.splitlines()] == [rows, rows], out.stdout
