@@ -96,9 +96,12 @@ enum { ISING_INIT_RANDOM = 0, ISING_INIT_SLAB_Y = 1, ISING_INIT_ALL_UP = 2 };
  *           films, each on its own few SMs).
  * AUTO      the autotuner's measurement for this film shape and record
  *           interval if there is one, else RESIDENT up to 1024 spins,
- *           CLUSTER up to 98304 (a film that qualifies for no cluster of two
- *           or more: RESIDENT up to 32768), GRID_1 above, and GRID_Q from
- *           2^18 words per half-sweep up. */
+ *           CLUSTER up to 98304 unless a CTA would hold too many words (films
+ *           of few layers, or of very short rows; a film that qualifies for no
+ *           cluster of two or more: RESIDENT up to 32768), GRID_1 otherwise,
+ *           and GRID_Q above 2^18 words per half-sweep: the best for a film
+ *           that has the GPU to itself (many small films at once belong in a
+ *           batch). */
 enum { ISING_SHAPE_AUTO = 0, ISING_SHAPE_RESIDENT = 1, ISING_SHAPE_GRID_1 = 2, ISING_SHAPE_GRID_2 = 3,
        ISING_SHAPE_GRID_Q = 4, ISING_SHAPE_CLUSTER = 5 };
 

@@ -397,9 +397,9 @@ int sweep_slab(ising* h, const SlabLaunch& l, uint64_t n, uint64_t step) {
 // The launch shape of an ising_sweep call: the pinned one, else the
 // autotuner's choice for this film shape and record interval, else the
 // resident kernel up to kResidentAutoSites spins, a cluster up to
-// kClusterAutoSites, one word per thread above up to kOneWordAutoWords, and
-// columns of two; a film that no cluster takes (one layer) is resident up to
-// kResidentOnlySites.
+// kClusterAutoSites and kClusterAutoWords per CTA, one word per thread above up
+// to kOneWordAutoWords, and columns of two; a film that no cluster of two takes
+// (one layer) is resident up to kResidentOnlySites and as many words.
 int resolve_shape(ising* h, uint32_t measure_every) {
   const FilmDesc& d = h->d();
   if (h->shape != ISING_SHAPE_AUTO) return h->shape;
@@ -409,8 +409,11 @@ int resolve_shape(ising* h, uint32_t measure_every) {
     return s;
   const uint64_t sites = (uint64_t)d.Lx * d.Ly * d.Lz;
   if (sites <= kResidentAutoSites && resident_smem_bytes(d)) return ISING_SHAPE_RESIDENT;
-  if (sites <= kClusterAutoSites && handle_cluster_size(h) > 1) return ISING_SHAPE_CLUSTER;
-  if (sites <= kResidentOnlySites && resident_smem_bytes(d)) return ISING_SHAPE_RESIDENT;
+  const uint64_t words = (measure_every == 1 ? 2 : 1) * kClusterAutoWords;  // of a CTA
+  const uint32_t C = sites <= kClusterAutoSites ? handle_cluster_size(h) : 0;
+  if (C > 1 && slab_work(d, C) <= words) return ISING_SHAPE_CLUSTER;
+  if (C == 1 && sites <= kResidentOnlySites && resident_smem_bytes(d) && slab_work(d, 1) <= words)
+    return ISING_SHAPE_RESIDENT;
   return launch_words(d) <= kOneWordAutoWords ? ISING_SHAPE_GRID_1 : ISING_SHAPE_GRID_Q;
 }
 

@@ -2128,8 +2128,7 @@ bool slab_tasks_fit(const FilmDesc& d, uint32_t C) {
   // columns: 576 words per CTA (48x96x64 on eight) 8.0 / 9.1 us, 768 (32x96x64 on
   // four) 9.9 / 9.1, 1536 (on two) 19.3 / 15.3; 1224 words of two calls (64x153x10
   // on eight) 7.5 / 8.3.
-  const uint64_t calls = d.W == 1 && slab_rows(d, C) == 1 ? d.last_calls : 8;  // of a word
-  return words * calls <= 8 * kTaskThreads && words <= 0xFFFFu && (uint64_t)d.Lx * d.Ly <= 0xFFFFu && d.W <= 0xFFFFu &&
+  return words * slab_calls(d, slab_rows(d, C)) <= 8 * kTaskThreads && words <= 0xFFFFu && (uint64_t)d.Lx * d.Ly <= 0xFFFFu && d.W <= 0xFFFFu &&
          slab_task_bytes(d, C) <= kClusterMaxSmem;
 }
 

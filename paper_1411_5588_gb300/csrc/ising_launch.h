@@ -150,6 +150,20 @@ __host__ __device__ inline uint32_t slab_rows(const FilmDesc& d, uint32_t C) {
   const uint64_t words = (uint64_t)((d.Lx + C - 1) / C) * d.Ly * d.W;
   return words <= 128 ? 1u : d.sl_pack;
 }
+// Philox calls of a word of film d in a slab of R rows per word.
+inline uint32_t slab_calls(const FilmDesc& d, uint32_t R) { return d.W == 1 ? R * d.last_calls : 8u; }
+// Work of a slab's half-sweep in words of eight calls: a word is its calls, and
+// about two more in loads and decisions.  Without a measurement a film takes the
+// slab path up to kClusterAutoWords of them per CTA, and up to twice that with a
+// record every sweep, which costs the grid some 3.4 us and the cluster 0.4.  Per
+// sweep, no records / a record each, cluster / one word per thread: 256
+// (4x128x128) 5.9 / 6.2 and 5.6 / 9.1 us, 384 (3x128x192) 6.5 / 6.8 and 5.3 / 8.8,
+// 490 (64x153x10) 7.5 / 8.0 and 5.2 / 8.4, 512 (2x128x256) 7.6 / 8.0 and 5.2 / 8.7.
+constexpr uint64_t kClusterAutoWords = 256;
+inline uint64_t slab_work(const FilmDesc& d, uint32_t C) {
+  const uint32_t rows = slab_rows(d, C);
+  return (uint64_t)((d.Lx + C - 1) / C) * (d.Ly / rows) * d.W * (slab_calls(d, rows) + 2) / 10;
+}
 // Columns of a slab (the largest of the cluster's) over at most tmax threads:
 // each layer's G groups (words, W of them per group) in equal columns of
 // `len` >= 2 steps, as short as one turn of the threads allows; with more than

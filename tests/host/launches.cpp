@@ -7,6 +7,7 @@
 //   tune Lx Ly Lz        the shapes AUTO takes: untuned, tuned (every candidate
 //                        taking no time, so that the first one wins), with a bulk
 //                        field, and without it again
+//   auto Lx Ly Lz every  the shape AUTO takes without a measurement
 //   film Lx Ly Lz shape H  a sweep of a handle; a line per launch: its form, and the
 //                        rows of a packed word
 //   grid items H0 H1 H2  half-sweeps of a set of a small, a medium and a large film
@@ -143,6 +144,13 @@ int main(int, char** a) {
   }
   ising* h = nullptr;
   ok(ising_create(atoi(a[1]), atoi(a[2]), atoi(a[3]), 1.0, 0.5, 3.0, 1, &h));
+  if (!strcmp(a[0], "auto")) {
+    int s = 0;
+    ok(ising_get_shape(h, (uint32_t)atoi(a[4]), &s));
+    printf("shape %d\n", s);
+    ok(ising_destroy(h));
+    return 0;
+  }
   if (!strcmp(a[0], "tune")) {
     g_quiet = true;
     tune(h);

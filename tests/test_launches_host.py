@@ -32,7 +32,7 @@ AUTO, RESIDENT, CLUSTER = 0, 1, 5
 # Sizes whose need differs between the three- and the seven-mask tables, by less
 # and by more than the launch's padding, and where the task form stops fitting.
 @pytest.mark.parametrize("Lx,Ly,Lz,shape", [
-    (8, 8, 8, AUTO), (24, 601, 4, AUTO), (64, 768, 2, AUTO), (64, 153, 10, AUTO), (41, 47, 34, RESIDENT),
+    (8, 8, 8, AUTO), (24, 601, 4, CLUSTER), (64, 768, 2, CLUSTER), (64, 153, 10, AUTO), (41, 47, 34, RESIDENT),
     (64, 128, 128, CLUSTER), (96, 192, 64, CLUSTER), (16, 150, 130, CLUSTER), (96, 192, 384, CLUSTER)])
 def test_launch_holds_the_present_tables(harness, Lx, Ly, Lz, shape):
     out = subprocess.run([harness, "slab", str(Lx), str(Ly), str(Lz), str(shape)], capture_output=True, text=True)
@@ -129,3 +129,15 @@ def test_thin_films_pack_where_they_fill_the_gpu(harness, Lx, Ly, Lz, rows, shap
     out = subprocess.run([harness, "film", str(Lx), str(Ly), str(Lz), str(shape), "0"], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     assert [int(l.split()[3]) for l in out.stdout.splitlines()] == [rows, rows], out.stdout
+
+
+@pytest.mark.parametrize("Lx,Ly,Lz,every,shape", [
+    (8, 8, 8, 1, RESIDENT), (16, 48, 32, 10, CLUSTER), (32, 48, 64, 0, CLUSTER), (32, 48, 64, 1, CLUSTER),
+    (4, 128, 128, 0, CLUSTER), (2, 128, 256, 0, 2), (2, 128, 256, 10, 2), (2, 128, 256, 1, CLUSTER), (3, 128, 192, 0, 2),
+    (64, 153, 10, 0, 2), (64, 153, 10, 1, CLUSTER), (2, 480, 34, 0, 2), (1, 64, 256, 0, RESIDENT),
+    (400, 30, 8, 0, 2), (400, 30, 8, 1, CLUSTER), (1, 500, 64, 0, 2),
+    (64, 128, 128, 0, 2), (120, 240, 1600, 0, 4)])
+def test_unmeasured_films_take_clusters_of_few_words(harness, Lx, Ly, Lz, every, shape):
+    out = subprocess.run([harness, "auto", str(Lx), str(Ly), str(Lz), str(every)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    assert out.stdout.split() == ["shape", str(shape)]
