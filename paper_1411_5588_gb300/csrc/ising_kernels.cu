@@ -1591,7 +1591,9 @@ __device__ __forceinline__ void slab_tasks(const Slab& s, const FilmDesc& d, con
                                            uint32_t n3, uint32_t* m, uint32_t c, uint32_t t, uint32_t me) {
   constexpr uint32_t B = 8 / R;
   constexpr int D = R == 1 ? 4 : 1;
-  if (4 * n_words > blockDim.x) {
+  // four lanes are the form bound by latency, and the code's main line: the other
+  // way round 8^3 takes 2.326 us per sweep instead of 2.310
+  if (__builtin_expect(4 * n_words > blockDim.x, 0)) {
     for (uint32_t i = me; i < (n_words + 31u & ~31u); i += blockDim.x) {  // whole warps
       const uint32_t n = min(i, n_words - 1), f = words[n].f, rw = words[n].row;
       const bool any7 = __any_sync(0xFFFFFFFFu, n >= n3);
