@@ -538,7 +538,7 @@ def main():
     ap.add_argument("--impl", default="gb300", choices=["gb300", "reference"])
     ap.add_argument("--no-extras", action="store_true", help="skip the batched/serving/e2e/cpu legs")
     ap.add_argument("--serve-jobs", type=int, default=2000)
-    ap.add_argument("--shape", default="auto", choices=["auto", "grid1", "grid2"],
+    ap.add_argument("--shape", default="auto", choices=["auto", "grid1", "grid2", "gridq"],
                     help="launch shape of the 120x240x1600 film (auto: the library's autotuner); profiling "
                          "pins the autotuner's normal pick because ncu's serialisation distorts its timing")
     ap.add_argument("--profile-set", choices=PROFILE_SETS,
@@ -579,7 +579,7 @@ def main():
     if args.shape == "auto":
         code_step, code_kernel = film.autotune(SWEEPS_PER_STEP), film.autotune(0)
     else:
-        code_step = code_kernel = {"grid1": ig.SHAPE_GRID_1, "grid2": ig.SHAPE_GRID_2}[args.shape]
+        code_step = code_kernel = {"grid1": ig.SHAPE_GRID_1, "grid2": ig.SHAPE_GRID_2, "gridq": ig.SHAPE_GRID_Q}[args.shape]
         film.set_shape(code_step)
     shape_step, shape_kernel = SHAPE_NAMES[code_step], SHAPE_NAMES[code_kernel]
     sites = WL.sites(job)

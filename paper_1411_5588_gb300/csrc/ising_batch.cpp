@@ -680,8 +680,8 @@ int ising_batch_autotune(ising_batch* b, int* shape) {
       bool ok = true;
       for (const Lane* l : b->lanes) {
         uint32_t smem = 0, threads = 0;
-              bool tasks = false;
-              ok = ok && lane_cluster_params(l, C, per_sm, &smem, &threads, &tasks) == ISING_OK;
+        bool tasks = false;
+        ok = ok && lane_cluster_params(l, C, per_sm, &smem, &threads, &tasks) == ISING_OK;
       }
       clear_error();
       if (ok) cands.push_back({ISING_SHAPE_CLUSTER, C});

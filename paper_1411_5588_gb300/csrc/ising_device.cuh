@@ -28,8 +28,6 @@ constexpr uint32_t kInitSweep = 0xFFFFFFFFu;
 
 enum : uint32_t { kYGapbc = 0, kYPbc = 1, kYApbc = 2 };
 
-// One film of a launch.  Lives in device memory; counters `sweep` and
-// `rec_next` are advanced by kernels so that captured graphs can be replayed.
 // Acceptance data of one row class, by k = the site's up neighbours (0 .. D):
 // dE of the two spins at one k are each other's negatives, so at most one of
 // the two moves costs energy.  It happens for a word u < t[k], or always
@@ -43,6 +41,8 @@ struct ClassDraw {
   uint32_t pad;
 };
 
+// One film of a launch.  Lives in device memory; counters `sweep` and
+// `rec_next` are advanced by kernels so that captured graphs can be replayed.
 struct FilmDesc {
   uint32_t Lx, Ly, Lz, n, W;   // n = Lz/2 sites per array, W words per array
   uint32_t Wp;                 // row stride in words (= W)

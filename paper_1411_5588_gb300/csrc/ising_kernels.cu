@@ -794,10 +794,11 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
 // the write overlaps the launch's other blocks.  The last block holds the
 // film's ragged end, so it has the fewest words; the first ones hold the pairs.
 //
-// The masks are drawn before pdl_wait, from the film's sweep counter.  Only
-// advance_kernel writes that, between chunks: the first launch of a chunk
-// (`first`) waits before it reads the counter and lets its successor start
-// only then, so every later launch of the chunk starts after the write.
+// The masks are drawn before pdl_wait, from the film's sweep counter.
+// advance_kernel writes that, and slab_store where a lane has swept in shared
+// memory, both between chunks: the first launch of a chunk (`first`) waits
+// before it reads the counter and lets its successor start only then, so every
+// later launch of the chunk starts after the write.
 enum : uint32_t { kUpdPlain = 0, kUpdAccumulate = 1, kUpdWriteRecord = 2 };
 
 __device__ __forceinline__ uint32_t last_update_block(const FilmDesc& d, uint32_t items) {
@@ -1890,10 +1891,11 @@ __global__ void init_kernel(FilmDesc F, uint32_t* __restrict__ pool, int kind, u
 // int8 canonical order <-> packed planes, a thread per word pair: the 64 bytes
 // z0 = 64 w .. 64 w + 63 of a row hold word w of both arrays, site l = 2 k and
 // 2 k + 1 of either in the k-th four of them.  They move in accesses of ALIGN
-// bytes (16, 4 or 1: the largest that divides both the address and Lz), so that
-// a warp reads or writes 2 KiB in one piece; a thread per site, and one per
-// word gathering every other byte, took 0.16 and 0.10 ms for the 46M-site film
-// where its 52 MB take 8 us.
+// bytes (16, 4 or 1: the largest that divides both the address and Lz).  A thread's
+// bytes lie side by side, so a warp's four accesses together cover 2 KiB, and
+// each of them half sectors; pack and unpack of the 46M-site film take 13 to 14 us
+// each where its 52 MB take 8.  A thread per site, and one per word gathering every
+// other byte, took 0.16 and 0.10 ms.
 template <uint32_t ALIGN>
 __device__ __forceinline__ uint32_t four_bytes(const int8_t* p, uint32_t left) {
   if (ALIGN >= 4) return *reinterpret_cast<const uint32_t*>(p);

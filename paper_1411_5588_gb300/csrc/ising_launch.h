@@ -102,9 +102,10 @@ __host__ __device__ inline uint32_t update_blocks(const FilmDesc& d, uint32_t it
 
 // Words a half-sweep's launch updates for film d, and the most for which, without
 // a measurement, a launch takes one word per thread: it is the shorter launch,
-// columns are the higher rate.  Per sweep, one word / columns of two (one film)
-// or of four (a batch's lane): 245760 words 15.7 / 16.5 us, 524288 33.2 / 28.1;
-// lanes of 245760 words 35.2 / 35.8, of 491520 68.1 / 61.7, of 806400 110 / 89.
+// columns are the higher rate.  Per sweep, one word / columns of two (one film):
+// 245760 words 15.7 / 16.6 us, 524288 33.2 / 28.2; one word / columns of four (a
+// batch's two lanes): 122880 words each 18.0 / 23.2, 245760 33.5 / 28.1, 491520
+// 67.3 / 53.7, 806400 110 / 88.  Film sets cross over a little below the line.
 constexpr uint64_t kOneWordAutoWords = 1ull << 18;
 inline uint64_t launch_words(const FilmDesc& d) { return (uint64_t)d.Lx * (d.Ly / d.pack) * d.W; }
 
