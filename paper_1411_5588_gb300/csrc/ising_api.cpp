@@ -219,14 +219,14 @@ uint32_t FilmSet::fin_grid() const { return std::min<uint32_t>(hh.n_films, (uint
 
 int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
   const uint32_t ug = upd_grid(), fg = fin_grid();
-  bool pack = false;
-  uint64_t words = 0, general = 0;
+  uint64_t words = 0, packed = 0, general = 0;
   for (const auto& d : h) {
-    pack = pack || d.pack > 1;
     words += launch_words(d);
+    if (d.pack > 1) packed += launch_words(d);
     if (!table_form(d)) general += launch_words(d);
   }
-  const bool look = 2 * general > words;
+  const bool pack = packed != 0;
+  const uint32_t form = set_form(items, ug, words, packed, general);
   bool prev_meas = false;
   for (uint32_t k = k0; k < k0 + n; k++) {
     bool meas = false;
@@ -238,8 +238,8 @@ int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
       }
     // records: half-sweep 1 accumulates the sums; the next half-sweep 0
     // writes them, or, after the last sweep of the call, a small kernel
-    ISG_CK(launch_update(L, ug, pool, 0, k, items, pack, look, part, rec, false, prev_meas ? k : 0, k == k0, stream));
-    ISG_CK(launch_update(L, ug, pool, 1, k, items, pack, look, part, rec, meas, 0, false, stream));
+    ISG_CK(launch_update(L, ug, pool, 0, k, items, form, pack, part, rec, false, prev_meas ? k : 0, k == k0, stream));
+    ISG_CK(launch_update(L, ug, pool, 1, k, items, form, pack, part, rec, meas, 0, false, stream));
     if (meas && k + 1 == k0 + n) ISG_CK(launch_record(L, fg, part, rec, k + 1, stream));
     prev_meas = meas;
   }

@@ -827,7 +827,7 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
   for (uint32_t i = threadIdx.x; i < kDescWords / 4; i += blockDim.x) dst[i] = src[i];
   __syncthreads();
   if (threadIdx.x == 0) s_d.sweep = __ldcg(&films[f].sweep);  // around L1: an earlier chunk's line may be there
-  if (FORM != kFormWord) fill_look(s_look, s_d.cls);
+  if (FORM == kFormColumnsLook || FORM == kFormWordLook) fill_look(s_look, s_d.cls);
   __syncthreads();
   const uint32_t t = s_d.sweep + k;
   if (!s_d.active || t > s_d.sweep_end || (MODE != kUpdWriteRecord && t >= s_d.sweep_end)) {
@@ -855,9 +855,10 @@ update_kernel(const FilmDesc* __restrict__ films, const uint32_t* __restrict__ o
     else if (PK && s_d.pack == 2) update_word<2, MEAS, LOOK>(s_d, s_look, pool, colour, t, at, meas, acc_of, wait);
     else update_word<1, MEAS, LOOK>(s_d, s_look, pool, colour, t, at, meas, acc_of, wait);
   } else {
-    if (PK && s_d.pack == 4) update_columns<4, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
-    else if (PK && s_d.pack == 2) update_columns<2, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
-    else update_columns<1, MEAS, true>(s_d, c, s_look, at, items, meas, acc_of, wait);
+    constexpr bool LOOK = FORM == kFormColumnsLook;
+    if (PK && s_d.pack == 4) update_columns<4, MEAS, LOOK>(s_d, c, s_look, at, items, meas, acc_of, wait);
+    else if (PK && s_d.pack == 2) update_columns<2, MEAS, LOOK>(s_d, c, s_look, at, items, meas, acc_of, wait);
+    else update_columns<1, MEAS, LOOK>(s_d, c, s_look, at, items, meas, acc_of, wait);
   }
 }
 
@@ -2013,6 +2014,12 @@ auto update_variant(uint32_t mode, bool pack) {
                                    : (pack ? update_kernel<kUpdPlain, true, FORM> : update_kernel<kUpdPlain, false, FORM>);
 }
 
+auto packed_columns_variant(uint32_t mode) {
+  return mode == kUpdAccumulate    ? update_kernel<kUpdAccumulate, true, kFormColumns>
+         : mode == kUpdWriteRecord ? update_kernel<kUpdWriteRecord, true, kFormColumns>
+                                   : update_kernel<kUpdPlain, true, kFormColumns>;
+}
+
 template <bool MEAS, uint32_t FORM>
 auto update_film_variant(uint32_t pack) {
   return pack == 4 ? update_film_kernel<4, MEAS, FORM>
@@ -2027,13 +2034,14 @@ auto update_film_variant(uint32_t pack, bool meas) {
 }  // namespace
 
 cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
-                          uint32_t items, bool pack, bool general, int64_t* part, int64_t* records, bool accumulate,
+                          uint32_t items, uint32_t form, bool pack, int64_t* part, int64_t* records, bool accumulate,
                           uint32_t rec_done, bool first, cudaStream_t st) {
   if (grid == 0) return cudaSuccess;
   const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
-  auto* kern = items != 1                         ? update_variant<kFormColumnsLook>(mode, pack)
-               : general && grid >= kLookBlocks ? update_variant<kFormWordLook>(mode, pack)
-                                                : update_variant<kFormWord>(mode, pack);
+  auto* kern = form == kFormColumns       ? packed_columns_variant(mode)
+               : form == kFormColumnsLook ? update_variant<kFormColumnsLook>(mode, pack)
+               : form == kFormWordLook    ? update_variant<kFormWordLook>(mode, pack)
+                                          : update_variant<kFormWord>(mode, pack);
   return launch_pdl(kern, grid, kFilmThreads, 0, st, (const FilmDesc*)L.films, (const uint32_t*)L.owner_upd,
                     pool, colour, k, items, part, records,
                     mode == kUpdWriteRecord ? rec_done : 0u, first ? 1u : 0u);

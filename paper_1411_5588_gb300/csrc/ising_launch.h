@@ -17,8 +17,8 @@ namespace isg {
 // 12.3 us on 32x96x64.
 //
 // Forms: columns by masks (single films without a bulk field), columns by
-// look-ups (single films in one, and film sets, whose walls would otherwise take
-// seven masks: 320 films of 32x96x64 60.1 us per sweep by masks, 53.7 by look-ups,
+// look-ups (single films in one, and most film sets, whose walls would otherwise
+// take seven masks: 320 films of 32x96x64 60.1 us per sweep by masks, 53.7 by look-ups,
 // in a field 85.7 and 52.8), one word by masks drawn ahead, and one word by
 // look-ups (kLookBlocks).
 //
@@ -47,6 +47,17 @@ __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
 // blocks 12.7 / 12.7, 5625 blocks 68.1 / 45.6.
 constexpr uint32_t kWaveWords = 8 * 152 * kFilmThreads;
 constexpr uint32_t kLookBlocks = kWaveWords / kFilmThreads + 1;
+// Form of a film set's launch: `words` words in all, `packed` of them in packed
+// rows, `general` of films in a bulk field.  In columns, sets of packed films go
+// by masks (40 films of 64x512x32 45.2 us per sweep, by look-ups 51.2; of
+// 128x512x16 55.7 and 57.3), all others by look-ups: blocks by masks beside blocks
+// by look-ups, in sets of thin and thick films, thrash the instruction cache (the
+// line-tension set, 62% packed, 45.7 us by look-ups, 52.5 mixed).
+inline uint32_t set_form(uint32_t items, uint32_t grid, uint64_t words, uint64_t packed, uint64_t general) {
+  const bool look = 2 * general > words;
+  if (items == 1) return look && grid >= kLookBlocks ? kFormWordLook : kFormWord;
+  return !look && 8 * packed > 7 * words ? kFormColumns : kFormColumnsLook;
+}
 constexpr int kMeasureBlock = 256;
 
 // Items a measurement block covers per layer before another block is added;
@@ -194,7 +205,8 @@ struct LaunchSet {
   LaunchHdr* hdr = nullptr;          // sizes
 };
 
-// items: the launch shape, matching the owner table's block size.  Records:
+// items: the launch shape, matching the owner table's block size; form: set_form's
+// (kFormColumns only with pack).  Records:
 // with accumulate (colour 1) the films that record after sweep k add their
 // record sums into their accumulators in part; with rec_done > 0 (colour 0) the
 // films that recorded after rec_done sweeps have that record written into
@@ -203,7 +215,7 @@ struct LaunchSet {
 // (FilmDesc::pack > 1).  first: the chunk's first launch, whose predecessor may
 // still be advancing the films' sweep counters.
 cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uint32_t colour, uint32_t k,
-                          uint32_t items, bool pack, bool general, int64_t* part, int64_t* records, bool accumulate,
+                          uint32_t items, uint32_t form, bool pack, int64_t* part, int64_t* records, bool accumulate,
                           uint32_t rec_done, bool first, cudaStream_t st);
 // One half-sweep of a single film whose descriptor (with `sweep` absolute) is
 // passed by value; acc (colour 1 of a recorded sweep, else null): the film's

@@ -10,6 +10,8 @@
 //   auto Lx Ly Lz every  the shape AUTO takes without a measurement
 //   film Lx Ly Lz shape H  a sweep of a handle; a line per launch: its form, and the
 //                        rows of a packed word
+//   thin items thick H   half-sweeps of eight films of 128x512x16 and, if thick, one
+//                        of 120x240x1600; printed like grid's
 //   grid items H0 H1 H2  half-sweeps of a set of a small, a medium and a large film
 //                        in those bulk fields; a line per launch: its grid, the
 //                        entries of the owner table, and its form
@@ -101,16 +103,19 @@ void ok(int rc) {
   if (rc) { printf("status %d: %s\n", rc, ising_last_error()); exit(1); }
 }
 
-// a small, a medium and a large film: more blocks than the GPU holds at once
-void grids(uint32_t items, char** H) {
+// two sweeps of a film set
+struct Size {
+  int Lx, Ly, Lz;
+  double H;
+};
+void set(uint32_t items, const std::vector<Size>& films) {
   isg::FilmSet fs;
   fs.items = items;
-  fs.h.resize(3);
-  const int L[3][3] = {{4, 6, 8}, {24, 30, 96}, {120, 240, 1600}};
-  for (int i = 0; i < 3; i++) {
+  fs.h.resize(films.size());
+  for (size_t i = 0; i < films.size(); i++) {
     memset(&fs.h[i], 0, sizeof fs.h[i]);
-    isg::fill_geometry(fs.h[i], L[i][0], L[i][1], L[i][2], ISING_Y_GAPBC, ISING_X_FREE, 1, i);
-    isg::build_tables(fs.h[i], 1.0, atof(H[i]), 0.5, 3.0);
+    isg::fill_geometry(fs.h[i], films[i].Lx, films[i].Ly, films[i].Lz, ISING_Y_GAPBC, ISING_X_FREE, 1, (uint32_t)i);
+    isg::build_tables(fs.h[i], 1.0, films[i].H, 0.5, 3.0);
   }
   ok(fs.init_device());
   fs.layout();
@@ -139,7 +144,13 @@ void tune(ising* h) {
 // slab: sweeps at J = 1, H = 0, then J = -1, J = 1, H = 0.3, H = 0
 int main(int, char** a) {
   if (!strcmp(*++a, "grid")) {
-    grids((uint32_t)atoi(a[1]), a + 2);
+    set((uint32_t)atoi(a[1]), {{4, 6, 8, atof(a[2])}, {24, 30, 96, atof(a[3])}, {120, 240, 1600, atof(a[4])}});
+    return 0;
+  }
+  if (!strcmp(*a, "thin")) {
+    std::vector<Size> films(8, Size{128, 512, 16, atof(a[3])});
+    if (atoi(a[2])) films.push_back({120, 240, 1600, 0.0});
+    set((uint32_t)atoi(a[1]), films);
     return 0;
   }
   ising* h = nullptr;

@@ -45,3 +45,20 @@ def test_sets(H, big, shape):
         assert np.array_equal(b.read_series(i), o.sweep(4, 2)), i
         assert np.array_equal(b.get_spins(i), o.get_spins()), i
     b.close()
+
+
+# Sets of packed films alone (columns by masks), some in a bulk field.
+@SHAPES
+def test_packed_sets(shape):
+    sizes = [(391, 1004, 10, 0.0), (5, 28, 2, 0.3), (33, 256, 20, 0.0), (7, 12, 6, -0.2), (32, 260, 30, 0.1)]
+    jobs = [dict(Lx=L[0], Ly=L[1], Lz=L[2], T=2.6, H1=0.4, H=L[3], seed=5, replica=i, init_kind=ig.INIT_RANDOM,
+                 measure_every=1 + i % 2) for i, L in enumerate(sizes)]
+    b = ig.Batch(jobs, lanes=1)
+    b.set_shape(shape)
+    b.sweep(4, False)
+    for i, j in enumerate(jobs):
+        o = O.Film(j["Lx"], j["Ly"], j["Lz"], 1.0, j["H1"], j["T"], j["seed"], H=j["H"], replica=i)
+        o.init(ig.INIT_RANDOM, 0.0)
+        assert np.array_equal(b.read_series(i), o.sweep(4, j["measure_every"])), i
+        assert np.array_equal(b.get_spins(i), o.get_spins()), i
+    b.close()
