@@ -219,14 +219,15 @@ uint32_t FilmSet::fin_grid() const { return std::min<uint32_t>(hh.n_films, (uint
 
 int FilmSet::enqueue_sweeps(uint32_t k0, uint32_t n) {
   const uint32_t ug = upd_grid(), fg = fin_grid();
-  uint64_t words = 0, packed = 0, general = 0;
+  bool pack = false;
+  uint64_t words = 0, brief = 0, general = 0;
   for (const auto& d : h) {
+    pack = pack || d.pack > 1;
     words += launch_words(d);
-    if (d.pack > 1) packed += launch_words(d);
+    if (short_words(d)) brief += launch_words(d);
     if (!table_form(d)) general += launch_words(d);
   }
-  const bool pack = packed != 0;
-  const uint32_t form = set_form(items, ug, words, packed, general);
+  const uint32_t form = set_form(items, ug, words, brief, general);
   bool prev_meas = false;
   for (uint32_t k = k0; k < k0 + n; k++) {
     bool meas = false;

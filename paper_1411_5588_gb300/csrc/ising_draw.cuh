@@ -207,9 +207,12 @@ __device__ __forceinline__ void look_up(uint32_t (&t)[4], const uint32_t* look, 
 
 // The mask [u < t_k] of a word whose counts k are known, class cl: one comparison
 // per site with a looked-up threshold, where the general form compares each site
-// with all seven.  The arguments are draw_masks'; FULL (R = 1): eight calls,
-// straight-line code, so that one pair's look-ups pass under another's draws.
-template <int R, bool FULL>
+// with all seven.  The arguments are draw_masks'.  HOW (R = 1): eight calls in
+// straight-line code, so that one pair's look-ups pass under another's draws; the
+// same with only the word's calls, in branches; or those as a loop, in fewer
+// registers.
+enum : int { kLookLoop, kLookBranches, kLookStraight };
+template <int R, int HOW>
 __device__ __forceinline__ uint32_t draw_looked_up(const Count& k, const uint32_t* look, uint32_t cl, uint32_t row,
                                                    uint32_t X, uint32_t c1, uint32_t ncalls, uint32_t sweep,
                                                    const uint32_t* rk0, const uint32_t* rk1) {
@@ -236,7 +239,7 @@ __device__ __forceinline__ uint32_t draw_looked_up(const Count& k, const uint32_
   const uint32_t y1 = (p1 & 0x33333333u) | ((k.c2 << 1) & 0x44444444u);
   const uint32_t y2 = ((p0 >> 2) & 0x33333333u) | (k.c2 & 0x44444444u);
   const uint32_t y3 = ((p1 >> 2) & 0x33333333u) | ((k.c2 >> 1) & 0x44444444u);
-  if constexpr (R == 1 && FULL) {
+  if constexpr (R == 1 && HOW == kLookStraight) {
     // calls q and q + 4 side by side
     const PhiloxRow3 p(row, sweep, X, rk0, rk1);
     auto two = [&](auto qc, uint32_t y) {
@@ -254,8 +257,8 @@ __device__ __forceinline__ uint32_t draw_looked_up(const Count& k, const uint32_
   } else if constexpr (R == 1) {
     // the same, for a row's only word with fewer than eight calls
     const PhiloxRow3 p(row, sweep, X, rk0, rk1);
-#pragma unroll 1
-    for (uint32_t q = 0; q < 4 && q < ncalls; q++) {
+    auto some = [&](uint32_t q) {
+      if (q >= ncalls) return;
       const uint32_t y = q == 0 ? y0 : q == 1 ? y1 : q == 2 ? y2 : y3;
       uint32_t s = 0;
       look_up(tu, look, ((y << 2) & 0x3C3C3C3Cu) | base);
@@ -268,6 +271,15 @@ __device__ __forceinline__ uint32_t draw_looked_up(const Count& k, const uint32_
       }
       put(s, I0{}, u, tu);
       acc |= s << q;
+    };
+    if constexpr (HOW == kLookBranches) {
+      some(0);
+      some(1);
+      some(2);
+      some(3);
+    } else {
+#pragma unroll 1
+      for (uint32_t q = 0; q < 4; q++) some(q);
     }
   } else {
     // row j's calls q and q + 1 side by side: bits b and b + 1 of a byte

@@ -245,18 +245,23 @@ __device__ __forceinline__ void draw_any(Drawn& o, bool any7, const ClassDraw& c
   }
 }
 
-// The sites of a word that flip, by look-ups.  eight: most words of the film have
-// eight calls, and all then take the straight-line form (a warp with one
-// row's partial last word has full ones too, and what is drawn beyond the
-// row's end is not valid).
-template <int R>
+// The sites of a word that flip, by look-ups.  Words of rows of several take the
+// straight-line form for eight calls, the partial last ones too (their warps
+// have full ones, and what is drawn beyond the row's end is not valid).  So do
+// rows of one partial word, in the grid kernels from five calls up (64 films of
+// 64x128x48, six calls: 28.4 us per sweep, 30.4 as a loop), on slabs from seven (300
+// films of 24x60x40, five calls, on a CTA each: 24.4 us in branches, 27.6 straight
+// and as a loop).
+template <int R, bool SLAB = false>
 __device__ __forceinline__ uint32_t look_and_decide(const Hood& h, const Count& k, const uint32_t* look, uint32_t ci,
                                                     const ClassDraw& cl, uint32_t row, uint32_t X, uint32_t w,
-                                                    uint32_t calls, bool eight, uint32_t sweep, const uint32_t* rk0,
-                                                    const uint32_t* rk1) {
+                                                    uint32_t calls, bool several, uint32_t sweep,
+                                                    const uint32_t* rk0, const uint32_t* rk1) {
   uint32_t m;
-  if (R == 1 && eight) m = draw_looked_up<R, true>(k, look, ci, row, X, 8u * w, 8u, sweep, rk0, rk1);
-  else m = draw_looked_up<R, false>(k, look, ci, row, X, 8u * w, calls, sweep, rk0, rk1);
+  if (R == 1 && (several || calls >= (SLAB ? 7u : 5u)))
+    m = draw_looked_up<R, kLookStraight>(k, look, ci, row, X, 8u * w, 8u, sweep, rk0, rk1);
+  else
+    m = draw_looked_up<R, SLAB ? kLookBranches : kLookLoop>(k, look, ci, row, X, 8u * w, calls, sweep, rk0, rk1);
   return flips_looked_up(h.S, k, m, cl);
 }
 
@@ -434,7 +439,7 @@ __device__ __forceinline__ void update_looked_up(const FilmCtx& c, const uint32_
     const Count k = count_up(h);
     const uint32_t v =
         h.S ^ (look_and_decide<R>(h, k, look, cl, c.cls[cl], (x - 1) * c.Ly + y - 1, (x + y + 1 + c.colour) & 1u, w,
-                                            calls, c.W > 1 || c.last_mask == 0xFFFFFFFFu, c.sweep, c.rk0, c.rk1) & valid);
+                                            calls, c.W > 1, c.sweep, c.rk0, c.rk1) & valid);
     store_rows<R>(c, x, y, w, v);
     if (MEAS && meas) {
       LayerSums q = word_sums(x, k, v, h.z0, valid, bond_slots(x, c.Lx, c.x_pbc));
@@ -765,7 +770,7 @@ __device__ __forceinline__ void update_columns(const FilmDesc& d, const FilmCtx&
       }
       const Count k = count_up(h);
       const uint32_t fl = look_and_decide<R>(h, k, look, ci, cl, row, (kx + n * R + 2 + c.colour) & 1u, w, calls,
-                                                            W > 1 || c.last_mask == 0xFFFFFFFFu, c.sweep, c.rk0, c.rk1);
+                                                            W > 1, c.sweep, c.rk0, c.rk1);
       row += R;
       settle(n, h, k, h.S ^ (fl & valid));
     }
@@ -1433,9 +1438,9 @@ __device__ __forceinline__ void slab_film(FilmDesc* Fg, const FilmDesc& d, uint3
         if (seam) h.yp = (h.yp & ~(valid1 << kSeam)) | (((pv ^ s.neg) & valid1) << kSeam);
         const Count k = count_up(h);
         const uint32_t ci = row_class(kx, s.Lx);
-        const uint32_t fl = look_and_decide<R>(h, k, look, ci, d.cls[ci], (kx - 1) * s.Ly + g * R,
+        const uint32_t fl = look_and_decide<R, true>(h, k, look, ci, d.cls[ci], (kx - 1) * s.Ly + g * R,
                                                      (kx + g * R + 2 + c) & 1u, col.w, col.w + 1 == s.W ? s.last_calls : 8u,
-                                                     s.W > 1 || s.last_mask == 0xFFFFFFFFu, t, d.rk0, d.rk1);
+                                                     s.W > 1, t, d.rk0, d.rk1);
         const uint32_t nv = h.S ^ (fl & valid);
         const uint32_t off = 4 * (c * s.pw + in_layer(g * s.W + col.w, s.lw, 70));
         if (CL && partner) sst<true>(s.lp[kx - 1] + off, nv);
@@ -2014,12 +2019,6 @@ auto update_variant(uint32_t mode, bool pack) {
                                    : (pack ? update_kernel<kUpdPlain, true, FORM> : update_kernel<kUpdPlain, false, FORM>);
 }
 
-auto packed_columns_variant(uint32_t mode) {
-  return mode == kUpdAccumulate    ? update_kernel<kUpdAccumulate, true, kFormColumns>
-         : mode == kUpdWriteRecord ? update_kernel<kUpdWriteRecord, true, kFormColumns>
-                                   : update_kernel<kUpdPlain, true, kFormColumns>;
-}
-
 template <bool MEAS, uint32_t FORM>
 auto update_film_variant(uint32_t pack) {
   return pack == 4 ? update_film_kernel<4, MEAS, FORM>
@@ -2038,7 +2037,7 @@ cudaError_t launch_update(const LaunchSet& L, uint32_t grid, uint32_t* pool, uin
                           uint32_t rec_done, bool first, cudaStream_t st) {
   if (grid == 0) return cudaSuccess;
   const uint32_t mode = accumulate && colour == 1 ? kUpdAccumulate : rec_done && colour == 0 ? kUpdWriteRecord : kUpdPlain;
-  auto* kern = form == kFormColumns       ? packed_columns_variant(mode)
+  auto* kern = form == kFormColumns       ? update_variant<kFormColumns>(mode, pack)
                : form == kFormColumnsLook ? update_variant<kFormColumnsLook>(mode, pack)
                : form == kFormWordLook    ? update_variant<kFormWordLook>(mode, pack)
                                           : update_variant<kFormWord>(mode, pack);

@@ -47,16 +47,20 @@ __host__ __device__ constexpr uint32_t column_len(uint32_t items) {
 // blocks 12.7 / 12.7, 5625 blocks 68.1 / 45.6.
 constexpr uint32_t kWaveWords = 8 * 152 * kFilmThreads;
 constexpr uint32_t kLookBlocks = kWaveWords / kFilmThreads + 1;
-// Form of a film set's launch: `words` words in all, `packed` of them in packed
-// rows, `general` of films in a bulk field.  In columns, sets of packed films go
-// by masks (40 films of 64x512x32 45.2 us per sweep, by look-ups 51.2; of
-// 128x512x16 55.7 and 57.3), all others by look-ups: blocks by masks beside blocks
-// by look-ups, in sets of thin and thick films, thrash the instruction cache (the
-// line-tension set, 62% packed, 45.7 us by look-ups, 52.5 mixed).
-inline uint32_t set_form(uint32_t items, uint32_t grid, uint64_t words, uint64_t packed, uint64_t general) {
+// Whether film d's words are short: rows of one word of at most five calls, packed
+// or not.
+inline bool short_words(const FilmDesc& d) { return d.W == 1 && d.last_calls <= 5; }
+// Form of a film set's launch: `words` words in all, `brief` of them short,
+// `general` of films in a bulk field.  In columns, sets of short words go by masks
+// (40 films of 64x512x32 44.9 us per sweep, by look-ups 51.2; of 128x512x16 55.2 and
+// 57.3; 64 of 64x129x40 24.4 and 28.4), all others by look-ups: blocks by masks
+// beside blocks by look-ups, in sets of thin and thick films, thrash the
+// instruction cache (the line-tension set, 62% short, 45.7 us by look-ups, 52.5
+// mixed).
+inline uint32_t set_form(uint32_t items, uint32_t grid, uint64_t words, uint64_t brief, uint64_t general) {
   const bool look = 2 * general > words;
   if (items == 1) return look && grid >= kLookBlocks ? kFormWordLook : kFormWord;
-  return !look && 8 * packed > 7 * words ? kFormColumns : kFormColumnsLook;
+  return !look && 8 * brief > 7 * words ? kFormColumns : kFormColumnsLook;
 }
 constexpr int kMeasureBlock = 256;
 
@@ -205,8 +209,8 @@ struct LaunchSet {
   LaunchHdr* hdr = nullptr;          // sizes
 };
 
-// items: the launch shape, matching the owner table's block size; form: set_form's
-// (kFormColumns only with pack).  Records:
+// items: the launch shape, matching the owner table's block size; form: set_form's.
+// Records:
 // with accumulate (colour 1) the films that record after sweep k add their
 // record sums into their accumulators in part; with rec_done > 0 (colour 0) the
 // films that recorded after rec_done sweeps have that record written into

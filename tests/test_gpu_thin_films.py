@@ -47,10 +47,12 @@ def test_sets(H, big, shape):
     b.close()
 
 
-# Sets of packed films alone (columns by masks), some in a bulk field.
+# Sets of short words alone (columns by masks), packed and not, some in a bulk field.
 @SHAPES
-def test_packed_sets(shape):
-    sizes = [(391, 1004, 10, 0.0), (5, 28, 2, 0.3), (33, 256, 20, 0.0), (7, 12, 6, -0.2), (32, 260, 30, 0.1)]
+@pytest.mark.parametrize("sizes", [
+    [(391, 1004, 10, 0.0), (5, 28, 2, 0.3), (33, 256, 20, 0.0), (7, 12, 6, -0.2), (32, 260, 30, 0.1)],
+    [(24, 61, 40, 0.0), (7, 13, 34, 0.3), (12, 31, 20, 0.0), (3, 2, 2, 0.0), (9, 47, 38, 0.0)]], ids=["packed", "rows"])
+def test_sets_of_short_words(sizes, shape):
     jobs = [dict(Lx=L[0], Ly=L[1], Lz=L[2], T=2.6, H1=0.4, H=L[3], seed=5, replica=i, init_kind=ig.INIT_RANDOM,
                  measure_every=1 + i % 2) for i, L in enumerate(sizes)]
     b = ig.Batch(jobs, lanes=1)

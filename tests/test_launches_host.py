@@ -145,7 +145,7 @@ def test_unmeasured_films_take_clusters_of_few_words(harness, Lx, Ly, Lz, every,
 
 @pytest.mark.parametrize("items,thick,H,form", [(0, 0, 0, MASKS), (2, 0, 0, MASKS), (0, 1, 0, COLUMNS_LOOK),
                                                 (0, 0, 0.2, COLUMNS_LOOK), (1, 0, 0, WORD)])
-def test_sets_of_packed_films_go_by_masks(harness, items, thick, H, form):
+def test_sets_of_short_words_go_by_masks(harness, items, thick, H, form):
     out = subprocess.run([harness, "thin", str(items), str(thick), str(H)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     assert [int(l.split()[5]) for l in out.stdout.splitlines()] == [form] * 4, out.stdout
