@@ -160,10 +160,10 @@ int FilmSet::init_device() {
 void FilmSet::layout(bool assign_part) {
   uint32_t ub = 0, mb = 0;
   size_t po = 0;
-  uint64_t words = 0;  // of the lanes' launches, a row each in thin films
-  for (const auto& d : h) words += (uint64_t)d.Lx * d.Ly * d.W * lanes;
+  uint64_t work = 0;  // of the lanes' launches
+  for (const auto& d : h) work += row_work(d) * lanes;
   for (auto& d : h) {
-    set_pack(d, grid_pack(d, words));
+    set_pack(d, grid_pack(d, work));
     d.upd_block_begin = ub;
     d.meas_block_begin = mb;
     if (assign_part) d.part_off = po;

@@ -76,22 +76,28 @@ __host__ __device__ inline uint64_t acc_offset(const FilmDesc& d) {
   return d.part_off + 2ull * d.Lx * d.meas_bpl;
 }
 
-// Rows that a thin film packs to a word in launches of `words` words with a row
-// each, side by side.  Packed words are fewer instructions per site, but a chain of all their
-// rows' Philox calls in a fraction of the threads: they pay once the rows fill
-// the GPU for longer than a wave (two and a half for four rows, whose calls are
-// two each), those of the launches beside it included.  Per sweep, a word per row
-// / packed: four rows 65536 rows (128x512x16) 6.3 / 12.4 us, 262144 (256x1024x16)
-// 10.6 / 14.1, 327680 12.0 / 14.4, 524288 17.0 / 14.4, 16 and 32 films of 64x256x16
-// (262144 and 524288) 10.4 / 12.9 and 20.0 / 17.3; two rows 65536 (128x512x32)
-// 6.1 / 9.4, 153600 7.3 / 10.1, 196608 9.0 / 9.2, 262144 12.2 / 10.0.  Two rows only in films of at least
-// kPack2Rows: a set of small ones is bound by its chains (the beta-integration
-// set's films of 1200-3000 rows lose 6% packed, the line-tension set's of 13824
-// gain).
+// Work of a half-sweep of film d with a row per word, in words of eight calls (a
+// word is its Philox calls, and about two more in loads and decisions).
+inline uint64_t row_work(const FilmDesc& d) {
+  return (uint64_t)d.Lx * d.Ly * d.W * ((d.W == 1 ? d.last_calls : 8u) + 2) / 10;
+}
+// Rows that a thin film packs to a word in launches of `work` words of eight calls
+// (row_work of all their films), side by side.  Packed words are fewer
+// instructions per site, but a chain of all their rows' calls in a fraction of
+// the threads: they pay once the work fills the GPU for a wave (four rows), or
+// three fifths of one (two).  Per sweep, a word per row / packed: four rows 65536
+// rows (128x512x16, 0.17 waves) 6.3 / 12.4 us, 262144 (256x1024x16, 0.67) 10.6 /
+// 14.1, 327680 (0.84) 12.0 / 14.4, 524288 (1.35) 17.0 / 14.4, 16 and 32 films of
+// 64x256x16 (0.67 and 1.35) 10.4 / 12.9 and 20.0 / 17.3, twenty films of the
+// line-tension set (1.08) 25.6 / 19.8; two rows 65536 (128x512x32, 0.25) 6.1 / 9.4,
+// 153600 (0.59) 7.3 / 10.1, 196608 (0.76) 9.0 / 9.2, 262144 (1.01) 12.2 / 10.0.  Two
+// rows only in films of at least kPack2Rows: a set of small ones is bound by its
+// chains (the beta-integration set's films of 1200-3000 rows lose 6% packed, the
+// line-tension set's of 13824 gain).
 constexpr uint32_t kPack2Rows = 8192;
-inline uint32_t grid_pack(const FilmDesc& d, uint64_t words) {
-  if (d.sl_pack == 4) return 2 * words > 5 * kWaveWords ? 4u : 1u;
-  return d.sl_pack == 2 && d.Lx * d.Ly >= kPack2Rows && words > kWaveWords ? 2u : 1u;
+inline uint32_t grid_pack(const FilmDesc& d, uint64_t work) {
+  if (d.sl_pack == 4) return work > kWaveWords ? 4u : 1u;
+  return d.sl_pack == 2 && d.Lx * d.Ly >= kPack2Rows && 5 * work > 3 * kWaveWords ? 2u : 1u;
 }
 
 // Columns of a film in the grid update kernels (of words, or of packed words of

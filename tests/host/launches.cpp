@@ -12,6 +12,8 @@
 //                        rows of a packed word
 //   thin items thick H   half-sweeps of eight films of 128x512x16 and, if thick, one
 //                        of 120x240x1600; printed like grid's
+//   pack n               the rows per word of n of each of the line-tension set's
+//                        sizes in one set
 //   grid items H0 H1 H2  half-sweeps of a set of a small, a medium and a large film
 //                        in those bulk fields; a line per launch: its grid, the
 //                        entries of the owner table, and its form
@@ -121,6 +123,8 @@ void set(uint32_t items, const std::vector<Size>& films) {
   fs.layout();
   ok(fs.upload());
   g_blocks = fs.hh.upd_blocks;
+  if (g_quiet)
+    for (const auto& d : fs.h) printf("rows %u\n", d.pack);
   ok(fs.enqueue_sweeps(0, 2));
 }
 
@@ -145,6 +149,14 @@ void tune(ising* h) {
 int main(int, char** a) {
   if (!strcmp(*++a, "grid")) {
     set((uint32_t)atoi(a[1]), {{4, 6, 8, atof(a[2])}, {24, 30, 96, atof(a[3])}, {120, 240, 1600, atof(a[4])}});
+    return 0;
+  }
+  if (!strcmp(*a, "pack")) {
+    std::vector<Size> films;
+    for (int i = 0; i < atoi(a[1]); i++)
+      for (int z : {16, 32, 48, 64, 96}) films.push_back({1536 / z, 9216 / z, z, 0.0});
+    g_quiet = true;
+    set(1, films);
     return 0;
   }
   if (!strcmp(*a, "thin")) {

@@ -149,3 +149,12 @@ def test_sets_of_short_words_go_by_masks(harness, items, thick, H, form):
     out = subprocess.run([harness, "thin", str(items), str(thick), str(H)], capture_output=True, text=True)
     assert out.returncode == 0, out.stdout + out.stderr
     assert [int(l.split()[5]) for l in out.stdout.splitlines()] == [form] * 4, out.stdout
+
+
+@pytest.mark.parametrize("n,rows", [(1, [1, 1, 1, 1, 1]), (3, [1, 2, 1, 1, 1]), (4, [4, 2, 1, 1, 1]), (16, [4, 2, 1, 1, 1])])
+def test_sets_of_thin_and_thick_films_pack_by_their_work(harness, n, rows):
+    """The thick films' words are eight calls each, the thinnest's two: a set fills
+    the GPU by its calls, not by its words."""
+    out = subprocess.run([harness, "pack", str(n)], capture_output=True, text=True)
+    assert out.returncode == 0, out.stdout + out.stderr
+    assert [int(l.split()[1]) for l in out.stdout.splitlines()] == rows * n, out.stdout
